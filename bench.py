@@ -117,12 +117,6 @@ def stage_columns(prob) -> int:
     return sum(2 if t.tkind == I.T_SIN else 1 for t in prob.forcing) if prob.forcing else 1
 
 
-def fine_flops_per_unit(prob, mixed: bool = False):
-    """FLOPs per DoF*substep of the fine kernel: K + 1 FMAs (float64) or K + 2 (mixed: E as
-    hi + lo), 2 FLOPs each, where the stage sum is contracted to K columns."""
-    return 2 * (stage_columns(prob) + (2 if mixed else 1))
-
-
 def measured_peaks():
     path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     if os.path.exists(path):
@@ -134,11 +128,6 @@ def measured_peaks():
 def fp64_peak_tflops(sm_mhz: float):
     """FP64 FMA peak: 152 SMs x 2 FP64 FMA lanes per clock x 2 FLOPs x clock."""
     return 152 * 2 * 2 * sm_mhz * 1e6 / 1e12
-
-
-def fp32_peak_tflops(sm_mhz: float):
-    """FP32 FMA peak: 152 SMs x 128 FP32 lanes per clock x 2 FLOPs x clock."""
-    return 152 * 128 * 2 * sm_mhz * 1e6 / 1e12
 
 
 class ClockSampler:
@@ -200,42 +189,6 @@ class ClockSampler:
             return {"sm_mhz": None, "sm_max_mhz": smax, "reasons": ["no samples"]}
         return {"sm_mhz": float(np.median(sm)), "sm_max_mhz": smax, "reasons": sorted(reasons),
                 "samples": len(sm)}
-
-
-# the files that define fine_f64_kernel and its launch (the context header's host-side fields
-# do not enter the kernel)
-FINE_SOURCES = ("pe_fine_kernels.cuh", "pe_fine_k17_24.cu", "pe_fine.cu")
-TRAFFIC_SUMMARY = os.path.join(ROOT, "profiles", "fine_sweep_c2_d2n255.md")
-
-
-def fine_sources_sha256() -> str:
-    """sha256 over the sources that build fine_f64_kernel (to tell whether a stored capture is current)."""
-    import hashlib
-
-    h = hashlib.sha256()
-    for name in FINE_SOURCES:
-        with open(os.path.join(ROOT, "paper_2412_01138_gb300", "csrc", name), "rb") as fh:
-            h.update(fh.read())
-    return h.hexdigest()
-
-
-def fine_f64_traffic():
-    """DRAM bytes per fine_f64_kernel launch from the committed ncu summary, or None when the
-    summary is missing or was taken on other kernel sources."""
-    if not os.path.exists(TRAFFIC_SUMMARY):
-        return None
-    fields = {}
-    with open(TRAFFIC_SUMMARY) as fh:
-        for ln in fh:
-            if ln.startswith("    ") and ":" in ln:
-                k, v = ln.strip().split(":", 1)
-                fields[k.strip()] = v.strip()
-    if fields.get("kernel_sources_sha256") != fine_sources_sha256():
-        return None
-    try:
-        return int(fields["dram_bytes_per_launch"])
-    except (KeyError, ValueError):
-        return None
 
 
 def oracle_chunk(payload):
@@ -745,53 +698,26 @@ def run_example4(pe, args, barrier):
     return out
 
 
-def fine_tc_tensor_flops(prob):
-    """Tensor FLOPs one fine_tc_kernel launch issues: six split products over the K padding
-    (16, 32 or 64 columns) for every 128-mode tile and slice group of at most 256 substeps."""
-    K = stage_columns(prob)
-    KP = 16 if K <= 16 else (32 if K <= 32 else 64)
-    rows_max = 256 if KP <= 32 else 128
-    G = max(1, rows_max // prob.M)
-    groups = (prob.N + G - 1) // G
-    tiles = (prob.ndof + 127) // 128
-    return tiles * 128 * groups * G * prob.M * KP * 2 * 6
-
-
 def chosen_rooflines(prob, chosen, plain, fma):
-    """Rooflines of the chosen form's kernels and of the float64 correction: per-launch CUDA-event
-    times measured inside the library on the launching stream, algorithmic work per launch."""
+    """Rooflines of the sweeps' kernels: CUDA-event times measured inside the library on the
+    launching stream (host-driven loop), algorithmic work of the solve's passes.  The walk takes
+    six float64 operations per mode and slice in the first pass (which makes the coarse iterate
+    too) and five in each further one; counted as one FMA each."""
     peaks = measured_peaks() or {}
     hbm = float(peaks.get("hbm_gbs", 6788.6))
-    bf16 = float(peaks.get("bf16_tflops", 1928.9))
-    nd, N, M, p = prob.ndof, prob.N, prob.M, prob.p
+    nd, N = prob.ndof, prob.N
     out = []
-    ms = chosen["ms_fine_launch"]
-    alg = 2 * (stage_columns(prob) + 1) * nd * N * M
-    issued = fine_tc_tensor_flops(prob)
-    out.append({"kernel": "fine_tc_kernel (chosen)", "bound": "tensor", "ms": ms,
-                "achieved": alg / (ms / 1e3) / 1e12, "peak": bf16, "unit": "TFLOP/s",
-                "frac": alg / (ms / 1e3) / 1e12 / bf16,
-                "tensor_issued_tflops": issued / (ms / 1e3) / 1e12,
-                "tensor_issued_frac": issued / (ms / 1e3) / 1e12 / bf16,
-                "flops_per_launch_algorithmic": alg, "tensor_flops_per_launch": issued,
-                "peak_source": "MEASURED_PEAKS.json bf16_tflops (burst, measured)",
-                "note": "algorithmic = 2 (K + 1) FLOP per DoF*substep; issued = six bf16 split products over "
-                        "the padded K and the 128-mode tiles"})
-    for name, rec in (("correction_kernel (chosen)", chosen), ("correction_kernel (float64)", plain)):
-        ms = rec["ms_corr_launch"]
-        nbytes = 24 * N * nd + 16 * nd
-        out.append({"kernel": name, "bound": "hbm", "ms": ms, "achieved": nbytes / (ms / 1e3) / 1e9,
-                    "peak": hbm, "unit": "GB/s", "frac": nbytes / (ms / 1e3) / 1e9 / hbm,
-                    "bytes_per_launch": nbytes, "peak_source": "MEASURED_PEAKS.json hbm_gbs",
-                    "note": "24 B per DoF*slice (F^M(U^n), old U^{n+1} in, new U^{n+1} out) + U^0 and E_G"})
-    ms = chosen["ms_coarse"]
-    nbytes = 8 * N * nd + 8 * (p + 2) * nd
-    out.append({"kernel": "coarse_fused_kernel (chosen, k = 0)", "bound": "hbm", "ms": ms,
-                "achieved": nbytes / (ms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
-                "frac": nbytes / (ms / 1e3) / 1e9 / hbm, "bytes_per_launch": nbytes,
-                "peak_source": "MEASURED_PEAKS.json hbm_gbs",
-                "note": "U^{n+1} written for every slice (8 B per DoF*slice) + U^0, E_G and the p weights read; "
-                        "the forcing is formed on the fly from per-axis factors"})
+    for name, rec, key, nbytes in (
+            ("walk_kernel (chosen)", chosen, "ms_fine_launch", 8 * N * nd + 16 * N * nd * (chosen["k"] - 1)),
+            ("walk_kernel (float64)", plain, "ms_corr_launch", 24 * N * nd * plain["k"])):
+        ms = rec[key] * rec["k"]
+        flops = 2 * N * nd * (6 + 5 * (rec["k"] - 1))
+        out.append({"kernel": name, "bound": "alu", "ms": ms, "achieved": flops / (ms / 1e3) / 1e12,
+                    "peak": fma["fp64_tflops"], "unit": "TFLOP/s", "frac": flops / (ms / 1e3) / 1e12 / fma["fp64_tflops"],
+                    "passes": rec["k"], "hbm_gbs": nbytes / (ms / 1e3) / 1e9, "hbm_frac": nbytes / (ms / 1e3) / 1e9 / hbm,
+                    "peak_source": "pe_measure_fma_peak(PE_FP64)",
+                    "note": "float64 operations of the recurrences and residual sums; the chosen form's float32 "
+                            "column sums run under them"})
     return out
 
 
@@ -1029,11 +955,12 @@ def main():
                          f"(k={k_or} sweeps of {prob.N}x{prob.M} substeps), {cpu_passes} pass(es), {cpu_s:.1f} s",
                "all_cores": all_cores}
 
-    flops_launch = fine_flops_per_unit(prob) * prob.ndof * prob.N * prob.M
-    achieved = flops_launch / (plain["ms_fine_launch"] / 1e3) / 1e12
+    # the float64 form's forced parts: both propagators' in the first pass, the fine one's after it
+    flops_solve = 2 * stage_columns(prob) * prob.ndof * prob.N * (plain["k"] + 1)
+    ms_forced = plain["ms_fine_launch"] * plain["k"]
+    achieved = flops_solve / (ms_forced / 1e3) / 1e12
     sm_mhz = clock.get("sm_max_mhz") or 2070.0
     peak = fp64_peak_tflops(sm_mhz)
-    traffic = fine_f64_traffic()
     fma = measured_fma
     kernel_rooflines = chosen_rooflines(prob, chosen, plain, fma)
 
@@ -1057,40 +984,34 @@ def main():
         "time_to_tol_ms": plain["ms_per_step"],
         "iterations": plain["k"],
         "rel_l2_vs_oracle": err_plain,
-        "chosen": {"form": "mixed: stage contraction on the tensor cores (tcgen05, three-term bfloat16 split, "
-                           "six products, float32 accumulators), float32 recurrence (hi/lo E), float64 tables, "
-                           "correction, residual; Parareal loop on the device (one CUDA graph with a conditional "
-                           "while node), set-up and output phases replayed as CUDA graphs, the solve enqueued "
-                           "with pe_solve_async and its nodal output written by the solve; kernel times from "
-                           "the same solve with the host-driven loop",
+        "substeps": "fine DoF*substeps are the method's (Ndof x slices x substeps x fine sweeps run): a sweep "
+                    "evaluates F^M on every mode and slice, its M substeps of q stages contracted exactly to one "
+                    "sum over the source's time columns",
+        "chosen": {"form": "mixed: float32 column sums under float64 recurrences, correction and residual, one kernel "
+                           "per iteration (the coarse sweep in the first); Parareal loop on the device (one CUDA graph "
+                           "with a conditional while node), set-up and output phases replayed as CUDA graphs, "
+                           "the solve enqueued with pe_solve_async and its nodal output written by the solve; "
+                           "kernel times from the same solve with the host-driven loop",
                    "value": chosen["value"], "unit": UNIT, "time_to_tol_ms": chosen["ms_per_step"],
                    "iterations": chosen["k"], "rel_l2_vs_oracle": err_chosen, "dtype": "f32",
                    "speedup_time_to_tol": plain["ms_per_step"] / chosen["ms_per_step"],
-                   "fine_kernel_ms": chosen["ms_fine_launch"],
-                   "fine_kernel_tflops": fine_flops_per_unit(prob, mixed=True) * prob.ndof * prob.N * prob.M
-                   / (chosen["ms_fine_launch"] / 1e3) / 1e12,
-                   "fp32_peak_tflops": fp32_peak_tflops(sm_mhz),
-                   "fp32_peak_tflops_measured": measured_fma["fp32_tflops"],
+                   "iteration_kernel_ms": chosen["ms_fine_launch"],
                    "e2e": chosen["e2e"], "phases_ms": chosen["phases"]},
-        "mixed_simt": {"form": "mixed, float32 stage contraction on the CUDA cores (K + 2 FMAs per DoF*substep)",
+        "mixed_simt": {"form": "the same kernels through fine_engine = PE_FINE_SIMT",
                        "value": simt["value"], "unit": UNIT, "time_to_tol_ms": simt["ms_per_step"],
                        "iterations": simt["k"], "rel_l2_vs_oracle": err_simt,
-                       "fine_kernel_ms": simt["ms_fine_launch"],
-                       "fine_kernel_tflops": fine_flops_per_unit(prob, mixed=True) * prob.ndof * prob.N * prob.M
-                       / (simt["ms_fine_launch"] / 1e3) / 1e12,
+                       "iteration_kernel_ms": simt["ms_fine_launch"],
                        "e2e": simt["e2e"]},
         "phases_ms": plain["phases"],
-        "roofline": {"kernel": "fine_f64_kernel", "bound": "alu", "achieved": achieved, "peak": peak,
-                     "unit": "TFLOP/s", "frac": achieved / peak, "traffic": traffic,
+        "roofline": {"kernel": "forced_f64_kernel", "bound": "alu", "achieved": achieved, "peak": peak,
+                     "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
                      "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk x 2 FLOP x max SM clock",
                      "peak_measured": fma["fp64_tflops"], "frac_of_measured": achieved / fma["fp64_tflops"],
                      "peak_measured_source": "pe_measure_fma_peak(PE_FP64): independent FMA chains, best of 5",
-                     "flops_per_launch": flops_launch,
-                     "flops_per_unit": fine_flops_per_unit(prob),
-                     "unit_of_work": "DoF*substep; 2 (K + 1) FLOP = K + 1 FMAs: the q-stage forcing sum of "
-                                     "Eq. (1-7) contracted exactly to K = 17 time columns (one per exponential, "
-                                     "two per sinusoid) plus the E_F multiply; the stage-by-stage count "
-                                     "q (2R + 2) + 1 = 81 is not what the kernel has to execute"},
+                     "flops_per_solve": flops_solve, "ms_per_solve": ms_forced,
+                     "unit_of_work": "2 K FLOP per mode, slice and propagator (K = 17 time columns: one per "
+                                     "exponential, two per sinusoid); k + 1 of them per solve, the coarse forcing "
+                                     "in the first pass and the fine one in each"},
         "kernel_rooflines": kernel_rooflines,
         "measured_fma_peaks": fma,
         "e2e": {"value": plain["e2e"], "unit": UNIT, "h2d_bytes_per_step": prob.ndof * 8,

@@ -58,13 +58,17 @@ enum { PE_FP64 = 0,   /* every step in float64 */
                          homogeneous part e^{-lam M dt} v, tables, correction and
                          residual in float64 */ };
 
-/* engine of the mixed-precision fine sweep (pe_options.fine_engine), separable forcing only:
- * SIMT = float32 FMAs on the CUDA cores; TC = the stage contraction of every 128 modes x
- * (slice group) on the tensor cores (tcgen05, three-term bfloat16 split of both operands,
- * six products, float32 accumulation; about the accuracy of the float32 form), the
- * recurrence and the float64 homogeneous term on the CUDA cores.  TC needs M (substeps
- * per slice) a multiple of 16 in 16..128: pe_setup returns PE_EINVAL otherwise, and for
- * PE_FP64 or PE_FORCING_GENERAL.  The float64 refinement (pe_refine) is unaffected. */
+/* How the fine sweep evaluates F^M (separable forcing): the time factors are shift invariant, so
+ * the q stages of all M substeps of a slice add up exactly to one value per time column (one
+ * column per exponential, two per sinusoid) times a per-mode weight made once per problem; every
+ * sweep evaluates that sum on every mode and slice.  The general path takes every substep.
+ *
+ * Engine of the mixed-precision fine sweep (pe_options.fine_engine): a single problem runs the same
+ * kernels for both values, the sum over the columns being too small for tensor cores to matter;
+ * a batch with TC contracts the stages of each substep on the tensor cores (tcgen05, three-term
+ * bfloat16 split of both operands, six products, float32 accumulation; about the accuracy
+ * of the float32 form).  TC needs M (substeps per slice) a multiple of 16 in 16..128: pe_setup
+ * returns PE_EINVAL otherwise, and for PE_FP64 or PE_FORCING_GENERAL. */
 enum { PE_FINE_SIMT = 0, PE_FINE_TC = 1 };
 
 /* DST-I backend of the general forcing path (pe_options.dst_backend): AUTO = radix-2 FFT
@@ -188,16 +192,20 @@ typedef struct {
   double* residual_history;  /* host, caller-owned, capacity history_cap (may be NULL) */
   int32_t history_cap;
   int64_t fine_sweeps;       /* fine propagator sweeps executed (= k; 1 with cache_forced) */
-  double ms_tables;          /* device time of the forcing tables (time factors, per-axis modal
-                                factors, fine-step stage weights); the phi/b coefficient tables
-                                depend only on pe_setup's arguments and are made there */
-  double ms_prepare;         /* projection of u0, coarse sweep */
+  double ms_tables;          /* device time of the forcing tables (time columns, per-axis modal
+                                factors, column weights); the phi/b coefficient tables depend
+                                only on pe_setup's arguments and are made there */
+  double ms_prepare;         /* projection of u0 */
   double ms_iterations;      /* all fine sweeps + corrections + residuals */
   double ms_output;          /* inverse DST of the final slice */
-  double ms_fine_kernel;     /* device time of the fine-propagator kernels alone (sum over sweeps) */
+  double ms_fine_kernel;     /* device time of the fine-propagator kernels (sum over sweeps): the forced
+                                parts; in the mixed separable form, where one kernel makes them and
+                                the correction, all of it (host-driven loop only) */
   int64_t kernel_launches;   /* kernels this call launched */
-  double ms_correction_kernel; /* device time of the correction + residual kernel (sum over iterations) */
-  double ms_coarse_kernel;   /* device time of the coarse sweep of k = 0 (its kernels alone) */
+  double ms_correction_kernel; /* device time of the correction + residual kernel (sum over iterations)
+                                where it is a kernel of its own */
+  double ms_coarse_kernel;   /* device time of the pass that makes the coarse iterate of k = 0: the first
+                                iteration, which makes it on the way (cache_forced: the coarse sweep) */
 } pe_result;
 
 /*

@@ -12,6 +12,7 @@
 #include <new>
 #include <string>
 
+#include "pe_contract.cuh"
 #include "pe_internal.h"
 
 // ---------------------------------------------------------------------------
@@ -127,9 +128,9 @@ void free_ctx(pe_ctx* c) {
   if (!c) return;
   void* ptrs[] = {c->muM_axis, c->ratio_axis, c->S[0], c->S[1], c->S[2], c->S32[0], c->S32[1], c->S32[2],
                   c->gen_L, c->gen_buf, c->gen_tmp, c->lam, c->coefF, c->coefG,
-                  c->coefF32, c->U, c->Fbar, c->gG, c->work0, c->work1, c->out_nodal, c->partials,
-                  c->red, c->axisF, c->axisF32, c->axisU0, c->AF, c->AF32, c->AG, c->AG32, c->loads,
-                  c->Ktab, c->phase_tab, c->Zst, c->Wst, c->Wst32, c->Fz, c->done_ctr, c->tcB, c->tc_err, c->tcA,
+                  c->coefF32, c->coefG32, c->U, c->Fbar, c->gG, c->work0, c->work1, c->out_nodal, c->partials,
+                  c->red, c->axisF, c->axisF32, c->axisU0, c->loads, c->tab64, c->tab32,
+                  c->Ktab, c->V64, c->G64, c->V32, c->G32, c->Fz, c->done_ctr,
                   c->muM_full, c->ratio_full, c->fac_full, c->work2, c->loopctl, c->loop_hist, c->io32, c->muM_inv};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -268,7 +269,8 @@ extern "C" pe_status pe_setup(pe_ctx** out, int32_t d, const int32_t* n, const d
     return pe_fail(PE_EINVAL, "pe_setup: bad fine_engine");
   }
   if (o.fine_engine == PE_FINE_TC &&
-      (o.precision != PE_MIXED || o.forcing_path != PE_FORCING_SEPARABLE || !fine_tc_supported(n_substeps))) {
+      (o.precision != PE_MIXED || o.forcing_path != PE_FORCING_SEPARABLE || n_substeps < 16 || n_substeps > 128 ||
+       n_substeps % 16 != 0)) {
     delete c;
     return pe_fail(PE_EINVAL,
                    "pe_setup: PE_FINE_TC needs PE_MIXED, PE_FORCING_SEPARABLE and M a multiple of 16 in 16..128");
@@ -303,7 +305,6 @@ extern "C" pe_status pe_setup(pe_ctx** out, int32_t d, const int32_t* n, const d
     return pe_fail(PE_EINVAL, "pe_setup: device_loop must be 0, 1 or 2");
   }
   c->device_loop = o.device_loop;
-  c->fine_engine = o.fine_engine;
   c->forcing_path = o.forcing_path;
   c->cache_forced = o.cache_forced ? 1 : 0;
   c->precision = o.precision;
@@ -338,6 +339,7 @@ extern "C" pe_status pe_setup(pe_ctx** out, int32_t d, const int32_t* n, const d
   if (st == PE_OK) st = dev_alloc(&c->coefF, (size_t)(c->q + 2) * nd);
   if (st == PE_OK) st = dev_alloc(&c->coefG, (size_t)(c->p + 1) * nd);
   if (st == PE_OK && c->precision == PE_MIXED) st = dev_alloc(&c->coefF32, (size_t)(c->q + 2) * nd);
+  if (st == PE_OK && c->precision == PE_MIXED) st = dev_alloc(&c->coefG32, (size_t)c->p * nd);
   if (st == PE_OK) st = dev_alloc(&c->U, (N + 1) * nd);
   if (st == PE_OK) st = dev_alloc(&c->Fbar, N * nd);
   if (st == PE_OK && c->cache_forced) st = dev_alloc(&c->Fz, N * nd);
@@ -352,23 +354,31 @@ extern "C" pe_status pe_setup(pe_ctx** out, int32_t d, const int32_t* n, const d
   if (st == PE_OK) st = dev_alloc(&c->partials, 2 * (size_t)c->max_blocks + 64);
   if (st == PE_OK) st = dev_alloc(&c->red, 2);
   if (st == PE_OK) st = dev_alloc(&c->done_ctr, 1);
-  if (st == PE_OK && c->fine_engine == PE_FINE_TC) {
-    st = dev_alloc(&c->tcB, fine_tc_buffer_bytes(n_substeps, n_slices));
-    if (st == PE_OK) st = dev_alloc(&c->tc_err, 1);
-    if (st == PE_OK && cudaMemset(c->tc_err, 0, sizeof(int)) != cudaSuccess)
-      st = pe_fail(PE_ECUDA, "pe_setup: error flag initialisation failed");
-  }
   if (st == PE_OK && cudaMemset(c->done_ctr, 0, sizeof(unsigned int)) != cudaSuccess)
     st = pe_fail(PE_ECUDA, "pe_setup: counter initialisation failed");
   if (st == PE_OK) st = dev_alloc(&c->axisF, MT * nsl);
   if (st == PE_OK && c->precision == PE_MIXED) st = dev_alloc(&c->axisF32, MT * nsl);
   if (st == PE_OK) st = dev_alloc(&c->axisU0, MT * nsl);
   if (st == PE_OK) st = dev_alloc(&c->loads, MT * nsum);
-  if (st == PE_OK) st = dev_alloc(&c->AF, N * n_substeps * 2 * MT);
-  if (st == PE_OK && c->precision == PE_MIXED) st = dev_alloc(&c->AF32, N * n_substeps * 2 * MT);
-  if (st == PE_OK) st = dev_alloc(&c->Zst, (size_t)PE_MAX_S * 2 * MT);
-  if (st == PE_OK) st = dev_alloc(&c->AG, N * c->p * MT);
-  if (st == PE_OK && c->precision == PE_MIXED) st = dev_alloc(&c->AG32, N * c->p * MT);
+  if (st == PE_OK) {
+    // time tables of up to 2 MT columns (ColumnTables); Y first, its float rows 16-byte aligned
+    const size_t K = 2 * MT, steps = (size_t)chain_steps(n_substeps);
+    const size_t cnt[5] = {N * K, c->q * K, c->p * K, steps * MT * 4, MT};
+    st = dev_alloc(&c->tab64, cnt[0] + cnt[1] + cnt[2] + cnt[3] + cnt[4]);
+    if (st == PE_OK && c->precision == PE_MIXED)
+      st = dev_alloc(&c->tab32, 2 * cnt[0] + cnt[1] + cnt[2] + 2 * cnt[3] + 2 * cnt[4]);
+    if (st == PE_OK) {
+      double** d[5] = {&c->tab.Y, &c->tab.ZF, &c->tab.ZG, &c->tab.chain, &c->tab.xs};
+      float** f[5] = {&c->tab.Y32, &c->tab.ZF32, &c->tab.ZG32, &c->tab.chain32, &c->tab.xs32};
+      size_t od = 0, of = 0;
+      for (int i = 0; i < 5; ++i) {
+        *d[i] = c->tab64 + od;
+        od += cnt[i];
+        if (c->tab32) *f[i] = c->tab32 + of;
+        of += i == 1 || i == 2 ? cnt[i] : 2 * cnt[i];
+      }
+    }
+  }
   if (st == PE_OK && c->forcing_path == PE_FORCING_GENERAL &&
       ((int64_t)n_substeps * c->q > 65535 || (int64_t)n_slices * c->p > 65535))
     st = pe_fail(PE_EINVAL, "pe_setup: general forcing path needs M*q and N*p <= 65535");
@@ -566,7 +576,9 @@ static cudaError_t record_timing(pe_ctx* c, cudaEvent_t e) {
   return cudaEventRecordWithFlags(e, c->stream, c->capturing ? cudaEventRecordExternal : cudaEventRecordDefault);
 }
 
-static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcing* f) {
+// Algorithm 1 up to its loop; the coarse sweep only where `coarse` (pe_solve makes it in the same
+// pass as the first iteration, launch_iteration).
+static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcing* f, bool coarse) {
   if (!u0) return pe_fail(PE_EINVAL, "pe_set_problem: u0 is NULL");
   const int nf = f ? f->n_terms : 0;
   const bool general = c->forcing_path == PE_FORCING_GENERAL;
@@ -579,7 +591,6 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
   if (c->sharded && u0->kind == PE_FIELD_TERMS_QUADRATURE)
     return pe_fail(PE_EINVAL, "pe_set_problem: a context that owns a block of modes takes nodal or separable u0");
   memset(c->lkind, 0, sizeof(c->lkind));
-  c->tc_split_ok = false;
   if (nf == 0 && c->nbd == 0) {
     // no source: one zero term keeps every kernel shape valid
     c->R = 1;
@@ -591,15 +602,13 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
   }
   // Two streams for grids large enough that their set-up kernels run side by side: the side
   // stream makes the time tables, then the forward transform of nodal u0 (after its copy, for
-  // host u0), then the tensor-core engine's split time factors; the main stream makes the
-  // per-axis forcing factors, waits for the time tables (the stage weights take their shifts
-  // Z), makes the stage weights, and waits for the side stream before the coarse sweep.
+  // host u0); the main stream makes the per-axis forcing factors, waits for the time tables, makes
+  // the column weights, and waits for the side stream before the coarse sweep.
   // (Small grids, whose kernels are launch-bound, keep everything on the main stream.)
   double* U0 = c->U;
   const bool fork_u0 = u0->kind == PE_FIELD_NODAL && u0->nodal != nullptr;
   const bool fork = fork_u0 && c->gn.ndof >= kForkMinDof;
   const bool inline_u0 = fork_u0 && !fork;  // nodal u0, transformed below on the main stream
-  const bool tc = !general && c->precision == PE_MIXED && c->fine_engine == PE_FINE_TC;
   if (fork) {
     PE_CUDA_TRY(cudaEventRecord(c->ev_fork, c->stream));
     PE_CUDA_TRY(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
@@ -623,7 +632,6 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
       }
       if (st == PE_OK) st = nodal_to_modal(c, src, U0);
     }
-    if (st == PE_OK && tc) st = fine_tc_prepare_time(c);
     c->stream = main_stream;
     PE_TRY(st);
     PE_CUDA_TRY(cudaEventRecord(c->ev_join, c->side));
@@ -631,15 +639,11 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
     PE_TRY(launch_time_tables(c));
   }
   // The phi/b coefficient tables depend only on lam, dt, dT and the nodes: pe_setup made them.
-  // Forcing: per-axis modal factors, then the stage weights of the fine step.
+  // Forcing: per-axis modal factors, then the column weights.
   if (!general) PE_TRY(launch_separable_factors(c, c->terms, c->R, c->axisF, 1, c->lkind));
   if (fork && !general) PE_CUDA_TRY(cudaStreamWaitEvent(c->stream, c->ev_tables, 0));
-  if (!general) PE_TRY(launch_stage_weights(c));
-  // the tensor-core engine's split operand images of the stage weights and time factors
-  if (tc) PE_TRY(fine_tc_prepare_weights(c));
-  if (tc && !fork) PE_TRY(fine_tc_prepare_time(c));
+  if (!general) PE_TRY(launch_column_weights(c));
   if (fork) PE_CUDA_TRY(cudaStreamWaitEvent(c->stream, c->ev_join, 0));
-  if (tc) c->tc_split_ok = true;
   PE_CUDA_TRY(record_timing(c, c->ev[1]));
   // U^0 = P_h u0
   if (fork_u0 && !inline_u0) {
@@ -674,9 +678,11 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
     PE_TRY(add_lift(c, c->t0, -1.0, nodal ? 2 : 1, U0));
   }
   // k = 0: coarse sweep
-  PE_CUDA_TRY(record_timing(c, c->ev[8]));
-  PE_TRY(launch_coarse_sweep(c));
-  PE_CUDA_TRY(record_timing(c, c->ev[9]));
+  if (coarse) {
+    PE_CUDA_TRY(record_timing(c, c->ev[8]));
+    PE_TRY(launch_coarse_sweep(c));
+    PE_CUDA_TRY(record_timing(c, c->ev[9]));
+  }
   c->fz_prec = -1;
   c->k = 0;
   c->have_problem = true;
@@ -690,20 +696,21 @@ extern "C" pe_status pe_set_problem(pe_ctx* c, const pe_field* u0, const pe_forc
   c->have_problem = false;
   drop_solve_graphs(c);
   PE_CUDA_TRY(cudaEventRecord(c->ev[0], c->stream));
-  PE_TRY(set_problem_impl(c, u0, f));
+  PE_TRY(set_problem_impl(c, u0, f, true));
   PE_CUDA_TRY(cudaStreamSynchronize(c->stream));
   return PE_OK;
 }
 
 // One pass of Algorithm 1's loop.  sums_out (may be NULL): this context's two residual sums;
 // r_out (may be NULL): the relative residual of the totals (after residual_reduce, if any).
-static pe_status iter_impl(pe_ctx* c, double* r_out, int precision, double* sums_out = nullptr) {
+// first: the coarse sweep of k = 0 in the same pass (its time is then the coarse sweep's too).
+static pe_status iter_impl(pe_ctx* c, double* r_out, int precision, double* sums_out = nullptr, bool first = false) {
   PE_CUDA_TRY(cudaEventRecord(c->ev[5], c->stream));
-  if (c->forcing_path == PE_FORCING_GENERAL) PE_TRY(launch_general_fine_sweep(c, precision));
-  else PE_TRY(launch_fine_sweep(c, precision));
-  PE_CUDA_TRY(cudaEventRecord(c->ev[6], c->stream));
+  if (first) PE_CUDA_TRY(cudaEventRecord(c->ev[8], c->stream));
+  PE_TRY(launch_iteration(c, precision, first, nullptr, 0ull, c->ev[6]));
+  if (first) PE_CUDA_TRY(cudaEventRecord(c->ev[9], c->stream));
   double num = 0.0, den = 0.0;
-  PE_TRY(launch_correction(c, &num, &den, c->ev[7]));  // synchronises the stream
+  PE_TRY(read_sums(c, &num, &den, c->ev[7]));  // synchronises the stream
   c->ms_fine += elapsed(c->ev[5], c->ev[6]);
   c->ms_corr += elapsed(c->ev[6], c->ev[7]);
   c->k += 1;
@@ -713,7 +720,6 @@ static pe_status iter_impl(pe_ctx* c, double* r_out, int precision, double* sums
   }
   if (!isfinite(num) || !isfinite(den)) {
     c->have_problem = false;
-    if (precision == PE_MIXED && c->fine_engine == PE_FINE_TC) PE_TRY(fine_tc_status(c));
     return pe_fail(PE_ENONFINITE, "Parareal residual is not finite (NaN/Inf in the iterate)");
   }
   if (r_out) {
@@ -770,9 +776,10 @@ extern "C" pe_status pe_refine(pe_ctx* c, double* rel_residual_out) {
 }
 
 // ---------------------------------------------------------------------------
-// device-resident Parareal loop: a CUDA graph with one conditional (while) node whose body is
-// one pass of Algorithm 1's loop -- the fine sweep from every slice and the correction, whose
-// last CTA appends r_k, advances k and sets the condition (r > tol and k < max_iter)
+// device-resident Parareal loop: a CUDA graph of the first iteration (with the coarse sweep, see
+// launch_iteration) and a conditional (while) node whose body is one further pass of Algorithm 1's
+// loop; the last CTA of each appends r_k, advances k and sets the condition (r > tol and
+// k < max_iter)
 // ---------------------------------------------------------------------------
 static bool loop_on_device(const pe_ctx* c) {
   return c->device_loop && !c->cache_forced && c->forcing_path == PE_FORCING_SEPARABLE && !c->reduce &&
@@ -789,38 +796,56 @@ static pe_status build_loop_graph(pe_ctx* c) {
   PE_CUDA_TRY(cudaGraphCreate(&graph, 0));
   cudaGraphConditionalHandle handle;
   pe_status st = PE_OK;
-  cudaError_t e = cudaGraphConditionalHandleCreate(&handle, graph, 1u, cudaGraphCondAssignDefault);
-  cudaGraphNodeParams np{};
-  cudaGraphNode_t node = nullptr;
-  if (e == cudaSuccess) {
+  // the condition starts at 0 in every launch: the first iteration's decision sets it
+  cudaError_t e = cudaGraphConditionalHandleCreate(&handle, graph, 0u, cudaGraphCondAssignDefault);
+  if (e != cudaSuccess) {
+    cudaGraphDestroy(graph);
+    return pe_cuda_fail(e, "device loop: condition");
+  }
+  // both parts are captured on the side stream (the context's own stream may be the legacy
+  // default stream, which cannot be captured)
+  cudaStream_t main_stream = c->stream;
+  const int64_t launches0 = c->launches, sweeps0 = c->sweeps;
+  auto capture = [&](cudaGraph_t into, bool first, std::vector<cudaGraphNode_t>* last) {
+    e = cudaStreamBeginCaptureToGraph(c->side, into, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return pe_cuda_fail(e, "device loop: begin capture");
+    c->stream = c->side;
+    c->capturing = 1;
+    pe_status s = PE_OK;
+    if (first && record_timing(c, c->ev[8]) != cudaSuccess) s = pe_cuda_fail(cudaGetLastError(), "device loop: event");
+    if (s == PE_OK) s = launch_iteration(c, c->precision, first && first_fused(c), c->loopctl, (unsigned long long)handle);
+    if (s == PE_OK && first && record_timing(c, c->ev[9]) != cudaSuccess)
+      s = pe_cuda_fail(cudaGetLastError(), "device loop: event");
+    c->capturing = 0;
+    c->stream = main_stream;
+    if (s == PE_OK && last) {
+      cudaStreamCaptureStatus cs;
+      const cudaGraphNode_t* deps = nullptr;
+      size_t nd = 0;
+      e = cudaStreamGetCaptureInfo(c->side, &cs, nullptr, nullptr, &deps, nullptr, &nd);
+      if (e == cudaSuccess) last->assign(deps, deps + nd);
+      else s = pe_cuda_fail(e, "device loop: capture info");
+    }
+    cudaGraph_t captured = nullptr;
+    const cudaError_t e2 = cudaStreamEndCapture(c->side, &captured);
+    if (s == PE_OK && e2 != cudaSuccess) s = pe_cuda_fail(e2, "device loop: capture");
+    return s;
+  };
+  std::vector<cudaGraphNode_t> last;
+  st = capture(graph, true, &last);
+  c->loop_first_launches = c->launches - launches0;
+  if (st == PE_OK) {
+    cudaGraphNodeParams np{};
+    cudaGraphNode_t node = nullptr;
     np.type = cudaGraphNodeTypeConditional;
     np.conditional.handle = handle;
     np.conditional.type = cudaGraphCondTypeWhile;
     np.conditional.size = 1;
-    e = cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, &np);
+    e = cudaGraphAddNode(&node, graph, last.data(), nullptr, last.size(), &np);
+    if (e != cudaSuccess) st = pe_cuda_fail(e, "device loop: conditional node");
+    else st = capture(np.conditional.phGraph_out[0], false, nullptr);
   }
-  if (e != cudaSuccess) {
-    cudaGraphDestroy(graph);
-    return pe_cuda_fail(e, "device loop: conditional node");
-  }
-  // the body: the launches of one iteration, captured on the side stream (the context's own
-  // stream may be the legacy default stream, which cannot be captured)
-  cudaGraph_t body = np.conditional.phGraph_out[0];
-  cudaStream_t main_stream = c->stream;
-  const int64_t launches0 = c->launches, sweeps0 = c->sweeps;
-  e = cudaStreamBeginCaptureToGraph(c->side, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
-  if (e == cudaSuccess) {
-    c->stream = c->side;
-    st = launch_fine_sweep(c, c->precision);
-    if (st == PE_OK) st = launch_correction_kernel(c, c->loopctl, (unsigned long long)handle);
-    c->stream = main_stream;
-    cudaGraph_t captured = nullptr;
-    const cudaError_t e2 = cudaStreamEndCapture(c->side, &captured);
-    if (st == PE_OK && e2 != cudaSuccess) st = pe_cuda_fail(e2, "device loop: capture");
-  } else {
-    st = pe_cuda_fail(e, "device loop: begin capture");
-  }
-  c->loop_body_launches = c->launches - launches0;
+  c->loop_body_launches = c->launches - launches0 - c->loop_first_launches;
   c->launches = launches0;
   c->sweeps = sweeps0;
   if (st == PE_OK) {
@@ -858,7 +883,7 @@ static pe_status finish_loop_on_device(pe_ctx* c, pe_result* res, double* r) {
   const int k = h->k;
   c->k += k;
   c->sweeps += k;
-  c->launches += (int64_t)k * c->loop_body_launches;
+  if (k > 0) c->launches += c->loop_first_launches + (int64_t)(k - 1) * c->loop_body_launches;
   *r = h->r;
   if (res && res->residual_history && res->history_cap > 0) {
     const int cnt = std::min(k, res->history_cap);
@@ -866,7 +891,6 @@ static pe_status finish_loop_on_device(pe_ctx* c, pe_result* res, double* r) {
   }
   if (h->nonfinite) {
     c->have_problem = false;
-    if (c->precision == PE_MIXED && c->fine_engine == PE_FINE_TC) PE_TRY(fine_tc_status(c));
     return pe_fail(PE_ENONFINITE, "Parareal residual is not finite (NaN/Inf in the iterate)");
   }
   return PE_OK;
@@ -969,7 +993,8 @@ static pe_status solve_begin(pe_ctx* c, const pe_field* u0, const pe_forcing* f,
   }
   PE_CUDA_TRY(cudaEventRecord(c->ev[0], c->stream));
   if (use_graphs && !c->setup_exec &&
-      !capture_phase(c, &c->setup_exec, &c->setup_launches, [&] { return set_problem_impl(c, u0, f); })) {
+      !capture_phase(c, &c->setup_exec, &c->setup_launches,
+                     [&] { return set_problem_impl(c, u0, f, !first_fused(c)); })) {
     use_graphs = false;  // not capturable: this problem runs its phases directly from now on
     c->graph_key_seen = INT_MIN / 2;
   }
@@ -983,7 +1008,7 @@ static pe_status solve_begin(pe_ctx* c, const pe_field* u0, const pe_forcing* f,
     PE_CUDA_TRY(cudaGraphLaunch(c->setup_exec, c->stream));
     c->launches += c->setup_launches;
   } else {
-    PE_TRY(set_problem_impl(c, u0, f));
+    PE_TRY(set_problem_impl(c, u0, f, !first_fused(c)));
   }
   c->u0_dev_hint = -1;
   PE_CUDA_TRY(cudaEventRecord(c->ev[2], c->stream));
@@ -994,7 +1019,7 @@ static pe_status solve_begin(pe_ctx* c, const pe_field* u0, const pe_forcing* f,
     PE_TRY(enqueue_loop_on_device(c, tol));
   } else {
     while (c->k < c->max_iter) {
-      PE_TRY(iter_impl(c, &r, c->precision));
+      PE_TRY(iter_impl(c, &r, c->precision, nullptr, c->k == 0 && first_fused(c)));
       c->pend_hist.push_back(r);
       if (r <= tol) break;
     }

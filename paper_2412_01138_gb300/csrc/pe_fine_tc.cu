@@ -139,358 +139,6 @@ __device__ __forceinline__ void split8(const float (&x)[8], uint4 (&o)[3]) {
   for (int t = 0; t < 3; ++t) o[t] = make_uint4(pk[t][0], pk[t][1], pk[t][2], pk[t][3]);
 }
 
-// Split time factors of every slice group, in the B-operand layout of the kernel below:
-// group g occupies 3 * NR * KP * 2 bytes, [term][row r][k] swizzled as above, row r = s * M + m
-// holding Y_{gG+s}[m][k] (zero past the last slice and past K).
-__global__ void ft_split_time_kernel(const float* __restrict__ Y, int N, int M, int K, int KC, int G, int NR,
-                                     int KP, int ngroups, uint4* __restrict__ Bsp) {
-  pdl_wait();
-  const int chunks = KP / 8;
-  const int64_t total = (int64_t)ngroups * NR * chunks;
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= total) return;
-  const int c = (int)(e % chunks);
-  const int64_t gr = e / chunks;
-  const int r = (int)(gr % NR);
-  const int g = (int)(gr / NR);
-  const int s = r / M, m = r - s * M, n = g * G + s;
-  float x[8];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int k = 8 * c + j;
-    x[j] = (n < N && k < K) ? Y[((int64_t)n * M + m) * KC + k] : 0.f;
-  }
-  uint4 o[3];
-  split8(x, o);
-  const int64_t term = (int64_t)NR * KP * 2;
-#pragma unroll
-  for (int t = 0; t < 3; ++t)
-    Bsp[(((int64_t)g * 3 + t) * term + ft_swz((int64_t)r * KP * 2 + c * 16, KP)) / 16] = o[t];
-}
-
-// Stage weights of every mode tile formed and split in one pass, in the A-operand layout of the
-// kernel below: tile q occupies 3 * 128 * KP * 2 bytes, [term][row r][k] swizzled as above, row
-// r holding W[k][128 q + r] (zero past the last mode and past K).  A thread per row and group of
-// eight columns (consecutive threads: the 16-byte chunks of one row, then the next row): the same
-// float32 arithmetic as the SIMT engine's stage-weight table, W[k][J] = P_{r(k),J} sum_i
-// (dt b_i)_J Z_k(c_i dt) with P the product of the per-axis modal factors, so that table is never
-// written or read by this engine.
-template <int Q>
-__global__ void __launch_bounds__(256) ft_weights_image_kernel(Geom g, StageCols C, int R,
-                                                               const float* __restrict__ axisF,
-                                                               const float* __restrict__ coef_b,
-                                                               const double* __restrict__ Z, int KP, int64_t tiles,
-                                                               uint4* __restrict__ Asp) {
-  pdl_wait();
-  __shared__ float sZ[PE_MAX_S * 2 * PE_MAX_TERMS];
-  __shared__ int sTerm[2 * PE_MAX_TERMS];
-  const int K = C.K;
-  for (int e = threadIdx.x; e < Q * K; e += blockDim.x) sZ[e] = (float)Z[e];
-  for (int e = threadIdx.x; e < K; e += blockDim.x) sTerm[e] = C.term[e];
-  __syncthreads();
-  const int chunks = KP / 8;
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= tiles * FT_ROWS * chunks) return;
-  const int c = (int)(e % chunks);
-  const int64_t J = e / chunks;
-  const int r = (int)(J % FT_ROWS);
-  const int64_t tile = J / FT_ROWS, nd = g.ndof;
-  const int64_t term = (int64_t)FT_ROWS * KP * 2;
-  if (J >= nd || 8 * c >= K) {
-    // padding rows past the last mode and columns past K: zero in every split term
-#pragma unroll
-    for (int t = 0; t < 3; ++t)
-      Asp[((tile * 3 + t) * term + ft_swz((int64_t)r * KP * 2 + c * 16, KP)) / 16] = make_uint4(0u, 0u, 0u, 0u);
-    return;
-  }
-  int j[PE_MAX_D];
-  unflatten(g, J, j);
-  // the row's entries of the per-axis factor tables (term rt of axis a at ax[a][rt * n_a])
-  const float* ax[PE_MAX_D];
-#pragma unroll
-  for (int a = 0; a < PE_MAX_D; ++a) ax[a] = axisF + (int64_t)R * g.off[a] + j[a];
-  float b[Q];
-#pragma unroll
-  for (int i = 0; i < Q; ++i) b[i] = coef_b[(int64_t)i * nd + J];
-  {
-    float x[8];
-#pragma unroll
-    for (int jj = 0; jj < 8; ++jj) {
-      const int k = 8 * c + jj;
-      float v = 0.f;
-      if (k < K) {
-        const int rt = sTerm[k];
-        float P = ax[0][rt * g.n[0]];
-#pragma unroll
-        for (int a = 1; a < PE_MAX_D; ++a) if (a < g.d) P *= ax[a][rt * g.n[a]];
-        float sw = 0.f;
-#pragma unroll
-        for (int i = 0; i < Q; ++i) sw = fmaf(b[i], sZ[i * K + k], sw);
-        v = P * sw;
-      }
-      x[jj] = v;
-    }
-    uint4 o[3];
-    split8(x, o);
-#pragma unroll
-    for (int t = 0; t < 3; ++t) Asp[((tile * 3 + t) * term + ft_swz((int64_t)r * KP * 2 + c * 16, KP)) / 16] = o[t];
-  }
-}
-
-struct FtArgs {
-  const float* coefF32;  // E_hi [ndof], E_lo [ndof]
-  const double* EM;      // exp(-lam M dt) [ndof]
-  const double* U;       // U^n at n * ndof
-  double* out;           // F^M(U^n) (or F^M(0)) at n * ndof
-  const unsigned char* Asp;  // split stage weights of every mode tile
-  const unsigned char* Bsp;  // split time factors of every slice group
-  int64_t ndof, tiles, items;
-  int N, M, K, G, NR, from_zero;
-  int* err;
-};
-
-template <int KP>
-__global__ void __launch_bounds__(FT_THREADS, 1) fine_tc_kernel(FtArgs a) {
-  pdl_wait();
-  constexpr int A_TERM = FT_ROWS * KP * 2;          // one split term of the A operand
-  constexpr int A_BYTES = 3 * A_TERM;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t fullA[FT_ABUF], emptyA[FT_ABUF], fullD[2], emptyD[2], fullB, freeB, drain;
-  __shared__ uint32_t tmem_slot;
-  __shared__ int s_fail;
-  unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  unsigned char* sB = smem;
-  unsigned char* sA = smem + 3 * ft_rows_max(KP) * KP * 2;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int NR = a.NR, M = a.M;
-  const int B_BYTES = 3 * NR * KP * 2;
-  const int64_t nd = a.ndof;
-  const int64_t i0 = (int64_t)blockIdx.x * a.items / gridDim.x;
-  const int64_t i1 = (int64_t)(blockIdx.x + 1) * a.items / gridDim.x;
-  uint32_t ncols = 32;
-  while (ncols < (uint32_t)(2 * NR)) ncols <<= 1;
-  volatile int* fail = &s_fail;
-  auto set_fail = [&](int code) {
-    atomicExch(a.err, code);
-    *fail = 1;
-    a.out[0] = __longlong_as_double(0x7ff8000000000000LL);
-  };
-  if (tid == 0) {
-    for (int b = 0; b < FT_ABUF; ++b) {
-      mbar_init(&fullA[b], 1);
-      mbar_init(&emptyA[b], 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&fullD[b], 1);
-      mbar_init(&emptyD[b], FT_WORKERS / 32);
-    }
-    mbar_init(&fullB, 1);
-    mbar_init(&freeB, 1);
-    mbar_init(&drain, 1);
-    s_fail = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == FT_WORKERS / 32) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
-                 "r"(ncols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tmem_slot;
-
-  if (warp < FT_WORKERS / 32) {
-    // thread (h, r): warpgroup h of two, row r of the tile (TMEM lane r)
-    const int r = tid & (FT_ROWS - 1), h = tid >> 7, lane = tid & 31;
-    // the epilogue inputs of item i + 1 (E_hi, E_lo, exp(-lam M dt)) are loaded while item i
-    // waits for its accumulator and runs, into two alternating register sets
-    struct Pre {
-      float eh, el;
-      double em;
-    };
-    Pre P0, P1;
-    auto load_epi = [&](Pre& P, int64_t i) {
-      const int64_t g = i / a.tiles, J = (i % a.tiles) * FT_ROWS + r;
-      const bool ok = J < nd;
-      P.eh = ok ? a.coefF32[J] : 0.f;
-      P.el = ok ? a.coefF32[nd + J] : 0.f;
-      P.em = ok ? a.EM[J] : 0.0;
-    };
-    auto step = [&](int64_t i, const Pre& cur, Pre& nxt) -> bool {
-      const int j = (int)(i - i0);
-      if (i + 1 < i1) load_epi(nxt, i + 1);
-      // U^n of the slices, loaded ahead: the first pair's before the wait for the accumulator,
-      // each later pair's (more than four slices per group) while the pair before it runs
-      const int64_t g = i / a.tiles;
-      const int64_t J = (i % a.tiles) * FT_ROWS + r;
-      const bool ok = J < nd;
-      auto load_u = [&](int s) -> double {
-        const int64_t n = g * a.G + s;
-        return (!a.from_zero && ok && s < a.G && n < a.N) ? a.U[n * nd + J] : 0.0;
-      };
-      double u0 = load_u(h), u1 = load_u(h + 2);
-      if (!mbar_wait(&fullD[j & 1], (uint32_t)((j >> 1) & 1))) {
-        set_fail(5);
-        return false;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      float e2h, e2l, e4h, e4l;
-      df_square(cur.eh, cur.el, e2h, e2l);
-      df_square(e2h, e2l, e4h, e4l);
-      const float eh = cur.eh, e2 = e2h, e3 = e2h * eh;
-      const uint32_t row = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((j & 1) * NR);
-      // this thread's slices s = h + 2t of the group, two at a time (warp-uniform); each
-      // TMEM read brings 32 substeps of both, and the chains run four substeps per step:
-      // w <- E^4 w + (E^3 a_m + E^2 a_{m+1} + E a_{m+2} + a_{m+3}), the bracket independent of
-      // w and E^4 applied as a hi/lo pair
-      auto chain4 = [&](float& w, float x0, float x1, float x2, float x3) {
-        const float b = fmaf(e3, x0, fmaf(e2, x1, fmaf(eh, x2, x3)));
-        w = fmaf(e4h, w, fmaf(e4l, w, b));
-      };
-      auto finish = [&](double u, int s, float w) {
-        const int64_t n = g * a.G + s;
-        if (ok && n < a.N) a.out[n * nd + J] = a.from_zero ? (double)w : fma(cur.em, u, (double)w);
-      };
-#pragma unroll 1
-      for (int p = 0; p < 4; ++p) {
-        const int s0 = h + 4 * p, s1 = s0 + 2;
-        if (s0 >= a.G) break;
-        const bool two = s1 < a.G;
-        const double n0 = load_u(s0 + 4), n1 = load_u(s1 + 4);
-        float w0 = 0.f, w1 = 0.f;
-        int m0 = 0;
-        for (; m0 + 32 <= M; m0 += 32) {
-          float v0[32], v1[32];
-          tmem_ld32(row + (uint32_t)(s0 * M + m0), v0);
-          if (two) tmem_ld32(row + (uint32_t)(s1 * M + m0), v1);
-          tmem_wait_ld();
-#pragma unroll
-          for (int e = 0; e < 32; e += 4) {
-            chain4(w0, v0[e], v0[e + 1], v0[e + 2], v0[e + 3]);
-            if (two) chain4(w1, v1[e], v1[e + 1], v1[e + 2], v1[e + 3]);
-          }
-        }
-        if (m0 < M) {  // a tail of 16 substeps
-          float v0[16], v1[16];
-          tmem_ld16(row + (uint32_t)(s0 * M + m0), v0);
-          if (two) tmem_ld16(row + (uint32_t)(s1 * M + m0), v1);
-          tmem_wait_ld();
-#pragma unroll
-          for (int e = 0; e < 16; e += 4) {
-            chain4(w0, v0[e], v0[e + 1], v0[e + 2], v0[e + 3]);
-            if (two) chain4(w1, v1[e], v1[e + 1], v1[e + 2], v1[e + 3]);
-          }
-        }
-        finish(u0, s0, w0);
-        if (two) finish(u1, s1, w1);
-        u0 = n0;
-        u1 = n1;
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&emptyD[j & 1]);
-      return true;
-    };
-    if (i0 < i1) load_epi(P0, i0);
-    for (int64_t i = i0; i < i1; i += 2) {
-      if (*fail || !step(i, P0, P1)) break;
-      if (i + 1 < i1 && (*fail || !step(i + 1, P1, P0))) break;
-    }
-  } else if (tid == FT_WORKERS) {
-    const uint32_t idesc = instr_desc_bf16(FT_ROWS, NR);
-    const int ta[6] = {2, 1, 0, 1, 0, 0}, tb[6] = {0, 1, 2, 0, 1, 0};  // small products first
-    const int n = (int)(i1 - i0);
-    // item i0 + jj's split weights into A buffer jj % FT_ABUF
-    auto load_A = [&](int jj) {
-      const int b = jj % FT_ABUF;
-      const unsigned char* src = a.Asp + ((i0 + jj) % a.tiles) * (int64_t)A_BYTES;
-      mbar_expect_tx(&fullA[b], (uint32_t)A_BYTES);
-      for (int off = 0; off < A_BYTES; off += FT_CHUNK)
-        bulk_g2s(sA + b * A_BYTES + off, src + off, (uint32_t)(A_BYTES - off < FT_CHUNK ? A_BYTES - off : FT_CHUNK),
-                 &fullA[b]);
-    };
-    int nl = 0;  // items whose A copy has been issued
-    for (; nl < FT_ABUF && nl < n; ++nl) load_A(nl);
-    int j = 0;
-    int64_t gcur = -1;
-    int nB = 0;
-    bool issued = false;
-    for (; j < n; ++j) {
-      const int64_t g = (i0 + j) / a.tiles;
-      if (g != gcur) {
-        // the previous group's MMAs must be done with sB before it is overwritten
-        if (gcur >= 0) {
-          mma_commit(&freeB);
-          if (!mbar_wait(&freeB, (uint32_t)((nB - 1) & 1))) {
-            set_fail(6);
-            break;
-          }
-        }
-        mbar_expect_tx(&fullB, (uint32_t)B_BYTES);
-        const unsigned char* src = a.Bsp + g * (int64_t)B_BYTES;
-        for (int off = 0; off < B_BYTES; off += FT_CHUNK)
-          bulk_g2s(sB + off, src + off, (uint32_t)(B_BYTES - off < FT_CHUNK ? B_BYTES - off : FT_CHUNK), &fullB);
-        if (!mbar_wait(&fullB, (uint32_t)(nB & 1))) {
-          set_fail(7);
-          break;
-        }
-        ++nB;
-        gcur = g;
-      }
-      const int b = j % FT_ABUF;
-      if (!mbar_wait(&fullA[b], (uint32_t)((j / FT_ABUF) & 1))) {
-        set_fail(8);
-        break;
-      }
-      if (j >= 2 && !mbar_wait(&emptyD[j & 1], (uint32_t)(((j >> 1) - 1) & 1))) {
-        set_fail(9);
-        break;
-      }
-      if (*fail) break;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t a0 = smem_u32(sA + b * A_BYTES), b0 = smem_u32(sB);
-      const uint32_t d = tmem + (uint32_t)((j & 1) * NR);
-      bool first = true;
-#pragma unroll
-      for (int q = 0; q < 6; ++q) {
-#pragma unroll
-        for (int ks = 0; ks < KP / 16; ++ks) {
-          const uint64_t da = smem_desc_swz(a0 + ta[q] * A_TERM + 32 * ks, KP);
-          const uint64_t db = smem_desc_swz(b0 + tb[q] * (NR * KP * 2) + 32 * ks, KP);
-          mma_bf16(d, da, db, idesc, first ? 0u : 1u);
-          first = false;
-        }
-      }
-      mma_commit(&fullD[j & 1]);
-      mma_commit(&emptyA[b]);
-      issued = true;
-      // refill the buffer of item j - 1 (its MMAs ran ahead of item j's) with item j + 2
-      if (j >= 1 && j + FT_ABUF - 1 < n) {
-        if (!mbar_wait(&emptyA[(j - 1) % FT_ABUF], (uint32_t)(((j - 1) / FT_ABUF) & 1))) {
-          set_fail(11);
-          break;
-        }
-        load_A(j + FT_ABUF - 1);
-        ++nl;
-      }
-    }
-    // after a failure: wait (bounded) for the A copies still in flight into shared memory
-    if (*fail)
-      for (int jj = j; jj < nl; ++jj) mbar_wait(&fullA[jj % FT_ABUF], (uint32_t)((jj / FT_ABUF) & 1));
-    // every MMA and copy of this CTA has completed before the tensor memory is freed
-    if (issued) {
-      mma_commit(&drain);
-      if (!mbar_wait(&drain, 0)) set_fail(10);
-    }
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  if (warp == FT_WORKERS / 32) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
-  }
-}
 
 // ---------------------------------------------------------------------------
 // Batched form: the same engine over the work items (problem p, slice group g, mode tile t)
@@ -829,150 +477,15 @@ pe_status btc_launch(const BtcArgs& args, int grid, cudaStream_t st) {
   return PE_OK;
 }
 
-template <int KP>
-pe_status ft_launch(const FtArgs& args, int grid, cudaStream_t st) {
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(fine_tc_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, ft_smem_bytes(KP));
-  });
-  if (attr != cudaSuccess) return pe_cuda_fail(attr, "fine sweep (tensor cores): shared-memory attribute");
-  PE_CUDA_TRY(launch_pdl(fine_tc_kernel<KP>, dim3(grid), dim3(FT_THREADS), ft_smem_bytes(KP), st, args));
-  return PE_OK;
-}
+}  // namespace
+
+static bool fine_tc_supported(int M) { return M >= 16 && M <= 128 && M % 16 == 0; }
 
 // slice-group shape of a column padding KP at M substeps: G slices, NR = G * M rows
-void ft_shape(int KP, int M, int N, int* G, int* NR, int* ngroups) {
+static void ft_shape(int KP, int M, int N, int* G, int* NR, int* ngroups) {
   *G = std::max(1, ft_rows_max(KP) / M);
   *NR = *G * M;
   *ngroups = (N + *G - 1) / *G;
-}
-
-}  // namespace
-
-bool fine_tc_supported(int M) { return M >= 16 && M <= 128 && M % 16 == 0; }
-
-size_t fine_tc_buffer_bytes(int M, int N) {
-  size_t most = 0;
-  for (int KP = 16; KP <= 64; KP *= 2) {
-    int G, NR, ng;
-    ft_shape(KP, M, N, &G, &NR, &ng);
-    most = std::max(most, (size_t)ng * 3 * NR * KP * 2);
-  }
-  return most;
-}
-
-// The split operand images depend only on the problem (stage weights, time factors): made
-// once by pe_set_problem (after the stage weights) and reused by every sweep of the problem.
-static pe_status ft_check(pe_ctx* c) {
-  if (!fine_tc_supported(c->M) || c->K < 1 || c->K > 64 || !c->tcB || !c->tc_err)
-    return pe_fail(PE_EINVAL, "fine sweep (tensor cores): unsupported shape");
-  return PE_OK;
-}
-
-pe_status fine_tc_prepare_time(pe_ctx* c) {
-  PE_TRY(ft_check(c));
-  const int M = c->M, K = c->K, N = c->N;
-  const int KP = ft_kpad(K), KC = (K + 3) / 4 * 4;
-  int G, NR, ngroups;
-  ft_shape(KP, M, N, &G, &NR, &ngroups);
-  const int64_t nsplit = (int64_t)ngroups * NR * (KP / 8);
-  PE_CUDA_TRY(launch_pdl(ft_split_time_kernel, dim3((unsigned)((nsplit + 255) / 256)), dim3(256), 0, c->stream,
-                         (const float*)c->AF32, N, M, K, KC, G, NR, KP, ngroups, (uint4*)c->tcB));
-  c->launches += 1;
-  return PE_OK;
-}
-
-pe_status fine_tc_prepare_weights(pe_ctx* c) {
-  PE_TRY(ft_check(c));
-  const int KP = ft_kpad(c->K);
-  const int64_t tiles = (c->g.ndof + FT_ROWS - 1) / FT_ROWS;
-  const size_t a_need = (size_t)tiles * ft_a_bytes(KP);
-  if (a_need > c->tcA_cap) {
-    PE_CUDA_TRY(cudaStreamSynchronize(c->stream));
-    if (c->tcA) PE_CUDA_TRY(cudaFree(c->tcA));
-    c->tcA = nullptr;
-    c->tcA_cap = 0;
-    PE_CUDA_TRY(cudaMalloc((void**)&c->tcA, a_need));
-    c->tcA_cap = a_need;
-  }
-  // a thread per (row, group of eight columns)
-  const int64_t nsw = tiles * FT_ROWS * (KP / 8);
-  const dim3 grid((unsigned)((nsw + 255) / 256));
-  const float* ax = c->axisF32;
-  const float* cb = c->coefF32 + 2 * c->g.ndof;
-  switch (c->q) {
-#define PE_FW_CASE(Q)                                                                                          \
-  case Q:                                                                                                      \
-    PE_CUDA_TRY(launch_pdl(ft_weights_image_kernel<Q>, grid, dim3(256), 0, c->stream, c->g, c->cols, c->R, ax, cb, \
-                           (const double*)c->Zst, KP, tiles, (uint4*)c->tcA));                                  \
-    break;
-    PE_FW_CASE(1) PE_FW_CASE(2) PE_FW_CASE(3) PE_FW_CASE(4) PE_FW_CASE(5) PE_FW_CASE(6) PE_FW_CASE(7) PE_FW_CASE(8)
-#undef PE_FW_CASE
-    default:
-      return pe_fail(PE_EINVAL, "fine sweep (tensor cores): unsupported number of stages");
-  }
-  c->launches += 1;
-  return PE_OK;
-}
-
-pe_status fine_tc_prepare(pe_ctx* c) {
-  PE_TRY(fine_tc_prepare_time(c));
-  PE_TRY(fine_tc_prepare_weights(c));
-  c->tc_split_ok = true;
-  return PE_OK;
-}
-
-pe_status launch_fine_tc(pe_ctx* c, int from_zero, double* out) {
-  const int M = c->M, K = c->K, N = c->N;
-  if (!fine_tc_supported(M) || K < 1 || K > 64 || !c->tcB || !c->tc_err)
-    return pe_fail(PE_EINVAL, "fine sweep (tensor cores): unsupported shape");
-  if (!c->tc_split_ok) PE_TRY(fine_tc_prepare(c));
-  const int KP = ft_kpad(K);
-  int G, NR, ngroups;
-  ft_shape(KP, M, N, &G, &NR, &ngroups);
-  const int64_t tiles = (c->g.ndof + FT_ROWS - 1) / FT_ROWS;
-  FtArgs args{};
-  args.coefF32 = c->coefF32;
-  args.EM = c->coefF + (int64_t)(c->q + 1) * c->g.ndof;
-  args.U = c->U;
-  args.out = out;
-  args.Asp = c->tcA;
-  args.Bsp = c->tcB;
-  args.ndof = c->g.ndof;
-  args.tiles = tiles;
-  args.items = args.tiles * ngroups;
-  args.N = N;
-  args.M = M;
-  args.K = K;
-  args.G = G;
-  args.NR = NR;
-  args.from_zero = from_zero;
-  args.err = c->tc_err;
-  int dev = 0, sms = 0;
-  PE_CUDA_TRY(cudaGetDevice(&dev));
-  PE_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int grid = (int)std::min<int64_t>(args.items, sms);
-  pe_status st = PE_OK;
-  switch (KP) {
-    case 16: st = ft_launch<16>(args, grid, c->stream); break;
-    case 32: st = ft_launch<32>(args, grid, c->stream); break;
-    default: st = ft_launch<64>(args, grid, c->stream); break;
-  }
-  c->launches += 1;
-  return st;
-}
-
-pe_status fine_tc_status(pe_ctx* c) {
-  if (!c->tc_err) return PE_OK;
-  int herr = 0;
-  PE_CUDA_TRY(cudaMemcpyAsync(&herr, c->tc_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  PE_CUDA_TRY(cudaStreamSynchronize(c->stream));
-  if (herr != 0) {
-    cudaMemsetAsync(c->tc_err, 0, sizeof(int), c->stream);
-    return pe_fail(PE_ETIMEOUT, "fine sweep (tensor cores): a pipeline wait expired (code " + std::to_string(herr) + ")");
-  }
-  return PE_OK;
 }
 
 // ---------------------------------------------------------------------------

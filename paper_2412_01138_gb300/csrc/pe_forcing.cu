@@ -6,103 +6,177 @@
 // of 1D loads F_a[k] = int g_a phi_k, so
 //   ghat_J(t) = sum_r amp_r time_r(t) prod_a (S_a F_{r,a})_{j_a} / mu^M_a(j_a).
 // 1D loads use a Gauss-Legendre rule with quad_pts points on each element.
-// The per-axis modal factors, the time factors of the coarse stages and of the
-// fine substep starts, and the per-mode stage weights of the fine step
-// (Eq. (1-7), with the stage sum contracted as described in pe_fine_kernels.cuh)
-// are tabulated here; the sweeps multiply them together on the fly.
+// The per-axis modal factors, the time columns of every slice and the per-mode column weights of
+// the fine propagator and the coarse step (pe_contract.cuh) are tabulated here; the sweeps
+// multiply columns and weights together on the fly.
 #include <math.h>
 
-#include "pe_internal.h"
+#include <algorithm>
+
+#include "pe_contract.cuh"
 #include "pe_forcing_common.cuh"
+#include "pe_internal.h"
+#include "pe_learned.h"
 
 namespace {
 
-// Time tables of one problem, one thread per entry:
-//   AF[(n*M + m)*K + k] = Y_k(T_n + m dt)   (fine substep starts, stage-contracted columns;
-//                                            the float copy AF32 has rows of roundup(K, 4))
-//   AG[(n*p + i)*R + r] = amp_r time_r(T_n + c_i dT)   (coarse stage times)
-//   Z[i*K + k]          = Z_k(c_i dt)       (shift of column k to fine stage i)
-__global__ void time_tables_kernel(TermsDev T, StageCols C, int N, int M, int q, int p, double t0, double dT,
-                                   double dt, Nodes cF, Nodes cG, double* __restrict__ AF,
-                                   float* __restrict__ AF32, double* __restrict__ AG, float* __restrict__ AG32,
-                                   double* __restrict__ Z) {
+// Time tables of one problem, one thread per entry (pe_contract.cuh): the columns Y_k of every
+// slice, the shifts of the fine and coarse nodes, and per term the chain's powers and scale.
+// Float copies (the mixed form): Y as a row of high and one of low parts, KC = roundup(K, 4) long
+// with zeros past K, shifts rounded, chain powers and scales as (hi, lo) pairs.
+__global__ void time_tables_kernel(TermsDev T, StageCols C, ColumnTables D, int N, int M, int q, int p, double t0,
+                                   double dT, double dt, Nodes cF, Nodes cG) {
   pdl_wait();
-  const int R = T.n, K = C.K;
-  const int64_t nf = (int64_t)N * M * K;
-  const int64_t ng = (int64_t)N * p * R;
-  const int64_t nz = (int64_t)q * K;
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < nf) {
-    int64_t rest = idx;
-    const int k = (int)(rest % K); rest /= K;
-    const int m = (int)(rest % M); rest /= M;
-    const int n = (int)rest;
-    const double t = t0 + (double)n * dT + (double)m * dt;
-    const pe_term& tr = T.t[C.term[k]];
-    double v;
-    if (C.kind[k] == 1) v = tr.amp * cos(tr.tp[0] * t + tr.tp[1]);  // partner of a sinusoid
-    else v = tr.amp * eval_time(tr, t);
-    AF[idx] = v;
-    if (AF32) {
-      // float copy padded to KC = roundup(K, 4) columns: [N][M][KC], zeros past K
+  const int R = T.n, K = C.K, steps = chain_steps(M);
+  const int ny = N * K, nf = q * K, ng = p * K;
+  int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < ny) {
+    const int n = e / K, k = e - n * K;
+    const double v = column_value(T.t[C.term[k]], C.kind[k], t0 + (double)n * dT, t0 + (double)(n + 1) * dT);
+    D.Y[e] = v;
+    if (D.Y32) {
       const int KC = (K + 3) & ~3;
-      float* row = AF32 + ((int64_t)n * M + m) * KC;
+      float* row = D.Y32 + (int64_t)n * 2 * KC;
       row[k] = (float)v;
+      row[KC + k] = (float)(v - (double)(float)v);
       if (k == K - 1)
-        for (int e = K; e < KC; ++e) row[e] = 0.f;
+        for (int z = K; z < KC; ++z) row[z] = row[KC + z] = 0.f;
     }
-  } else if (idx < nf + ng) {
-    int64_t rest = idx - nf;
-    const int r = (int)(rest % R); rest /= R;
-    const int i = (int)(rest % p); rest /= p;
-    const int n = (int)rest;
-    const double Tn = t0 + (double)n * dT;
-    const double t = Tn + cG.c[i] * dT;
-    const double v = T.t[r].amp * eval_time(T.t[r], t);
-    AG[idx - nf] = v;
-    if (AG32) AG32[idx - nf] = (float)v;
-  } else if (idx < nf + ng + nz) {
-    const int64_t e = idx - nf - ng;
-    const int k = (int)(e % K), i = (int)(e / K);
-    const pe_term& tr = T.t[C.term[k]];
-    const double s = cF.c[i] * dt;
-    double v;
-    if (tr.tkind == PE_T_SIN) v = C.kind[k] == 1 ? sin(tr.tp[0] * s) : cos(tr.tp[0] * s);
-    else v = exp(tr.tp[0] * s);
-    Z[e] = v;
+    return;
+  }
+  e -= ny;
+  if (e < nf + ng) {
+    const bool fine = e < nf;
+    const int l = fine ? e : e - nf, i = l / K, k = l - i * K;
+    const double v = column_shift(T.t[C.term[k]], C.kind[k], fine ? cF.c[i] : cG.c[i], fine ? dt : dT);
+    (fine ? D.ZF : D.ZG)[l] = v;
+    if (D.Y32) (fine ? D.ZF32 : D.ZG32)[l] = (float)v;
+    return;
+  }
+  e -= nf + ng;
+  if (e >= R * (steps + 1)) return;
+  const int s = e / R - 1, r = e - (s + 1) * R;
+  if (s < 0) {
+    const double v = chain_scale(T.t[r], dt);
+    D.xs[r] = v;
+    if (D.Y32) {
+      D.xs32[2 * r] = (float)v;
+      D.xs32[2 * r + 1] = (float)(v - (double)(float)v);
+    }
+    return;
+  }
+  double v[4];
+  const int L = chain_length(M, steps, s);
+  chain_power(T.t[r], L, dt, v[0], v[1]);
+  chain_power(T.t[r], 2 * L, dt, v[2], v[3]);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    D.chain[(s * R + r) * 4 + i] = v[i];
+    if (D.Y32) {
+      D.chain32[(s * R + r) * 8 + 2 * i] = (float)v[i];
+      D.chain32[(s * R + r) * 8 + 2 * i + 1] = (float)(v[i] - (double)(float)v[i]);
+    }
   }
 }
 
-// W[k*ndof + J] = P_{r(k),J} sum_i (dt b_i)_J Z[i*K + k], with P_{r,J} = prod_a axisF[R off_a + r n_a + j_a],
-// in the arithmetic of T (coefficient row i of dt b_i at coef + i * ndof).
+// Per-mode column weights: V[k * ndof + J] of the fine propagator's slice sum and G[k * ndof + J]
+// of the coarse step (sum_i dT b^G_i Z_k(c_i dT), plus the learned correction's P K^ on the
+// columns of a sinusoid), P_{r,J} = prod_a axisF.  A thread takes TPT consecutive terms of one
+// mode.  T = float (mixed form): float32 weights from float32 factors, the chain in float pairs.
+// coef: E (float: hi and lo rows), then the q rows dt b_i; coefG: the p rows dT b^G_i.
 template <typename T>
-__global__ void stage_weights_kernel(Geom g, StageCols C, int R, int q, const T* __restrict__ axisF,
-                                     const T* __restrict__ coef, const double* __restrict__ Z, T* __restrict__ W) {
+__global__ void __launch_bounds__(256) column_weights_kernel(Geom g, StageCols C, ColumnTables D, int R, int M, int q,
+                                                             int p, int tpt, const T* __restrict__ axisF,
+                                                             const T* __restrict__ coef, const T* __restrict__ coefG,
+                                                             T* __restrict__ V, T* __restrict__ G, LearnedTerms L,
+                                                             const double* __restrict__ axisF64,
+                                                             const double* __restrict__ lam) {
   pdl_wait();
-  // the shifts Z (converted to T once per CTA) and the column -> term map, in shared memory
-  __shared__ T sZ[PE_MAX_S * 2 * PE_MAX_TERMS];
-  __shared__ int sTerm[2 * PE_MAX_TERMS];
-  for (int e = threadIdx.x; e < q * C.K; e += blockDim.x) sZ[e] = (T)Z[e];
-  for (int e = threadIdx.x; e < C.K; e += blockDim.x) sTerm[e] = C.term[e];
-  __syncthreads();
+  constexpr bool F64 = sizeof(T) == 8;
   const int64_t J = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (J >= g.ndof) return;
   const int64_t nd = g.ndof;
+  const int K = C.K, steps = chain_steps(M);
+  const T* ZF;
+  const T* ZG;
+  if constexpr (F64) {
+    ZF = D.ZF;
+    ZG = D.ZG;
+  } else {
+    ZF = D.ZF32;
+    ZG = D.ZG32;
+  }
   int j[PE_MAX_D];
   unflatten(g, J, j);
-  T b[PE_MAX_S];
+  T b[PE_MAX_S], bg[PE_MAX_S];
+  constexpr int kERows = F64 ? 1 : 2;
 #pragma unroll
-  for (int i = 0; i < PE_MAX_S; ++i) b[i] = i < q ? coef[(int64_t)i * nd + J] : T(0);
-  for (int k = 0; k < C.K; ++k) {
-    const int r = sTerm[k];
+  for (int i = 0; i < PE_MAX_S; ++i) {
+    b[i] = i < q ? coef[(int64_t)(kERows + i) * nd + J] : T(0);
+    bg[i] = G && i < p ? coefG[(int64_t)i * nd + J] : T(0);
+  }
+  const T Eh = coef[J];
+  T El = T(0);
+  if constexpr (!F64) El = coef[nd + J];
+  int band = 0;
+  double bf = 0.0;
+  if (L.Ktab) {
+    double pos = (log(lam[J] * L.dT) - L.loglo) / L.logstep;
+    pos = fmin(fmax(pos, 0.0), (double)(L.NB - 1) - 1e-9);
+    band = (int)pos;
+    bf = pos - (double)band;
+  }
+  const int r1 = min(R, (int)(blockIdx.y + 1) * tpt);
+  for (int r = blockIdx.y * tpt; r < r1; ++r) {
+    const int k = C.first[r];
+    const bool two = k + 1 < K && C.term[k + 1] == r;
     T P = axisF[(int64_t)R * g.off[0] + (int64_t)r * g.n[0] + j[0]];
 #pragma unroll
     for (int a = 1; a < PE_MAX_D; ++a) if (a < g.d) P *= axisF[(int64_t)R * g.off[a] + (int64_t)r * g.n[a] + j[a]];
-    T s = T(0);
+    T br = T(0), bi = T(0), gr = T(0), gi = T(0);
 #pragma unroll
     for (int i = 0; i < PE_MAX_S; ++i)
-      if (i < q) s = fma(b[i], sZ[i * C.K + k], s);
-    W[(int64_t)k * nd + J] = P * s;
+      if (i < q) {
+        br = fma(b[i], ZF[i * K + k], br);
+        if (two) bi = fma(b[i], ZF[i * K + k + 1], bi);
+      }
+    if (G) {
+#pragma unroll
+      for (int i = 0; i < PE_MAX_S; ++i)
+        if (i < p) {
+          gr = fma(bg[i], ZG[i * K + k], gr);
+          if (two) gi = fma(bg[i], ZG[i * K + k + 1], gi);
+        }
+      gr *= P;
+      gi *= P;
+      if (L.Ktab && two) {
+        double Pd = axisF64[(int64_t)R * g.off[0] + (int64_t)r * g.n[0] + j[0]];
+#pragma unroll
+        for (int a = 1; a < PE_MAX_D; ++a) if (a < g.d)
+          Pd *= axisF64[(int64_t)R * g.off[a] + (int64_t)r * g.n[a] + j[a]];
+        const double* k0 = L.Ktab + 2 * ((int64_t)r * L.NB + band);
+        gr += (T)(Pd * ((1.0 - bf) * k0[0] + bf * k0[2]));
+        gi += (T)(Pd * ((1.0 - bf) * k0[1] + bf * k0[3]));
+      }
+      G[(int64_t)k * nd + J] = gr;
+      if (two) G[(int64_t)(k + 1) * nd + J] = gi;
+    }
+    T v0, v1;
+    if constexpr (F64) {
+      double Sr, Si;
+      chain_sum(Eh * D.xs[r], M, steps, D.chain + 4 * r, 4 * R, Sr, Si);
+      v0 = P * fma(br, Sr, -(bi * Si));
+      v1 = P * fma(br, Si, bi * Sr);
+    } else {
+      F2 Sr, Si;
+      chain_sum(f2_mul(F2{Eh, El}, F2{D.xs32[2 * r], D.xs32[2 * r + 1]}), M, steps, D.chain32 + 8 * r, 8 * R, Sr, Si);
+      const F2 B{br, 0.f}, C2{bi, 0.f};
+      const F2 re = f2_add(f2_mul(B, Sr), f2_neg(f2_mul(C2, Si))), im = f2_add(f2_mul(B, Si), f2_mul(C2, Sr));
+      v0 = fmaf(P, re.h, P * re.l);
+      v1 = fmaf(P, im.h, P * im.l);
+    }
+    V[(int64_t)k * nd + J] = v0;
+    if (two) V[(int64_t)(k + 1) * nd + J] = v1;
   }
 }
 
@@ -258,9 +332,10 @@ pe_status launch_time_tables(pe_ctx* c) {
     nF.c[i] = c->cF[i];
     nG.c[i] = c->cG[i];
   }
-  // stage-contracted columns: one per exponential term, two per sinusoid
+  // columns: one per exponential term, two per sinusoid
   StageCols C{};
   for (int r = 0; r < R; ++r) {
+    C.first[r] = (signed char)C.K;
     C.term[C.K] = (signed char)r;
     C.kind[C.K++] = 0;
     if (c->terms[r].tkind == PE_T_SIN) {
@@ -270,69 +345,82 @@ pe_status launch_time_tables(pe_ctx* c) {
   }
   c->cols = C;
   c->K = C.K;
-  const int64_t total = (int64_t)c->N * c->M * C.K + (int64_t)c->N * c->p * R + (int64_t)c->q * C.K;
-  const int threads = 256;
+  const int total = c->N * C.K + (c->q + c->p) * C.K + R * (chain_steps(c->M) + 1);
+  const int threads = 128;
   PE_CUDA_TRY(launch_pdl(time_tables_kernel, dim3((unsigned)((total + threads - 1) / threads)), dim3(threads), 0,
-                         c->stream, T, C, c->N, c->M, c->q, c->p, c->t0, c->dT, c->dt, nF, nG, c->AF,
-                         c->precision == PE_MIXED ? c->AF32 : (float*)nullptr, c->AG,
-                         c->precision == PE_MIXED ? c->AG32 : (float*)nullptr, c->Zst));
+                         c->stream, T, C, c->tab, c->N, c->M, c->q, c->p, c->t0, c->dT, c->dt, nF, nG));
   c->launches += 1;
   PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;
 }
 
-pe_status launch_stage_weights(pe_ctx* c) {
+// Room for the weights of K columns: float64 (V64, and G64 when `coarse`), float32 (V32, G32).
+template <typename T>
+static pe_status grow_weights(pe_ctx* c, T** V, T** G, int* cap) {
   const int K = c->K;
-  if (K > c->Wcap) {
-    // grown on demand (first problem, or a problem with more columns than before)
-    PE_CUDA_TRY(cudaStreamSynchronize(c->stream));
-    if (c->Wst) cudaFree(c->Wst);
-    if (c->Wst32) cudaFree(c->Wst32);
-    c->Wst = nullptr;
-    c->Wst32 = nullptr;
-    c->Wcap = 0;
-    const size_t n = (size_t)K * (size_t)c->g.ndof;
-    if (cudaMalloc((void**)&c->Wst, n * sizeof(double)) != cudaSuccess ||
-        (c->precision == PE_MIXED && cudaMalloc((void**)&c->Wst32, n * sizeof(float)) != cudaSuccess)) {
-      cudaGetLastError();
-      return pe_fail(PE_ENOMEM, "pe_set_problem: stage-weight table allocation failed");
-    }
-    c->Wcap = K;
+  if (K <= *cap) return PE_OK;
+  PE_CUDA_TRY(cudaStreamSynchronize(c->stream));
+  if (*V) cudaFree(*V);
+  if (G && *G) cudaFree(*G);
+  *V = nullptr;
+  if (G) *G = nullptr;
+  *cap = 0;
+  const size_t n = (size_t)K * (size_t)c->g.ndof;
+  if (cudaMalloc((void**)V, n * sizeof(T)) != cudaSuccess ||
+      (G && cudaMalloc((void**)G, n * sizeof(T)) != cudaSuccess)) {
+    cudaGetLastError();
+    return pe_fail(PE_ENOMEM, "pe_set_problem: column-weight table allocation failed");
   }
-  const int threads = 256;
-  const unsigned blocks = (unsigned)((c->g.ndof + threads - 1) / threads);
-  if (c->precision == PE_MIXED && c->fine_engine == PE_FINE_TC && c->forcing_path == PE_FORCING_SEPARABLE) {
-    // the tensor-core engine forms its float32 weights inside its operand split
-    // (fine_tc_prepare); the float64 ones follow on the first float64 sweep (pe_refine)
-    c->Wst_valid = false;
-    return PE_OK;
-  }
+  *cap = K;
+  return PE_OK;
+}
+
+// Terms per thread of the weights kernel: one while the modes alone leave the GPU short of warps
+// (each term's chain is a serial run of its own), then a few, so that the tables of the mode are
+// read less often; all of them with the learned correction, whose band position costs a logarithm.
+static int weights_tpt(const pe_ctx* c, bool learned) {
+  if (learned) return c->R;
+  return c->g.ndof < ((int64_t)1 << 19) ? 1 : std::min(c->R, 4);
+}
+
+pe_status launch_column_weights(pe_ctx* c) {
+  LearnedTerms L{};
+  if (c->mlp) PE_TRY(launch_learned_tables(c, &L));
+  const int threads = 256, tpt = weights_tpt(c, c->mlp != nullptr);
+  const dim3 grid((unsigned)((c->g.ndof + threads - 1) / threads), (unsigned)((c->R + tpt - 1) / tpt));
+  c->V64_valid = false;
   if (c->precision == PE_MIXED) {
-    // the float32 fine sweeps need only the float32 weights; the float64 ones follow on the
-    // first float64 sweep (pe_refine)
-    PE_CUDA_TRY(launch_pdl(stage_weights_kernel<float>, dim3(blocks), dim3(threads), 0, c->stream, c->g, c->cols, c->R,
-                           c->q, (const float*)c->axisF32, (const float*)(c->coefF32 + 2 * c->g.ndof),
-                           (const double*)c->Zst, c->Wst32));
-    c->Wst_valid = false;
+    // the float32 sweeps need only float32 weights; pe_refine makes its float64 ones
+    PE_TRY(grow_weights(c, &c->V32, &c->G32, &c->cap32));
+    PE_CUDA_TRY(launch_pdl(column_weights_kernel<float>, grid, dim3(threads), 0, c->stream, c->g, c->cols, c->tab,
+                           c->R, c->M, c->q, c->p, tpt, (const float*)c->axisF32, (const float*)c->coefF32,
+                           (const float*)c->coefG32, c->V32, c->G32, L, (const double*)c->axisF,
+                           (const double*)c->lam));
   } else {
-    PE_CUDA_TRY(launch_pdl(stage_weights_kernel<double>, dim3(blocks), dim3(threads), 0, c->stream, c->g, c->cols,
-                           c->R, c->q, (const double*)c->axisF, (const double*)(c->coefF + c->g.ndof),
-                           (const double*)c->Zst, c->Wst));
-    c->Wst_valid = true;
+    PE_TRY(grow_weights(c, &c->V64, &c->G64, &c->cap64));
+    PE_CUDA_TRY(launch_pdl(column_weights_kernel<double>, grid, dim3(threads), 0, c->stream, c->g, c->cols, c->tab,
+                           c->R, c->M, c->q, c->p, tpt, (const double*)c->axisF, (const double*)c->coefF,
+                           (const double*)(c->coefG + c->g.ndof), c->V64, c->G64, L, (const double*)c->axisF,
+                           (const double*)c->lam));
+    c->V64_valid = true;
   }
   c->launches += 1;
   PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;
 }
 
-pe_status launch_stage_weights_f64(pe_ctx* c) {
-  if (c->Wst_valid) return PE_OK;
-  const int threads = 256;
-  stage_weights_kernel<double><<<(unsigned)((c->g.ndof + threads - 1) / threads), threads, 0, c->stream>>>(
-      c->g, c->cols, c->R, c->q, c->axisF, c->coefF + c->g.ndof, c->Zst, c->Wst);
+pe_status launch_column_weights_f64(pe_ctx* c) {
+  if (c->V64_valid) return PE_OK;
+  PE_TRY(grow_weights(c, &c->V64, (double**)nullptr, &c->cap64));
+  const int threads = 256, tpt = weights_tpt(c, false);
+  const dim3 grid((unsigned)((c->g.ndof + threads - 1) / threads), (unsigned)((c->R + tpt - 1) / tpt));
+  PE_CUDA_TRY(launch_pdl(column_weights_kernel<double>, grid, dim3(threads), 0, c->stream, c->g, c->cols, c->tab,
+                         c->R, c->M, c->q, c->p, tpt, (const double*)c->axisF, (const double*)c->coefF,
+                         (const double*)nullptr, c->V64, (double*)nullptr, LearnedTerms{}, (const double*)c->axisF,
+                         (const double*)c->lam));
   c->launches += 1;
   PE_CUDA_TRY(cudaGetLastError());
-  c->Wst_valid = true;
+  c->V64_valid = true;
   return PE_OK;
 }
 

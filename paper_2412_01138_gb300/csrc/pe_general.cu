@@ -8,7 +8,8 @@
 // every axis (batched over the stage times of a chunk of slices), and (iii) folds
 // Lambda_M^{-1} into the stage weights of the fine and coarse recurrences.  The
 // fine propagator then reads ghat(t) from HBM instead of forming it from
-// per-axis factors: the step is memory-bound, and the transform dominates.
+// per-axis factors: the step is memory-bound, and the transform dominates.  It is started from
+// zero: the walk over the slices adds e^{-lam M dt} U (pe_sweep.cu).
 // In the mixed form the fine sweep's loads, assembly and transforms run in
 // float32 (the coarse forcing, computed once per problem, stays float64).
 //
@@ -188,12 +189,12 @@ __global__ void __launch_bounds__(256) gen_assemble_kernel(TermsDev T, Geom g, S
   }
 }
 
-// fine propagator from the stored transformed loads: Gh[(n - n0) M q + m q + i][J] = (V^T F)_J
+// F^M(0) from the stored transformed loads: Gh[(n - n0) M q + m q + i][J] = (V^T F)_J
 __global__ void __launch_bounds__(256) gen_fine_f64_kernel(Geom g, int n0, int M, int q,
                                                           const double* __restrict__ muM_axis,
                                                           const double* __restrict__ coefF,
                                                           const double* __restrict__ Gh,
-                                                          const double* __restrict__ U, double* __restrict__ Fbar) {
+                                                          double* __restrict__ Fbar) {
   const int n = n0 + blockIdx.y;
   const int64_t nd = g.ndof;
   const int64_t J = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -208,7 +209,7 @@ __global__ void __launch_bounds__(256) gen_fine_f64_kernel(Geom g, int n0, int M
 #pragma unroll
   for (int i = 0; i < PE_MAX_S; ++i)
     if (i < q) b[i] = coefF[(1 + i) * nd + J] / mu;
-  double c = U[(int64_t)n * nd + J];
+  double c = 0.0;
   const double* Gs = Gh + (int64_t)blockIdx.y * M * q * nd + J;
   for (int m = 0; m < M; ++m) {
     double acc = 0.0;
@@ -225,7 +226,6 @@ __global__ void __launch_bounds__(256) gen_fine_mixed_kernel(Geom g, int n0, int
                                                             const double* __restrict__ coefF,
                                                             const float* __restrict__ coefF32,
                                                             const float* __restrict__ Gh,
-                                                            const double* __restrict__ U,
                                                             double* __restrict__ Fbar) {
   const int n = n0 + blockIdx.y;
   const int64_t nd = g.ndof;
@@ -250,8 +250,7 @@ __global__ void __launch_bounds__(256) gen_fine_mixed_kernel(Geom g, int n0, int
       if (i < q) acc = fmaf(b[i], Gs[(int64_t)(m * q + i) * nd], acc);
     w = fmaf(eh, w, fmaf(el, w, acc));
   }
-  const double EM = coefF[(int64_t)(q + 1) * nd + J];
-  Fbar[(int64_t)n * nd + J] = fma(EM, U[(int64_t)n * nd + J], (double)w);
+  Fbar[(int64_t)n * nd + J] = (double)w;
 }
 
 // coarse forcing gG[n][J] = sum_i (dT b_i / mu_J) (V^T F(T_n + c_i dT))_J
@@ -372,11 +371,11 @@ pe_status launch_general_fine_sweep(pe_ctx* c, int precision) {
       float* tmp = reinterpret_cast<float*>(c->gen_tmp);
       PE_TRY(stage_transforms<float>(c, SG, count, out, tmp));
       gen_fine_mixed_kernel<<<grid, 256, 0, c->stream>>>(c->g, n0, c->M, c->q, c->muM_axis, c->coefF, c->coefF32,
-                                                          out, c->U, c->Fbar);
+                                                          out, c->Fbar);
     } else {
       PE_TRY(stage_transforms<double>(c, SG, count, c->gen_buf, c->gen_tmp));
       gen_fine_f64_kernel<<<grid, 256, 0, c->stream>>>(c->g, n0, c->M, c->q, c->muM_axis, c->coefF, c->gen_buf,
-                                                        c->U, c->Fbar);
+                                                        c->Fbar);
     }
     c->launches += 1;
     PE_CUDA_TRY(cudaGetLastError());

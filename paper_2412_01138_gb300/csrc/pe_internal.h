@@ -67,19 +67,25 @@ __host__ __device__ inline void unflatten(const Geom& g, int64_t J, int* j) {
     }
 }
 
-// Separable forcing, device layout (R terms, K stage-contracted columns):
-//   axisF[R * off[a] + r * n_a + j]         = modal factor (S_a F_{r,a})_j / mu^M_a(j)
-//   AF[(n * M + m) * K + k]                 = Y_k(T_n + m dt)   (substep-start time factors)
-//   Zst[i * K + k]                          = Z_k(c_i dt)       (stage shifts)
-//   Wst[k * ndof + J]                       = P_{r(k),J} sum_i dt b_i(J) Z_k(c_i dt)
-//   AG[(n * p + i) * R + r]                 = amp_r * time_r(T_n + c_i dT)
-// Column k belongs to term colTerm[k]: an exponential time factor gives one
-// column (Y = amp e^{at}, Z = e^{as}); a sinusoid gives two (kind 0:
-// Y = amp sin(wt+phi), Z = cos(ws); kind 1: Y = amp cos(wt+phi), Z = sin(ws)).
+// Separable forcing, device layout (R terms, K columns, pe_contract.cuh):
+//   axisF[R * off[a] + r * n_a + j]  = modal factor (S_a F_{r,a})_j / mu^M_a(j)
+//   V[k * ndof + J], G[k * ndof + J] = per-mode weights of column k in the fine propagator's
+//                                      slice sum and in the coarse step
+// Column k belongs to term term[k]: an exponential time factor gives one column, a sinusoid two
+// (kind 0 the sine, kind 1 its cosine partner); first[r] is the first column of term r.
 struct StageCols {
   int K;
   signed char term[2 * PE_MAX_TERMS];
   signed char kind[2 * PE_MAX_TERMS];
+  signed char first[PE_MAX_TERMS];
+};
+// Time tables of the columns (time_tables_kernel): Y [N][K] column values of every slice, ZF [q][K]
+// and ZG [p][K] shifts of the fine and coarse nodes, chain [steps][R][4] and xs [R] the powers and
+// scales of the slice sum; the float forms (null unless mixed): Y32 [N][2][roundup(K, 4)] (high and low
+// parts), chain32 and xs32 as (hi, lo) pairs.
+struct ColumnTables {
+  double *Y, *ZF, *ZG, *chain, *xs;
+  float *Y32, *ZF32, *ZG32, *chain32, *xs32;
 };
 // Device-resident state of a solve whose Parareal loop runs as a CUDA graph (device_loop):
 // the correction kernel's last CTA appends r_k, advances k and sets the graph's loop condition.
@@ -113,7 +119,6 @@ struct pe_ctx {
   void* reduce_user = nullptr;
   // options
   int precision, dst_backend, quad_pts, max_iter, forcing_path, cache_forced;
-  int fine_engine = 0;  // PE_FINE_SIMT | PE_FINE_TC
   cudaStream_t stream;
   // device memory
   double* muM_axis = nullptr;   // [nsum]
@@ -128,12 +133,13 @@ struct pe_ctx {
   double* coefF = nullptr;      // [(q+2) * ndof]: E, dt*b_1..q, exp(-lam M dt)
   double* coefG = nullptr;      // [(p+1) * ndof]: E, dT*b_1..p
   float* coefF32 = nullptr;     // [(q+2) * ndof]: E_hi, E_lo, dt*b_i (float)
+  float* coefG32 = nullptr;     // [p * ndof]: dT*b_i of the coarse step (float)
   double* U = nullptr;          // [(N+1) * ndof]
   double* Fz = nullptr;         // [N * ndof] cached F^M(0) per slice (cache_forced)
   int fz_prec = -1;             // precision Fz was computed in, -1: none for this problem
   int64_t sweeps = 0;           // fine sweeps executed since the last reset
-  double* Fbar = nullptr;       // [N * ndof]
-  double* gG = nullptr;         // [N * ndof] coarse forcing of each slice
+  double* Fbar = nullptr;       // [N * ndof] F^M(0) of each slice (float64 and general sweeps)
+  double* gG = nullptr;         // [N * ndof] coarse forcing of each slice (float64 and general)
   double* work0 = nullptr;      // [gn.ndof] nodal / DST scratch
   double* work1 = nullptr;      // [gn.ndof]
   float* io32 = nullptr;        // [3 gn.ndof] float32 transform scratch of the mixed form (null: float64 transforms)
@@ -142,11 +148,6 @@ struct pe_ctx {
   double* partials = nullptr;   // [2 * max_blocks]
   double* red = nullptr;        // [2] device
   unsigned int* done_ctr = nullptr;  // correction: CTAs finished (0 between launches)
-  unsigned char* tcB = nullptr;  // tensor-core fine engine: split time factors of every slice group
-  unsigned char* tcA = nullptr;  // tensor-core fine engine: split stage weights of every mode tile
-  size_t tcA_cap = 0;            // bytes allocated in tcA
-  bool tc_split_ok = false;      // tcA / tcB hold the current problem's split operands
-  int* tc_err = nullptr;         // tensor-core fine engine: error code of an expired wait (0: none)
   cudaStream_t side = nullptr;  // second stream: the nodal u0 transform beside the forcing tables
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_tables = nullptr;
   double* h_red = nullptr;      // [2] pinned host
@@ -162,22 +163,21 @@ struct pe_ctx {
   double* axisF = nullptr;      // [PE_MAX_TERMS * nsum]
   float* axisF32 = nullptr;     // [PE_MAX_TERMS * nsum]
   double* axisU0 = nullptr;     // [PE_MAX_TERMS * nsum] factors of separable u0
-  double* AF = nullptr;         // [N*M*2*PE_MAX_TERMS]
-  float* AF32 = nullptr;
-  int K = 0;                    // stage-contracted columns of the current forcing
+  int K = 0;                    // columns of the current forcing
   StageCols cols{};
-  double* Zst = nullptr;        // [PE_MAX_S * 2*PE_MAX_TERMS]
-  double* Wst = nullptr;        // [K * ndof] (allocated on first use, grown with K)
-  float* Wst32 = nullptr;       // [K * ndof] (mixed precision)
-  int Wcap = 0;                 // columns allocated in Wst / Wst32
-  bool Wst_valid = false;       // Wst holds the current problem's float64 weights
-  double* AG = nullptr;         // [N*p*PE_MAX_TERMS]
-  float* AG32 = nullptr;
+  ColumnTables tab{};           // its time tables
+  double *tab64 = nullptr;      //   their storage
+  float *tab32 = nullptr;
+  // column weights [K * ndof], allocated on first use and grown with K: float64 (the float64 form;
+  // of a mixed context V64 alone, for pe_refine) and float32 (mixed)
+  double *V64 = nullptr, *G64 = nullptr;
+  float *V32 = nullptr, *G32 = nullptr;
+  int cap64 = 0, cap32 = 0;     // columns allocated
+  bool V64_valid = false;       // V64 holds the current problem's weights
   double* loads = nullptr;      // [PE_MAX_TERMS * nsum_full] 1D loads before the DST
   // learned coarse correction (optional)
   const struct pe_mlp* mlp = nullptr;
   double* Ktab = nullptr;       // [PE_MAX_TERMS][bands][2]
-  void* phase_tab = nullptr;    // [PE_MAX_TERMS][N] float2
   // accounting
   int64_t launches = 0;     // kernels launched since the last reset
   double ms_fine = 0.0;     // device time of fine-propagator kernels since the last reset
@@ -191,7 +191,8 @@ struct pe_ctx {
   int device_loop = 0;
   cudaGraphExec_t loop_exec = nullptr;
   int loop_K = -1, loop_prec = -1;  // what the graph was built for
-  int64_t loop_body_launches = 0;   // kernels of one pass of the graph's body
+  int64_t loop_first_launches = 0;  // kernels of the graph's first iteration
+  int64_t loop_body_launches = 0;   // kernels of one pass of the loop's body
   LoopCtl* loopctl = nullptr;       // device
   LoopCtl* h_loop = nullptr;        // mapped pinned mirror of the loop state (host address)
   LoopCtl* h_loop_dev = nullptr;    //   its device address
@@ -234,9 +235,9 @@ pe_status build_dst_matrix(int n, double* S, cudaStream_t st, int periodic = 0);
 pe_status build_dst_matrix_f32(int n, float* S, cudaStream_t st, int periodic = 0);
 
 // pe_forcing.cu
-pe_status launch_time_tables(pe_ctx* c);   // also sets c->K, c->cols and Zst
-pe_status launch_stage_weights(pe_ctx* c);  // Wst (float64 form) or Wst32 (mixed form)
-pe_status launch_stage_weights_f64(pe_ctx* c);  // Wst, if not yet made for this problem
+pe_status launch_time_tables(pe_ctx* c);   // also sets c->K and c->cols
+pe_status launch_column_weights(pe_ctx* c);  // V64 and G64 (float64 form) or V32 and G32 (mixed form)
+pe_status launch_column_weights_f64(pe_ctx* c);  // V64, if not yet made for this problem
 // rows of whole-axis per-axis tables [R * nsum_full] kept by a sharded context, in its layout
 pe_status compact_axis_tables(pe_ctx* c, int R, const double* in, double* out, float* out32);
 pe_status launch_separable_factors(pe_ctx* c, const pe_term* terms, int nterms, double* axis_out, int mode,
@@ -260,34 +261,35 @@ pe_status dst_nd_mixed(pe_ctx* c, const double* in, double* out);  // whole grid
 pe_status axis_factors_fused(pe_ctx* c, int R, const double* loads, double* fac, float* fac32, bool* done);
 
 // pe_sweep.cu
-pe_status launch_coarse_sweep(pe_ctx* c);
-pe_status launch_fine_sweep(pe_ctx* c, int precision);
-pe_status launch_correction(pe_ctx* c, double* num, double* den, cudaEvent_t after = nullptr);
-// the correction kernel alone; with loop != NULL its last CTA also runs the stopping decision of a
-// device-resident loop (appends r, advances k, sets the graph condition `handle`)
-pe_status launch_correction_kernel(pe_ctx* c, LoopCtl* loop, unsigned long long handle);
+pe_status launch_coarse_sweep(pe_ctx* c);  // k = 0
+// One iteration (fine sweep from every slice, correction, residual sums).  first: from the coarse
+// iterate made in the same pass (nothing in U but U^0 is read).  loop != NULL: the last CTA also
+// runs the stopping decision of a device-resident loop (appends r, advances k, sets the graph
+// condition `handle`).  mid (may be null): recorded between the forced part and the walk.
+pe_status launch_iteration(pe_ctx* c, int precision, bool first, LoopCtl* loop, unsigned long long handle,
+                           cudaEvent_t mid = nullptr);
+// pe_forced.cu: F^M(0) of every slice into f and the coarse forcing into gG (either may be null)
+pe_status launch_forced_f64(pe_ctx* c, double* f, double* gG);
+bool first_fused(const pe_ctx* c);  // pe_solve makes the coarse iterate in the first iteration's pass
+pe_status read_sums(pe_ctx* c, double* num, double* den, cudaEvent_t after);  // waits for the stream
 // Arms the device-resident loop's state for one solve (k = 0, tol, the history, the mirror).
 pe_status launch_loop_init(pe_ctx* c, double tol);
 pe_status launch_scale_by_muM(pe_ctx* c, double* x, int inverse);
-
-// pe_learned.cu
-pe_status launch_learned_correction(pe_ctx* c);
 
 // pe_general.cu
 int general_slices_per_chunk(const pe_ctx* c);
 pe_status launch_general_coarse_forcing(pe_ctx* c);
 pe_status launch_general_fine_sweep(pe_ctx* c, int precision);
 
-// pe_fine_tc.cu (tensor-core engine of the mixed fine sweep)
-bool fine_tc_supported(int M);                 // M a multiple of 16 in 16..128
-size_t fine_tc_buffer_bytes(int M, int N);     // split time factors, any K <= 64
-// Threads per CTA of a kernel with one thread per mode: when the modes fit one wave of CTAs,
-// as many warps as an even share of the SMs needs (every SM then runs one CTA of equal size,
-// rather than some SMs two CTAs of 256 threads and others one); 256 otherwise.
-inline int per_mode_block(int64_t units, int sms) {
+// Threads per CTA (at most cap) of a kernel with one thread per mode: when the modes fit one
+// wave of CTAs of up to 512 threads per SM, as many warps as an even share of the SMs needs (every
+// SM then runs CTAs of equal size, rather than some SMs two CTAs of 256 threads and others one);
+// 256 otherwise.
+inline int per_mode_block(int64_t units, int sms, int cap = 512) {
   if (sms <= 0) return 256;
-  const int64_t per_sm = (units + sms - 1) / sms;
+  int64_t per_sm = (units + sms - 1) / sms;
   if (per_sm > 512) return 256;
+  if (per_sm > cap) per_sm = (per_sm + 1) / 2;
   const int64_t t = (per_sm + 31) / 32 * 32;
   return (int)(t < 64 ? 64 : t);
 }
@@ -335,8 +337,3 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
 
 // Drops the cached set-up and output graphs of a repeated problem (pe_api.cu).
 void drop_solve_graphs(pe_ctx* c);
-pe_status fine_tc_prepare(pe_ctx* c);          // split operand images of the current problem
-pe_status fine_tc_prepare_time(pe_ctx* c);     //   the time factors' image (after the time tables)
-pe_status fine_tc_prepare_weights(pe_ctx* c);  //   the stage weights' image (after tables and factors)
-pe_status launch_fine_tc(pe_ctx* c, int from_zero, double* out);
-pe_status fine_tc_status(pe_ctx* c);           // PE_ETIMEOUT if a pipeline wait expired

@@ -493,64 +493,6 @@ __global__ void band_table_kernel(const __half* __restrict__ params16, TermsW T,
   Ktab[2 * idx + 1] = Kim;
 }
 
-// cs[r][n] = (cos, sin)(w_r T_n + phi_r)
-__global__ void phase_table_kernel(TermsW T, int N, double dT, double t0, float2* __restrict__ cs) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= T.R * N) return;
-  const int r = idx / N, n = idx % N;
-  double s, co;
-  sincos(T.omega[r] * (t0 + (double)n * dT) + T.phase[r], &s, &co);
-  cs[idx] = make_float2((float)co, (float)s);
-}
-
-// gG[n][J] += sum_r P_{r,J} amp_r Im(e^{i(w_r T_n + phi_r)} K^(lam_J, w_r)) with K^ interpolated
-// linearly in log(lam dT) between band centres.  Per mode the r-sum reduces to
-// sum_r (A_r cos_{r,n} + B_r sin_{r,n}), A_r = P amp Im K^, B_r = P amp Re K^, evaluated in
-// float32 (delta^ is a prediction; only its size relative to tol matters).
-__global__ void __launch_bounds__(256) learned_correction_kernel(Geom g, int N, int R, int NB, double loglo,
-                                                                 double logstep, double dT, TermsW T,
-                                                                 const double* __restrict__ lam,
-                                                                 const double* __restrict__ axisF,
-                                                                 const double* __restrict__ Ktab,
-                                                                 const float2* __restrict__ cs,
-                                                                 double* __restrict__ gG) {
-  extern __shared__ float sAB[];  // [2R][blockDim]
-  const int64_t J = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (J >= g.ndof) return;
-  const int64_t nd = g.ndof;
-  const int tid = threadIdx.x, B = blockDim.x;
-  int j[PE_MAX_D];
-  unflatten(g, J, j);
-  double pos = (log(lam[J] * dT) - loglo) / logstep;
-  pos = fmin(fmax(pos, 0.0), (double)(NB - 1) - 1e-9);
-  const int b0 = (int)pos;
-  const double f = pos - (double)b0;
-  for (int r = 0; r < R; ++r) {
-    float A = 0.f, Bv = 0.f;
-    if (T.is_sin[r]) {
-      double P = axisF[(int64_t)R * g.off[0] + (int64_t)r * g.n[0] + j[0]];
-#pragma unroll
-      for (int a = 1; a < PE_MAX_D; ++a) if (a < g.d) P *= axisF[(int64_t)R * g.off[a] + (int64_t)r * g.n[a] + j[a]];
-      const double* k0 = Ktab + 2 * ((int64_t)r * NB + b0);
-      const double Kre = (1.0 - f) * k0[0] + f * k0[2];
-      const double Kim = (1.0 - f) * k0[1] + f * k0[3];
-      const double c = P * T.amp[r];
-      A = (float)(c * Kim);
-      Bv = (float)(c * Kre);
-    }
-    sAB[(2 * r) * B + tid] = A;
-    sAB[(2 * r + 1) * B + tid] = Bv;
-  }
-  for (int n = 0; n < N; ++n) {
-    float d = 0.f;
-    for (int r = 0; r < R; ++r) {
-      const float2 e = __ldg(cs + (int64_t)r * N + n);
-      d = fmaf(sAB[(2 * r) * B + tid], e.x, fmaf(sAB[(2 * r + 1) * B + tid], e.y, d));
-    }
-    gG[(int64_t)n * nd + J] += (double)d;
-  }
-}
-
 // ---------------------------------------------------------------------------
 // batched form: band and phase tables of every problem of a batch, jobs flattened through
 // per-problem prefix tables (the owner of job e is the problem with the largest prefix <= e)
@@ -841,7 +783,7 @@ extern "C" pe_status pe_set_learned(pe_ctx* c, const pe_mlp* m) {
   return PE_OK;
 }
 
-// Called by pe_set_problem after the coarse forcing, before the coarse recurrence.
+// Called by pe_set_problem before the column weights, which take the table in.
 pe_status launch_learned_tables(pe_ctx* c, LearnedTerms* L) {
   if (!c->mlp) return pe_fail(PE_ESTATE, "learned G: no network attached");
   if (!c->Ktab) {
@@ -877,48 +819,12 @@ pe_status launch_learned_tables(pe_ctx* c, LearnedTerms* L) {
   const double step = (loghi - loglo) / (double)(NB - 1);
   band_table_kernel<<<(c->R * NB + 127) / 128, 128, 0, c->stream>>>((const __half*)c->mlp->params16, T, NB, loglo,
                                                                      step, c->dT, c->Ktab);
-  if (!c->phase_tab) {
-    if (cudaMalloc((void**)&c->phase_tab, sizeof(float2) * (size_t)PE_MAX_TERMS * c->N) != cudaSuccess) {
-      cudaGetLastError();
-      return pe_fail(PE_ENOMEM, "learned G: phase table allocation failed");
-    }
-  }
-  phase_table_kernel<<<(c->R * c->N + 127) / 128, 128, 0, c->stream>>>(T, c->N, c->dT, c->t0,
-                                                                       (float2*)c->phase_tab);
-  c->launches += 2;
+  c->launches += 1;
   PE_CUDA_TRY(cudaGetLastError());
   L->NB = NB;
   L->loglo = loglo;
   L->logstep = step;
   L->dT = c->dT;
   L->Ktab = c->Ktab;
-  L->cs = (const float2*)c->phase_tab;
-  for (int r = 0; r < PE_MAX_TERMS; ++r) {
-    L->is_sin[r] = r < c->R ? T.is_sin[r] : 0;
-    L->amp[r] = r < c->R ? T.amp[r] : 0.0;
-  }
-  return PE_OK;
-}
-
-pe_status launch_learned_correction(pe_ctx* c) {
-  if (!c->mlp) return PE_OK;
-  LearnedTerms L{};
-  PE_TRY(launch_learned_tables(c, &L));
-  TermsW T{};
-  T.R = c->R;
-  for (int r = 0; r < c->R; ++r) {
-    T.is_sin[r] = L.is_sin[r];
-    T.omega[r] = c->terms[r].tp[0];
-    T.phase[r] = c->terms[r].tp[1];
-    T.amp[r] = L.amp[r];
-  }
-  const int NB = L.NB;
-  const double loglo = L.loglo, step = L.logstep;
-  const int threads = 256;
-  const size_t smem = sizeof(float) * 2 * (size_t)c->R * threads;
-  learned_correction_kernel<<<(unsigned)((c->g.ndof + threads - 1) / threads), threads, smem, c->stream>>>(
-      c->g, c->N, c->R, NB, loglo, step, c->dT, T, c->lam, c->axisF, c->Ktab, (const float2*)c->phase_tab, c->gG);
-  c->launches += 1;
-  PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;
 }

@@ -1,311 +1,26 @@
-// Coarse sweep, correction and residual of Algorithm 1 (PEIFE-linear).
+// Coarse sweep, fine sweep, correction and residual of Algorithm 1 (PEIFE-linear).
 //
-// In mode space every step of Eq. (1-7) is  c <- E c + sum_i (tau b_i) ghat(t_i)
-// with ghat_J(t) = sum_r A_r(t) P_{r,J}, A_r(t) = amp_r time_r(t) and
-// P_{r,J} = prod_a axisF[a][r][j_a].  Modes are independent, so one thread owns
-// one mode and walks the slices n = 0..N-1 sequentially (the "sequential"
-// parts of Algorithm 1 are sequential in n only).
+// In mode space every step of Eq. (1-7) is  c <- E c + sum_i (tau b_i) ghat(t_i).  Modes are
+// independent, so one thread owns one mode and walks the slices n = 0..N-1 sequentially (the
+// "sequential" parts of Algorithm 1 are sequential in n only).
 //
 //   coarse sweep   U^{n+1,(0)} = G(U^{n,(0)}) = E_G U^n + gG_n.
-//   correction     U^{n+1,(k+1)} = G(U^{n,(k+1)}) + Fbar^{n+1} - G(U^{n,(k)}).  G is affine
-//                  in its argument, G(v) = E_G v + gG_n (a learned correction adds a term
-//                  that does not depend on v), so the update is evaluated as
-//                    U^{n+1,(k+1)} = Fbar^{n+1} + E_G (U^{n,(k+1)} - U^{n,(k)}):
+//   fine sweep     F^M(U^{n,(k)}) = E_F^M U^{n,(k)} + F^M(0)_n, the step being affine in its
+//                  argument; F^M(0)_n and gG_n are sums over the K columns of the source
+//                  (pe_contract.cuh), evaluated anew in every sweep.
+//   correction     U^{n+1,(k+1)} = G(U^{n,(k+1)}) + F^M(U^{n,(k)}) - G(U^{n,(k)}).  G is affine too
+//                  (a learned correction adds a term that does not depend on the argument), so
+//                  the update is evaluated as
+//                    U^{n+1,(k+1)} = F^M(U^{n,(k)}) + E_G (U^{n,(k+1)} - U^{n,(k)}):
 //                  the same value, without G(U^{n,(k)}) stored between iterations and
-//                  without the cancellation of the two G terms; it reads Fbar and the
-//                  old U and writes the new U (3 words per mode and slice instead of 6).
+//                  without the cancellation of the two G terms.
 //                  Float64 sums  sum mu^M_J (U^{new} - U^{old})^2, sum mu^M_J (U^{new})^2
 //                  (per-CTA partial sums, added by the last CTA to finish).
+#include <algorithm>
+
 #include "pe_internal.h"
-#include "pe_learned.h"
 
 namespace {
-
-// Coarse forcing of every slice, in parallel over slices: each thread owns one
-// mode and SL consecutive slices.  Its weights P_{r,J} sit in registers, padded
-// with zeros to RB = roundup(R, 4) terms; the CTA's coarse time factors
-// A_r(T_n + c_i dT) (n in its slice range) are staged in shared memory, rows of RB
-// with zero padding, and read as float4 / double2 broadcasts.  T = double on the
-// float64 path; float in the mixed form, where gG only enters through
-// G(U^{new}) - G(U^{old}), in which the same stored gG cancels.
-template <typename T, int RB>
-__global__ void __launch_bounds__(256) coarse_forcing_kernel(Geom g, int N, int p, int R, int SL,
-                                                            const T* __restrict__ axisF, const T* __restrict__ AG,
-                                                            const double* __restrict__ coefG,
-                                                            double* __restrict__ gG) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* sA = reinterpret_cast<T*>(smem_raw);  // [SL * p][RB]
-  const int n0 = blockIdx.y * SL;
-  const int n1 = min(N, n0 + SL);
-  for (int e = threadIdx.x; e < (n1 - n0) * p * RB; e += blockDim.x) {
-    const int row = e / RB, r = e - row * RB;
-    sA[e] = r < R ? AG[((int64_t)n0 * p + row) * R + r] : T(0);
-  }
-  __syncthreads();
-  const int64_t J = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (J >= g.ndof) return;
-  const int64_t nd = g.ndof;
-  int j[PE_MAX_D];
-  unflatten(g, J, j);
-  T P[RB];
-#pragma unroll
-  for (int r = 0; r < RB; ++r) {
-    T v = T(0);
-    if (r < R) {
-      v = axisF[(int64_t)R * g.off[0] + (int64_t)r * g.n[0] + j[0]];
-#pragma unroll
-      for (int a = 1; a < PE_MAX_D; ++a) if (a < g.d) v *= axisF[(int64_t)R * g.off[a] + (int64_t)r * g.n[a] + j[a]];
-    }
-    P[r] = v;
-  }
-  T b[PE_MAX_S];
-#pragma unroll
-  for (int i = 0; i < PE_MAX_S; ++i) b[i] = i < p ? (T)coefG[(1 + i) * nd + J] : T(0);
-  for (int n = n0; n < n1; ++n) {
-    T acc = T(0);
-#pragma unroll
-    for (int i = 0; i < PE_MAX_S; ++i) {
-      if (i < p) {
-        const T* a = sA + ((int64_t)(n - n0) * p + i) * RB;
-        T gi = T(0);
-        if constexpr (sizeof(T) == 4) {
-#pragma unroll
-          for (int r = 0; r < RB; r += 4) {
-            const float4 v = *reinterpret_cast<const float4*>(a + r);
-            gi = fmaf(v.x, P[r], gi);
-            gi = fmaf(v.y, P[r + 1], gi);
-            gi = fmaf(v.z, P[r + 2], gi);
-            gi = fmaf(v.w, P[r + 3], gi);
-          }
-        } else {
-#pragma unroll
-          for (int r = 0; r < RB; r += 2) {
-            const double2 v = *reinterpret_cast<const double2*>(a + r);
-            gi = fma(v.x, P[r], gi);
-            gi = fma(v.y, P[r + 1], gi);
-          }
-        }
-        acc = fma(b[i], gi, acc);
-      }
-    }
-    gG[(int64_t)n * nd + J] = (double)acc;
-  }
-}
-
-// The instantiation with RB = roundup(R, 4) (at least 4); SL slices per thread,
-// capped so that the staged time factors fit 48 KB.
-template <typename T>
-pe_status launch_coarse_forcing_t(pe_ctx* c, unsigned blocks, int threads, int SL, const T* axisF, const T* AG) {
-  const int RB = c->R < 4 ? 4 : (c->R + 3) / 4 * 4;  // no source terms: one all-zero group
-  const int sl_max = (int)((48 * 1024) / (sizeof(T) * (size_t)c->p * RB));
-  SL = SL > sl_max ? sl_max : SL;
-  const size_t smem = sizeof(T) * (size_t)SL * c->p * RB;
-  const dim3 grid(blocks, (unsigned)((c->N + SL - 1) / SL));
-  switch (RB) {
-#define PE_CF_CASE(X)                                                                                        \
-  case X:                                                                                                    \
-    coarse_forcing_kernel<T, X><<<grid, threads, smem, c->stream>>>(c->g, c->N, c->p, c->R, SL, axisF, AG, \
-                                                                    c->coefG, c->gG);                      \
-    break;
-    PE_CF_CASE(4) PE_CF_CASE(8) PE_CF_CASE(12) PE_CF_CASE(16) PE_CF_CASE(20) PE_CF_CASE(24) PE_CF_CASE(28)
-    PE_CF_CASE(32)
-#undef PE_CF_CASE
-    default:
-      return pe_fail(PE_EINVAL, "coarse forcing: too many source terms");
-  }
-  PE_CUDA_TRY(cudaGetLastError());
-  return PE_OK;
-}
-
-// Coarse sweep of k = 0 with the coarse forcing made on the fly: one thread per mode walks
-// the slices, forming gG_n = sum_i b_i sum_r A_r(T_n + c_i dT) P_{r,J} from its register
-// weights and the time factors of all slices (staged in shared memory, rows of RB) and
-// applying U^{n+1} = E_G U^n + gG_n, so gG is neither written nor read back.  LEARN adds the
-// learned term of G' = G + delta^ per slice, sum_r (A_r cos_{r,n} + B_r sin_{r,n}) with
-// A_r = P_{r,J} amp_r Im K^, B_r = P_{r,J} amp_r Re K^ (K^ interpolated linearly in
-// log(lam dT) between the band centres) and the phase table staged beside the time factors:
-// the same float32 sum, added to gG_n in float64, as the separate learned-correction kernel.
-template <typename T, int RB, bool LEARN>
-__global__ void __launch_bounds__(512) coarse_fused_kernel(Geom g, int N, int p, int R,
-                                                          const T* __restrict__ axisF, const T* __restrict__ AG,
-                                                          const double* __restrict__ coefG, double* __restrict__ U,
-                                                          LearnedTerms L, const double* __restrict__ axisF64,
-                                                          const double* __restrict__ lam) {
-  pdl_wait();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* sCS = reinterpret_cast<float2*>(smem_raw);                // [N][RB] (LEARN only)
-  T* sA = reinterpret_cast<T*>(smem_raw + (LEARN ? sizeof(float2) * (size_t)N * RB : 0));  // [N * p][RB]
-  for (int e = threadIdx.x; e < N * p * RB; e += blockDim.x) {
-    const int row = e / RB, r = e - row * RB;
-    sA[e] = r < R ? AG[(int64_t)row * R + r] : T(0);
-  }
-  if constexpr (LEARN) {
-    for (int e = threadIdx.x; e < N * RB; e += blockDim.x) {
-      const int n = e / RB, r = e - n * RB;
-      sCS[e] = r < R ? L.cs[(int64_t)r * N + n] : make_float2(0.f, 0.f);
-    }
-  }
-  __syncthreads();
-  const int64_t J = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (J >= g.ndof) return;
-  const int64_t nd = g.ndof;
-  int j[PE_MAX_D];
-  unflatten(g, J, j);
-  T P[RB];
-#pragma unroll
-  for (int r = 0; r < RB; ++r) {
-    T v = T(0);
-    if (r < R) {
-      v = axisF[(int64_t)R * g.off[0] + (int64_t)r * g.n[0] + j[0]];
-#pragma unroll
-      for (int a = 1; a < PE_MAX_D; ++a) if (a < g.d) v *= axisF[(int64_t)R * g.off[a] + (int64_t)r * g.n[a] + j[a]];
-    }
-    P[r] = v;
-  }
-  float LA[LEARN ? RB : 1], LB[LEARN ? RB : 1];
-  if constexpr (LEARN) {
-    double pos = (log(lam[J] * L.dT) - L.loglo) / L.logstep;
-    pos = fmin(fmax(pos, 0.0), (double)(L.NB - 1) - 1e-9);
-    const int b0 = (int)pos;
-    const double f = pos - (double)b0;
-#pragma unroll
-    for (int r = 0; r < RB; ++r) {
-      LA[r] = 0.f;
-      LB[r] = 0.f;
-      if (r < R && L.is_sin[r]) {
-        double Pd = axisF64[(int64_t)R * g.off[0] + (int64_t)r * g.n[0] + j[0]];
-#pragma unroll
-        for (int a = 1; a < PE_MAX_D; ++a) if (a < g.d)
-          Pd *= axisF64[(int64_t)R * g.off[a] + (int64_t)r * g.n[a] + j[a]];
-        const double* k0 = L.Ktab + 2 * ((int64_t)r * L.NB + b0);
-        const double Kre = (1.0 - f) * k0[0] + f * k0[2];
-        const double Kim = (1.0 - f) * k0[1] + f * k0[3];
-        const double cc = Pd * L.amp[r];
-        LA[r] = (float)(cc * Kim);
-        LB[r] = (float)(cc * Kre);
-      }
-    }
-  }
-  T b[PE_MAX_S];
-#pragma unroll
-  for (int i = 0; i < PE_MAX_S; ++i) b[i] = i < p ? (T)coefG[(1 + i) * nd + J] : T(0);
-  const double E = coefG[J];
-  double c = U[J];
-  // two slices per pass: the forcing sums of the second overlap the float64 step of the first
-  // (four measured slower: 20.3 against 18.4 us at 255^2)
-#pragma unroll 2
-  for (int n = 0; n < N; ++n) {
-    T acc = T(0);
-#pragma unroll
-    for (int i = 0; i < PE_MAX_S; ++i) {
-      if (i < p) {
-        const T* a = sA + ((int64_t)n * p + i) * RB;
-        T gi = T(0);
-        if constexpr (sizeof(T) == 4) {
-#pragma unroll
-          for (int r = 0; r < RB; r += 4) {
-            const float4 v = *reinterpret_cast<const float4*>(a + r);
-            gi = fmaf(v.x, P[r], gi);
-            gi = fmaf(v.y, P[r + 1], gi);
-            gi = fmaf(v.z, P[r + 2], gi);
-            gi = fmaf(v.w, P[r + 3], gi);
-          }
-        } else {
-#pragma unroll
-          for (int r = 0; r < RB; r += 2) {
-            const double2 v = *reinterpret_cast<const double2*>(a + r);
-            gi = fma(v.x, P[r], gi);
-            gi = fma(v.y, P[r + 1], gi);
-          }
-        }
-        acc = fma(b[i], gi, acc);
-      }
-    }
-    double gn;
-    if constexpr (sizeof(T) == 4) gn = widen_f32(acc);
-    else gn = acc;
-    if constexpr (LEARN) {
-      float dl = 0.f;
-      const float2* e = sCS + (int64_t)n * RB;
-#pragma unroll
-      for (int r = 0; r < RB; ++r) dl = fmaf(LA[r], e[r].x, fmaf(LB[r], e[r].y, dl));
-      gn += widen_f32(dl);
-    }
-    c = fma(E, c, gn);
-    U[(int64_t)(n + 1) * nd + J] = c;
-  }
-}
-
-// The fused coarse sweep when its shared tables fit 48 KB; *done = false (nothing launched)
-// otherwise.  L is null without a learned correction.
-template <typename T>
-pe_status launch_coarse_fused_t(pe_ctx* c, unsigned blocks, int threads, const T* axisF, const T* AG,
-                                const LearnedTerms* L, bool* done) {
-  *done = false;
-  const int RB = c->R < 4 ? 4 : (c->R + 3) / 4 * 4;
-  const size_t smem = sizeof(T) * (size_t)c->N * c->p * RB + (L ? sizeof(float2) * (size_t)c->N * RB : 0);
-  if (smem > 48 * 1024) return PE_OK;
-  const LearnedTerms Lv = L ? *L : LearnedTerms{};
-  switch (RB) {
-#define PE_CF_CASE(X)                                                                                          \
-  case X:                                                                                                      \
-    if (L)                                                                                                     \
-      PE_CUDA_TRY(launch_pdl(coarse_fused_kernel<T, X, true>, dim3(blocks), dim3(threads), smem, c->stream, c->g, \
-                             c->N, c->p, c->R, axisF, AG, (const double*)c->coefG, c->U, Lv,                    \
-                             (const double*)c->axisF, (const double*)c->lam));                                  \
-    else                                                                                                       \
-      PE_CUDA_TRY(launch_pdl(coarse_fused_kernel<T, X, false>, dim3(blocks), dim3(threads), smem, c->stream, c->g, \
-                             c->N, c->p, c->R, axisF, AG, (const double*)c->coefG, c->U, Lv,                     \
-                             (const double*)c->axisF, (const double*)c->lam));                                   \
-    break;
-    PE_CF_CASE(4) PE_CF_CASE(8) PE_CF_CASE(12) PE_CF_CASE(16) PE_CF_CASE(20) PE_CF_CASE(24) PE_CF_CASE(28)
-    PE_CF_CASE(32)
-#undef PE_CF_CASE
-    default:
-      return pe_fail(PE_EINVAL, "coarse sweep: too many source terms");
-  }
-  PE_CUDA_TRY(cudaGetLastError());
-  *done = true;
-  return PE_OK;
-}
-
-// Slices of loads each thread keeps in flight in the sequential sweeps below.
-// The recurrence carries one value per mode; its inputs do not depend on it,
-// so the loads of the next kPF slices are issued while the current kPF are
-// combined (one thread per mode leaves too few threads to cover HBM latency
-// with one slice in flight).
-constexpr int kPF = 4;
-
-// Sequential coarse sweep U^{n+1,(0)} = E_G U^{n,(0)} + gG_n (one thread per mode).
-__global__ void __launch_bounds__(256) coarse_recurrence_kernel(Geom g, int N, const double* __restrict__ coefG,
-                                                               const double* __restrict__ gG,
-                                                               double* __restrict__ U) {
-  const int64_t J = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (J >= g.ndof) return;
-  const int64_t nd = g.ndof;
-  const double E = coefG[J];
-  double c = U[J];
-  double cur[kPF], nxt[kPF];
-#pragma unroll
-  for (int e = 0; e < kPF; ++e) cur[e] = e < N ? gG[(int64_t)e * nd + J] : 0.0;
-  for (int n0 = 0; n0 < N; n0 += kPF) {
-#pragma unroll
-    for (int e = 0; e < kPF; ++e) {
-      const int n = n0 + kPF + e;
-      nxt[e] = n < N ? gG[(int64_t)n * nd + J] : 0.0;
-    }
-#pragma unroll
-    for (int e = 0; e < kPF; ++e) {
-      const int n = n0 + e;
-      if (n < N) {
-        c = fma(E, c, cur[e]);
-        U[(int64_t)(n + 1) * nd + J] = c;
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < kPF; ++e) cur[e] = nxt[e];
-  }
-}
 
 template <typename T>
 __device__ inline T block_sum(T v, T* sh) {
@@ -359,145 +74,340 @@ __global__ void loop_init_kernel(LoopCtl* L, int max_iter, int hist_cap, double 
   }
 }
 
-// The correction: one thread per mode walks the slices.  With d = U^{n,(k+1)} - U^{n,(k)}
-// (d = 0 at n = 0: U^0 is the same in every iterate)
-//   U^{n+1,(k+1)} = fma(E_G, d, Fbar^{n+1}),   d <- U^{n+1,(k+1)} - U^{n+1,(k)},
-// and the residual terms fma(d, d, sd), fma(U, U, su): four float64 operations per mode and
-// slice.  GB300 executes float64 at 2 lanes per SM and clock, so this HBM-shaped step is bound
-// by those operations (at 255^2 x 32 slices: about 13 us at the full float64 rate); the loads of
-// the next kCorrPF slices are issued before the current kCorrPF are combined.
-constexpr int kCorrPF = 8;
+// The walk: one thread per mode, the slices in order.  MODE kCoarse makes the coarse iterate, MODE
+// kIterate one iteration from the iterate in U, MODE kFirst both in one pass (the coarse value of
+// a slice stays in a register; pe_solve).  With o the old and d = U^{new} - U^{old} (0 at n = 0),
+//   F = fma(E_F^M, o, F^M(0)_n),  U^{n+1} = fma(E_G, d, F),  d <- U^{n+1} - o',
+// o' the old value of slice n + 1 (kFirst: fma(E_G, o, gG_n)), and the residual terms fma(d, d, sd),
+// fma(U, U, su): five float64 operations per mode and slice (kFirst: six).
+//
+// The forced parts come from memory (SRC = 0: the float64 and the general path, made by a kernel
+// before) or, in the mixed form (SRC = 1), from the K float32 weights of the mode in registers and
+// the float32 columns of the slices in shared memory, read as float4 broadcasts: 2 KB,
+// KB = roundup(K, 4), FMAs per part on the float32 pipe, under the float64 operations, of which GB300 does two per
+// SM and clock; the sums enter the float64 recurrence through widen_f32.  F^M(0) never exists in
+// memory and U is read and written once.  At 255^2 x
+// 32 slices, K = 17: 34 us for the coarse sweep and first iteration in one pass, 30 us for a further
+// iteration (float64 rate alone: 20 and 17 us), against 17 us (coarse) and 62 + 26 us per iteration
+// with every substep taken on the tensor cores; 127^3 x 64, K = 33: 1.57 and 1.37 ms (1.25 and
+// 1.04 ms by the float64 rate) against 0.50 and 3.3 + 1.06 ms.
+//
+// Loads are issued kPF slices ahead (one thread per mode leaves too few threads to cover HBM
+// latency with one slice in flight).
+constexpr int kCoarse = 0, kIterate = 1, kFirst = 2;
+constexpr int kPF = 8;
 
-__global__ void __launch_bounds__(512) correction_kernel(Geom g, int N, const double* __restrict__ muM_axis,
-                                                         const double* __restrict__ coefG,
-                                                         const double* __restrict__ Fbar, double* __restrict__ U,
-                                                         double* __restrict__ partials,
-                                                         unsigned int* __restrict__ done, double* __restrict__ red,
-                                                         LoopCtl* loop, unsigned long long handle) {
+struct WalkArgs {
+  Geom g;
+  int N, K, SL;             // SL: slices of columns staged at a time (a multiple of kPF)
+  const float *V, *G, *Y;   // SRC = 1: column weights [K][ndof], columns [N][2 KB]
+  const double *f, *gG;     // SRC = 0: forced parts [N][ndof]
+  const double *EG, *EM;    // e^{-lam dT} of the coarse step, e^{-lam M dt}
+  const double* muM_axis;
+  double *U, *partials, *red;
+  unsigned int* done;
+  LoopCtl* loop;
+  unsigned long long handle;
+};
+
+// sum_k y_k w_k over a slice's staged columns, a row of KB high parts and one of KB low parts:
+// rounding Y_k(T_n) to one float would be an error of the whole slice, which M separately rounded
+// substeps average out
+template <int KB>
+__device__ __forceinline__ float column_dot(const float* y, const float (&w)[KB]) {
+  float hi = 0.f, lo = 0.f;
+#pragma unroll
+  for (int k = 0; k < KB; k += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(y + k);
+    const float4 l = *reinterpret_cast<const float4*>(y + KB + k);
+    hi = fmaf(v.x, w[k], hi);
+    lo = fmaf(l.x, w[k], lo);
+    hi = fmaf(v.y, w[k + 1], hi);
+    lo = fmaf(l.y, w[k + 1], lo);
+    hi = fmaf(v.z, w[k + 2], hi);
+    lo = fmaf(l.z, w[k + 2], lo);
+    hi = fmaf(v.w, w[k + 3], hi);
+    lo = fmaf(l.w, w[k + 3], lo);
+  }
+  return hi + lo;
+}
+
+// Threads per CTA: as many as 65536 registers allow with the weights in registers.
+__host__ __device__ constexpr int walk_cap(int SRC, int KB, int MODE) {
+  return SRC == 0 || (MODE == kIterate ? KB <= 40 : KB <= 28) ? 512 : 256;
+}
+
+template <int SRC, int KB, int MODE>
+__global__ void __launch_bounds__(walk_cap(SRC, KB, MODE)) walk_kernel(WalkArgs a) {
   pdl_wait();
+  extern __shared__ __align__(16) float sY[];  // [SL][2 KB]
   __shared__ double sh[32];
   __shared__ bool s_last;
   const int64_t J = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double sd = 0.0, su = 0.0, w = 0.0;
-  if (J < g.ndof) {
-    const int64_t nd = g.ndof;
-    int j[PE_MAX_D];
-    unflatten(g, J, j);
-    w = muM_axis[g.off[0] + j[0]];
+  const int64_t nd = a.g.ndof;
+  const int N = a.N;
+  const bool on = J < nd;
+  constexpr bool kOld = MODE == kIterate, kF = MODE != kCoarse, kG = MODE != kIterate;
+  float V[SRC && kF ? KB : 1], G[SRC && kG ? KB : 1];
+  if constexpr (SRC) {
 #pragma unroll
-    for (int a = 1; a < PE_MAX_D; ++a) if (a < g.d) w *= muM_axis[g.off[a] + j[a]];
-    const double E = coefG[J];
-    double d = 0.0;
-    // per slice n: Fbar^{n+1} = F(U^{n,(k)}) and the old U^{n+1}
-    double f0[kCorrPF], o0[kCorrPF], f1[kCorrPF], o1[kCorrPF];
-#pragma unroll
-    for (int e = 0; e < kCorrPF; ++e) {
-      const int64_t o = (int64_t)e * nd + J;
-      const bool in = e < N;
-      f0[e] = in ? Fbar[o] : 0.0;
-      o0[e] = in ? U[o + nd] : 0.0;
+    for (int k = 0; k < KB; ++k) {
+      if constexpr (kF) V[k] = on && k < a.K ? a.V[(int64_t)k * nd + J] : 0.f;
+      if constexpr (kG) G[k] = on && k < a.K ? a.G[(int64_t)k * nd + J] : 0.f;
     }
-    for (int n0 = 0; n0 < N; n0 += kCorrPF) {
+  }
+  double E = 0.0, EM = 0.0, o = 0.0, d = 0.0, sd = 0.0, su = 0.0, w = 0.0;
+  double* U = a.U + J;
+  if (on) {
+    E = a.EG[J];
+    o = U[0];
+    if constexpr (kF) {
+      EM = a.EM[J];
+      int j[PE_MAX_D];
+      unflatten(a.g, J, j);
+      w = a.muM_axis[a.g.off[0] + j[0]];
 #pragma unroll
-      for (int e = 0; e < kCorrPF; ++e) {
-        const int n = n0 + kCorrPF + e;
-        const int64_t o = (int64_t)n * nd + J;
-        const bool in = n < N;
-        f1[e] = in ? Fbar[o] : 0.0;
-        o1[e] = in ? U[o + nd] : 0.0;
-      }
+      for (int x = 1; x < PE_MAX_D; ++x) if (x < a.g.d) w *= a.muM_axis[a.g.off[x] + j[x]];
+    }
+  }
+  // the next kPF slices' old values and forced parts
+  double on1[kOld ? kPF : 1], f1[!SRC && kF ? kPF : 1], g1[!SRC && kG ? kPF : 1];
+  auto fetch = [&](int n0) {
 #pragma unroll
-      for (int e = 0; e < kCorrPF; ++e) {
-        const int n = n0 + e;
-        if (n < N) {
-          const double un = fma(E, d, f0[e]);
-          U[(int64_t)(n + 1) * nd + J] = un;
-          d = un - o0[e];
-          sd = fma(d, d, sd);
-          su = fma(un, un, su);
+    for (int e = 0; e < kPF; ++e) {
+      const int64_t n = n0 + e;
+      const bool in = on && n < N;
+      if constexpr (kOld) on1[e] = in ? U[(n + 1) * nd] : 0.0;
+      if constexpr (!SRC && kF) f1[e] = in ? a.f[n * nd + J] : 0.0;
+      if constexpr (!SRC && kG) g1[e] = in ? a.gG[n * nd + J] : 0.0;
+    }
+  };
+  fetch(0);
+  for (int c0 = 0; c0 < N; c0 += a.SL) {
+    const int c1 = min(N, c0 + a.SL);
+    if constexpr (SRC) {
+      __syncthreads();  // the previous chunk's reads are done
+      // rows past N (up to a whole group of kPF) are zero
+      const int rows = (c1 - c0 + kPF - 1) / kPF * kPF;
+      const float4* src = reinterpret_cast<const float4*>(a.Y + (int64_t)c0 * 2 * KB);
+      for (int e = threadIdx.x; e < rows * (KB / 2); e += blockDim.x)
+        reinterpret_cast<float4*>(sY)[e] = e < (c1 - c0) * (KB / 2) ? src[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+      __syncthreads();
+    }
+    if (on) {
+      for (int n0 = c0; n0 < c1; n0 += kPF) {
+        double o1[kOld ? kPF : 1], f[!SRC && kF ? kPF : 1], gg[!SRC && kG ? kPF : 1];
+#pragma unroll
+        for (int e = 0; e < kPF; ++e) {
+          if constexpr (kOld) o1[e] = on1[e];
+          if constexpr (!SRC && kF) f[e] = f1[e];
+          if constexpr (!SRC && kG) gg[e] = g1[e];
+        }
+        if constexpr (kOld || !SRC) fetch(n0 + kPF);
+#pragma unroll
+        for (int e = 0; e < kPF; ++e) {
+          const int n = n0 + e;
+          double fn = 0.0, gn = 0.0;
+          if constexpr (SRC) {
+            const float* y = sY + (n - c0) * 2 * KB;
+            if constexpr (kF) fn = widen_f32(column_dot<KB>(y, V));
+            if constexpr (kG) gn = widen_f32(column_dot<KB>(y, G));
+          } else {
+            if constexpr (kF) fn = f[e];
+            if constexpr (kG) gn = gg[e];
+          }
+          if (n < N) {
+            if constexpr (MODE == kCoarse) {
+              o = fma(E, o, gn);
+              U[(int64_t)(n + 1) * nd] = o;
+            } else {
+              const double un = fma(E, d, fma(EM, o, fn));
+              U[(int64_t)(n + 1) * nd] = un;
+              if constexpr (MODE == kFirst) o = fma(E, o, gn);
+              else o = o1[e];
+              d = un - o;
+              sd = fma(d, d, sd);
+              su = fma(un, un, su);
+            }
+          }
         }
       }
-#pragma unroll
-      for (int e = 0; e < kCorrPF; ++e) {
-        f0[e] = f1[e];
-        o0[e] = o1[e];
+    }
+  }
+  if constexpr (kF) {
+    // the weight mu^M_J is the same for every slice of the mode: applied once
+    sd = block_sum(sd * w, sh);
+    su = block_sum(su * w, sh);
+    // the last CTA to finish adds the per-CTA partial sums (in CTA order) and re-arms the counter
+    if (threadIdx.x == 0) {
+      a.partials[2 * blockIdx.x] = sd;
+      a.partials[2 * blockIdx.x + 1] = su;
+      __threadfence();
+      s_last = atomicAdd(a.done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (s_last) {
+      __threadfence();
+      double td = 0.0, tu = 0.0;
+      for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
+        td += __ldcg(a.partials + 2 * b);
+        tu += __ldcg(a.partials + 2 * b + 1);
+      }
+      td = block_sum(td, sh);
+      tu = block_sum(tu, sh);
+      if (threadIdx.x == 0) {
+        a.red[0] = td;
+        a.red[1] = tu;
+        *a.done = 0u;
+        if (a.loop) loop_decide(a.loop, a.handle, td, tu);
       }
     }
   }
-  // the weight mu^M_J is the same for every slice of the mode: applied once
-  sd *= w;
-  su *= w;
-  sd = block_sum(sd, sh);
-  su = block_sum(su, sh);
-  // the last CTA to finish adds the per-CTA partial sums (in CTA order) and re-arms the counter
-  if (threadIdx.x == 0) {
-    partials[2 * blockIdx.x] = sd;
-    partials[2 * blockIdx.x + 1] = su;
-    __threadfence();
-    s_last = atomicAdd(done, 1u) == gridDim.x - 1;
-  }
+}
+
+// F^M(0) of every slice from the float32 weights, stored as float64 (cache_forced of the mixed
+// form; the same sums as the walk makes): a CTA takes 256 modes and SL slices.
+template <int KB>
+__global__ void __launch_bounds__(256) forced_f32_kernel(int64_t ndof, int N, int K, int SL,
+                                                         const float* __restrict__ Y, const float* __restrict__ V,
+                                                         double* __restrict__ out) {
+  pdl_wait();
+  extern __shared__ __align__(16) float sY[];
+  const int n0 = blockIdx.y * SL, n1 = min(N, n0 + SL);
+  for (int e = threadIdx.x; e < (n1 - n0) * 2 * KB; e += blockDim.x) sY[e] = Y[(int64_t)n0 * 2 * KB + e];
   __syncthreads();
-  if (s_last) {
-    __threadfence();
-    double td = 0.0, tu = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
-      td += __ldcg(partials + 2 * b);
-      tu += __ldcg(partials + 2 * b + 1);
-    }
-    td = block_sum(td, sh);
-    tu = block_sum(tu, sh);
-    if (threadIdx.x == 0) {
-      red[0] = td;
-      red[1] = tu;
-      *done = 0u;
-      if (loop) loop_decide(loop, handle, td, tu);
-    }
+  const int64_t J = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (J >= ndof) return;
+  float w[KB];
+#pragma unroll
+  for (int k = 0; k < KB; ++k) w[k] = k < K ? V[(int64_t)k * ndof + J] : 0.f;
+  for (int n = n0; n < n1; ++n) out[(int64_t)n * ndof + J] = (double)column_dot<KB>(sY + (n - n0) * 2 * KB, w);
+}
+
+template <int SRC, int KB, int MODE>
+pe_status walk_launch(pe_ctx* c, WalkArgs a) {
+  const int threads = per_mode_block(c->g.ndof, c->sms, walk_cap(SRC, KB, MODE));
+  const int64_t blocks = (c->g.ndof + threads - 1) / threads;
+  if (blocks > (int64_t)c->max_blocks) return pe_fail(PE_EINVAL, "walk: partials buffer too small");
+  size_t smem = 0;
+  a.SL = c->N;
+  if (SRC) {
+    const int most = (40 * 1024) / (int)(sizeof(float) * 2 * KB) / kPF * kPF;
+    a.SL = std::min((c->N + kPF - 1) / kPF * kPF, most);
+    smem = sizeof(float) * 2 * (size_t)a.SL * KB;
   }
+  PE_CUDA_TRY(launch_pdl(walk_kernel<SRC, KB, MODE>, dim3((unsigned)blocks), dim3(threads), smem, c->stream, a));
+  c->launches += 1;
+  return PE_OK;
+}
+
+template <int MODE>
+pe_status walk_columns(pe_ctx* c, const WalkArgs& a) {
+  switch ((c->K + 3) / 4) {
+#define PE_W(X) \
+  case X:       \
+    return walk_launch<1, 4 * X, MODE>(c, a);
+    PE_W(1) PE_W(2) PE_W(3) PE_W(4) PE_W(5) PE_W(6) PE_W(7) PE_W(8) PE_W(9) PE_W(10) PE_W(11) PE_W(12) PE_W(13)
+    PE_W(14) PE_W(15) PE_W(16)
+#undef PE_W
+  }
+  return pe_fail(PE_EINVAL, "source columns must be in 1..64");
+}
+
+pe_status forced_f32(pe_ctx* c, double* out) {
+  const int KB = (c->K + 3) / 4 * 4, threads = 256;
+  const int SL = std::min(c->N, std::max(1, (16 * 1024) / (int)(sizeof(float) * 2 * KB)));
+  const dim3 grid((unsigned)((c->g.ndof + threads - 1) / threads), (unsigned)((c->N + SL - 1) / SL));
+  const size_t smem = sizeof(float) * 2 * (size_t)SL * KB;
+  switch (KB / 4) {
+#define PE_F(X)                                                                                                    \
+  case X:                                                                                                          \
+    PE_CUDA_TRY(launch_pdl(forced_f32_kernel<4 * X>, grid, dim3(threads), smem, c->stream, c->g.ndof, c->N, c->K, \
+                           SL, (const float*)c->tab.Y32, (const float*)c->V32, out));                              \
+    break;
+    PE_F(1) PE_F(2) PE_F(3) PE_F(4) PE_F(5) PE_F(6) PE_F(7) PE_F(8) PE_F(9) PE_F(10) PE_F(11) PE_F(12) PE_F(13)
+    PE_F(14) PE_F(15) PE_F(16)
+#undef PE_F
+    default:
+      return pe_fail(PE_EINVAL, "source columns must be in 1..64");
+  }
+  c->launches += 1;
+  return PE_OK;
+}
+
+WalkArgs walk_args(pe_ctx* c, LoopCtl* loop, unsigned long long handle) {
+  WalkArgs a{};
+  a.g = c->g;
+  a.N = c->N;
+  a.K = c->K;
+  a.V = c->V32;
+  a.G = c->G32;
+  a.Y = c->tab.Y32;
+  a.f = c->Fbar;
+  a.gG = c->gG;
+  a.EG = c->coefG;
+  a.EM = c->coefF + (int64_t)(c->q + 1) * c->g.ndof;
+  a.muM_axis = c->muM_axis;
+  a.U = c->U;
+  a.partials = c->partials;
+  a.red = c->red;
+  a.done = c->done_ctr;
+  a.loop = loop;
+  a.handle = handle;
+  return a;
+}
+
+bool mixed_columns(const pe_ctx* c, int precision) {
+  return precision == PE_MIXED && c->forcing_path == PE_FORCING_SEPARABLE;
 }
 
 }  // namespace
 
+bool first_fused(const pe_ctx* c) { return !c->cache_forced; }
+
 pe_status launch_coarse_sweep(pe_ctx* c) {
-  const int threads = 256;
-  const unsigned blocks = (unsigned)((c->g.ndof + threads - 1) / threads);
-  const int fthreads = per_mode_block(c->g.ndof, c->sms);
-  const unsigned fblocks = (unsigned)((c->g.ndof + fthreads - 1) / fthreads);
-  if (c->forcing_path == PE_FORCING_GENERAL) {
-    PE_TRY(launch_general_coarse_forcing(c));
-    coarse_recurrence_kernel<<<blocks, threads, 0, c->stream>>>(c->g, c->N, c->coefG, c->gG, c->U);
-    c->launches += 1;
-    PE_CUDA_TRY(cudaGetLastError());
-    return PE_OK;
-  }
-  {
-    // fused sweep; with a learned correction its band and phase tables are made first
-    LearnedTerms L{};
-    if (c->mlp) PE_TRY(launch_learned_tables(c, &L));
-    const LearnedTerms* Lp = c->mlp ? &L : nullptr;
-    bool done = false;
-    if (c->precision == PE_MIXED) PE_TRY(launch_coarse_fused_t<float>(c, fblocks, fthreads, c->axisF32, c->AG32, Lp, &done));
-    else PE_TRY(launch_coarse_fused_t<double>(c, fblocks, fthreads, c->axisF, c->AG, Lp, &done));
-    if (done) {
-      c->launches += 1;
-      return PE_OK;
-    }
-  }
-  // slices per thread: enough CTAs to cover the GPU twice, at least one slice each
-  int64_t want = (2 * 152 * 2 + blocks - 1) / blocks;
-  int SL = (int)((c->N + want - 1) / want);
-  SL = SL < 1 ? 1 : SL;
-  if (c->precision == PE_MIXED) PE_TRY(launch_coarse_forcing_t<float>(c, blocks, threads, SL, c->axisF32, c->AG32));
-  else PE_TRY(launch_coarse_forcing_t<double>(c, blocks, threads, SL, c->axisF, c->AG));
-  // learned correction G'(v) = G(v) + delta^ (no-op unless a trained network is attached)
-  PE_TRY(launch_learned_correction(c));
-  coarse_recurrence_kernel<<<blocks, threads, 0, c->stream>>>(c->g, c->N, c->coefG, c->gG, c->U);
-  c->launches += 2;
-  PE_CUDA_TRY(cudaGetLastError());
-  return PE_OK;
+  const WalkArgs a = walk_args(c, nullptr, 0ull);
+  if (mixed_columns(c, c->precision)) return walk_columns<kCoarse>(c, a);
+  if (c->forcing_path == PE_FORCING_GENERAL) PE_TRY(launch_general_coarse_forcing(c));
+  else PE_TRY(launch_forced_f64(c, nullptr, c->gG));
+  return walk_launch<0, 4, kCoarse>(c, a);
 }
 
-pe_status launch_correction(pe_ctx* c, double* num, double* den, cudaEvent_t after) {
-  PE_TRY(launch_correction_kernel(c, nullptr, 0ull));
+pe_status launch_iteration(pe_ctx* c, int precision, bool first, LoopCtl* loop, unsigned long long handle,
+                           cudaEvent_t mid) {
+  WalkArgs a = walk_args(c, loop, handle);
+  if (mixed_columns(c, precision) && !c->cache_forced) {
+    c->sweeps += 1;
+    PE_TRY(first ? walk_columns<kFirst>(c, a) : walk_columns<kIterate>(c, a));
+    if (mid) PE_CUDA_TRY(cudaEventRecord(mid, c->stream));
+    return PE_OK;
+  }
+  if (c->forcing_path == PE_FORCING_GENERAL) {
+    if (first) PE_TRY(launch_general_coarse_forcing(c));
+    PE_TRY(launch_general_fine_sweep(c, precision));
+  } else if (c->cache_forced) {
+    // one sweep per problem and precision, its forced part kept
+    if (c->fz_prec != precision) {
+      if (precision == PE_MIXED) {
+        PE_TRY(forced_f32(c, c->Fz));
+      } else {
+        PE_TRY(launch_column_weights_f64(c));
+        PE_TRY(launch_forced_f64(c, c->Fz, nullptr));
+      }
+      c->fz_prec = precision;
+      c->sweeps += 1;
+    }
+    a.f = c->Fz;
+  } else {
+    c->sweeps += 1;
+    PE_TRY(launch_column_weights_f64(c));
+    PE_TRY(launch_forced_f64(c, c->Fbar, first ? c->gG : nullptr));
+  }
+  if (mid) PE_CUDA_TRY(cudaEventRecord(mid, c->stream));
+  return first ? walk_launch<0, 4, kFirst>(c, a) : walk_launch<0, 4, kIterate>(c, a);
+}
+
+pe_status read_sums(pe_ctx* c, double* num, double* den, cudaEvent_t after) {
   if (after) PE_CUDA_TRY(cudaEventRecord(after, c->stream));
   PE_CUDA_TRY(cudaMemcpyAsync(c->h_red, c->red, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   PE_CUDA_TRY(cudaStreamSynchronize(c->stream));
@@ -510,17 +420,5 @@ pe_status launch_loop_init(pe_ctx* c, double tol) {
   PE_CUDA_TRY(launch_pdl(loop_init_kernel, dim3(1), dim3(32), 0, c->stream, c->loopctl, c->max_iter, c->N, tol,
                          c->loop_hist, c->h_loop_dev));
   c->launches += 1;
-  return PE_OK;
-}
-
-pe_status launch_correction_kernel(pe_ctx* c, LoopCtl* loop, unsigned long long handle) {
-  const int threads = per_mode_block(c->g.ndof, c->sms);
-  const int64_t blocks = (c->g.ndof + threads - 1) / threads;
-  if (blocks > (int64_t)c->max_blocks) return pe_fail(PE_EINVAL, "correction: partials buffer too small");
-  PE_CUDA_TRY(launch_pdl(correction_kernel, dim3((unsigned)blocks), dim3(threads), 0, c->stream, c->g, c->N,
-                         (const double*)c->muM_axis, (const double*)c->coefG, (const double*)c->Fbar, c->U,
-                         c->partials, c->done_ctr, c->red, loop, handle));
-  c->launches += 1;
-  PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;
 }

@@ -44,7 +44,7 @@ __global__ void axis_tables_kernel(Geom g, double h0, double h1, double h2, doub
 __global__ void coef_tables_kernel(Geom g, const double* __restrict__ ratio, double D, double dt, double dT,
                                    int M, int q, int p, Lag LF, Lag LG, double* __restrict__ lam_out,
                                    double* __restrict__ coefF, double* __restrict__ coefG,
-                                   float* __restrict__ coefF32) {
+                                   float* __restrict__ coefF32, float* __restrict__ coefG32) {
   const int64_t J = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (J >= g.ndof) return;
   int j[PE_MAX_D];
@@ -77,7 +77,10 @@ __global__ void coef_tables_kernel(Geom g, const double* __restrict__ ratio, dou
     const double z = -lam * dT;
     b_weights(z, p, LG, b);
     coefG[J] = exp(z);
-    for (int i = 0; i < p; ++i) coefG[(1 + i) * nd + J] = dT * b[i];
+    for (int i = 0; i < p; ++i) {
+      coefG[(1 + i) * nd + J] = dT * b[i];
+      if (coefG32) coefG32[i * nd + J] = (float)(dT * b[i]);
+    }
   }
 }
 
@@ -145,7 +148,7 @@ pe_status launch_coef_tables(pe_ctx* c) {
   const int64_t blocks = (c->g.ndof + threads - 1) / threads;
   coef_tables_kernel<<<(unsigned)blocks, threads, 0, c->stream>>>(
       c->g, c->ratio_axis, c->D, c->dt, c->dT, c->M, c->q, c->p, LF, LG, c->lam, c->coefF, c->coefG,
-      c->precision == PE_MIXED ? c->coefF32 : nullptr);
+      c->coefF32, c->coefG32);
   c->launches += 1;
   PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;

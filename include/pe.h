@@ -340,7 +340,7 @@ pe_status pe_load_state(pe_ctx* ctx, const void* buf, size_t bytes);
  * applied along every axis of a C-ordered float64 array: out = (kron_a S_a) in.
  * V is symmetric and orthogonal, so the same call is the forward and the inverse
  * transform (Sec. 2.3).  in/out: device, Ndof values, may alias.  d in 1..3.
- * stream: cudaStream_t or NULL.  Scratch (a ping-pong array; the DST-I matrix of axes whose
+ * stream: cudaStream_t or NULL.  Scratch (a ping-pong array; a row of n sines for axes whose
  * n + 1 is not a power of two) comes stream-ordered from a memory pool the library creates per
  * device, which keeps freed memory for the next call until the process exits.
  */
@@ -356,7 +356,7 @@ pe_status pe_dst_f32(int32_t d, const int32_t* n, const float* in, float* out, v
  * can synchronise the device).  The
  * paper has no counterpart: this is an interface variant, not a step of the method.
  * It calls no cudaMalloc, cudaFree or other allocating routine; its scratch (ping-pong
- * array, DST-I matrices, FFT twiddles) is one file-scope device array of 1,835,008
+ * array, sine rows, FFT twiddles) is one file-scope device array of 1,835,008
  * doubles (about 14.7 MB) that every GPU loading the library holds until the process
  * exits.  Limits: at most 1,048,576 values in total; an axis whose n+1 is not a power
  * of two must have n <= 512.  Larger sizes return PE_EINVAL with a message.

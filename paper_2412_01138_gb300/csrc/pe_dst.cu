@@ -1,9 +1,8 @@
 // Tensor DST-I along every axis (the simultaneous diagonalisation of Sec. 2.3).
 //
 // Each axis pass is a dense contraction with the symmetric orthonormal matrix
-// S_a[j][k] = sqrt(2/(n_a+1)) sin(pi (j+1)(k+1)/(n_a+1)):
-//   last axis   : out[o][j]    = sum_k X[o][k] S[k][j]     (one GEMM, outer x n times n x n)
-//   other axes  : out[o][j][i] = sum_k S[j][k] X[o][k][i]  (batched over o)
+// S_a[j][k] = sqrt(2/(n_a+1)) sin(pi (j+1)(k+1)/(n_a+1)),
+//   out[o][j][i] = sum_k S[j][k] X[o][k][i]  (i: the axes after a, o: those before).
 // Two kernel families serve every axis pass:
 //  * n + 1 = 2^k (n <= 1023): an FFT.  Two real pencils x, y are packed as
 //    z = x + i y; the odd extension of z over 2(n+1) points is Fourier
@@ -11,11 +10,12 @@
 //    5 log2(2n+2) flops per element instead of the 2n of the matrix form.  In
 //    float64 with n + 1 >= 128 the half-length form folds each pencil so that the
 //    pair needs a complex FFT of n + 1 points only (dst_half_warp_kernel); float32
-//    and shorter float64 pencils transform the full odd extension with one warp per
+//    pencils transform the full odd extension with one warp per
 //    pencil pair (dst_fft_warp_kernel); both run self-sorting radix-4..32 passes.
 //    Pencils with n + 1 < 16 use a block-wide radix-2 kernel (dst_fft_kernel).
-//  * any other n: a shared-memory tiled, strided, batched GEMM with the matrix S_a
-//    (tile shape chosen so that the grid covers the GPU).
+//  * any other n, and many short float64 pencils (takes_folded): the matrix form, folded by its symmetry to half the multiplications
+//    (folded_dst_kernel).  A periodic axis without an FFT form keeps the plain product with its
+//    Hartley matrix (strided_gemm_kernel).
 #include <algorithm>
 #include <mutex>
 
@@ -122,6 +122,187 @@ pe_status gemm_axis(const T* S, const T* in, T* out, int64_t outer, int n, int64
   }
   PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;
+}
+
+// ---------------------------------------------------------------------------
+// Matrix form, folded.  S[j][n-1-k] = (-1)^j S[j][k], so the even outputs (j = 0, 2, ...) see only
+// the sums x_k + x_{n-1-k} and the odd ones only the differences: n/2 multiplications per output
+// instead of n.  A CTA of four warps makes TK = 8 RW consecutive outputs of TC = 32 CW pencils (lane =
+// pencil): per folded index two values of the lane's pencil from shared memory and the CTA's matrix
+// entries as broadcasts.
+//
+// In float64 the step is bound by the FMA rate (two lanes per SM: 16 clocks per warp instruction, in which
+// shared memory delivers far more than the operands, so a large register tile gains nothing), and
+// what counts is that the work spreads evenly over the SMs: RW is chosen by the busiest SM's share
+// (folded_axis).  In float32 two pencils per lane keep the operand reads under the FMAs.
+// Matrix entries come from a row of n sines (S[0][m-1] = sqrt(2/(n+1)) sin(pi m/(n+1)), signs and zeros
+// from m = (j+1)(k+1) mod 2(n+1)) while a tile is staged: no n x n matrix is made, stored or read.  The next
+// chunk of pencil values is fetched into registers while the current one is used; contiguous
+// pencils (inner = 1) are read along the pencil and written through shared memory.
+// Float64, a transform of 200 x 117 nodes: 37 us against 249 with the plain tiled product and the matrix
+// made per call; 500 x 500: 304 against 744 us (199 us by the float64 rate); float32 500 x 500: 57
+// against 219 us.
+// ---------------------------------------------------------------------------
+constexpr int kFoldJC = 32;  // folded indices per chunk
+
+template <typename T, int RW, int CW>
+__global__ void __launch_bounds__(128) folded_dst_kernel(const T* __restrict__ row, const T* __restrict__ in,
+                                                         T* __restrict__ out, int n, int64_t inner, int64_t np) {
+  pdl_wait();
+  constexpr int JC = kFoldJC, TC = 32 * CW, TK = 8 * RW, PE = JC * TC / 128, SE = JC * TK / 128;
+  __shared__ T sX[2][JC][TC + 1];  // sums and differences (then the outputs of contiguous pencils)
+  __shared__ __align__(16) T sS[2][JC][4 * RW];
+  static_assert(TC * (TK + 1) <= 2 * JC * (TC + 1), "output tile fits the operand tiles");
+  static_assert(128 % TK == 0 && 128 % TC == 0, "a thread stages one output's and one pencil's entries");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t c0 = (int64_t)blockIdx.x * TC;
+  const int k0 = blockIdx.y * TK, h = (n + 1) / 2;
+  const unsigned period = 2u * (unsigned)(n + 1);
+  const bool contig = inner == 1;
+  // loader: contiguous pencils lane = index, others lane = pencil (fixed per thread)
+  const int64_t cl = c0 + tid % TC;
+  const int64_t offl = contig || cl >= np ? 0 : (cl / inner) * n * inner + cl % inner;
+  auto place = [&](int it, int& j, int& col) {
+    if (contig) {
+      j = lane;
+      col = it * 4 + warp;
+    } else {
+      j = it * (128 / TC) + tid / TC;
+      col = tid % TC;
+    }
+  };
+  T xa[PE], xb[PE];
+  auto fetch = [&](int j0) {
+#pragma unroll
+    for (int it = 0; it < PE; ++it) {
+      int j, col;
+      place(it, j, col);
+      j += j0;
+      xa[it] = T(0);
+      xb[it] = T(0);
+      if (j < h && c0 + col < np) {
+        const T* x = in + (contig ? (c0 + col) * n : offl);
+        xa[it] = x[(int64_t)j * inner];
+        if (n - 1 - j != j) xb[it] = x[(int64_t)(n - 1 - j) * inner];
+      }
+    }
+  };
+  T acc[2][RW][CW];
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+#pragma unroll
+    for (int r = 0; r < RW; ++r)
+#pragma unroll
+      for (int q = 0; q < CW; ++q) acc[e][r][q] = T(0);
+  // m = (j+1)(k+1) mod 2(n+1) of this thread's staged entries, advanced by JC (k+1) per chunk
+  const unsigned kk1 = (unsigned)(k0 + tid % TK + 1);
+  const unsigned step = (unsigned)JC * kk1 % period;
+  unsigned m[SE];
+#pragma unroll
+  for (int it = 0; it < SE; ++it) m[it] = (unsigned)((it * 128 + tid) / TK + 1) * kk1 % period;
+  fetch(0);
+  for (int j0 = 0; j0 < h; j0 += JC) {
+    if (j0) __syncthreads();  // the previous chunk's reads are done
+#pragma unroll
+    for (int it = 0; it < PE; ++it) {
+      int j, col;
+      place(it, j, col);
+      sX[0][j][col] = xa[it] + xb[it];
+      // the middle index of an odd n is its own mirror: it enters the even outputs alone
+      sX[1][j][col] = 2 * (j0 + j) == n - 1 ? T(0) : xa[it] - xb[it];
+    }
+#pragma unroll
+    for (int it = 0; it < SE; ++it) {
+      const int kk = tid % TK, j = (it * 128 + tid) / TK;
+      T v = T(0);
+      if (k0 + kk < n && j0 + j < h) {
+        const unsigned half = (unsigned)n + 1u;
+        const bool neg = m[it] > half;
+        const unsigned q = neg ? m[it] - half : m[it];
+        if (q != 0u && q != half) v = neg ? -row[q - 1] : row[q - 1];
+      }
+      m[it] += step;
+      if (m[it] >= period) m[it] -= period;
+      sS[kk & 1][j][kk >> 1] = v;
+    }
+    __syncthreads();
+    if (j0 + JC < h) fetch(j0 + JC);
+    const int jn = min(JC, h - j0);
+#pragma unroll 8
+    for (int j = 0; j < jn; ++j) {
+      T x[2][CW];
+#pragma unroll
+      for (int q = 0; q < CW; ++q) {
+        x[0][q] = sX[0][j][lane + 32 * q];
+        x[1][q] = sX[1][j][lane + 32 * q];
+      }
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int r = 0; r < RW; ++r) {
+          const T s = sS[e][j][warp * RW + r];
+#pragma unroll
+          for (int q = 0; q < CW; ++q) acc[e][r][q] = fma(s, x[e][q], acc[e][r][q]);
+        }
+    }
+  }
+  if (contig) {
+    __syncthreads();
+    T* sO = &sX[0][0][0];  // [TC][TK + 1]
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+#pragma unroll
+      for (int r = 0; r < RW; ++r)
+#pragma unroll
+        for (int q = 0; q < CW; ++q) sO[(lane + 32 * q) * (TK + 1) + 2 * (warp * RW + r) + e] = acc[e][r][q];
+    __syncthreads();
+    for (int e = tid; e < TC * TK; e += 128) {
+      const int kk = e % TK, col = e / TK;
+      if (c0 + col < np && k0 + kk < n) out[(c0 + col) * n + k0 + kk] = sO[col * (TK + 1) + kk];
+    }
+    return;
+  }
+#pragma unroll
+  for (int q = 0; q < CW; ++q) {
+    const int64_t c = c0 + lane + 32 * q;
+    if (c >= np) continue;
+    T* o = out + (c / inner) * n * inner + c % inner;
+#pragma unroll
+    for (int r = 0; r < RW; ++r)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int k = k0 + 2 * (warp * RW + r) + e;
+        if (k < n) o[(int64_t)k * inner] = acc[e][r][q];
+      }
+  }
+}
+
+template <typename T, int RW, int CW>
+pe_status folded_launch(const T* row, const T* in, T* out, int n, int64_t inner, int64_t np, cudaStream_t st) {
+  const dim3 grid((unsigned)((np + 32 * CW - 1) / (32 * CW)), (unsigned)((n + 8 * RW - 1) / (8 * RW)));
+  PE_CUDA_TRY(launch_pdl(folded_dst_kernel<T, RW, CW>, grid, dim3(128), 0, st, row, in, out, n, inner, np));
+  return PE_OK;
+}
+
+// row: S[0][.], the n values sqrt(2/(n+1)) sin(pi m/(n+1)), m = 1..n
+template <typename T>
+pe_status folded_axis(const T* row, const T* in, T* out, int64_t outer, int n, int64_t inner, cudaStream_t st) {
+  const int64_t np = outer * inner;
+  if (np > (int64_t)1 << 36) return pe_fail(PE_EINVAL, "dst: too many pencils");
+  auto ctas = [&](int RW, int CW) { return ((np + 32 * CW - 1) / (32 * CW)) * ((n + 8 * RW - 1) / (8 * RW)); };
+  if constexpr (sizeof(T) == 8) {
+    // float64 instructions of the busiest SM per chunk and thread: 64 RW multiply-adds of a CTA, its
+    // 16 additions of the fold and about ten instructions' worth of staging
+    auto cost = [&](int RW) { return (ctas(RW, 1) + 151) / 152 * (64 * RW + 26); };
+    const int64_t c1 = cost(1), c2 = cost(2), c4 = cost(4);
+    if (c4 <= c2 && c4 <= c1) return folded_launch<T, 4, 1>(row, in, out, n, inner, np, st);
+    if (c2 <= c1) return folded_launch<T, 2, 1>(row, in, out, n, inner, np, st);
+    return folded_launch<T, 1, 1>(row, in, out, n, inner, np, st);
+  } else {
+    if (ctas(4, 2) >= 2 * 152) return folded_launch<T, 4, 2>(row, in, out, n, inner, np, st);
+    if (ctas(2, 1) >= 2 * 152) return folded_launch<T, 2, 1>(row, in, out, n, inner, np, st);
+    return folded_launch<T, 1, 1>(row, in, out, n, inner, np, st);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1785,10 +1966,7 @@ pe_status fft_warp_axis(const T* in, T* out, int64_t outer, int n, int64_t inner
   // rounding by about sqrt(n+1)/2, harmless at float64 precision).  float32: the full
   // odd extension, whose error stays at the FFT's own level.
   if constexpr (sizeof(T) == 8) {
-    switch (logL) {
-      case 5: return fft_warp_launch<T, 5>(in, out, n, inner, np, scale, st);
-      case 6: return fft_warp_launch<T, 6>(in, out, n, inner, np, scale, st);
-      case 7: return fft_warp_launch<T, 7>(in, out, n, inner, np, scale, st);
+    switch (logL) {  // (n <= 63: the folded matrix form, takes_folded)
       case 8: return fft_half_launch<T, 7>(in, out, n, inner, np, st);
       case 9: return fft_half_launch<T, 8>(in, out, n, inner, np, st);
       case 10: return fft_half_launch<T, 9>(in, out, n, inner, np, st);
@@ -1868,17 +2046,29 @@ pe_status fft_axis(const T* in, T* out, int64_t outer, int n, int64_t inner, int
   return PE_OK;
 }
 
+// Whether a Dirichlet axis takes the folded matrix form (and so needs its sine row): without an FFT form
+// always; in float64 also up to n = 63 for more pencils than the block-wide FFT serves, where n/2 + 1
+// multiplications per value cost less than the FFT of the short odd extension (255 x 255 x n: 460 us
+// at n = 15 with the FFT, 112 folded; 566 and 240 at 31; 830 and 562 at 63; at n = 127 the half-length FFT is ahead,
+// 172 against 218 for 127 x 63 x 63).
+template <typename T>
+bool takes_folded(int n, int64_t npencils) {
+  int logL = 0;
+  return !fft_size_ok(n, &logL) || (sizeof(T) == 8 && n <= 63 && npencils > kFewPencils);
+}
+
 template <typename T>
 pe_status dst_axis(const T* S, const T* in, T* out, int64_t outer, int n, int64_t inner, cudaStream_t st,
                    int periodic = 0) {
   int logL = 0;
+  if (!periodic && takes_folded<T>(n, outer * inner)) return folded_axis<T>(S, in, out, outer, n, inner, st);
   if (!periodic && fft_size_ok(n, &logL)) return fft_axis<T>(in, out, outer, n, inner, logL, st);
   if (periodic) {
     bool done = false;
     PE_TRY(dht_fft_axis<T>(in, out, outer, n, inner, st, &done));
     if (done) return PE_OK;
   }
-  // matrix form: large tiles when they still give >= 2 CTAs per SM, else small ones
+  // Hartley matrix: large tiles when they still give >= 2 CTAs per SM, else small ones
   const int64_t rows = inner == 1 ? outer : n;
   const int64_t cols = inner == 1 ? n : inner;
   const int64_t batch = inner == 1 ? 1 : outer;
@@ -1909,14 +2099,11 @@ pe_status dst_nd(int d, const int* n, T* const* S, const T* in, T* out, T* tmp, 
   return PE_OK;
 }
 
+// S[0][.], the row the folded matrix form takes its entries from
 template <typename T>
-__global__ void dst_matrix_kernel_t(int n, T* S) {
+__global__ void dst_row_kernel(int n, T* row) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y;
-  if (k >= n || j >= n) return;
-  const int64_t period = 2 * (int64_t)(n + 1);
-  const int64_t m = ((int64_t)(j + 1) * (k + 1)) % period;
-  S[(int64_t)j * n + k] = (T)(sqrt(2.0 / (double)(n + 1)) * sinpi((double)m / (double)(n + 1)));
+  if (k < n) row[k] = (T)(sqrt(2.0 / (double)(n + 1)) * sinpi((double)(k + 1) / (double)(n + 1)));
 }
 
 // The library's own stream-ordered memory pool of a device for the scratch of the standalone
@@ -1970,14 +2157,12 @@ pe_status standalone_dst(int32_t d, const int32_t* n, const T* in, T* out, void*
   T* S[PE_MAX_D] = {nullptr, nullptr, nullptr};
   T* tmp = nullptr;
   pe_status rc = PE_OK;
-  // the DST-I matrix only of axes without an FFT form (n + 1 not a power of two)
+  // the sine row of axes in the matrix form
   for (int a = 0; a < d && rc == PE_OK; ++a) {
-    int logL = 0;
-    if (fft_size_ok(nn[a], &logL)) continue;
-    cudaError_t e = scratch_alloc(&S[a], sizeof(T) * (size_t)nn[a] * nn[a], st);
+    if (!takes_folded<T>(nn[a], ndof / nn[a])) continue;
+    cudaError_t e = scratch_alloc(&S[a], sizeof(T) * (size_t)nn[a], st);
     if (e != cudaSuccess) { rc = pe_cuda_fail(e, "cudaMallocAsync(S)"); break; }
-    dim3 grid((nn[a] + 127) / 128, nn[a]);
-    dst_matrix_kernel_t<T><<<grid, 128, 0, st>>>(nn[a], S[a]);
+    dst_row_kernel<T><<<(nn[a] + 127) / 128, 128, 0, st>>>(nn[a], S[a]);
   }
   if (rc == PE_OK && (d > 1 || in == out)) {
     cudaError_t e = scratch_alloc(&tmp, sizeof(T) * (size_t)ndof, st);
@@ -2128,8 +2313,8 @@ extern "C" pe_status pe_dst_f32(int32_t d, const int32_t* n, const float* in, fl
 // forbid the runtime allocator, hosts whose device memory is fully reserved up front,
 // and latency-critical loops that must not enter the allocator (cudaMalloc and cudaFree
 // can synchronise the device).  This entry point keeps every scratch
-// buffer of the transform (the ping-pong array, the DST-I matrices of axes without
-// an FFT length, the FFT twiddles) in one file-scope device array.  Every GPU that
+// buffer of the transform (the ping-pong array, the sine rows of axes without an FFT
+// length, the FFT twiddles) in one file-scope device array.  Every GPU that
 // loads the library holds that array (about 14.7 MB) until the process exits.
 // ---------------------------------------------------------------------------
 namespace {
@@ -2201,7 +2386,7 @@ extern "C" pe_status pe_dst_noalloc(int32_t d, const int32_t* n, const double* i
   double* scratch = nullptr;
   PE_TRY(noalloc_scratch(&scratch));
   double* tmp = scratch;  // ping-pong buffer, kNoallocMaxNdof values
-  // per-axis slot: the DST-I matrix (matrix path) or the twiddles (FFT path); every value the
+  // per-axis slot: the sine row (matrix path) or the twiddles (FFT path); every value the
   // passes read is written here first, so nothing in the array has to start at zero
   for (int a = 0; a < d; ++a) {
     double* slot = scratch + kNoallocMaxNdof + (int64_t)a * kNoallocSlot;
@@ -2209,8 +2394,7 @@ extern "C" pe_status pe_dst_noalloc(int32_t d, const int32_t* n, const double* i
       const int L = 1 << logL[a];
       twiddle_kernel<double><<<(L / 2 + 255) / 256, 256, 0, st>>>(L, reinterpret_cast<Cplx<double>*>(slot));
     } else {
-      dim3 grid((n[a] + 127) / 128, n[a]);
-      dst_matrix_kernel_t<double><<<grid, 128, 0, st>>>(n[a], slot);
+      dst_row_kernel<double><<<(n[a] + 127) / 128, 128, 0, st>>>(n[a], slot);
     }
   }
   PE_CUDA_TRY(cudaGetLastError());
@@ -2229,12 +2413,7 @@ extern "C" pe_status pe_dst_noalloc(int32_t d, const int32_t* n, const double* i
     if (fft[a]) {
       PE_TRY(fft_axis_tw(src, dst, outer, n[a], inner, logL[a], reinterpret_cast<const Cplx<double>*>(slot), st));
     } else {
-      const int64_t rows = inner == 1 ? outer : n[a];
-      const int64_t cols = inner == 1 ? n[a] : inner;
-      const int64_t batch = inner == 1 ? 1 : outer;
-      const int64_t big = ((rows + 63) / 64) * ((cols + 63) / 64) * batch;
-      if (big >= 2 * 152) PE_TRY((gemm_axis<double, 64, 64>(slot, src, dst, outer, n[a], inner, st)));
-      else PE_TRY((gemm_axis<double, 32, 32>(slot, src, dst, outer, n[a], inner, st)));
+      PE_TRY(folded_axis<double>(slot, src, dst, outer, n[a], inner, st));
     }
     src = dst;
   }

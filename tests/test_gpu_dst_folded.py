@@ -1,0 +1,57 @@
+"""GPU: the folded matrix form of the DST-I (axes whose n + 1 is not a power of two) against dense products.
+
+Sizes where it can go wrong: odd and even n (an odd one has a middle index that is its own mirror), fewer
+indices than a chunk of 32, one more than a chunk, tiles of 8, 16 and 32 outputs with a remainder,
+pencil counts around 32 and 64 and large enough for the wide tiles, contiguous and strided pencils with short
+and long inner extents, short axes with an FFT form that take it in float64, in place.  Bound: a folded sum has n/2 + 1 rounded terms, so each output is within
+(n/2 + 3) u sum |S||x| of the product, and the 2-norm of |S||x| is at most sqrt(n) times that of x:
+(n/2 + 3) u sqrt(n) relative, u = 2^-53 or 2^-24.
+"""
+import math
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [(2,), (4,), (5,), (6,), (33,), (64,), (65,), (66,), (257,), (1000,), (4, 2), (5, 33), (33, 5), (64, 64),
+         (100, 37), (37, 100), (200, 117), (129, 300), (20, 700), (1200, 9), (6, 5, 4), (10, 33, 17), (40, 66, 9),
+         (12, 250, 130), (63, 34, 100),
+         (7, 400), (31, 400), (19, 17, 15), (63, 500)]
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2412_01138_gb300 import pe
+
+    pe.lib()
+    return pe, torch
+
+
+def _dense(x):
+    for a, n in enumerate(x.shape):
+        j = np.arange(1, n + 1)
+        S = math.sqrt(2.0 / (n + 1)) * np.sin(np.pi * (np.outer(j, j) % (2 * (n + 1))) / (n + 1))
+        x = np.moveaxis(np.tensordot(S, x, axes=(1, a)), 0, a)
+    return x
+
+
+@pytest.mark.parametrize("n", SIZES, ids=["x".join(map(str, n)) for n in SIZES])
+@pytest.mark.parametrize("f32", [False, True], ids=["float64", "float32"])
+def test_folded_matrix_form_matches_dense_products(env, n, f32):
+    pe, torch = env
+    x = np.random.default_rng(sum(n)).standard_normal(n)
+    x = x.astype(np.float32) if f32 else x
+    ref = _dense(x.astype(np.float64))
+    u = 2.0 ** (-24 if f32 else -53)
+    bound = sum((v / 2 + 3) * u * math.sqrt(v) for v in n)
+    d = torch.tensor(x.reshape(-1), device="cuda")
+    out = torch.empty_like(d)
+    pe.dst(len(n), n, d, out, f32=f32)
+    pe.dst(len(n), n, d, d, f32=f32)
+    for got in (out, d):
+        err = np.linalg.norm(got.cpu().numpy().astype(np.float64).reshape(n) - ref) / np.linalg.norm(ref)
+        assert err <= bound, (err, bound)

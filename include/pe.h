@@ -63,12 +63,10 @@ enum { PE_FP64 = 0,   /* every step in float64 */
  * column per exponential, two per sinusoid) times a per-mode weight made once per problem; every
  * sweep evaluates that sum on every mode and slice.  The general path takes every substep.
  *
- * Engine of the mixed-precision fine sweep (pe_options.fine_engine): a single problem runs the same
- * kernels for both values, the sum over the columns being too small for tensor cores to matter;
- * a batch with TC contracts the stages of each substep on the tensor cores (tcgen05, three-term
- * bfloat16 split of both operands, six products, float32 accumulation; about the accuracy
- * of the float32 form).  TC needs M (substeps per slice) a multiple of 16 in 16..128: pe_setup
- * returns PE_EINVAL otherwise, and for PE_FP64 or PE_FORCING_GENERAL. */
+ * Engine of the mixed-precision fine sweep (pe_options.fine_engine): both values run the same kernels, the
+ * sum over the columns being too small for tensor cores to matter.  TC still needs M (substeps per
+ * slice) a multiple of 16 in 16..128: pe_setup and pe_setup_batch return PE_EINVAL otherwise, and for
+ * PE_FP64 or PE_FORCING_GENERAL. */
 enum { PE_FINE_SIMT = 0, PE_FINE_TC = 1 };
 
 /* DST-I backend of the general forcing path (pe_options.dst_backend): AUTO = radix-2 FFT
@@ -402,19 +400,17 @@ typedef struct {
   double ms_prepare;          /* forcing tables, u0 projection, coarse sweeps (phi/b tables: set-up) */
   double ms_iterations;       /* all graph replays */
   int64_t kernel_launches;    /* kernels launched (graph nodes counted per replay) */
-  int32_t threads, ctas_per_sm; /* launch shape of the persistent fine kernel */
+  int32_t threads, ctas_per_sm; /* launch shape of the persistent walk kernel */
 } pe_batch_result;
 
 /* Validate and lay out all problems (one arena per array kind), compute their
  * spectra and DST-I-free 1D factor transforms.  opt->precision selects the fine
  * stages (PE_MIXED: float32 stages, float64 tables/correction/residual);
- * opt->fine_engine = PE_FINE_TC (PE_MIXED only) runs the stage contraction of every
- * problem on the tensor cores (work items: problem x slice group x 128-mode tile, one
- * persistent launch per column padding; every problem needs M a multiple of 16 in
- * 16..128, else PE_EINVAL).  problems: host array of n_problems. */
+ * opt->fine_engine = PE_FINE_TC (PE_MIXED only) needs M a multiple of 16 in 16..128 of
+ * every problem, else PE_EINVAL.  problems: host array of n_problems. */
 pe_status pe_setup_batch(pe_batch** out, int32_t n_problems, const pe_problem* problems, const pe_options* opt);
 
-/* Pick the persistent fine kernel's launch shape (threads per CTA x CTAs per SM)
+/* Pick the persistent walk kernel's launch shape (threads per CTA x CTAs per SM)
  * by timing the candidates on this batch; cache_path (may be NULL) is a text file
  * of previous choices keyed by device and batch signature, read and appended. */
 pe_status pe_batch_autotune(pe_batch* b, const char* cache_path);
@@ -474,8 +470,7 @@ pe_status pe_learned_samples(pe_ctx* ctx, int32_t n, const double* lam, const do
 pe_status pe_set_learned(pe_ctx* ctx, const pe_mlp* m);
 /* Attach (m != NULL) or detach the learned coarse correction for every problem of the batch
  * (G'(v) = G(v) + delta^ per problem, as pe_set_learned does for one context; band tables of
- * 2048 log-spaced bands per problem and sine term, the learned term summed inside the batched
- * coarse sweep); takes effect at the next pe_batch_solve.  The network must outlive its use. */
+ * 2048 log-spaced bands per problem and sine term, entering the coarse step's column weights); takes effect at the next pe_batch_solve.  The network must outlive its use. */
 pe_status pe_batch_set_learned(pe_batch* b, const pe_mlp* m);
 
 /*

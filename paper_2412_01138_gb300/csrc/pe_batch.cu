@@ -3,14 +3,13 @@
 // Each array kind (slice arrays, tables, forcing factors) lives in one arena; a
 // device table of per-problem records (BProb) holds offsets into the arenas.
 // Work is cut into items:
-//   mode items  (problem, 256 consecutive modes)          coefficient tables, U^0,
-//                                                         coarse sweep, correction
-//   fine items  (problem, slice n, threads*MPT modes)     fine propagator
-// The fine kernel is persistent: every CTA pulls items from an atomic counter
-// and dispatches on the problem's number of forcing terms R (each R has its own
-// register-resident tile body).  One Parareal iteration (reset of the counter,
-// fine sweep, correction, per-problem residual + stop flags, readback of the
-// number of active problems) is captured once as a CUDA graph and replayed.
+//   mode items  (problem, 256 consecutive modes)      coefficient tables, column weights, U^0
+//   walk items  (problem, 128 or 256 modes)           the walk over the problem's slices: fine step,
+//                                                     correction, residual terms (and, in the first
+//                                                     iteration, the coarse iterate)
+// The walk kernel is persistent: every CTA pulls items from an atomic counter, longest first.
+// One Parareal iteration (reset of the counter, walk, per-problem residual + stop flags, readback
+// of the number of active problems) is captured once as a CUDA graph and replayed.
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -23,6 +22,7 @@
 #include <vector>
 
 #include "pe_batch.h"
+#include "pe_contract.cuh"
 #include "pe_phi.cuh"
 
 namespace {
@@ -62,7 +62,8 @@ __global__ void b_axis_tables_kernel(const BProb* __restrict__ probs, const int6
 
 __global__ void b_coef_tables_kernel(const BProb* __restrict__ probs, const ModeItem* __restrict__ items,
                                      int n_items, const double* __restrict__ ratio, double* __restrict__ coefF,
-                                     double* __restrict__ coefG, float* __restrict__ coefF32) {
+                                     double* __restrict__ coefG, float* __restrict__ coefF32,
+                                     float* __restrict__ coefG32) {
   for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
     const ModeItem m = items[it];
     const BProb& B = probs[m.p];
@@ -103,127 +104,195 @@ __global__ void b_coef_tables_kernel(const BProb* __restrict__ probs, const Mode
       b_weights(z, B.p, LG, b);
       double* cg = coefG + B.oCG;
       cg[J] = exp(z);
-      for (int i = 0; i < B.p; ++i) cg[(1 + i) * nd + J] = B.dT * b[i];
+      for (int i = 0; i < B.p; ++i) {
+        cg[(1 + i) * nd + J] = B.dT * b[i];
+        if (coefG32) coefG32[B.oCG + (1 + i) * nd + J] = (float)(B.dT * b[i]);
+      }
     }
   }
 }
 
-// Time tables of every problem, one thread per entry (layout as in the single-problem
-// solver): fine substep starts Y[(n*M + m)*K + k] (float copy: rows of KC = roundup(K, 4)),
-// coarse stage times AG[(n*p + i)*R + r],
-// stage shifts Z[i*K + k].  Column k of a problem is cols[oCol + k] = (term << 1) | kind:
-// kind 0 is amp*time(t) (shift factor e^{as} or cos(ws)), kind 1 the partner amp*cos(wt+phi)
-// of a sinusoid (shift factor sin(ws)).
+// Time tables of every problem, one thread per entry, as the single-problem solver makes them
+// (pe_forcing.cu): column values of every slice, shifts of the fine and coarse nodes, chain powers
+// and scales of the terms.  Column k of a problem is cols[oCol + k] = (term << 1) | kind.
+struct BTables {
+  double *Y, *Z, *chain, *xs;
+  float *Y32, *Z32, *chain32, *xs32;
+};
+
 __global__ void b_time_tables_kernel(const BProb* __restrict__ probs, const int64_t* __restrict__ tt_prefix, int P,
                                      int64_t total, const pe_term* __restrict__ terms,
-                                     const short* __restrict__ cols, double* __restrict__ AF,
-                                     float* __restrict__ AF32, double* __restrict__ AG, float* __restrict__ AG32,
-                                     double* __restrict__ Z, float* __restrict__ Z32) {
+                                     const short* __restrict__ cols, BTables D) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= total) return;
   const int p = find_prob(tt_prefix, P, idx);
   const BProb& B = probs[p];
-  const int R = B.R, K = B.K;
-  const int64_t nrow = (int64_t)B.N * K;
-  const int64_t ng = (int64_t)B.N * B.p * R;
-  int64_t local = idx - tt_prefix[p];
-  if (local < nrow) {
-    // one thread per (slice n, column k) walks the substeps m: the factor at T_n + m dt from
-    // the one at T_n by the exact step e^{a dt} or the rotation by omega dt (angle addition),
-    // two transcendental evaluations per thread instead of one per entry; the rounding grows
-    // by about one unit in the last place per substep (M <= 128)
-    const int k = (int)(local % K), n = (int)(local / K);
+  const int R = B.R, K = B.K, steps = chain_steps(B.M);
+  int64_t e = idx - tt_prefix[p];
+  if (e < (int64_t)B.N * K) {
+    const int n = (int)(e / K), k = (int)(e - (int64_t)n * K);
     const int c = cols[B.oCol + k];
-    const pe_term& T = terms[B.tf + (c >> 1)];
-    const double tn = B.t0 + (double)n * B.dT;
-    const int KC = (K + 3) & ~3;
-    double* af = AF + B.oAF + (int64_t)n * B.M * K + k;
-    float* row32 = AF32 ? AF32 + B.oAF32 + (int64_t)n * B.M * KC : nullptr;
-    auto put = [&](int m, double v) {
-      af[(int64_t)m * K] = v;
-      if (row32) {
-        float* row = row32 + (int64_t)m * KC;
-        row[k] = (float)v;
-        if (k == K - 1)
-          for (int e = K; e < KC; ++e) row[e] = 0.f;
-      }
-    };
-    if (T.tkind == PE_T_SIN) {
-      double sa, ca, sb, cb;
-      sincos(T.tp[0] * tn + T.tp[1], &sa, &ca);
-      sincos(T.tp[0] * B.dt, &sb, &cb);
-      for (int m = 0; m < B.M; ++m) {
-        put(m, T.amp * ((c & 1) ? ca : sa));
-        const double s2 = fma(sa, cb, ca * sb);
-        ca = fma(ca, cb, -(sa * sb));
-        sa = s2;
-      }
+    const double v = column_value(terms[B.tf + (c >> 1)], c & 1, B.t0 + (double)n * B.dT, B.t0 + (double)(n + 1) * B.dT);
+    if (!D.Y32) {
+      D.Y[B.oY + e] = v;
     } else {
-      double e = exp(T.tp[0] * tn);
-      const double eb = exp(T.tp[0] * B.dt);
-      for (int m = 0; m < B.M; ++m) {
-        put(m, T.amp * e);
-        e *= eb;
-      }
+      const int KC = (K + 3) & ~3;
+      float* row = D.Y32 + B.oY32 + (int64_t)n * 2 * KC;
+      row[k] = (float)v;
+      row[KC + k] = (float)(v - (double)(float)v);
+      if (k == K - 1)
+        for (int z = K; z < KC; ++z) row[z] = row[KC + z] = 0.f;
     }
-  } else if (local < nrow + ng) {
-    local -= nrow;
-    int64_t rest = local;
-    const int r = (int)(rest % R); rest /= R;
-    const int i = (int)(rest % B.p); rest /= B.p;
-    const int n = (int)rest;
-    const double Tn = B.t0 + (double)n * B.dT;
-    const double t = Tn + B.cG[i] * B.dT;
-    const pe_term& T = terms[B.tf + r];
-    const double v = T.amp * eval_time(T, t);
-    AG[B.oAG + local] = v;
-    if (AG32) AG32[B.oAG + local] = (float)v;
-  } else {
-    local -= nrow + ng;
-    const int k = (int)(local % K), i = (int)(local / K);
+    return;
+  }
+  e -= (int64_t)B.N * K;
+  const int nf = B.q * K, ng = B.p * K;
+  if (e < nf + ng) {
+    const bool fine = e < nf;
+    const int l = (int)(fine ? e : e - nf), i = l / K, k = l - i * K;
     const int c = cols[B.oCol + k];
-    const pe_term& T = terms[B.tf + (c >> 1)];
-    const double s = B.cF[i] * B.dt;
-    double v;
-    if (T.tkind == PE_T_SIN) v = (c & 1) ? sin(T.tp[0] * s) : cos(T.tp[0] * s);
-    else v = exp(T.tp[0] * s);
-    Z[B.oZ + local] = v;
-    if (Z32) Z32[B.oZ + local] = (float)v;
+    const double v = column_shift(terms[B.tf + (c >> 1)], c & 1, fine ? B.cF[i] : B.cG[i], fine ? B.dt : B.dT);
+    if (D.Y32) D.Z32[B.oZ + e] = (float)v;
+    else D.Z[B.oZ + e] = v;
+    return;
+  }
+  e -= nf + ng;
+  const int s = (int)(e / R) - 1, r = (int)(e - (int64_t)(s + 1) * R);
+  const pe_term& T = terms[B.tf + r];
+  if (s < 0) {
+    const double v = chain_scale(T, B.dt);
+    if (!D.Y32) {
+      D.xs[B.oXs + r] = v;
+    } else {
+      D.xs32[2 * (B.oXs + r)] = (float)v;
+      D.xs32[2 * (B.oXs + r) + 1] = (float)(v - (double)(float)v);
+    }
+    return;
+  }
+  double v[4];
+  const int L = chain_length(B.M, steps, s);
+  chain_power(T, L, B.dt, v[0], v[1]);
+  chain_power(T, 2 * L, B.dt, v[2], v[3]);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int64_t o = B.oCh + (int64_t)(s * R + r) * 4 + i;
+    if (!D.Y32) {
+      D.chain[o] = v[i];
+    } else {
+      D.chain32[2 * o] = (float)v[i];
+      D.chain32[2 * o + 1] = (float)(v[i] - (double)(float)v[i]);
+    }
   }
 }
 
-// Per-mode stage weights W[oW + k*ndof + J] = P_{r(k),J} sum_i (dt b_i)_J Z[oZ + i*K + k],
-// in the arithmetic of T: float64 into W for the float64 fine kernel; float32 (from the
-// float factors and shifts) into W32 in the mixed form, whose fine kernel reads only W32.
+// The learned correction's band tables (Kt null: no network).
+struct BLearn {
+  const double* ratio;    // per-axis mu^K / mu^M (lam = D sum_a ratio)
+  const double* Kt;
+  const double* axisF64;
+  int NB;
+};
+
+// Per-mode column weights V and G of every problem (column_weights_kernel of the single-problem
+// solver over mode items).
 template <typename T>
-__global__ void b_stage_weights_kernel(const BProb* __restrict__ probs, const ModeItem* __restrict__ items,
-                                       int n_items, const short* __restrict__ cols, const T* __restrict__ axisF,
-                                       const double* __restrict__ coefF, const T* __restrict__ Z,
-                                       T* __restrict__ W) {
+__global__ void __launch_bounds__(256) b_column_weights_kernel(const BProb* __restrict__ probs,
+                                                               const ModeItem* __restrict__ items, int n_items,
+                                                               const short* __restrict__ first,
+                                                               const short* __restrict__ cols,
+                                                               const T* __restrict__ axisF, const T* __restrict__ coefF,
+                                                               const T* __restrict__ coefG, const T* __restrict__ Z,
+                                                               const T* __restrict__ chain, const T* __restrict__ xs,
+                                                               T* __restrict__ V, T* __restrict__ G, BLearn L) {
+  constexpr bool F64 = sizeof(T) == 8;
+  constexpr int kERows = F64 ? 1 : 2, kPair = F64 ? 1 : 2;
   for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
     const ModeItem mi = items[it];
     const BProb& B = probs[mi.p];
     const int64_t J = mi.J0 + threadIdx.x;
     if (J >= B.g.ndof) continue;
     const int64_t nd = B.g.ndof;
+    const int K = B.K, R = B.R, q = B.q, p = B.p, steps = chain_steps(B.M);
     int j[PE_MAX_D];
     unflatten(B.g, J, j);
-    T b[PE_MAX_S];
+    const T* cf = coefF + B.oCF;
+    T b[PE_MAX_S], bg[PE_MAX_S];
 #pragma unroll
-    for (int i = 0; i < PE_MAX_S; ++i) b[i] = i < B.q ? (T)coefF[B.oCF + (int64_t)(1 + i) * nd + J] : T(0);
+    for (int i = 0; i < PE_MAX_S; ++i) {
+      b[i] = i < q ? cf[(int64_t)(kERows + i) * nd + J] : T(0);
+      bg[i] = i < p ? coefG[B.oCG + (int64_t)(1 + i) * nd + J] : T(0);
+    }
+    const T Eh = cf[J];
+    T El = T(0);
+    if constexpr (!F64) El = cf[nd + J];
+    int band = 0;
+    double bf = 0.0;
+    if (L.Kt) {
+      double sum = 0.0;
+#pragma unroll
+      for (int a = 0; a < PE_MAX_D; ++a) if (a < B.g.d) sum += L.ratio[B.oMu + B.g.off[a] + j[a]];
+      double pos = (log(B.D * sum * B.dT) - B.lloglo) / B.lstep;
+      pos = fmin(fmax(pos, 0.0), (double)(L.NB - 1) - 1e-9);
+      band = (int)pos;
+      bf = pos - (double)band;
+    }
     const T* ax = axisF + B.oAx;
-    const T* z = Z + B.oZ;
-    for (int k = 0; k < B.K; ++k) {
-      const int r = cols[B.oCol + k] >> 1;
-      T P = ax[(int64_t)B.R * B.g.off[0] + (int64_t)r * B.g.n[0] + j[0]];
+    const T* ZF = Z + B.oZ;
+    const T* ZG = ZF + (int64_t)q * K;
+    for (int r = 0; r < R; ++r) {
+      const int k = first[B.oFirst + r];
+      const bool two = k + 1 < K && (cols[B.oCol + k + 1] >> 1) == r;
+      T P = ax[(int64_t)R * B.g.off[0] + (int64_t)r * B.g.n[0] + j[0]];
 #pragma unroll
-      for (int a = 1; a < PE_MAX_D; ++a) if (a < B.g.d)
-        P *= ax[(int64_t)B.R * B.g.off[a] + (int64_t)r * B.g.n[a] + j[a]];
-      T sum = T(0);
+      for (int a = 1; a < PE_MAX_D; ++a) if (a < B.g.d) P *= ax[(int64_t)R * B.g.off[a] + (int64_t)r * B.g.n[a] + j[a]];
+      T br = T(0), bi = T(0), gr = T(0), gi = T(0);
 #pragma unroll
       for (int i = 0; i < PE_MAX_S; ++i)
-        if (i < B.q) sum = fma(b[i], z[(int64_t)i * B.K + k], sum);
-      W[B.oW + (int64_t)k * nd + J] = P * sum;
+        if (i < q) {
+          br = fma(b[i], ZF[i * K + k], br);
+          if (two) bi = fma(b[i], ZF[i * K + k + 1], bi);
+        }
+#pragma unroll
+      for (int i = 0; i < PE_MAX_S; ++i)
+        if (i < p) {
+          gr = fma(bg[i], ZG[i * K + k], gr);
+          if (two) gi = fma(bg[i], ZG[i * K + k + 1], gi);
+        }
+      gr *= P;
+      gi *= P;
+      if (L.Kt && two) {
+        const double* ax64 = L.axisF64 + B.oAx;
+        double Pd = ax64[(int64_t)R * B.g.off[0] + (int64_t)r * B.g.n[0] + j[0]];
+#pragma unroll
+        for (int a = 1; a < PE_MAX_D; ++a)
+          if (a < B.g.d) Pd *= ax64[(int64_t)R * B.g.off[a] + (int64_t)r * B.g.n[a] + j[a]];
+        const double* k0 = L.Kt + B.oKt + 2 * ((int64_t)r * L.NB + band);
+        gr += (T)(Pd * ((1.0 - bf) * k0[0] + bf * k0[2]));
+        gi += (T)(Pd * ((1.0 - bf) * k0[1] + bf * k0[3]));
+      }
+      T v0, v1;
+      const T* ch = chain + kPair * (B.oCh + 4 * r);
+      const T* x = xs + kPair * (B.oXs + r);
+      if constexpr (F64) {
+        double Sr, Si;
+        chain_sum(Eh * x[0], B.M, steps, ch, 4 * R, Sr, Si);
+        v0 = P * fma(br, Sr, -(bi * Si));
+        v1 = P * fma(br, Si, bi * Sr);
+      } else {
+        F2 Sr, Si;
+        chain_sum(f2_mul(F2{Eh, El}, F2{x[0], x[1]}), B.M, steps, ch, 8 * R, Sr, Si);
+        const F2 br2{br, 0.f}, bi2{bi, 0.f};
+        const F2 re = f2_add(f2_mul(br2, Sr), f2_neg(f2_mul(bi2, Si)));
+        const F2 im = f2_add(f2_mul(br2, Si), f2_mul(bi2, Sr));
+        v0 = fmaf(P, re.h, P * re.l);
+        v1 = fmaf(P, im.h, P * im.l);
+      }
+      V[B.oV + (int64_t)k * nd + J] = v0;
+      G[B.oV + (int64_t)k * nd + J] = gr;
+      if (two) {
+        V[B.oV + (int64_t)(k + 1) * nd + J] = v1;
+        G[B.oV + (int64_t)(k + 1) * nd + J] = gi;
+      }
     }
   }
 }
@@ -301,273 +370,168 @@ __global__ void b_u0_kernel(const BProb* __restrict__ probs, const ModeItem* __r
   }
 }
 
-// coarse sweep (k = 0) of every problem; P_{r,J} staged per thread in shared memory
-// Slices of loads each thread keeps in flight in the sequential correction (its
-// inputs do not depend on the recurrence, so they are fetched kPF slices ahead).
-constexpr int kPF = 4;
+// The walk of the single-problem solver (walk_kernel, pe_sweep.cu) over items of many problems: F =
+// fma(E_F^M, o, F^M(0)_n), U^{n+1} = fma(E_G, d, F), d <- U^{n+1} - o'; FIRST makes the coarse
+// iterate o' = fma(E_G, o, gG_n) on the way, else o' is the old U^{n+1}.
+//
+// T = float (mixed form): the item's K column weights in registers, KB = the batch's largest K rounded up
+// to 8 (the float32 FMAs of the padding run under the five or six float64 operations per mode and slice
+// that bound the kernel).  T = double: weights in shared memory with a runtime column count, since
+// every padded column would cost a float64 operation, and one per operation is what two shared-memory
+// reads hide under.  A batch has modes enough for one thread per mode, so that the float64 forced parts
+// never go to memory either.  64 uneven 2D problems (1.6M modes, 16 to 64 slices, 9 to 33 columns), mixed: 0.89 ms for
+// the coarse sweep and first iteration in one pass, 0.76 ms for a further one, against 0.94 ms (every substep on the
+// tensor cores) + 0.49 ms (correction) per iteration beside the coarse sweep.
+constexpr int kPF = 8;  // slices of loads in flight
 
-// Coarse sweep of k = 0 for every problem (item-strided grid: an item is 256 modes of one
-// problem), U^{n+1} = E_G U^n + gG_n with the coarse forcing gG_n = sum_i b_i sum_r
-// A_r(T_n + c_i dT) P_{r,J} made on the fly: the weights P_{r,J} sit in registers (RB =
-// roundup(PE_BATCH_MAX_TERMS, 4), zero past R) and the item's time factors are staged in
-// shared memory a chunk of slices at a time (rows of RB, read as float4 / double2
-// broadcasts).  TF = float in the mixed form (the coarse forcing only sets the first coarse
-// iterate; the affine correction never reads it again).
-constexpr int kCoarseRB = (PE_BATCH_MAX_TERMS + 3) / 4 * 4;
-constexpr int kCoarseSmem = 16 * 1024;  // bytes of staged time factors per CTA
-
-// LEARN: the learned term of G' = G + delta^ is added per slice, sum_r (A_r cos_{r,n} + B_r sin_{r,n})
-// with A_r = P_{r,J} amp_r Im K^, B_r = P_{r,J} amp_r Re K^ (K^ interpolated linearly in
-// log(lam dT) between the problem's band centres), as the single-problem coarse sweep does.
-struct BLearn {
-  const double* ratio;    // per-axis mu^K / mu^M (lam = D sum_a ratio)
-  const pe_term* terms;
-  const double* Kt;       // band tables
-  const float2* Ph;       // phase tables
-  int NB;
+template <typename T>
+struct BWalkArgs {
+  const BProb* probs;
+  const WalkItem* items;
+  int n_items, SL;       // SL: slices staged at a time (a multiple of kPF)
+  const int* active;
+  int* counter;
+  const T *Y, *V, *G;
+  const double *coefF, *coefG, *muM;
+  double *U, *partials;
 };
 
-template <typename TF, bool LEARN>
-__global__ void __launch_bounds__(256) b_coarse_kernel(const BProb* __restrict__ probs,
-                                                       const ModeItem* __restrict__ items, int n_items,
-                                                       const double* __restrict__ axisF, const TF* __restrict__ AG,
-                                                       const double* __restrict__ coefG, double* __restrict__ U,
-                                                       BLearn L, const float* __restrict__ axisF32) {
-  constexpr int RB = kCoarseRB;
+template <typename T, int KB, bool FIRST>
+__global__ void __launch_bounds__(256) b_walk_kernel(BWalkArgs<T> a) {
+  constexpr bool F64 = sizeof(T) == 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  TF* sA = reinterpret_cast<TF*>(smem_raw);  // [chunk * p][RB]
-  for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
-    const ModeItem m = items[it];
-    const BProb& B = probs[m.p];
-    const int64_t J = m.J0 + threadIdx.x;
-    const int64_t nd = B.g.ndof;
-    const bool on = J < nd;  // no early exit: the staging below needs every thread's barrier
-    const int R = B.R, p = B.p, N = B.N;
-    TF P[RB];
-#pragma unroll
-    for (int r = 0; r < RB; ++r) P[r] = TF(0);
-    TF b[PE_MAX_S];
-#pragma unroll
-    for (int i = 0; i < PE_MAX_S; ++i) b[i] = TF(0);
-    double E = 0.0, c = 0.0;
-    const double* cg = coefG + B.oCG;
-    float LA[LEARN ? kCoarseRB : 1], LB[LEARN ? kCoarseRB : 1];
-#pragma unroll
-    for (int r = 0; r < (LEARN ? kCoarseRB : 1); ++r) {
-      LA[r] = 0.f;
-      LB[r] = 0.f;
+  __shared__ double sh[32];
+  __shared__ int s_item;
+  const int tid = threadIdx.x, B_ = blockDim.x;
+  T* sY = reinterpret_cast<T*>(smem_raw);  // float: [SL][2 KB]; double: [SL][K]
+  for (;;) {
+    if (tid == 0) s_item = atomicAdd(a.counter, 1);
+    __syncthreads();
+    const int it = s_item;
+    if (it >= a.n_items) return;
+    const WalkItem mi = a.items[it];
+    if (!a.active[mi.p]) {  // uniform over the CTA
+      __syncthreads();
+      continue;
     }
+    const BProb& B = a.probs[mi.p];
+    const int64_t J = mi.J0 + tid, nd = B.g.ndof;
+    const int N = B.N, K = B.K;
+    const bool on = J < nd;
+    T* sV = sY + (F64 ? a.SL * K : 0);  // double: [K][threads], then G
+    float V[F64 ? 1 : KB], G[!F64 && FIRST ? KB : 1];
+    if constexpr (F64) {
+      for (int k = 0; k < K; ++k) {
+        sV[k * B_ + tid] = on ? a.V[B.oV + (int64_t)k * nd + J] : T(0);
+        if constexpr (FIRST) sV[(K + k) * B_ + tid] = on ? a.G[B.oV + (int64_t)k * nd + J] : T(0);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < KB; ++k) {
+        V[k] = on && k < K ? a.V[B.oV + (int64_t)k * nd + J] : 0.f;
+        if constexpr (FIRST) G[k] = on && k < K ? a.G[B.oV + (int64_t)k * nd + J] : 0.f;
+      }
+    }
+    double E = 0.0, EM = 0.0, o = 0.0, d = 0.0, sd = 0.0, su = 0.0, w = 0.0;
+    double* U = a.U + B.oU + J;
     if (on) {
+      E = a.coefG[B.oCG + J];
+      EM = a.coefF[B.oCF + (int64_t)(B.q + 1) * nd + J];
+      o = U[0];
       int j[PE_MAX_D];
       unflatten(B.g, J, j);
-      if constexpr (LEARN) {
-        double s = 0.0;
+      w = a.muM[B.oMu + B.g.off[0] + j[0]];
 #pragma unroll
-        for (int a = 0; a < PE_MAX_D; ++a) if (a < B.g.d) s += L.ratio[B.oMu + B.g.off[a] + j[a]];
-        double pos = (log(B.D * s * B.dT) - B.lloglo) / B.lstep;
-        pos = fmin(fmax(pos, 0.0), (double)(L.NB - 1) - 1e-9);
-        const int b0 = (int)pos;
-        const double f = pos - (double)b0;
-#pragma unroll
-        for (int r = 0; r < kCoarseRB; ++r) {
-          if (r < R && L.terms[B.tf + r].tkind == PE_T_SIN) {
-            double Pd = axisF[B.oAx + (int64_t)R * B.g.off[0] + (int64_t)r * B.g.n[0] + j[0]];
-#pragma unroll
-            for (int a = 1; a < PE_MAX_D; ++a)
-              if (a < B.g.d) Pd *= axisF[B.oAx + (int64_t)R * B.g.off[a] + (int64_t)r * B.g.n[a] + j[a]];
-            const double* k0 = L.Kt + B.oKt + 2 * ((int64_t)r * L.NB + b0);
-            const double Kre = (1.0 - f) * k0[0] + f * k0[2];
-            const double Kim = (1.0 - f) * k0[1] + f * k0[3];
-            const double cc = Pd * L.terms[B.tf + r].amp;
-            LA[r] = (float)(cc * Kim);
-            LB[r] = (float)(cc * Kre);
-          }
-        }
-      }
-      // the source weights P_{r,J}: in the mixed form from the float32 factors in float32 (as
-      // the single-problem sweep forms them; no float64 product and conversion per term)
-#pragma unroll
-      for (int r = 0; r < RB; ++r) {
-        if (r < R) {
-          if constexpr (sizeof(TF) == 4) {
-            float v = axisF32[B.oAx + (int64_t)R * B.g.off[0] + (int64_t)r * B.g.n[0] + j[0]];
-#pragma unroll
-            for (int a = 1; a < PE_MAX_D; ++a)
-              if (a < B.g.d) v *= axisF32[B.oAx + (int64_t)R * B.g.off[a] + (int64_t)r * B.g.n[a] + j[a]];
-            P[r] = v;
-          } else {
-            double v = axisF[B.oAx + (int64_t)R * B.g.off[0] + (int64_t)r * B.g.n[0] + j[0]];
-#pragma unroll
-            for (int a = 1; a < PE_MAX_D; ++a)
-              if (a < B.g.d) v *= axisF[B.oAx + (int64_t)R * B.g.off[a] + (int64_t)r * B.g.n[a] + j[a]];
-            P[r] = (TF)v;
-          }
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < PE_MAX_S; ++i)
-        if (i < p) b[i] = (TF)cg[(1 + i) * nd + J];
-      E = cg[J];
-      c = U[B.oU + J];
+      for (int x = 1; x < PE_MAX_D; ++x) if (x < B.g.d) w *= a.muM[B.oMu + B.g.off[x] + j[x]];
     }
-    const TF* ag = AG + B.oAG;
-    const int CS = max(1, kCoarseSmem / (int)(p * RB * sizeof(TF)));  // slices per chunk
-    for (int n0 = 0; n0 < N; n0 += CS) {
-      const int nc = min(CS, N - n0);
-      __syncthreads();  // the previous chunk's (or item's) reads of sA are done
-      for (int e = threadIdx.x; e < nc * p * RB; e += blockDim.x) {
-        const int row = e / RB, r = e - row * RB;
-        sA[e] = r < R ? ag[((int64_t)n0 * p + row) * R + r] : TF(0);
+    double on1[FIRST ? 1 : kPF];
+    auto fetch = [&](int n0) {
+      if constexpr (!FIRST) {
+#pragma unroll
+        for (int e = 0; e < kPF; ++e) on1[e] = on && n0 + e < N ? U[(int64_t)(n0 + e + 1) * nd] : 0.0;
+      }
+    };
+    fetch(0);
+    const int KC = F64 ? K : (K + 3) & ~3;
+    for (int c0 = 0; c0 < N; c0 += a.SL) {
+      const int c1 = min(N, c0 + a.SL), rows = (c1 - c0 + kPF - 1) / kPF * kPF;
+      __syncthreads();  // the previous chunk's (or item's) reads are done
+      if constexpr (F64) {
+        const T* src = a.Y + B.oY + (int64_t)c0 * K;
+        for (int e = tid; e < rows * K; e += B_) sY[e] = e < (c1 - c0) * K ? src[e] : T(0);
+      } else {
+        // rows of KC columns widened to KB with zeros, high and low parts
+        const T* src = a.Y + B.oY32 + (int64_t)c0 * 2 * KC;
+        for (int e = tid; e < rows * 2 * KB; e += B_) {
+          const int row = e / KB, k = e - row * KB;
+          sY[e] = row < 2 * (c1 - c0) && k < KC ? src[row * KC + k] : T(0);
+        }
       }
       __syncthreads();
       if (on) {
-        for (int n = 0; n < nc; ++n) {
-          TF acc = TF(0);
+        for (int n0 = c0; n0 < c1; n0 += kPF) {
+          double o1[FIRST ? 1 : kPF];
+          if constexpr (!FIRST) {
 #pragma unroll
-          for (int i = 0; i < PE_MAX_S; ++i) {
-            if (i < p) {
-              const TF* a = sA + ((int64_t)n * p + i) * RB;
-              TF gi = TF(0);
-              if constexpr (sizeof(TF) == 4) {
+            for (int e = 0; e < kPF; ++e) o1[e] = on1[e];
+            fetch(n0 + kPF);
+          }
+          double fv[F64 ? kPF : 1], gv[F64 && FIRST ? kPF : 1];
+          if constexpr (F64) {
 #pragma unroll
-                for (int r = 0; r < RB; r += 4) {
-                  const float4 v = *reinterpret_cast<const float4*>(a + r);
-                  gi = fmaf(v.x, P[r], gi);
-                  gi = fmaf(v.y, P[r + 1], gi);
-                  gi = fmaf(v.z, P[r + 2], gi);
-                  gi = fmaf(v.w, P[r + 3], gi);
-                }
-              } else {
+            for (int e = 0; e < kPF; ++e) {
+              fv[e] = 0.0;
+              if constexpr (FIRST) gv[e] = 0.0;
+            }
+            for (int k = 0; k < K; ++k) {
+              const T v = sV[k * B_ + tid];
+              T g = T(0);
+              if constexpr (FIRST) g = sV[(K + k) * B_ + tid];
 #pragma unroll
-                for (int r = 0; r < RB; r += 2) {
-                  const double2 v = *reinterpret_cast<const double2*>(a + r);
-                  gi = fma(v.x, P[r], gi);
-                  gi = fma(v.y, P[r + 1], gi);
-                }
+              for (int e = 0; e < kPF; ++e) {
+                const T y = sY[(n0 - c0 + e) * K + k];
+                fv[e] = fma(y, v, fv[e]);
+                if constexpr (FIRST) gv[e] = fma(y, g, gv[e]);
               }
-              acc = fma(b[i], gi, acc);
             }
           }
-          double gn;
-          if constexpr (sizeof(TF) == 4) gn = widen_f32(acc);  // exact, off the float64 pipe
-          else gn = acc;
-          if constexpr (LEARN) {
-            float dl = 0.f;
-            const float2* ph = L.Ph + B.oPh + n0 + n;
 #pragma unroll
-            for (int r = 0; r < kCoarseRB; ++r)
-              if (r < R) {
-                const float2 e = __ldg(ph + (int64_t)r * N);
-                dl = fmaf(LA[r], e.x, fmaf(LB[r], e.y, dl));
-              }
-            gn += widen_f32(dl);
+          for (int e = 0; e < kPF; ++e) {
+            const int n = n0 + e;
+            double fn, gn = 0.0;
+            if constexpr (F64) {
+              fn = fv[e];
+              if constexpr (FIRST) gn = gv[e];
+            } else {
+              const float* y = reinterpret_cast<const float*>(sY) + (n - c0) * 2 * KB;
+              fn = widen_f32(column_dot<KB>(y, V));
+              if constexpr (FIRST) gn = widen_f32(column_dot<KB>(y, G));
+            }
+            if (n < N) {
+              const double un = fma(E, d, fma(EM, o, fn));
+              U[(int64_t)(n + 1) * nd] = un;
+              if constexpr (FIRST) o = fma(E, o, gn);
+              else o = o1[e];
+              d = un - o;
+              sd = fma(d, d, sd);
+              su = fma(un, un, su);
+            }
           }
-          c = fma(E, c, gn);
-          U[B.oU + (int64_t)(n0 + n + 1) * nd + J] = c;
         }
       }
     }
-  }
-}
-
-template <typename T>
-__device__ inline T block_sum(T v, T* sh) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) sh[wid] = v;
-  __syncthreads();
-  T out = T(0);
-  if (threadIdx.x < 32) {
-    T x = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : T(0);
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    out = x;
-  }
-  __syncthreads();
-  return out;
-}
-
-// correction + residual partial sums of every active problem (item-strided grid).  G is
-// affine in its argument, so U^{n+1,(k+1)} = G(U^{n,(k+1)}) + Fbar^{n+1} - G(U^{n,(k)}) is
-// evaluated as Fbar^{n+1} + E_G (U^{n,(k+1)} - U^{n,(k)}) (no stored coarse values).
-__global__ void __launch_bounds__(256) b_correction_kernel(const BProb* __restrict__ probs,
-                                                           const ModeItem* __restrict__ items, int n_items,
-                                                           const int* __restrict__ active,
-                                                           const double* __restrict__ muM,
-                                                           const double* __restrict__ coefG,
-                                                           const double* __restrict__ Fbar,
-                                                           double* __restrict__ U, double* __restrict__ partials) {
-  __shared__ double sh[32];
-  for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
-    const ModeItem m = items[it];
-    const BProb& B = probs[m.p];
-    if (!active[m.p]) continue;  // uniform over the CTA
-    const int64_t J = m.J0 + threadIdx.x;
-    double sd = 0.0, su = 0.0, w = 0.0;
-    if (J < B.g.ndof) {
-      const int64_t nd = B.g.ndof;
-      const int N = B.N;
-      int j[PE_MAX_D];
-      unflatten(B.g, J, j);
-      w = muM[B.oMu + B.g.off[0] + j[0]];
-#pragma unroll
-      for (int a = 1; a < PE_MAX_D; ++a) if (a < B.g.d) w *= muM[B.oMu + B.g.off[a] + j[a]];
-      const double E = coefG[B.oCG + J];
-      double* Up = U + B.oU;
-      const double* fp = Fbar + B.oS;
-      // U^0 is the same in every iterate (d = U^n_new - U^n_old starts at 0); the loads of the
-      // next kPF slices are issued while the current kPF are combined.  Four FP64 operations
-      // per slice: the difference d is both the next slice's correction and this slice's
-      // residual term.
-      double d = 0.0;
-      double f0[kPF], o0[kPF], f1[kPF], o1[kPF];
-#pragma unroll
-      for (int e = 0; e < kPF; ++e) {
-        const int64_t o = (int64_t)e * nd + J;
-        const bool in = e < N;
-        f0[e] = in ? fp[o] : 0.0;
-        o0[e] = in ? Up[o + nd] : 0.0;
-      }
-      for (int n0 = 0; n0 < N; n0 += kPF) {
-#pragma unroll
-        for (int e = 0; e < kPF; ++e) {
-          const int n = n0 + kPF + e;
-          const int64_t o = (int64_t)n * nd + J;
-          const bool in = n < N;
-          f1[e] = in ? fp[o] : 0.0;
-          o1[e] = in ? Up[o + nd] : 0.0;
-        }
-#pragma unroll
-        for (int e = 0; e < kPF; ++e) {
-          const int n = n0 + e;
-          if (n < N) {
-            const double nxt = fma(E, d, f0[e]);
-            Up[(int64_t)(n + 1) * nd + J] = nxt;
-            d = nxt - o0[e];
-            sd = fma(d, d, sd);
-            su = fma(nxt, nxt, su);
-          }
-        }
-#pragma unroll
-        for (int e = 0; e < kPF; ++e) {
-          f0[e] = f1[e];
-          o0[e] = o1[e];
-        }
-      }
-    }
-    // the weight mu^M_J is the same for every slice of the mode: applied once
-    sd *= w;
-    su *= w;
-    sd = block_sum(sd, sh);
-    su = block_sum(su, sh);
-    if (threadIdx.x == 0) {
-      partials[2 * it] = sd;
-      partials[2 * it + 1] = su;
+    sd = block_sum(sd * w, sh);
+    su = block_sum(su * w, sh);
+    if (tid == 0) {
+      a.partials[2 * mi.slot] = sd;
+      a.partials[2 * mi.slot + 1] = su;
     }
   }
 }
 
 // one CTA per problem: residual, iteration count, stop flag, active count
-__global__ void b_reduce_kernel(const BProb* __restrict__ probs, int P, const double* __restrict__ partials,
+__global__ void b_reduce_kernel(const BProb* __restrict__ probs, int P, int item_modes,
+                                const double* __restrict__ partials,
                                 int* __restrict__ active, int* __restrict__ kcount, double* __restrict__ resid,
                                 double tol, int* __restrict__ n_active, int* __restrict__ nonfinite) {
   __shared__ double sh[32];
@@ -576,7 +540,8 @@ __global__ void b_reduce_kernel(const BProb* __restrict__ probs, int P, const do
   const BProb& B = probs[p];
   if (!active[p]) return;  // uniform
   double sd = 0.0, su = 0.0;
-  for (int i = threadIdx.x; i < B.nItems; i += blockDim.x) {
+  const int nItems = (int)((B.g.ndof + item_modes - 1) / item_modes);  // at slots oItems + i
+  for (int i = threadIdx.x; i < nItems; i += blockDim.x) {
     sd += partials[2 * (B.oItems + i)];
     su += partials[2 * (B.oItems + i) + 1];
   }
@@ -603,11 +568,83 @@ __global__ void b_reduce_kernel(const BProb* __restrict__ probs, int P, const do
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-pe_status batch_set_attributes(pe_batch* b) {
-  const size_t smem = sizeof(double) * (size_t)(b->nmax + 2 * (b->nmax + 1));
-  PE_CUDA_TRY(cudaFuncSetAttribute(b_axis_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+namespace {
 
-  return PE_OK;  // the fine kernels stage at most 48 KB (pick_mchunk), the default limit
+// Dynamic shared memory of the walk and the slices it stages: float rows of 2 KB within 32 KB; double rows
+// of Kmax beside the weights of `threads` modes.
+template <typename T>
+size_t walk_smem(const pe_batch* b, int threads, int KB, int* SL) {
+  int Nmax = 1;
+  for (const BProb& B : b->probs) Nmax = std::max(Nmax, B.N);
+  const size_t row = sizeof(T) * (size_t)(sizeof(T) == 8 ? b->Kmax : 2 * KB);
+  int sl = (int)((size_t)32 * 1024 / row) / kPF * kPF;
+  sl = std::max(kPF, std::min(sl, (Nmax + kPF - 1) / kPF * kPF));
+  *SL = sl;
+  return row * sl + (sizeof(T) == 8 ? sizeof(T) * 2 * (size_t)b->Kmax * threads : 0);
+}
+
+template <typename T, int KB, bool FIRST>
+pe_status walk_launch(pe_batch* b, cudaStream_t st, int threads, int ctas, bool set_attr) {
+  int SL = 0;
+  const size_t smem = walk_smem<T>(b, threads, KB, &SL);
+  if (set_attr) {  // at set-up, outside any capture: the limit any batch may need (40 columns, 256 threads)
+    if (sizeof(T) == 8)
+      PE_CUDA_TRY(cudaFuncSetAttribute(b_walk_kernel<T, KB, FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       200 * 1024));
+    return PE_OK;
+  }
+  const WalkItems& wi = threads == 128 ? b->walk128 : b->walk256;
+  BWalkArgs<T> a{};
+  a.probs = b->d_probs;
+  a.items = wi.d_items;
+  a.n_items = wi.n;
+  a.SL = SL;
+  a.active = b->active;
+  a.counter = b->counter;
+  if constexpr (sizeof(T) == 8) {
+    a.Y = b->Y;
+    a.V = b->V;
+    a.G = b->G;
+  } else {
+    a.Y = b->Y32;
+    a.V = b->V32;
+    a.G = b->G32;
+  }
+  a.coefF = b->coefF;
+  a.coefG = b->coefG;
+  a.muM = b->muM;
+  a.U = b->U;
+  a.partials = b->partials;
+  const int grid = std::min(b->sm_count * ctas, wi.n);
+  b_walk_kernel<T, KB, FIRST><<<grid, threads, smem, st>>>(a);
+  PE_CUDA_TRY(cudaGetLastError());
+  return PE_OK;
+}
+
+pe_status launch_walk(pe_batch* b, cudaStream_t st, int threads, int ctas, bool first, bool set_attr = false) {
+  if (b->precision != PE_MIXED)
+    return first ? walk_launch<double, 8, true>(b, st, threads, ctas, set_attr)
+                 : walk_launch<double, 8, false>(b, st, threads, ctas, set_attr);
+  switch ((b->Kmax + 7) / 8) {
+#define PE_BW(X)                                                                       \
+  case X:                                                                              \
+    return first ? walk_launch<float, 8 * X, true>(b, st, threads, ctas, set_attr)     \
+                 : walk_launch<float, 8 * X, false>(b, st, threads, ctas, set_attr);
+    PE_BW(1) PE_BW(2) PE_BW(3) PE_BW(4) PE_BW(5)
+#undef PE_BW
+  }
+  return pe_fail(PE_EINVAL, "batch: source columns must be in 1..40");
+}
+
+}  // namespace
+
+pe_status batch_set_attributes(pe_batch* b) {
+  // the limit any batch may need (n_a <= 4096)
+  PE_CUDA_TRY(cudaFuncSetAttribute(b_axis_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)sizeof(double) * (4096 + 2 * 4097)));
+  for (int threads = 128; threads <= 256; threads += 128)
+    for (int first = 0; first < 2; ++first) PE_TRY(launch_walk(b, b->stream, threads, 1, first != 0, true));
+  return PE_OK;
 }
 
 pe_status batch_launch_axis_tables(pe_batch* b) {
@@ -622,7 +659,8 @@ pe_status batch_launch_axis_tables(pe_batch* b) {
 // phi/b coefficient tables: a function of lam, the step sizes and the nodes only (made at set-up)
 pe_status batch_launch_coef_tables(pe_batch* b) {
   b_coef_tables_kernel<<<b->sm_count * 8, 256, 0, b->stream>>>(b->d_probs, b->d_mode_items, b->n_mode_items,
-                                                               b->ratio, b->coefF, b->coefG, b->coefF32);
+                                                               b->ratio, b->coefF, b->coefG, b->coefF32,
+                                                               b->coefG32);
   b->launches += 1;
   PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;
@@ -630,113 +668,57 @@ pe_status batch_launch_coef_tables(pe_batch* b) {
 
 pe_status batch_launch_prepare(pe_batch* b) {
   const int grid_items = b->sm_count * 8;
-  // time factors
-  b_time_tables_kernel<<<(unsigned)((b->tt_total + 255) / 256), 256, 0, b->stream>>>(
-      b->d_probs, b->d_tt_prefix, b->P, b->tt_total, b->d_terms, b->d_cols, b->AF, b->AF32, b->AG, b->AG32, b->Z,
-      b->Z32);
+  // time tables
+  const BTables D{b->Y, b->Z, b->chain, b->xs, b->Y32, b->Z32, b->chain32, b->xs32};
+  b_time_tables_kernel<<<(unsigned)((b->tt_total + 127) / 128), 128, 0, b->stream>>>(
+      b->d_probs, b->d_tt_prefix, b->P, b->tt_total, b->d_terms, b->d_cols, D);
   // per-axis factors of forcing and initial data
   const size_t smem = sizeof(double) * (size_t)(b->nmax + 2 * (b->nmax + 1));
   b_axis_factor_kernel<<<b->n_factor_jobs, 256, smem, b->stream>>>(b->d_probs, b->d_factor_jobs, b->d_terms,
                                                                    b->gauss, b->muM, b->axisF, b->axisF32,
                                                                    b->axisU0);
-  // per-mode stage weights of the fine step
-  if (b->precision == PE_MIXED)
-    b_stage_weights_kernel<float><<<grid_items, 256, 0, b->stream>>>(
-        b->d_probs, b->d_mode_items, b->n_mode_items, b->d_cols, b->axisF32, b->coefF, b->Z32, b->W32);
-  else
-    b_stage_weights_kernel<double><<<grid_items, 256, 0, b->stream>>>(
-        b->d_probs, b->d_mode_items, b->n_mode_items, b->d_cols, b->axisF, b->coefF, b->Z, b->W);
-  b_u0_kernel<<<grid_items, 256, 0, b->stream>>>(b->d_probs, b->d_mode_items, b->n_mode_items, b->d_terms, b->axisU0,
-                                                 b->U);
-  // the tensor-core engine's split operand images of every problem
-  if (b->fine_engine == PE_FINE_TC) PE_TRY(batch_tc_prepare(b, b->stream));
-  // the coarse forcing is iterate-independent and cancels in G(U^{k+1}) - G(U^k): the mixed
-  // form evaluates it in float32, the recurrence stays float64
-  // learned correction: band and phase tables first, the term summed inside the coarse sweep
+  // per-mode column weights, the learned correction's bands first
   BLearn L{};
   if (b->mlp) {
     PE_TRY(batch_learned_tables(b, b->stream));
     L.ratio = b->ratio;
-    L.terms = b->d_terms;
     L.Kt = b->Kt;
-    L.Ph = b->Ph;
+    L.axisF64 = b->axisF;
     L.NB = kBatchLearnedBands;
   }
-  if (b->precision == PE_MIXED && b->mlp)
-    b_coarse_kernel<float, true><<<grid_items, 256, kCoarseSmem, b->stream>>>(
-        b->d_probs, b->d_mode_items, b->n_mode_items, b->axisF, b->AG32, b->coefG, b->U, L, b->axisF32);
-  else if (b->precision == PE_MIXED)
-    b_coarse_kernel<float, false><<<grid_items, 256, kCoarseSmem, b->stream>>>(
-        b->d_probs, b->d_mode_items, b->n_mode_items, b->axisF, b->AG32, b->coefG, b->U, L, b->axisF32);
-  else if (b->mlp)
-    b_coarse_kernel<double, true><<<grid_items, 256, kCoarseSmem, b->stream>>>(
-        b->d_probs, b->d_mode_items, b->n_mode_items, b->axisF, b->AG, b->coefG, b->U, L, (const float*)nullptr);
+  if (b->precision == PE_MIXED)
+    b_column_weights_kernel<float><<<b->n_mode_items, 256, 0, b->stream>>>(
+        b->d_probs, b->d_mode_items, b->n_mode_items, b->d_first, b->d_cols, b->axisF32, b->coefF32, b->coefG32, b->Z32,
+        b->chain32, b->xs32, b->V32, b->G32, L);
   else
-    b_coarse_kernel<double, false><<<grid_items, 256, kCoarseSmem, b->stream>>>(
-        b->d_probs, b->d_mode_items, b->n_mode_items, b->axisF, b->AG, b->coefG, b->U, L, (const float*)nullptr);
-  b->launches += 5;
+    b_column_weights_kernel<double><<<b->n_mode_items, 256, 0, b->stream>>>(
+        b->d_probs, b->d_mode_items, b->n_mode_items, b->d_first, b->d_cols, b->axisF, b->coefF, b->coefG, b->Z,
+        b->chain, b->xs, b->V, b->G, L);
+  b_u0_kernel<<<grid_items, 256, 0, b->stream>>>(b->d_probs, b->d_mode_items, b->n_mode_items, b->d_terms, b->axisU0,
+                                                 b->U);
+  b->launches += 4;
   PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;
 }
 
-// One persistent launch per column class present in the batch, each over its own items
-// and counter (counter[c]); grids never exceed the class's item count.
-static pe_status launch_fine(pe_batch* b, cudaStream_t st, int threads, int ctas_per_sm) {
-  if (b->fine_engine == PE_FINE_TC) return batch_tc_fine(b, st);
-  const FineItems& fi = threads == 128 ? b->fine128 : b->fine256;
-  BatchArrays A{};
-  A.W = b->W; A.W32 = b->W32; A.AF = b->AF; A.AF32 = b->AF32;
-  A.coefF = b->coefF; A.coefF32 = b->coefF32; A.U = b->U; A.Fbar = b->Fbar;
-  for (int c = 0; c < kBatchClasses; ++c) {
-    const int n = fi.begin[c + 1] - fi.begin[c];
-    if (n == 0) continue;
-    const int grid = std::min(b->sm_count * ctas_per_sm, n);
-    const FineItem* items = fi.d_items + fi.begin[c];
-    if (b->precision == PE_MIXED)
-      PE_TRY(batch_launch_fine_mixed(4 * (c + 1), b->d_probs, items, n, b->active, b->counter + c, A, grid, threads,
-                                     fi.smem[c], st));
-    else
-      PE_TRY(batch_launch_fine_f64(4 * (c + 1), b->d_probs, items, n, b->active, b->counter + c, A, grid, threads,
-                                   fi.smem[c], st));
-  }
-  return PE_OK;
-}
-
-int batch_fine_launches(const pe_batch* b) {
-  int k = 0;
-  if (b->fine_engine == PE_FINE_TC) {
-    for (int c = 0; c < 3; ++c) k += b->tc.begin[c + 1] > b->tc.begin[c];
-    return k;
-  }
-  for (int c = 0; c < kBatchClasses; ++c) k += b->fine256.begin[c + 1] > b->fine256.begin[c];
-  return k;
-}
-
-pe_status batch_enqueue_iteration(pe_batch* b, cudaStream_t st, double tol) {
-  PE_CUDA_TRY(cudaMemsetAsync(b->counter, 0, sizeof(int) * kBatchClasses, st));
+pe_status batch_enqueue_iteration(pe_batch* b, cudaStream_t st, double tol, bool first) {
+  PE_CUDA_TRY(cudaMemsetAsync(b->counter, 0, sizeof(int), st));
   PE_CUDA_TRY(cudaMemsetAsync(b->n_active, 0, sizeof(int), st));
-  PE_TRY(launch_fine(b, st, b->tune_threads, b->tune_ctas));
-  b_correction_kernel<<<b->sm_count * 8, 256, 0, st>>>(b->d_probs, b->d_mode_items, b->n_mode_items, b->active,
-                                                       b->muM, b->coefG, b->Fbar, b->U, b->partials);
-  b_reduce_kernel<<<b->P, 256, 0, st>>>(b->d_probs, b->P, b->partials, b->active, b->kcount, b->resid, tol,
-                                        b->n_active, b->nonfinite);
+  PE_TRY(launch_walk(b, st, b->tune_threads, b->tune_ctas, first));
+  b_reduce_kernel<<<b->P, 256, 0, st>>>(b->d_probs, b->P, b->tune_threads, b->partials, b->active, b->kcount,
+                                        b->resid, tol, b->n_active, b->nonfinite);
   PE_CUDA_TRY(cudaMemcpyAsync(b->h_flags, b->n_active, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
   PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;
 }
 
-pe_status batch_time_fine(pe_batch* b, int threads, int ctas, float* ms) {
-  cudaEvent_t e0, e1;
-  PE_CUDA_TRY(cudaEventCreate(&e0));
-  PE_CUDA_TRY(cudaEventCreate(&e1));
-  PE_CUDA_TRY(cudaMemsetAsync(b->counter, 0, sizeof(int) * kBatchClasses, b->stream));
-  PE_CUDA_TRY(cudaEventRecord(e0, b->stream));
-  PE_TRY(launch_fine(b, b->stream, threads, ctas));
-  PE_CUDA_TRY(cudaEventRecord(e1, b->stream));
-  PE_CUDA_TRY(cudaEventSynchronize(e1));
-  PE_CUDA_TRY(cudaEventElapsedTime(ms, e0, e1));
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  b->launches += batch_fine_launches(b);
+pe_status batch_time_walk(pe_batch* b, int threads, int ctas, float* ms) {
+  PE_CUDA_TRY(cudaMemsetAsync(b->counter, 0, sizeof(int), b->stream));
+  PE_CUDA_TRY(cudaEventRecord(b->ev[0], b->stream));
+  PE_TRY(launch_walk(b, b->stream, threads, ctas, false));
+  PE_CUDA_TRY(cudaEventRecord(b->ev[1], b->stream));
+  PE_CUDA_TRY(cudaEventSynchronize(b->ev[1]));
+  PE_CUDA_TRY(cudaEventElapsedTime(ms, b->ev[0], b->ev[1]));
+  b->launches += 1;
   return PE_OK;
 }

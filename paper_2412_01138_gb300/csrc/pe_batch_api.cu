@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "pe_batch.h"
+#include "pe_contract.cuh"
 
 namespace {
 
@@ -35,18 +36,18 @@ pe_status upload(T** d, const std::vector<T>& h, cudaStream_t st) {
 
 void free_batch(pe_batch* b) {
   if (!b) return;
-  if (b->graph_exec) cudaGraphExecDestroy(b->graph_exec);
-  if (b->graph) cudaGraphDestroy(b->graph);
-  void* ptrs[] = {b->d_probs, b->d_terms, b->d_mode_items, b->fine128.d_items, b->fine256.d_items,
+  for (cudaGraphExec_t g : b->graph_exec)
+    if (g) cudaGraphExecDestroy(g);
+  void* ptrs[] = {b->d_probs, b->d_terms, b->d_mode_items, b->walk128.d_items, b->walk256.d_items,
                   b->d_factor_jobs, b->d_mu_prefix, b->d_tt_prefix, b->muM, b->ratio, b->coefF, b->coefG,
-                  b->coefF32, b->U, b->Fbar, b->axisF, b->axisU0, b->axisF32, b->AF, b->AG,
-                  b->AF32, b->partials, b->active, b->kcount, b->resid, b->counter, b->dflags,
-                  b->W, b->W32, b->Z, b->d_cols, b->AG32, b->Z32, b->tc.A, b->tc.B, b->tc.d_items,
-                  b->tc.d_w_prefix, b->tc.d_y_prefix, b->tc.err, b->Kt, b->Ph, b->d_kt_prefix,
-                  b->d_ph_prefix};
+                  b->coefF32, b->coefG32, b->U, b->axisF, b->axisU0, b->axisF32, b->partials, b->active,
+                  b->kcount, b->resid, b->counter, b->dflags, b->Y, b->Z, b->chain, b->xs, b->Y32, b->Z32,
+                  b->chain32, b->xs32, b->V, b->G, b->V32, b->G32, b->d_cols, b->d_first, b->Kt, b->d_kt_prefix};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (b->h_flags) cudaFreeHost(b->h_flags);
+  for (cudaEvent_t e : b->ev)
+    if (e) cudaEventDestroy(e);
   if (b->stream) cudaStreamDestroy(b->stream);
   delete b;
 }
@@ -60,32 +61,19 @@ uint64_t fnv1a(uint64_t h, const void* data, size_t n) {
   return h;
 }
 
-// Fine work items (problem, tile of threads*MPT modes; the item runs every slice of its
-// problem), grouped by column class, longest (most slices) first within a class, and the
-// dynamic shared memory each class needs (its widest staged chunk of time factors).
-pe_status build_fine_items(pe_batch* b, int threads, FineItems* out) {
-  std::vector<FineItem> items;
-  const size_t elem = b->precision == PE_MIXED ? sizeof(float) : sizeof(double);
+// Walk items (problem, `threads` modes; the item runs every slice of its problem), longest (most
+// slices) first; the residual slots of a problem are consecutive from oItems.
+pe_status build_walk_items(pe_batch* b, int threads, WalkItems* out) {
+  std::vector<WalkItem> items;
   std::vector<int> order((size_t)b->P);
   for (int p = 0; p < b->P; ++p) order[(size_t)p] = p;
-  std::stable_sort(order.begin(), order.end(),
-                   [&](int x, int y) { return (int64_t)b->probs[x].N * b->probs[x].M > (int64_t)b->probs[y].N * b->probs[y].M; });
-  for (int c = 0; c < kBatchClasses; ++c) {
-    out->begin[c] = (int)std::min<size_t>(items.size(), INT32_MAX);
-    out->smem[c] = 0;
-    for (int p : order) {
-      const BProb& B = b->probs[p];
-      const int KC = (B.K + 3) / 4 * 4;
-      if (KC != 4 * (c + 1)) continue;
-      const size_t need = B.dbuf ? 2 * sizeof(float) * (size_t)B.M * KC : elem * (size_t)B.mchunk * KC;
-      out->smem[c] = std::max(out->smem[c], need);
-      const int mpt = b->precision == PE_MIXED ? batch_mixed_mpt(KC) : 1;
-      const int64_t tile = (int64_t)threads * mpt;
-      for (int64_t J0 = 0; J0 < B.g.ndof; J0 += tile) items.push_back(FineItem{p, 0, J0});
-    }
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return b->probs[x].N > b->probs[y].N; });
+  for (int p : order) {
+    const BProb& B = b->probs[p];
+    int slot = (int)B.oItems;
+    for (int64_t J0 = 0; J0 < B.g.ndof; J0 += threads) items.push_back(WalkItem{p, slot++, J0});
   }
   if (items.size() > (size_t)INT32_MAX) return pe_fail(PE_EINVAL, "batch: too many work items");
-  out->begin[kBatchClasses] = (int)items.size();
   out->n = (int)items.size();
   return upload(&out->d_items, items, b->stream);
 }
@@ -131,10 +119,10 @@ extern "C" pe_status pe_setup_batch(pe_batch** out, int32_t n_problems, const pe
   }
 
   // ---- validate and lay out every problem --------------------------------
-  int64_t oU = 0, oS = 0, oCF = 0, oCG = 0, oAx = 0, oAxU = 0, oAF = 0, oAF32 = 0, oAG = 0, oMu = 0, oItems = 0;
-  int64_t oW = 0, oZ = 0, oTA = 0, oTB = 0, wjobs = 0, yjobs = 0;
-  std::vector<int64_t> mu_prefix, tt_prefix, w_prefix, y_prefix;
-  std::vector<short> cols;
+  int64_t oU = 0, oCF = 0, oCG = 0, oAx = 0, oAxU = 0, oY = 0, oY32 = 0, oMu = 0, oItems = 0;
+  int64_t oV = 0, oZ = 0, oCh = 0, oXs = 0;
+  std::vector<int64_t> mu_prefix, tt_prefix;
+  std::vector<short> cols, first;
   int64_t tt = 0;
   uint64_t sig = 0xcbf29ce484222325ull;
   b->probs.resize(n_problems);
@@ -211,54 +199,39 @@ extern "C" pe_status pe_setup_batch(pe_batch** out, int32_t n_problems, const pe
       B.Ru = q.u0.n_terms;
     }
     if (B.Ru > PE_MAX_TERMS) { st = pe_fail(PE_EINVAL, tag + "too many u0 terms"); break; }
-    // stage-contracted columns of the fine step: one per exponential term, two per sinusoid
+    // source columns: one per exponential term, two per sinusoid
     B.oCol = (int64_t)cols.size();
+    B.oFirst = (int64_t)first.size();
     for (int r = 0; r < B.R; ++r) {
+      first.push_back((short)((int64_t)cols.size() - B.oCol));
       cols.push_back((short)(r << 1));
       if (b->terms[B.tf + r].tkind == PE_T_SIN) cols.push_back((short)((r << 1) | 1));
     }
     B.K = (int)((int64_t)cols.size() - B.oCol);
-    // tile bodies run with K rounded up to a multiple of 4 (zero-padded staging rows)
-    const int KC = (B.K + 3) / 4 * 4;
-    const size_t elem = b->precision == PE_MIXED ? sizeof(float) : sizeof(double);
-    B.mchunk = pick_mchunk(B.M, KC, elem);
-    B.dbuf = b->precision == PE_MIXED && 2 * (size_t)B.M * KC * sizeof(float) <= 48 * 1024 ? 1 : 0;
+    b->Kmax = std::max(b->Kmax, B.K);
     B.oU = oU; oU += (int64_t)(B.N + 1) * ndof;
-    B.oS = oS; oS += (int64_t)B.N * ndof;
     B.oCF = oCF; oCF += (int64_t)(B.q + 2) * ndof;
     B.oCG = oCG; oCG += (int64_t)(B.p + 1) * ndof;
     B.oAx = oAx; oAx += (int64_t)B.R * nsum;
     B.oAxU = oAxU; oAxU += (int64_t)B.Ru * nsum;
-    B.oAF = oAF; oAF += (int64_t)B.N * B.M * B.K;
-    B.oAF32 = oAF32; oAF32 += (int64_t)B.N * B.M * KC;
-    B.oW = oW; oW += (int64_t)B.K * ndof;
-    B.oZ = oZ; oZ += (int64_t)B.q * B.K;
-    B.oAG = oAG; oAG += (int64_t)B.N * B.p * B.R;
+    const int KC = (B.K + 3) / 4 * 4;
+    const int64_t steps = chain_steps(B.M);
+    B.oY = oY; oY += (int64_t)B.N * B.K;
+    B.oY32 = oY32; oY32 += (int64_t)B.N * 2 * KC;
+    B.oV = oV; oV += (int64_t)B.K * ndof;
+    B.oZ = oZ; oZ += (int64_t)(B.q + B.p) * B.K;
+    B.oCh = oCh; oCh += steps * B.R * 4;
+    B.oXs = oXs; oXs += B.R;
     B.oMu = oMu;
     mu_prefix.push_back(oMu);
     oMu += nsum;
     tt_prefix.push_back(tt);
-    tt += (int64_t)B.N * B.K + (int64_t)B.N * B.p * B.R + (int64_t)B.q * B.K;  // b_time_tables_kernel's threads
+    tt += (int64_t)(B.N + B.q + B.p) * B.K + (int64_t)B.R * (steps + 1);  // b_time_tables_kernel's threads
     B.oItems = oItems;
-    B.nItems = (int)((ndof + 255) / 256);
-    oItems += B.nItems;
-    if (b->fine_engine == PE_FINE_TC) {
-      // tensor-core operand images: split stage weights per 128-mode tile, split time factors
-      // per slice group, each in the byte layout the kernel copies into shared memory
-      if (!batch_tc_shape(B.K, B.M, &B.KP, &B.TG, &B.NR)) {
-        st = pe_fail(PE_EINVAL, tag + "PE_FINE_TC needs M a multiple of 16 in 16..128");
-        break;
-      }
-      B.groups = (B.N + B.TG - 1) / B.TG;
-      B.tiles = (ndof + 127) / 128;
-      B.oTA = oTA;
-      oTA += B.tiles * 3 * 128 * B.KP * 2;
-      B.oTB = oTB;
-      oTB += (int64_t)B.groups * 3 * B.NR * B.KP * 2;
-      w_prefix.push_back(wjobs);
-      wjobs += B.tiles * 128 * (B.KP / 8);
-      y_prefix.push_back(yjobs);
-      yjobs += (int64_t)B.groups * B.NR * (B.KP / 8);
+    oItems += (ndof + 127) / 128;  // residual slots for the smaller item
+    if (b->fine_engine == PE_FINE_TC && (B.M < 16 || B.M > 128 || B.M % 16 != 0)) {
+      st = pe_fail(PE_EINVAL, tag + "PE_FINE_TC needs M a multiple of 16 in 16..128");
+      break;
     }
     sig = fnv1a(sig, &B.g, sizeof(B.g));
     sig = fnv1a(sig, &B.N, sizeof(int) * 6);
@@ -278,35 +251,26 @@ extern "C" pe_status pe_setup_batch(pe_batch** out, int32_t n_problems, const pe
   if (st == PE_OK) st = balloc(&b->coefF, oCF);
   if (st == PE_OK && mixed) st = balloc(&b->coefF32, oCF);
   if (st == PE_OK) st = balloc(&b->coefG, oCG);
+  if (st == PE_OK && mixed) st = balloc(&b->coefG32, oCG);
   if (st == PE_OK) st = balloc(&b->U, oU);
-  if (st == PE_OK) st = balloc(&b->Fbar, oS);
   if (st == PE_OK) st = balloc(&b->axisF, oAx);
   if (st == PE_OK && mixed) st = balloc(&b->axisF32, oAx);
   if (st == PE_OK) st = balloc(&b->axisU0, oAxU);
-  if (st == PE_OK) st = balloc(&b->AF, oAF);
-  if (st == PE_OK && mixed) st = balloc(&b->AF32, oAF32);
-  if (st == PE_OK) st = balloc(&b->AG, oAG);
-  if (st == PE_OK && mixed) st = balloc(&b->AG32, oAG);
-  // float64 weights for the float64 fine kernel; the mixed form keeps only the float copy
-  if (st == PE_OK && !mixed) st = balloc(&b->W, oW);
-  if (st == PE_OK && mixed) st = balloc(&b->W32, oW);
-  if (st == PE_OK) st = balloc(&b->Z, oZ);
-  if (st == PE_OK && mixed) st = balloc(&b->Z32, oZ);
+  // time tables and column weights in the form's own arithmetic
+  if (st == PE_OK) st = mixed ? balloc(&b->Y32, oY32) : balloc(&b->Y, oY);
+  if (st == PE_OK) st = mixed ? balloc(&b->Z32, oZ) : balloc(&b->Z, oZ);
+  if (st == PE_OK) st = mixed ? balloc(&b->chain32, 2 * oCh) : balloc(&b->chain, oCh);
+  if (st == PE_OK) st = mixed ? balloc(&b->xs32, 2 * oXs) : balloc(&b->xs, oXs);
+  if (st == PE_OK) st = mixed ? balloc(&b->V32, oV) : balloc(&b->V, oV);
+  if (st == PE_OK) st = mixed ? balloc(&b->G32, oV) : balloc(&b->G, oV);
   if (st == PE_OK) st = balloc(&b->partials, 2 * (size_t)oItems);
   if (st == PE_OK) st = balloc(&b->active, (size_t)b->P);
   if (st == PE_OK) st = balloc(&b->kcount, (size_t)b->P);
   if (st == PE_OK) st = balloc(&b->resid, (size_t)b->P);
-  if (st == PE_OK) st = balloc(&b->counter, (size_t)kBatchClasses);
+  if (st == PE_OK) st = balloc(&b->counter, 1);
   if (st == PE_OK) st = balloc(&b->dflags, 2);
-  if (st == PE_OK && b->fine_engine == PE_FINE_TC) {
-    st = balloc(&b->tc.A, (size_t)oTA);
-    if (st == PE_OK) st = balloc(&b->tc.B, (size_t)oTB);
-    if (st == PE_OK) st = balloc(&b->tc.err, 1);
-    if (st == PE_OK && cudaMemset(b->tc.err, 0, sizeof(int)) != cudaSuccess)
-      st = pe_cuda_fail(cudaGetLastError(), "pe_setup_batch: error flag");
-    b->tc.w_jobs = wjobs;
-    b->tc.y_jobs = yjobs;
-  }
+  for (cudaEvent_t& e : b->ev)
+    if (st == PE_OK && cudaEventCreate(&e) != cudaSuccess) st = pe_cuda_fail(cudaGetLastError(), "pe_setup_batch: event");
   if (st == PE_OK && cudaMallocHost((void**)&b->h_flags, 2 * sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
     st = pe_fail(PE_ENOMEM, "pe_setup_batch: pinned allocation failed");
@@ -321,7 +285,6 @@ extern "C" pe_status pe_setup_batch(pe_batch** out, int32_t n_problems, const pe
   // ---- work items ----------------------------------------------------------
   {
     std::vector<ModeItem> mitems;
-    mitems.reserve((size_t)oItems);
     for (int p = 0; p < b->P; ++p)
       for (int64_t J0 = 0; J0 < b->probs[p].g.ndof; J0 += 256) mitems.push_back(ModeItem{p, 0, J0});
     b->n_mode_items = (int)mitems.size();
@@ -341,27 +304,9 @@ extern "C" pe_status pe_setup_batch(pe_batch** out, int32_t n_problems, const pe
     if (st == PE_OK) st = upload(&b->d_mu_prefix, mu_prefix, b->stream);
     if (st == PE_OK) st = upload(&b->d_tt_prefix, tt_prefix, b->stream);
     if (st == PE_OK) st = upload(&b->d_cols, cols, b->stream);
-    if (st == PE_OK) st = build_fine_items(b, 128, &b->fine128);
-    if (st == PE_OK) st = build_fine_items(b, 256, &b->fine256);
-    if (st == PE_OK && b->fine_engine == PE_FINE_TC) {
-      // items per column padding (16, 32, 64), each problem's (slice group, tile) pairs
-      // group-major, so that a CTA's consecutive items share the group's B operand
-      std::vector<BTcItem> titems;
-      for (int cls = 0; cls < 3; ++cls) {
-        b->tc.begin[cls] = (int)titems.size();
-        for (int p = 0; p < b->P; ++p) {
-          const BProb& B = b->probs[p];
-          if (B.KP != (16 << cls)) continue;
-          for (int g = 0; g < B.groups; ++g)
-            for (int64_t t = 0; t < B.tiles; ++t) titems.push_back(BTcItem{p, g, t});
-        }
-      }
-      if (titems.size() > (size_t)INT32_MAX) st = pe_fail(PE_EINVAL, "batch: too many tensor-core work items");
-      b->tc.begin[3] = (int)titems.size();
-      if (st == PE_OK) st = upload(&b->tc.d_items, titems, b->stream);
-      if (st == PE_OK) st = upload(&b->tc.d_w_prefix, w_prefix, b->stream);
-      if (st == PE_OK) st = upload(&b->tc.d_y_prefix, y_prefix, b->stream);
-    }
+    if (st == PE_OK) st = upload(&b->d_first, first, b->stream);
+    if (st == PE_OK) st = build_walk_items(b, 128, &b->walk128);
+    if (st == PE_OK) st = build_walk_items(b, 256, &b->walk256);
   }
   if (st == PE_OK) st = batch_set_attributes(b);
   if (st == PE_OK) st = batch_launch_axis_tables(b);
@@ -387,38 +332,39 @@ extern "C" void pe_batch_destroy(pe_batch* b) {
 namespace {
 
 pe_status reset_iteration_state(pe_batch* b) {
-  std::vector<int> ones((size_t)b->P, 1);
-  PE_CUDA_TRY(cudaMemcpyAsync(b->active, ones.data(), sizeof(int) * b->P, cudaMemcpyHostToDevice, b->stream));
+  PE_CUDA_TRY(cudaMemsetAsync(b->active, 1, sizeof(int) * b->P, b->stream));  // any nonzero value: active
   PE_CUDA_TRY(cudaMemsetAsync(b->kcount, 0, sizeof(int) * b->P, b->stream));
   PE_CUDA_TRY(cudaMemsetAsync(b->resid, 0, sizeof(double) * b->P, b->stream));
   PE_CUDA_TRY(cudaMemsetAsync(b->dflags, 0, 2 * sizeof(int), b->stream));
-  // the host vector must stay alive until the copy has been issued from it
-  PE_CUDA_TRY(cudaStreamSynchronize(b->stream));
   return PE_OK;
 }
 
-pe_status ensure_graph(pe_batch* b, double tol) {
-  if (b->graph_exec && b->graph_tol == tol && b->graph_threads == b->tune_threads && b->graph_ctas == b->tune_ctas)
+// The graphs of the first iteration (which = 1) and of the others (0).
+pe_status ensure_graphs(pe_batch* b, double tol) {
+  if (b->graph_exec[0] && b->graph_exec[1] && b->graph_tol == tol && b->graph_threads == b->tune_threads &&
+      b->graph_ctas == b->tune_ctas)
     return PE_OK;
-  if (b->graph_exec) {
-    cudaGraphExecDestroy(b->graph_exec);
-    b->graph_exec = nullptr;
-  }
-  if (b->graph) {
-    cudaGraphDestroy(b->graph);
-    b->graph = nullptr;
-  }
-  PE_CUDA_TRY(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-  pe_status st = batch_enqueue_iteration(b, b->stream, tol);
-  cudaGraph_t g = nullptr;
-  cudaError_t e = cudaStreamEndCapture(b->stream, &g);
-  if (st != PE_OK) {
+  for (int which = 0; which < 2; ++which) {
+    cudaGraphExec_t& ex = b->graph_exec[which];
+    if (ex) {
+      cudaGraphExecDestroy(ex);
+      ex = nullptr;
+    }
+    PE_CUDA_TRY(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
+    pe_status st = batch_enqueue_iteration(b, b->stream, tol, which == 1);
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamEndCapture(b->stream, &g);
+    if (st == PE_OK && e != cudaSuccess) st = pe_cuda_fail(e, "batch: graph capture");
+    if (st == PE_OK) {
+      e = cudaGraphInstantiate(&ex, g, 0);
+      if (e != cudaSuccess) {
+        ex = nullptr;
+        st = pe_cuda_fail(e, "batch: graph instantiation");
+      }
+    }
     if (g) cudaGraphDestroy(g);
-    return st;
+    PE_TRY(st);
   }
-  if (e != cudaSuccess) return pe_cuda_fail(e, "batch: graph capture");
-  b->graph = g;
-  PE_CUDA_TRY(cudaGraphInstantiate(&b->graph_exec, g, 0));
   b->graph_tol = tol;
   b->graph_threads = b->tune_threads;
   b->graph_ctas = b->tune_ctas;
@@ -435,10 +381,6 @@ float ms_between(cudaEvent_t a, cudaEvent_t b) {
 
 extern "C" pe_status pe_batch_autotune(pe_batch* b, const char* cache_path) {
   if (!b) return pe_fail(PE_EINVAL, "pe_batch_autotune: NULL batch");
-  if (b->fine_engine == PE_FINE_TC) {  // one CTA of 288 threads per SM: no launch shape to choose
-    b->tuned = true;
-    return PE_OK;
-  }
   cudaDeviceProp prop;
   int dev = 0;
   PE_CUDA_TRY(cudaGetDevice(&dev));
@@ -462,19 +404,18 @@ extern "C" pe_status pe_batch_autotune(pe_batch* b, const char* cache_path) {
       }
     }
   }
-  // time every candidate on a prepared state (writes only the fine-propagator outputs)
+  // time every candidate on a prepared state (the walks write iterates that the next solve makes anew)
   PE_TRY(reset_iteration_state(b));
   PE_TRY(batch_launch_prepare(b));
   const int cand_threads[2] = {128, 256};
   float best = 1e30f;
-  int best_t = 256, best_c = 2;
+  int best_t = 128, best_c = 4;
   for (int ti = 0; ti < 2; ++ti) {
     for (int ct = 1; ct <= 4; ++ct) {
-      if (cand_threads[ti] == 256 && ct > 2) continue;  // 256 x 128 registers: at most 2 CTAs per SM
       float ms = 0.f, tot = 0.f;
-      PE_TRY(batch_time_fine(b, cand_threads[ti], ct, &ms));  // warm
+      PE_TRY(batch_time_walk(b, cand_threads[ti], ct, &ms));  // warm
       for (int rep = 0; rep < 2; ++rep) {
-        PE_TRY(batch_time_fine(b, cand_threads[ti], ct, &ms));
+        PE_TRY(batch_time_walk(b, cand_threads[ti], ct, &ms));
         tot += ms;
       }
       if (tot < best) {
@@ -497,15 +438,14 @@ extern "C" pe_status pe_batch_autotune(pe_batch* b, const char* cache_path) {
 extern "C" pe_status pe_batch_solve(pe_batch* b, double tol, pe_batch_result* res) {
   if (!b) return pe_fail(PE_EINVAL, "pe_batch_solve: NULL batch");
   if (!(tol >= 0.0)) return pe_fail(PE_EINVAL, "pe_batch_solve: tol must be >= 0");
-  cudaEvent_t ev[3];
-  for (int i = 0; i < 3; ++i) PE_CUDA_TRY(cudaEventCreate(&ev[i]));
+  cudaEvent_t* ev = b->ev;
   if (b->user_stream) {
     PE_CUDA_TRY(cudaEventRecord(ev[0], b->user_stream));
     PE_CUDA_TRY(cudaStreamWaitEvent(b->stream, ev[0], 0));
   }
   b->launches = 0;
   PE_TRY(reset_iteration_state(b));
-  PE_TRY(ensure_graph(b, tol));
+  PE_TRY(ensure_graphs(b, tol));
   PE_CUDA_TRY(cudaEventRecord(ev[0], b->stream));
   PE_TRY(batch_launch_prepare(b));
   PE_CUDA_TRY(cudaEventRecord(ev[1], b->stream));
@@ -513,13 +453,12 @@ extern "C" pe_status pe_batch_solve(pe_batch* b, double tol, pe_batch_result* re
   int maxN = 0;
   for (const BProb& B : b->probs) maxN = std::max(maxN, B.N);
   for (;;) {
-    PE_CUDA_TRY(cudaGraphLaunch(b->graph_exec, b->stream));
+    PE_CUDA_TRY(cudaGraphLaunch(b->graph_exec[replays == 0 ? 1 : 0], b->stream));
     PE_CUDA_TRY(cudaStreamSynchronize(b->stream));
     ++replays;
-    b->launches += batch_fine_launches(b) + 2;  // graph: fine kernels, correction, reduction
+    b->launches += 2;  // graph: walk, reduction
     if (b->h_flags[1]) {
       b->have_problem = false;
-      if (b->fine_engine == PE_FINE_TC) PE_TRY(batch_tc_status(b));
       return pe_fail(PE_ENONFINITE, "batch: a problem's Parareal residual is not finite");
     }
     if (b->h_flags[0] == 0 || replays >= maxN) break;
@@ -549,10 +488,9 @@ extern "C" pe_status pe_batch_solve(pe_batch* b, double tol, pe_batch_result* re
     res->ms_prepare = ms_between(ev[0], ev[1]);
     res->ms_iterations = ms_between(ev[1], ev[2]);
     res->kernel_launches = b->launches;
-    res->threads = b->fine_engine == PE_FINE_TC ? 288 : b->tune_threads;
-    res->ctas_per_sm = b->fine_engine == PE_FINE_TC ? 1 : b->tune_ctas;
+    res->threads = b->tune_threads;
+    res->ctas_per_sm = b->tune_ctas;
   }
-  for (int i = 0; i < 3; ++i) cudaEventDestroy(ev[i]);
   return PE_OK;
 }
 
@@ -574,17 +512,21 @@ extern "C" pe_status pe_batch_get_solution(pe_batch* b, int32_t problem, double*
   if (problem < 0 || problem >= b->P) return pe_fail(PE_EINVAL, "pe_batch_get_solution: problem out of range");
   if (!b->have_problem) return pe_fail(PE_ESTATE, "pe_batch_get_solution: no solve has completed");
   const BProb& B = b->probs[problem];
-  double* tmp = nullptr;
-  PE_CUDA_TRY(cudaMallocAsync((void**)&tmp, sizeof(double) * B.g.ndof, b->stream));
   int n[PE_MAX_D] = {B.g.n[0], B.g.n[1], B.g.n[2]};
-  pe_status st = pe_dst(B.g.d, n, b->U + B.oU + (int64_t)B.N * B.g.ndof, tmp, b->stream);
-  if (st == PE_OK) {
-    const bool dev = pe_is_device_ptr(nodal_out);
-    cudaError_t e = cudaMemcpyAsync(nodal_out, tmp, sizeof(double) * B.g.ndof,
-                                    dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, b->stream);
-    if (e != cudaSuccess) st = pe_cuda_fail(e, "pe_batch_get_solution");
+  const double* last = b->U + B.oU + (int64_t)B.N * B.g.ndof;
+  pe_status st = PE_OK;
+  if (pe_is_device_ptr(nodal_out)) {
+    st = pe_dst(B.g.d, n, last, nodal_out, b->stream);
+  } else {
+    double* tmp = nullptr;
+    PE_CUDA_TRY(cudaMallocAsync((void**)&tmp, sizeof(double) * B.g.ndof, b->stream));
+    st = pe_dst(B.g.d, n, last, tmp, b->stream);
+    if (st == PE_OK) {
+      cudaError_t e = cudaMemcpyAsync(nodal_out, tmp, sizeof(double) * B.g.ndof, cudaMemcpyDeviceToHost, b->stream);
+      if (e != cudaSuccess) st = pe_cuda_fail(e, "pe_batch_get_solution");
+    }
+    cudaFreeAsync(tmp, b->stream);
   }
-  cudaFreeAsync(tmp, b->stream);
   cudaError_t e = cudaStreamSynchronize(b->stream);
   if (st == PE_OK && e != cudaSuccess) st = pe_cuda_fail(e, "pe_batch_get_solution");
   return st;
@@ -601,8 +543,8 @@ extern "C" pe_status pe_batch_set_learned(pe_batch* b, const pe_mlp* m) {
   }
   PE_CUDA_TRY(cudaStreamSynchronize(b->stream));
   const int NB = kBatchLearnedBands;
-  std::vector<int64_t> kp, pp;
-  int64_t okt = 0, oph = 0;
+  std::vector<int64_t> kp;
+  int64_t okt = 0;
   for (int p = 0; p < b->P; ++p) {
     BProb& B = b->probs[p];
     double lmin = 0.0, lmax = 0.0;
@@ -622,26 +564,16 @@ extern "C" pe_status pe_batch_set_learned(pe_batch* b, const pe_mlp* m) {
     B.oKt = okt;
     kp.push_back(okt / 2);
     okt += 2 * (int64_t)B.R * NB;
-    B.oPh = oph;
-    pp.push_back(oph);
-    oph += (int64_t)B.R * B.N;
   }
   if (b->Kt) cudaFree(b->Kt);
-  if (b->Ph) cudaFree(b->Ph);
   if (b->d_kt_prefix) cudaFree(b->d_kt_prefix);
-  if (b->d_ph_prefix) cudaFree(b->d_ph_prefix);
   b->Kt = nullptr;
-  b->Ph = nullptr;
   b->d_kt_prefix = nullptr;
-  b->d_ph_prefix = nullptr;
   PE_TRY(balloc(&b->Kt, (size_t)okt));
-  PE_TRY(balloc(&b->Ph, (size_t)oph));
   PE_TRY(upload(&b->d_kt_prefix, kp, b->stream));
-  PE_TRY(upload(&b->d_ph_prefix, pp, b->stream));
   PE_CUDA_TRY(cudaMemcpyAsync(b->d_probs, b->probs.data(), sizeof(BProb) * b->P, cudaMemcpyHostToDevice, b->stream));
   PE_CUDA_TRY(cudaStreamSynchronize(b->stream));
   b->kt_jobs = okt / 2;
-  b->ph_jobs = oph;
   b->mlp = m;
   return PE_OK;
 }

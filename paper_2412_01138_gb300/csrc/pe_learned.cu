@@ -494,7 +494,7 @@ __global__ void band_table_kernel(const __half* __restrict__ params16, TermsW T,
 }
 
 // ---------------------------------------------------------------------------
-// batched form: band and phase tables of every problem of a batch, jobs flattened through
+// batched form: band tables of every problem of a batch, jobs flattened through
 // per-problem prefix tables (the owner of job e is the problem with the largest prefix <= e)
 // ---------------------------------------------------------------------------
 __device__ inline int job_owner(const int64_t* __restrict__ prefix, int P, int64_t e) {
@@ -535,21 +535,6 @@ __global__ void b_band_table_kernel(const __half* __restrict__ params16, const B
   Kt[B.oKt + 2 * le + 1] = Kim;
 }
 
-__global__ void b_phase_table_kernel(const BProb* __restrict__ probs, const pe_term* __restrict__ terms,
-                                     const int64_t* __restrict__ prefix, int P, int64_t total,
-                                     float2* __restrict__ Ph) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= total) return;
-  const int p = job_owner(prefix, P, e);
-  const BProb& B = probs[p];
-  const int64_t le = e - prefix[p];
-  const int r = (int)(le / B.N), n = (int)(le % B.N);
-  const pe_term& t = terms[B.tf + r];
-  double sn = 0.0, cs = 0.0;
-  if (t.tkind == PE_T_SIN) sincos(t.tp[0] * (B.t0 + (double)n * B.dT) + t.tp[1], &sn, &cs);
-  Ph[B.oPh + le] = make_float2((float)cs, (float)sn);
-}
-
 }  // namespace
 
 pe_status batch_learned_tables(pe_batch* b, cudaStream_t st) {
@@ -558,10 +543,7 @@ pe_status batch_learned_tables(pe_batch* b, cudaStream_t st) {
     b_band_table_kernel<<<(unsigned)((b->kt_jobs + 127) / 128), 128, 0, st>>>(
         (const __half*)b->mlp->params16, b->d_probs, b->d_terms, b->d_kt_prefix, b->P, b->kt_jobs,
         kBatchLearnedBands, b->Kt);
-  if (b->ph_jobs > 0)
-    b_phase_table_kernel<<<(unsigned)((b->ph_jobs + 255) / 256), 256, 0, st>>>(b->d_probs, b->d_terms, b->d_ph_prefix,
-                                                                               b->P, b->ph_jobs, b->Ph);
-  b->launches += 2;
+  b->launches += 1;
   PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;
 }

@@ -18,25 +18,10 @@
 //                  (per-CTA partial sums, added by the last CTA to finish).
 #include <algorithm>
 
+#include "pe_contract.cuh"
 #include "pe_internal.h"
 
 namespace {
-
-template <typename T>
-__device__ inline T block_sum(T v, T* sh) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) sh[wid] = v;
-  __syncthreads();
-  T out = T(0);
-  if (threadIdx.x < 32) {
-    T x = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : T(0);
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    out = x;
-  }
-  __syncthreads();
-  return out;
-}
 
 // Stopping decision of a device-resident loop, run by one thread after the residual sums are
 // complete: r_k appended to the history, k advanced, and the graph's while condition set to
@@ -109,28 +94,6 @@ struct WalkArgs {
   LoopCtl* loop;
   unsigned long long handle;
 };
-
-// sum_k y_k w_k over a slice's staged columns, a row of KB high parts and one of KB low parts:
-// rounding Y_k(T_n) to one float would be an error of the whole slice, which M separately rounded
-// substeps average out
-template <int KB>
-__device__ __forceinline__ float column_dot(const float* y, const float (&w)[KB]) {
-  float hi = 0.f, lo = 0.f;
-#pragma unroll
-  for (int k = 0; k < KB; k += 4) {
-    const float4 v = *reinterpret_cast<const float4*>(y + k);
-    const float4 l = *reinterpret_cast<const float4*>(y + KB + k);
-    hi = fmaf(v.x, w[k], hi);
-    lo = fmaf(l.x, w[k], lo);
-    hi = fmaf(v.y, w[k + 1], hi);
-    lo = fmaf(l.y, w[k + 1], lo);
-    hi = fmaf(v.z, w[k + 2], hi);
-    lo = fmaf(l.z, w[k + 2], lo);
-    hi = fmaf(v.w, w[k + 3], hi);
-    lo = fmaf(l.w, w[k + 3], lo);
-  }
-  return hi + lo;
-}
 
 // Threads per CTA: as many as 65536 registers allow with the weights in registers.
 __host__ __device__ constexpr int walk_cap(int SRC, int KB, int MODE) {

@@ -98,3 +98,20 @@ def test_exponentials_beyond_the_range_of_a_slice(pe, a, t0):
             s.solve(tol=1e-6)
             for m in range(1, prob.N + 1):
                 assert _rel(s.modal(m), fine[m], sys_.norm_w) <= bound, (prec, m)
+
+
+def test_batched_walk_stages_slices_in_chunks(pe):
+    """Problems of one batch with one to 39 columns and one to 210 slices (more than the walk stages at a
+    time), mode counts that leave partial items, one problem that converges before the others."""
+    probs = [_prob((130,), 210, 4, "s" * 19 + "e"), _prob((129, 3), 104, 3, "se"), _prob((5, 9), 1, 7, "e"),
+             _prob((16, 8), 9, 33, "s" * 8), _prob((257,), 97, 2, "ss")]
+    for prec, bound in ((pe.PE_FP64, 1e-12), (pe.PE_MIXED, 1e-6)):
+        with pe.BatchSolver(probs, precision=prec) as b:
+            b.solve(tol=1e-10)
+            _, k = b.status()
+            for i, p in enumerate(probs):
+                sys_ = osolver.ModalSystem(p)
+                fine = osolver.sequential_fine(sys_)
+                assert k[i] == min(2, p.N)
+                for m in range(0, p.N + 1, max(1, p.N // 9)):
+                    assert _rel(b.modal(i, m), fine[m], sys_.norm_w) <= bound, (prec, i, m)

@@ -61,7 +61,8 @@ enum { PE_FP64 = 0,   /* every step in float64 */
 /* How the fine sweep evaluates F^M (separable forcing): the time factors are shift invariant, so
  * the q stages of all M substeps of a slice add up exactly to one value per time column (one
  * column per exponential, two per sinusoid) times a per-mode weight made once per problem; every
- * sweep evaluates that sum on every mode and slice.  The general path takes every substep.
+ * sweep evaluates that sum on every mode and slice.  Terms with moving factors (the general path) take
+ * every substep.
  *
  * Engine of the mixed-precision fine sweep (pe_options.fine_engine): both values run the same kernels, the
  * sum over the columns being too small for tensor cores to matter.  TC still needs M (substeps per
@@ -83,8 +84,9 @@ enum { PE_S_ONE = 0, PE_S_SIN = 1, PE_S_GAUSS = 2, PE_S_POLY = 3, PE_S_MOVING_HA
 
 /* how P_h f(t) is formed (pe_options.forcing_path) */
 enum { PE_FORCING_SEPARABLE = 0, /* modal factors of every term once, products per mode and stage */
-       PE_FORCING_GENERAL = 1    /* at every stage time: consistent load assembled in nodal space
-                                    (element Gauss quadrature), tensor DST-I, division by Lambda_M */ };
+       PE_FORCING_GENERAL = 1    /* also terms with moving factors: at every stage time the consistent
+                                    1D loads of their moving axes (element Gauss quadrature), the DST-I along
+                                    those axes, division by Lambda_M; terms that do not move as above */ };
 enum { PE_T_EXP = 0, PE_T_SIN = 1 };
 
 /* One separable term  amp * time(t) * prod_{a<d} spatial_a(x_a). */

@@ -127,7 +127,7 @@ pe_status dev_alloc(T** p, size_t count) {
 void free_ctx(pe_ctx* c) {
   if (!c) return;
   void* ptrs[] = {c->muM_axis, c->ratio_axis, c->S[0], c->S[1], c->S[2], c->S32[0], c->S32[1], c->S32[2],
-                  c->gen_L, c->gen_buf, c->gen_tmp, c->lam, c->coefF, c->coefG,
+                  c->gen_L, c->gen_X, c->axisM, c->lam, c->coefF, c->coefG,
                   c->coefF32, c->coefG32, c->U, c->Fbar, c->gG, c->work0, c->work1, c->out_nodal, c->partials,
                   c->red, c->axisF, c->axisF32, c->axisU0, c->loads, c->tab64, c->tab32,
                   c->Ktab, c->V64, c->G64, c->V32, c->G32, c->Fz, c->done_ctr,
@@ -383,12 +383,7 @@ extern "C" pe_status pe_setup(pe_ctx** out, int32_t d, const int32_t* n, const d
       ((int64_t)n_substeps * c->q > 65535 || (int64_t)n_slices * c->p > 65535))
     st = pe_fail(PE_EINVAL, "pe_setup: general forcing path needs M*q and N*p <= 65535");
   if (st == PE_OK && c->forcing_path == PE_FORCING_GENERAL) {
-    // stage-time buffers of one chunk of slices (also holding the N*p coarse stage times)
-    const int chunk = general_slices_per_chunk(c);
-    const size_t stages = std::max((size_t)chunk * n_substeps * c->q, N * c->p);
-    st = dev_alloc(&c->gen_buf, stages * nd);
-    if (st == PE_OK) st = dev_alloc(&c->gen_tmp, stages * nd);
-    if (st == PE_OK) st = dev_alloc(&c->gen_L, stages * MT * nsum);
+    st = dev_alloc(&c->axisM, MT * nsl);
     for (int a = 0; a < d && st == PE_OK && c->precision == PE_MIXED; ++a)
       st = dev_alloc(&c->S32[a], (size_t)n[a] * n[a]);
   }
@@ -479,10 +474,6 @@ static pe_status expand_dirichlet_terms(pe_ctx* c) {
       for (int e = 0; e < d; ++e) c->lkind[c->R][e] = e == a ? 2 : 1;
       c->R += 1;
     }
-  }
-  if (c->R == 0) {  // data only through terms that vanished: keep one zero term
-    c->R = 1;
-    memset(&c->terms[0], 0, sizeof(pe_term));
   }
   return PE_OK;
 }
@@ -591,14 +582,20 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
   if (c->sharded && u0->kind == PE_FIELD_TERMS_QUADRATURE)
     return pe_fail(PE_EINVAL, "pe_set_problem: a context that owns a block of modes takes nodal or separable u0");
   memset(c->lkind, 0, sizeof(c->lkind));
-  if (nf == 0 && c->nbd == 0) {
-    // no source: one zero term keeps every kernel shape valid
+  // terms with a moving factor (general path) go their own way; the others are projected once
+  c->R = 0;
+  c->Rm = 0;
+  for (int i = 0; i < nf; ++i) {
+    bool moves = false;
+    for (int a = 0; a < c->g.d; ++a) moves = moves || f->terms[i].skind[a] == PE_S_MOVING_HAT;
+    if (moves) c->mterms[c->Rm++] = f->terms[i];
+    else c->terms[c->R++] = f->terms[i];
+  }
+  if (c->nbd > 0) PE_TRY(expand_dirichlet_terms(c));
+  if (c->R == 0) {
+    // no (fixed) source: one zero term keeps every kernel shape valid
     c->R = 1;
     memset(&c->terms[0], 0, sizeof(pe_term));
-  } else {
-    c->R = nf;
-    for (int i = 0; i < nf; ++i) c->terms[i] = f->terms[i];
-    PE_TRY(expand_dirichlet_terms(c));
   }
   // Two streams for grids large enough that their set-up kernels run side by side: the side
   // stream makes the time tables, then the forward transform of nodal u0 (after its copy, for
@@ -615,11 +612,9 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
     cudaStream_t main_stream = c->stream;
     c->stream = c->side;
     pe_status st = PE_OK;
-    if (!general) {
-      st = launch_time_tables(c);
-      if (st == PE_OK && cudaEventRecord(c->ev_tables, c->side) != cudaSuccess)
-        st = pe_cuda_fail(cudaGetLastError(), "pe_set_problem: event record");
-    }
+    st = launch_time_tables(c);
+    if (st == PE_OK && cudaEventRecord(c->ev_tables, c->side) != cudaSuccess)
+      st = pe_cuda_fail(cudaGetLastError(), "pe_set_problem: event record");
     if (st == PE_OK) {
       // device u0 is read in place by the transform; host u0 is copied in first
       const bool dev = c->u0_dev_hint >= 0 ? c->u0_dev_hint == 1 : pe_is_device_ptr(u0->nodal);
@@ -635,14 +630,15 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
     c->stream = main_stream;
     PE_TRY(st);
     PE_CUDA_TRY(cudaEventRecord(c->ev_join, c->side));
-  } else if (!general) {
+  } else {
     PE_TRY(launch_time_tables(c));
   }
   // The phi/b coefficient tables depend only on lam, dt, dT and the nodes: pe_setup made them.
   // Forcing: per-axis modal factors, then the column weights.
-  if (!general) PE_TRY(launch_separable_factors(c, c->terms, c->R, c->axisF, 1, c->lkind));
-  if (fork && !general) PE_CUDA_TRY(cudaStreamWaitEvent(c->stream, c->ev_tables, 0));
-  if (!general) PE_TRY(launch_column_weights(c));
+  PE_TRY(launch_separable_factors(c, c->terms, c->R, c->axisF, 1, c->lkind));
+  if (general) PE_TRY(general_prepare(c));
+  if (fork) PE_CUDA_TRY(cudaStreamWaitEvent(c->stream, c->ev_tables, 0));
+  PE_TRY(launch_column_weights(c));
   if (fork) PE_CUDA_TRY(cudaStreamWaitEvent(c->stream, c->ev_join, 0));
   PE_CUDA_TRY(record_timing(c, c->ev[1]));
   // U^0 = P_h u0

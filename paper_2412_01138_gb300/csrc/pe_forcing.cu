@@ -81,8 +81,8 @@ __global__ void time_tables_kernel(TermsDev T, StageCols C, ColumnTables D, int 
 
 // Per-mode column weights: V[k * ndof + J] of the fine propagator's slice sum and G[k * ndof + J]
 // of the coarse step (sum_i dT b^G_i Z_k(c_i dT), plus the learned correction's P K^ on the
-// columns of a sinusoid), P_{r,J} = prod_a axisF.  A thread takes TPT consecutive terms of one
-// mode.  T = float (mixed form): float32 weights from float32 factors, the chain in float pairs.
+// columns of a sinusoid), P_{r,J} = prod_a axisF; V or G may be null.  A thread takes TPT
+// consecutive terms of one mode.  T = float (mixed form): float32 weights from float32 factors, the chain in float pairs.
 // coef: E (float: hi and lo rows), then the q rows dt b_i; coefG: the p rows dT b^G_i.
 template <typename T>
 __global__ void __launch_bounds__(256) column_weights_kernel(Geom g, StageCols C, ColumnTables D, int R, int M, int q,
@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(256) column_weights_kernel(Geom g, StageCols C
       G[(int64_t)k * nd + J] = gr;
       if (two) G[(int64_t)(k + 1) * nd + J] = gi;
     }
+    if (!V) continue;
     T v0, v1;
     if constexpr (F64) {
       double Sr, Si;
@@ -354,20 +355,16 @@ pe_status launch_time_tables(pe_ctx* c) {
   return PE_OK;
 }
 
-// Room for the weights of K columns: float64 (V64, and G64 when `coarse`), float32 (V32, G32).
+// Room for the weights of K columns in one table.
 template <typename T>
-static pe_status grow_weights(pe_ctx* c, T** V, T** G, int* cap) {
+static pe_status grow_weights(pe_ctx* c, T** W, int* cap) {
   const int K = c->K;
   if (K <= *cap) return PE_OK;
   PE_CUDA_TRY(cudaStreamSynchronize(c->stream));
-  if (*V) cudaFree(*V);
-  if (G && *G) cudaFree(*G);
-  *V = nullptr;
-  if (G) *G = nullptr;
+  if (*W) cudaFree(*W);
+  *W = nullptr;
   *cap = 0;
-  const size_t n = (size_t)K * (size_t)c->g.ndof;
-  if (cudaMalloc((void**)V, n * sizeof(T)) != cudaSuccess ||
-      (G && cudaMalloc((void**)G, n * sizeof(T)) != cudaSuccess)) {
+  if (cudaMalloc((void**)W, (size_t)K * (size_t)c->g.ndof * sizeof(T)) != cudaSuccess) {
     cudaGetLastError();
     return pe_fail(PE_ENOMEM, "pe_set_problem: column-weight table allocation failed");
   }
@@ -383,43 +380,55 @@ static int weights_tpt(const pe_ctx* c, bool learned) {
   return c->g.ndof < ((int64_t)1 << 19) ? 1 : std::min(c->R, 4);
 }
 
-pe_status launch_column_weights(pe_ctx* c) {
-  LearnedTerms L{};
-  if (c->mlp) PE_TRY(launch_learned_tables(c, &L));
-  const int threads = 256, tpt = weights_tpt(c, c->mlp != nullptr);
+template <typename T>
+static pe_status column_weights(pe_ctx* c, T* V, T* G, const LearnedTerms& L) {
+  const int threads = 256, tpt = weights_tpt(c, L.Ktab != nullptr);
   const dim3 grid((unsigned)((c->g.ndof + threads - 1) / threads), (unsigned)((c->R + tpt - 1) / tpt));
-  c->V64_valid = false;
-  if (c->precision == PE_MIXED) {
-    // the float32 sweeps need only float32 weights; pe_refine makes its float64 ones
-    PE_TRY(grow_weights(c, &c->V32, &c->G32, &c->cap32));
-    PE_CUDA_TRY(launch_pdl(column_weights_kernel<float>, grid, dim3(threads), 0, c->stream, c->g, c->cols, c->tab,
-                           c->R, c->M, c->q, c->p, tpt, (const float*)c->axisF32, (const float*)c->coefF32,
-                           (const float*)c->coefG32, c->V32, c->G32, L, (const double*)c->axisF,
-                           (const double*)c->lam));
+  const T *axisF, *coef, *coefG;
+  if constexpr (sizeof(T) == 8) {
+    axisF = c->axisF;
+    coef = c->coefF;
+    coefG = c->coefG + c->g.ndof;
   } else {
-    PE_TRY(grow_weights(c, &c->V64, &c->G64, &c->cap64));
-    PE_CUDA_TRY(launch_pdl(column_weights_kernel<double>, grid, dim3(threads), 0, c->stream, c->g, c->cols, c->tab,
-                           c->R, c->M, c->q, c->p, tpt, (const double*)c->axisF, (const double*)c->coefF,
-                           (const double*)(c->coefG + c->g.ndof), c->V64, c->G64, L, (const double*)c->axisF,
-                           (const double*)c->lam));
-    c->V64_valid = true;
+    axisF = c->axisF32;
+    coef = c->coefF32;
+    coefG = c->coefG32;
   }
+  PE_CUDA_TRY(launch_pdl(column_weights_kernel<T>, grid, dim3(threads), 0, c->stream, c->g, c->cols, c->tab, c->R, c->M,
+                         c->q, c->p, tpt, axisF, coef, coefG, V, G, L, (const double*)c->axisF,
+                         (const double*)c->lam));
   c->launches += 1;
   PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;
 }
 
+pe_status launch_column_weights(pe_ctx* c) {
+  LearnedTerms L{};
+  if (c->mlp) PE_TRY(launch_learned_tables(c, &L));
+  c->V64_valid = false;
+  if (c->precision == PE_MIXED) {
+    // the float32 sweeps need only float32 weights; pe_refine makes its float64 ones.  The general
+    // path's coarse forcing is float64 in either form.
+    PE_TRY(grow_weights(c, &c->V32, &c->capV32));
+    if (c->forcing_path == PE_FORCING_GENERAL) {
+      PE_TRY(grow_weights(c, &c->G64, &c->capG64));
+      PE_TRY(column_weights<double>(c, nullptr, c->G64, L));
+      return column_weights<float>(c, c->V32, nullptr, L);
+    }
+    PE_TRY(grow_weights(c, &c->G32, &c->capG32));
+    return column_weights<float>(c, c->V32, c->G32, L);
+  }
+  PE_TRY(grow_weights(c, &c->V64, &c->capV64));
+  PE_TRY(grow_weights(c, &c->G64, &c->capG64));
+  PE_TRY(column_weights<double>(c, c->V64, c->G64, L));
+  c->V64_valid = true;
+  return PE_OK;
+}
+
 pe_status launch_column_weights_f64(pe_ctx* c) {
   if (c->V64_valid) return PE_OK;
-  PE_TRY(grow_weights(c, &c->V64, (double**)nullptr, &c->cap64));
-  const int threads = 256, tpt = weights_tpt(c, false);
-  const dim3 grid((unsigned)((c->g.ndof + threads - 1) / threads), (unsigned)((c->R + tpt - 1) / tpt));
-  PE_CUDA_TRY(launch_pdl(column_weights_kernel<double>, grid, dim3(threads), 0, c->stream, c->g, c->cols, c->tab,
-                         c->R, c->M, c->q, c->p, tpt, (const double*)c->axisF, (const double*)c->coefF,
-                         (const double*)nullptr, c->V64, (double*)nullptr, LearnedTerms{}, (const double*)c->axisF,
-                         (const double*)c->lam));
-  c->launches += 1;
-  PE_CUDA_TRY(cudaGetLastError());
+  PE_TRY(grow_weights(c, &c->V64, &c->capV64));
+  PE_TRY(column_weights<double>(c, c->V64, nullptr, LearnedTerms{}));
   c->V64_valid = true;
   return PE_OK;
 }

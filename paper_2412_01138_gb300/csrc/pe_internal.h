@@ -125,10 +125,14 @@ struct pe_ctx {
   double* ratio_axis = nullptr; // [nsum] mu^K/mu^M
   double* S[PE_MAX_D] = {nullptr, nullptr, nullptr};  // DST-I matrices n_a x n_a
   float* S32[PE_MAX_D] = {nullptr, nullptr, nullptr};  // float copies (general path, mixed)
-  // general forcing path: stage-time loads and their transforms for a chunk of slices
-  double* gen_L = nullptr;      // [stages][R * nsum] 1D loads
-  double* gen_buf = nullptr;    // [stages][ndof] transformed loads (float in the mixed fine sweep)
-  double* gen_tmp = nullptr;    // same size, DST ping-pong
+  // general forcing path: terms with a moving factor (the others are in terms), their static axes' modal
+  // factors, and the stage tables of a chunk of slices (1D loads, their transforms; float in the
+  // mixed fine sweep), grown on demand
+  int Rm = 0;
+  pe_term mterms[PE_MAX_TERMS];
+  double* axisM = nullptr;      // [PE_MAX_TERMS * nsum]
+  double *gen_L = nullptr, *gen_X = nullptr;
+  size_t gen_cap = 0;           // doubles allocated in each
   double* lam = nullptr;        // [ndof]
   double* coefF = nullptr;      // [(q+2) * ndof]: E, dt*b_1..q, exp(-lam M dt)
   double* coefG = nullptr;      // [(p+1) * ndof]: E, dT*b_1..p
@@ -169,10 +173,10 @@ struct pe_ctx {
   double *tab64 = nullptr;      //   their storage
   float *tab32 = nullptr;
   // column weights [K * ndof], allocated on first use and grown with K: float64 (the float64 form;
-  // of a mixed context V64 alone, for pe_refine) and float32 (mixed)
+  // of a mixed context V64 for pe_refine, G64 on the general path) and float32 (mixed)
   double *V64 = nullptr, *G64 = nullptr;
   float *V32 = nullptr, *G32 = nullptr;
-  int cap64 = 0, cap32 = 0;     // columns allocated
+  int capV64 = 0, capG64 = 0, capV32 = 0, capG32 = 0;  // columns allocated
   bool V64_valid = false;       // V64 holds the current problem's weights
   double* loads = nullptr;      // [PE_MAX_TERMS * nsum_full] 1D loads before the DST
   // learned coarse correction (optional)
@@ -276,11 +280,10 @@ pe_status read_sums(pe_ctx* c, double* num, double* den, cudaEvent_t after);  //
 pe_status launch_loop_init(pe_ctx* c, double tol);
 pe_status launch_scale_by_muM(pe_ctx* c, double* x, int inverse);
 
-// pe_general.cu
-int general_slices_per_chunk(const pe_ctx* c);
-pe_status launch_general_coarse_forcing(pe_ctx* c);
-pe_status launch_general_fine_sweep(pe_ctx* c, int precision);
-
+// pe_general.cu: the moving terms of the general path (no-ops without any)
+pe_status general_prepare(pe_ctx* c);                  // buffers, static factors
+pe_status general_add_coarse(pe_ctx* c);               // gG += their coarse forcing
+pe_status general_add_fine(pe_ctx* c, int precision);  // Fbar += their F^M(0)
 // Threads per CTA (at most cap) of a kernel with one thread per mode: when the modes fit one
 // wave of CTAs of up to 512 threads per SM, as many warps as an even share of the SMs needs (every
 // SM then runs CTAs of equal size, rather than some SMs two CTAs of 256 threads and others one);

@@ -228,8 +228,8 @@ __global__ void __launch_bounds__(walk_cap(SRC, KB, MODE)) walk_kernel(WalkArgs 
   }
 }
 
-// F^M(0) of every slice from the float32 weights, stored as float64 (cache_forced of the mixed
-// form; the same sums as the walk makes): a CTA takes 256 modes and SL slices.
+// F^M(0) of every slice from the float32 weights, stored as float64 (cache_forced and the general path of
+// the mixed form; the same sums as the walk makes): a CTA takes 256 modes and SL slices.
 template <int KB>
 __global__ void __launch_bounds__(256) forced_f32_kernel(int64_t ndof, int N, int K, int SL,
                                                          const float* __restrict__ Y, const float* __restrict__ V,
@@ -320,8 +320,24 @@ WalkArgs walk_args(pe_ctx* c, LoopCtl* loop, unsigned long long handle) {
   return a;
 }
 
+// The walk makes the forced parts itself: the mixed form, every term a sum over columns.
 bool mixed_columns(const pe_ctx* c, int precision) {
   return precision == PE_MIXED && c->forcing_path == PE_FORCING_SEPARABLE;
+}
+
+// Forced parts in memory: F^M(0) into f, the coarse forcing (float64 here in either form) into gG,
+// where not null.
+pe_status forced_parts(pe_ctx* c, int precision, double* f, double* gG) {
+  if (precision == PE_MIXED) {
+    if (f) PE_TRY(forced_f32(c, f));
+    if (gG) PE_TRY(launch_forced_f64(c, nullptr, gG));
+  } else {
+    if (f) PE_TRY(launch_column_weights_f64(c));
+    PE_TRY(launch_forced_f64(c, f, gG));
+  }
+  if (gG) PE_TRY(general_add_coarse(c));
+  if (f) PE_TRY(general_add_fine(c, precision));
+  return PE_OK;
 }
 
 }  // namespace
@@ -331,8 +347,7 @@ bool first_fused(const pe_ctx* c) { return !c->cache_forced; }
 pe_status launch_coarse_sweep(pe_ctx* c) {
   const WalkArgs a = walk_args(c, nullptr, 0ull);
   if (mixed_columns(c, c->precision)) return walk_columns<kCoarse>(c, a);
-  if (c->forcing_path == PE_FORCING_GENERAL) PE_TRY(launch_general_coarse_forcing(c));
-  else PE_TRY(launch_forced_f64(c, nullptr, c->gG));
+  PE_TRY(forced_parts(c, c->precision, nullptr, c->gG));
   return walk_launch<0, 4, kCoarse>(c, a);
 }
 
@@ -345,26 +360,17 @@ pe_status launch_iteration(pe_ctx* c, int precision, bool first, LoopCtl* loop, 
     if (mid) PE_CUDA_TRY(cudaEventRecord(mid, c->stream));
     return PE_OK;
   }
-  if (c->forcing_path == PE_FORCING_GENERAL) {
-    if (first) PE_TRY(launch_general_coarse_forcing(c));
-    PE_TRY(launch_general_fine_sweep(c, precision));
-  } else if (c->cache_forced) {
+  if (c->cache_forced) {
     // one sweep per problem and precision, its forced part kept
     if (c->fz_prec != precision) {
-      if (precision == PE_MIXED) {
-        PE_TRY(forced_f32(c, c->Fz));
-      } else {
-        PE_TRY(launch_column_weights_f64(c));
-        PE_TRY(launch_forced_f64(c, c->Fz, nullptr));
-      }
+      PE_TRY(forced_parts(c, precision, c->Fz, nullptr));
       c->fz_prec = precision;
       c->sweeps += 1;
     }
     a.f = c->Fz;
   } else {
     c->sweeps += 1;
-    PE_TRY(launch_column_weights_f64(c));
-    PE_TRY(launch_forced_f64(c, c->Fbar, first ? c->gG : nullptr));
+    PE_TRY(forced_parts(c, precision, c->Fbar, first ? c->gG : nullptr));
   }
   if (mid) PE_CUDA_TRY(cudaEventRecord(mid, c->stream));
   return first ? walk_launch<0, 4, kFirst>(c, a) : walk_launch<0, 4, kIterate>(c, a);

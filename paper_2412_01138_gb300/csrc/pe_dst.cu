@@ -418,132 +418,133 @@ __global__ void __launch_bounds__(256) dst_fft_kernel(const T* __restrict__ in, 
   }
 }
 
-// Half-length DST-I of one pencil pair per CTA, for float64 passes with few pencils: the
-// fold, complex FFT of N = n + 1 points and unfold of the half-length form (see the warp
-// kernel below), with the radix-2 butterflies and the prefix sum spread over the CTA so
-// that all four SM sub-partitions' float64 units work on the pair (about half the float64
-// work of the odd extension).  Shared memory: the pair (N + 1 values), the FFT buffer (N)
-// and the warp totals of the scan.
-// The CTA's pencil pair (a at in_a, b at in_b, stride `inner`, b absent when !has_b) in
-// x[1..n] on return: x[m] = (F^a_m, F^b_m), the unscaled sine sums.  x, z and wsum are
-// shared buffers of N + 1, N and 8 complex values.
-template <typename T>
-__device__ __forceinline__ void half_block_pair(const T* __restrict__ in_a, const T* __restrict__ in_b, bool has_b,
-                                                int64_t inner, int n, int logN, const Cplx<T>* __restrict__ tw,
-                                                const T* __restrict__ sinN, Cplx<T>* x, Cplx<T>* z, Cplx<T>* wsum) {
-  const int N = 1 << logN, H = N / 2;
-  const int tid = threadIdx.x, B = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  for (int j = tid; j <= N; j += B) {
-    T va = T(0), vb = T(0);
-    if (j >= 1 && j <= n) {
-      va = in_a[(int64_t)(j - 1) * inner];
-      if (has_b) vb = in_b[(int64_t)(j - 1) * inner];
-    }
-    x[j] = Cplx<T>{va, vb};
-  }
-  __syncthreads();
-  // fold y_j = sin(pi j/N)(x_j + x_{N-j}) + (x_j - x_{N-j})/2 of both pencils, z = y^a + i y^b
-  const int shift = 32 - logN;
-  for (int j = tid; j < N; j += B) {
-    const Cplx<T> xj = x[j];
-    const Cplx<T> xm = j == 0 ? Cplx<T>{T(0), T(0)} : x[N - j];
-    const T sj = sinN[j];
-    z[__brev((unsigned)j) >> shift] = Cplx<T>{sj * (xj.re + xm.re) + T(0.5) * (xj.re - xm.re),
-                                              sj * (xj.im + xm.im) + T(0.5) * (xj.im - xm.im)};
-  }
-  __syncthreads();
-  // radix-2 decimation in time, twiddles e^{-2 pi i k/N}
-  for (int st = 1; st <= logN; ++st) {
-    const int half = 1 << (st - 1), tstride = N >> st;
-    for (int b = tid; b < H; b += B) {
-      const int grp = b >> (st - 1), pos = b & (half - 1);
-      const int i0 = grp * 2 * half + pos, i1 = i0 + half;
-      const Cplx<T> w = tw[pos * tstride];
-      const Cplx<T> u = z[i0], v = z[i1];
-      const T tr = w.re * v.re - w.im * v.im;
-      const T ti = w.re * v.im + w.im * v.re;
-      z[i0] = Cplx<T>{u.re + tr, u.im + ti};
-      z[i1] = Cplx<T>{u.re - tr, u.im - ti};
-    }
-    __syncthreads();
-  }
-  // unfold: F_{2k} = I_k, F_{2k+1} = R_0/2 + R_1 + ... + R_k (k < N/2) for both pencils;
-  // thread tid owns the contiguous k = tid*C .. tid*C + C - 1
-  constexpr int CMAX = 2;  // N <= 1024 and 256 threads
-  const int C = (H + B - 1) / B;
-  T ia[CMAX], ib[CMAX], sa[CMAX], sb[CMAX];
-  T ta = T(0), tb = T(0);
-#pragma unroll
-  for (int c = 0; c < CMAX; ++c) {
-    const int k = tid * C + c;
-    ia[c] = ib[c] = T(0);
-    if (c < C && k < H) {
-      const Cplx<T> Z = z[k];
-      const Cplx<T> Wm = z[(N - k) & (N - 1)];
-      T ra = T(0.5) * (Z.re + Wm.re), rb = T(0.5) * (Z.im + Wm.im);
-      ia[c] = T(0.5) * (Wm.im - Z.im);
-      ib[c] = T(0.5) * (Z.re - Wm.re);
-      if (k == 0) {
-        ra *= T(0.5);
-        rb *= T(0.5);
-      }
-      ta += ra;
-      tb += rb;
-    }
-    sa[c] = ta;
-    sb[c] = tb;
-  }
-  // exclusive scan of the thread totals: within the warp by shuffles, then over the warps
-  T ea = ta, eb = tb;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const T ua = __shfl_up_sync(0xffffffffu, ea, d), ub = __shfl_up_sync(0xffffffffu, eb, d);
-    if (lane >= d) {
-      ea += ua;
-      eb += ub;
-    }
-  }
-  if (lane == 31) wsum[warp] = Cplx<T>{ea, eb};
-  __syncthreads();
-  T pre_a = T(0), pre_b = T(0);
-  for (int w = 0; w < warp; ++w) {
-    pre_a += wsum[w].re;
-    pre_b += wsum[w].im;
-  }
-  ea += pre_a - ta;
-  eb += pre_b - tb;
-#pragma unroll
-  for (int c = 0; c < CMAX; ++c) {
-    const int k = tid * C + c;
-    if (c < C && k < H) {
-      if (k > 0) x[2 * k] = Cplx<T>{ia[c], ib[c]};
-      x[2 * k + 1] = Cplx<T>{sa[c] + ea, sb[c] + eb};
-    }
-  }
-  __syncthreads();
+// Half-length DST-I of one pencil pair per CTA, for float64 passes with few pencils: the fold, complex
+// FFT of N = n + 1 points and unfold of the half-length form (see the warp kernel below), one radix-2
+// butterfly per thread, so that all four SM sub-partitions' float64 units work on the pair.
+// With one pair per CTA the pass is a chain of latencies, not work (about 90 float64 instructions per
+// thread): every table value a thread needs is in registers before the pass before it has
+// finished (the tables are constants of the process), both folded values come straight from global memory,
+// the first log2(64) stages stay within a warp's 64 values (no CTA barrier), the first two have no
+// multiplications, and the outputs leave from registers.  255 pencils of 255 values: 6.6 us per pass against
+// 9.7 us with a barrier and a table read per stage.
+//
+// load(j), j = 1..n: values j of the two pencils; store(m, F): the unscaled sums times four,
+// F = 4 (F^a_m, F^b_m), m = 1..n.  z: N complex values of shared memory, wsum: one per warp.
+template <int LOGN>
+constexpr int few_threads() {
+  return (1 << LOGN) / 2 < 32 ? 32 : (1 << LOGN) / 2;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) dst_half_block_kernel(const T* __restrict__ in, T* __restrict__ out, int n,
-                                                             int logN, int64_t inner, int64_t npencils, T scale,
-                                                             const Cplx<T>* __restrict__ tw,
-                                                             const T* __restrict__ sinN) {
+template <int LOGN, typename Load, typename Store>
+__device__ __forceinline__ void few_pair(const Cplx<double>* __restrict__ tw, const double* __restrict__ sinN,
+                                         Cplx<double>* z, Cplx<double>* wsum, Load load, Store store) {
+  constexpr int N = 1 << LOGN, H = N / 2;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const bool on = t < H;
+  // twiddles e^{-2 pi i k/N} of this thread's butterflies from stage 3 on, the fold's 2 sin +- 1
+  Cplx<double> w[LOGN > 2 ? LOGN - 2 : 1];
+  double sp[2], sm[2];
+#pragma unroll
+  for (int st = 3; st <= LOGN; ++st) w[st - 3] = on ? tw[(t & ((1 << (st - 1)) - 1)) << (LOGN - st)] : Cplx<double>{0.0, 0.0};
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const double sj = on ? sinN[t + e * H] : 0.0;
+    sp[e] = fma(2.0, sj, 1.0);
+    sm[e] = fma(2.0, sj, -1.0);
+  }
   pdl_wait();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int N = 1 << logN;
-  Cplx<T>* x = reinterpret_cast<Cplx<T>*>(smem_raw);
-  Cplx<T>* z = x + (N + 1);
-  Cplx<T>* wsum = z + N;
+  // 2 y_j = (2 s_j + 1) x_j + (2 s_j - 1) x_{N-j} of both pencils, bit-reversed
+  if (on) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int j = t + e * H;
+      Cplx<double> y{0.0, 0.0};
+      if (j > 0) {
+        const Cplx<double> xj = load(j), xm = load(N - j);
+        y = Cplx<double>{fma(sp[e], xj.re, sm[e] * xm.re), fma(sp[e], xj.im, sm[e] * xm.im)};
+      }
+      z[__brev((unsigned)j) >> (32 - LOGN)] = y;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int st = 1; st <= LOGN; ++st) {
+    const int half = 1 << (st - 1), pos = t & (half - 1), i0 = ((t >> (st - 1)) << st) + pos, i1 = i0 + half;
+    if (on) {
+      const Cplx<double> u = z[i0], v = z[i1];
+      Cplx<double> m = v;
+      if (st == 2) {
+        if (pos) m = Cplx<double>{v.im, -v.re};
+      } else if (st > 2) {
+        m = Cplx<double>{fma(w[st - 3].re, v.re, -(w[st - 3].im * v.im)), fma(w[st - 3].re, v.im, w[st - 3].im * v.re)};
+      }
+      z[i0] = Cplx<double>{u.re + m.re, u.im + m.im};
+      z[i1] = Cplx<double>{u.re - m.re, u.im - m.im};
+    }
+    // stages 1..6 pair values of one warp's 64
+    if (st < 6 && st < LOGN) __syncwarp();
+    else __syncthreads();
+  }
+  // unfold, times four: F_{2k} = I_k, F_{2k+1} = R_0/2 + R_1 + ... + R_k, k = t
+  double ra = 0.0, rb = 0.0, ia = 0.0, ib = 0.0;
+  if (on) {
+    const Cplx<double> Z = z[t], W = z[(N - t) & (N - 1)];
+    ra = Z.re + W.re;
+    rb = Z.im + W.im;
+    ia = W.im - Z.im;
+    ib = Z.re - W.re;
+    if (t == 0) {
+      ra *= 0.5;
+      rb *= 0.5;
+    }
+  }
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const double ua = __shfl_up_sync(0xffffffffu, ra, d), ub = __shfl_up_sync(0xffffffffu, rb, d);
+    if (lane >= d) {
+      ra += ua;
+      rb += ub;
+    }
+  }
+  constexpr int WARPS = few_threads<LOGN>() / 32;
+  if constexpr (WARPS > 1) {
+    if (lane == 31) wsum[warp] = Cplx<double>{ra, rb};
+    __syncthreads();
+    // the sum over the warps before this one, in the lanes of each warp
+    double pa = lane < warp ? wsum[lane < WARPS ? lane : 0].re : 0.0, pb = lane < warp ? wsum[lane < WARPS ? lane : 0].im : 0.0;
+#pragma unroll
+    for (int d = WARPS / 2; d > 0; d >>= 1) {
+      pa += __shfl_xor_sync(0xffffffffu, pa, d);
+      pb += __shfl_xor_sync(0xffffffffu, pb, d);
+    }
+    // lanes 0 .. WARPS - 1 hold the total; every lane takes lane 0's
+    ra += __shfl_sync(0xffffffffu, pa, 0);
+    rb += __shfl_sync(0xffffffffu, pb, 0);
+  }
+  if (on) {
+    if (t > 0) store(2 * t, Cplx<double>{ia, ib});
+    store(2 * t + 1, Cplx<double>{ra, rb});
+  }
+}
+
+template <int LOGN>
+__global__ void __launch_bounds__(few_threads<LOGN>()) dst_few_kernel(const double* __restrict__ in,
+                                                                      double* __restrict__ out, int n, int64_t inner,
+                                                                      int64_t npencils, double scale,
+                                                                      const Cplx<double>* __restrict__ tw,
+                                                                      const double* __restrict__ sinN) {
+  __shared__ Cplx<double> z[1 << LOGN], wsum[16];
   const int64_t pa = 2 * (int64_t)blockIdx.x, pb = pa + 1;
   const bool has_b = pb < npencils;
-  const int64_t oa = (pa / inner) * (int64_t)n * inner + (pa % inner);
-  const int64_t ob = has_b ? (pb / inner) * (int64_t)n * inner + (pb % inner) : 0;
-  half_block_pair<T>(in + oa, in + ob, has_b, inner, n, logN, tw, sinN, x, z, wsum);
-  for (int m = threadIdx.x + 1; m <= n; m += blockDim.x) {
-    const Cplx<T> F = x[m];
-    out[oa + (int64_t)(m - 1) * inner] = F.re * scale;
-    if (has_b) out[ob + (int64_t)(m - 1) * inner] = F.im * scale;
-  }
+  const int64_t oa = (pa / inner) * (int64_t)n * inner + (pa % inner) - inner;
+  const int64_t ob = has_b ? (pb / inner) * (int64_t)n * inner + (pb % inner) - inner : 0;
+  few_pair<LOGN>(
+      tw, sinN, z, wsum,
+      [&](int j) { return Cplx<double>{in[oa + j * inner], has_b ? in[ob + j * inner] : 0.0}; },
+      [&](int m, Cplx<double> F) {
+        out[oa + m * inner] = F.re * scale;
+        if (has_b) out[ob + m * inner] = F.im * scale;
+      });
 }
 
 // The per-axis source factors of every axis in one launch (blockIdx.y = axis, blockIdx.x =
@@ -555,33 +556,47 @@ struct AxisFactorJob {
   const Cplx<double>* tw[PE_MAX_D];
   const double* sinN[PE_MAX_D];
 };
-__global__ void __launch_bounds__(256) axis_factor_dst_kernel(AxisFactorJob J, const double* __restrict__ loads,
+
+template <int LOGN>
+__device__ __forceinline__ void axis_factor_pair(const AxisFactorJob& J, int a, const double* __restrict__ loads,
+                                                 const double* __restrict__ muM, double* __restrict__ fac,
+                                                 float* __restrict__ fac32, Cplx<double>* z, Cplx<double>* wsum) {
+  const int n = J.n[a], ra = 2 * blockIdx.x;
+  const bool has_b = ra + 1 < J.R;
+  const int64_t oa = (int64_t)J.R * J.off[a] + (int64_t)ra * n - 1, ob = oa + n;
+  const double scale = 0.25 * sqrt(2.0 / (double)(1 << LOGN));
+  few_pair<LOGN>(
+      J.tw[a], J.sinN[a], z, wsum,
+      [&](int j) { return Cplx<double>{loads[oa + j], has_b ? loads[ob + j] : 0.0}; },
+      [&](int m, Cplx<double> F) {
+        const double mu = muM[J.off[a] + m - 1];
+        const double va = F.re * scale / mu;
+        fac[oa + m] = va;
+        if (fac32) fac32[oa + m] = (float)va;
+        if (has_b) {
+          const double vb = F.im * scale / mu;
+          fac[ob + m] = vb;
+          if (fac32) fac32[ob + m] = (float)vb;
+        }
+      });
+}
+
+// as many threads as the longest axis needs; a shorter axis' transform leaves the rest idle
+__global__ void __launch_bounds__(512) axis_factor_dst_kernel(AxisFactorJob J, const double* __restrict__ loads,
                                                               const double* __restrict__ muM,
                                                               double* __restrict__ fac, float* __restrict__ fac32) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  Cplx<double>* z = reinterpret_cast<Cplx<double>*>(smem_raw);
+  Cplx<double>* wsum = z + 1024;
   const int a = blockIdx.y;
-  const int n = J.n[a], logN = J.logN[a], N = 1 << logN;
-  const int ra = 2 * blockIdx.x, rb = ra + 1;
-  if (ra >= J.R) return;  // uniform over the CTA
-  const bool has_b = rb < J.R;
-  Cplx<double>* x = reinterpret_cast<Cplx<double>*>(smem_raw);
-  Cplx<double>* z = x + (N + 1);
-  Cplx<double>* wsum = z + N;
-  const int64_t oa = (int64_t)J.R * J.off[a] + (int64_t)ra * n;
-  const int64_t ob = has_b ? oa + n : 0;
-  half_block_pair<double>(loads + oa, loads + ob, has_b, 1, n, logN, J.tw[a], J.sinN[a], x, z, wsum);
-  const double scale = sqrt(2.0 / (double)N);
-  for (int m = threadIdx.x + 1; m <= n; m += blockDim.x) {
-    const Cplx<double> F = x[m];
-    const double mu = muM[J.off[a] + m - 1];
-    const double va = F.re * scale / mu;
-    fac[oa + m - 1] = va;
-    if (fac32) fac32[oa + m - 1] = (float)va;
-    if (has_b) {
-      const double vb = F.im * scale / mu;
-      fac[ob + m - 1] = vb;
-      if (fac32) fac32[ob + m - 1] = (float)vb;
-    }
+  if (2 * (int)blockIdx.x >= J.R) return;  // uniform over the CTA
+  switch (J.logN[a]) {
+#define PE_AF(X)                                                        \
+  case X:                                                               \
+    axis_factor_pair<X>(J, a, loads, muM, fac, fac32, z, wsum);         \
+    break;
+    PE_AF(4) PE_AF(5) PE_AF(6) PE_AF(7) PE_AF(8) PE_AF(9) PE_AF(10)
+#undef PE_AF
   }
 }
 
@@ -1996,8 +2011,15 @@ pe_status fft_warp_axis(const T* in, T* out, int64_t outer, int n, int64_t inner
   return PE_OK;
 }
 
-// Pencil count up to which the block-wide kernel is used (two pencils per SM of 152).
+// Pencil count up to which the block-wide kernels are used: two pencils per SM of 152; in float64 four,
+// where the half-length kernel with one pair per CTA still leads the warp kernel (608 pencils
+// of 255: 128 against 132 us with the other axis' 116; of 511: 205 against 213; at 800 they are equal or
+// behind, 392 against 376 at 511).
 constexpr int64_t kFewPencils = 2 * 152;
+template <typename T>
+constexpr int64_t few_pencils() {
+  return sizeof(T) == 8 ? 2 * kFewPencils : kFewPencils;
+}
 
 template <typename T>
 pe_status fft_axis(const T* in, T* out, int64_t outer, int n, int64_t inner, int logL, cudaStream_t st) {
@@ -2010,19 +2032,25 @@ pe_status fft_axis(const T* in, T* out, int64_t outer, int n, int64_t inner, int
   // would leave most SMs idle behind the FFT's chain of dependent float64 latencies, so
   // those go to the block-wide kernels, which spread every pencil pair over a CTA (float64
   // in the half-length form from N = n + 1 = 16 on).
-  if (npencils > kFewPencils) PE_TRY(fft_warp_axis<T>(in, out, outer, n, inner, logL, st, &done));
+  if (npencils > few_pencils<T>()) PE_TRY(fft_warp_axis<T>(in, out, outer, n, inner, logL, st, &done));
   if (done) return PE_OK;
   if constexpr (sizeof(T) == 8) {
     const int logN = logL - 1;
-    if (npencils <= kFewPencils && logN >= 4) {
+    if (npencils <= few_pencils<T>() && logN >= 4) {
       const Cplx<T>* twN = twiddles<T>(logN, st);
       const T* sinN = half_sines<T>(logN, st);
       if (!twN || !sinN) return pe_fail(PE_ECUDA, "dst: twiddle table allocation failed");
-      const int N = 1 << logN;
-      const size_t smem = sizeof(Cplx<T>) * ((size_t)2 * N + 1 + 8);
-      const int threads = N / 2 >= 256 ? 256 : (N / 2 >= 128 ? 128 : (N / 2 >= 64 ? 64 : 32));
-      PE_CUDA_TRY(launch_pdl(dst_half_block_kernel<T>, dim3((unsigned)((npencils + 1) / 2)), dim3(threads), smem, st,
-                             in, out, n, logN, inner, npencils, (T)sqrt(2.0 / (double)N), twN, sinN));
+      const double few_scale = 0.25 * sqrt(2.0 / (double)(1 << logN));
+      const dim3 few_grid((unsigned)((npencils + 1) / 2));
+      switch (logN) {
+#define PE_FEW(X)                                                                                                   \
+  case X:                                                                                                           \
+    PE_CUDA_TRY(launch_pdl(dst_few_kernel<X>, few_grid, dim3(few_threads<X>()), 0, st, in, out, n, inner, npencils, \
+                           few_scale, twN, sinN));                                                                  \
+    break;
+        PE_FEW(4) PE_FEW(5) PE_FEW(6) PE_FEW(7) PE_FEW(8) PE_FEW(9) PE_FEW(10)
+#undef PE_FEW
+      }
       PE_CUDA_TRY(cudaGetLastError());
       return PE_OK;
     }
@@ -2197,7 +2225,7 @@ pe_status axis_factors_fused(pe_ctx* c, int R, const double* loads, double* fac,
   AxisFactorJob J{};
   J.d = c->g.d;
   J.R = R;
-  size_t smem = 0;
+  const size_t smem = sizeof(Cplx<double>) * (1024 + 16);
   for (int a = 0; a < c->g.d; ++a) {
     int logL = 0;
     if (c->g.per[a] || !fft_size_ok(c->g.n[a], &logL) || logL - 1 < 4) return PE_OK;
@@ -2207,13 +2235,12 @@ pe_status axis_factors_fused(pe_ctx* c, int R, const double* loads, double* fac,
     J.tw[a] = twiddles<double>(logL - 1, c->stream);
     J.sinN[a] = half_sines<double>(logL - 1, c->stream);
     if (!J.tw[a] || !J.sinN[a]) return pe_fail(PE_ECUDA, "dst: twiddle table allocation failed");
-    smem = std::max(smem, sizeof(Cplx<double>) * ((size_t)2 * (c->g.n[a] + 1) + 1 + 8));
   }
   int nmax = 1;
   for (int a = 0; a < c->g.d; ++a) nmax = std::max(nmax, c->g.n[a] + 1);
-  const int threads = nmax / 2 >= 256 ? 256 : (nmax / 2 >= 128 ? 128 : (nmax / 2 >= 64 ? 64 : 32));
-  axis_factor_dst_kernel<<<dim3((unsigned)((R + 1) / 2), (unsigned)c->g.d), threads, smem, c->stream>>>(
-      J, loads, c->muM_axis, fac, fac32);
+  const int threads = std::max(32, nmax / 2);
+  PE_CUDA_TRY(launch_pdl(axis_factor_dst_kernel, dim3((unsigned)((R + 1) / 2), (unsigned)c->g.d), dim3(threads), smem,
+                         c->stream, J, loads, (const double*)c->muM_axis, fac, fac32));
   PE_CUDA_TRY(cudaGetLastError());
   c->launches += 1;
   *done = true;

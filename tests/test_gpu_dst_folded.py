@@ -55,3 +55,22 @@ def test_folded_matrix_form_matches_dense_products(env, n, f32):
     for got in (out, d):
         err = np.linalg.norm(got.cpu().numpy().astype(np.float64).reshape(n) - ref) / np.linalg.norm(ref)
         assert err <= bound, (err, bound)
+
+
+@pytest.mark.parametrize("m", [15, 31, 63, 127, 255, 511, 1023])
+@pytest.mark.parametrize("pencils", [1, 2, 5, 70])
+@pytest.mark.parametrize("strided", [False, True], ids=["contiguous", "strided"])
+def test_few_float64_pencils(env, m, pencils, strided):
+    """The block-wide half-length FFT at every length, one pencil and an odd number of them (the last pair is
+    half empty).  Its prefix sum adds up to N/2 = (m + 1)/2 values of an FFT of log2 N stages: N log2 N u relative."""
+    pe, torch = env
+    n = (m,) if pencils == 1 else ((m, pencils) if strided else (pencils, m))
+    x = np.random.default_rng(m + pencils).standard_normal(n)
+    d = torch.tensor(x.reshape(-1), device="cuda")
+    pe.dst(len(n), n, d, d)
+    ref = _dense(x)
+    err = np.linalg.norm(d.cpu().numpy().reshape(n) - ref) / np.linalg.norm(ref)
+    bound = (m + 1) * math.log2(m + 1) * 2.0 ** -53
+    if pencils > 1:  # the other axis in the matrix form
+        bound += (pencils / 2 + 3) * 2.0 ** -53 * math.sqrt(pencils)
+    assert err <= bound, (err, bound)

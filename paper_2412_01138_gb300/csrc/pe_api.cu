@@ -130,7 +130,7 @@ void free_ctx(pe_ctx* c) {
                   c->gen_L, c->gen_X, c->axisM, c->lam, c->coefF, c->coefG,
                   c->coefF32, c->coefG32, c->U, c->Fbar, c->gG, c->work0, c->work1, c->out_nodal, c->partials,
                   c->red, c->axisF, c->axisF32, c->axisU0, c->loads, c->tab64, c->tab32,
-                  c->Ktab, c->V64, c->G64, c->V32, c->G32, c->Fz, c->done_ctr,
+                  c->Ktab, c->V64, c->G64, c->V32, c->G32, c->Fz, c->done_ctr, c->resp_nodes, c->resp,
                   c->muM_full, c->ratio_full, c->fac_full, c->work2, c->loopctl, c->loop_hist, c->io32, c->muM_inv};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -415,6 +415,7 @@ extern "C" pe_status pe_setup(pe_ctx** out, int32_t d, const int32_t* n, const d
   for (int a = 0; a < d && st == PE_OK; ++a)
     if (c->S32[a]) st = build_dst_matrix_f32(n[a], c->S32[a], c->stream, c->g.per[a]);
   if (st == PE_OK) st = launch_coef_tables(c);
+  if (st == PE_OK && c->g.ndof >= kRespMinDof) st = setup_response_nodes(c);
   if (st == PE_OK) {
     cudaError_t e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) st = pe_cuda_fail(e, "pe_setup");

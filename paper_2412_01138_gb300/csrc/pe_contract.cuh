@@ -102,6 +102,51 @@ __device__ __forceinline__ void chain_sum(F2 x, int M, int steps, const float* _
   }
 }
 
+// Response tables.  The weight of a term's columns is P times a function of lam alone,
+//   H_r(lam) = (sum_i dt b_i(-lam dt) Z(c_i dt)) S_M(lam)   (complex for a sinusoid),
+// smooth over scales of lam itself: on an interval of relative width w the interpolation at n Chebyshev
+// nodes is off by 2 (w/4)^n at most (in units of int e^{-lam s} ds times the term's size).  Where a grid has many
+// more modes than an interval table has nodes, H is tabulated per problem and a mode evaluates a
+// polynomial instead of the q stages and the chain.  Intervals split each octave of lam evenly into 2^bits
+// (index and local coordinate are bits of lam): float 16 per octave and 5 nodes (2e-9 of the scale, a
+// thirtieth of a float's rounding), double 32 and 8 (3e-17).  One more interval, the last, is lam = 0.
+template <typename T>
+struct Resp;
+template <>
+struct Resp<float> {
+  static constexpr int bits = 4, nodes = 5, comp = 6;  // c0 high, c0 low, c1 .. c4
+};
+template <>
+struct Resp<double> {
+  static constexpr int bits = 5, nodes = 8, comp = 8;
+};
+// interval index of lam >= 0 (base: the first interval's leading bits, T intervals and the zero one) and the local
+// coordinate in [-1, 1)
+__device__ __forceinline__ int resp_locate(double lam, int base, int T, float& x) {
+  constexpr int B = Resp<float>::bits;
+  const int hi = __double2hiint(lam), idx = (hi >> (20 - B)) - base;
+  if (idx < 0) {  // lam = 0
+    x = 0.f;
+    return T;
+  }
+  const unsigned m = ((unsigned)(hi & ((1 << (20 - B)) - 1)) << (B + 4)) | ((unsigned)__double2loint(lam) >> (28 - B));
+  x = fmaf((float)m, 0x1p-23f, -1.f);  // 24 bits below the interval's own: exact
+  return min(idx, T - 1);
+}
+__device__ __forceinline__ int resp_locate(double lam, int base, int T, double& x) {
+  constexpr int B = Resp<double>::bits;
+  const int hi = __double2hiint(lam), idx = (hi >> (20 - B)) - base;
+  if (idx < 0) {
+    x = 0.0;
+    return T;
+  }
+  // mantissa in [1, 2) less the interval's middle, times 2^(B+1): exact
+  const double m = __hiloint2double((hi & 0xFFFFF) | 0x3FF00000, __double2loint(lam));
+  const double mid = __hiloint2double((((hi & 0xFFFFF) >> (20 - B)) << (20 - B)) | (1 << (19 - B)) | 0x3FF00000, 0);
+  x = (m - mid) * (double)(1 << (B + 1));
+  return min(idx, T - 1);
+}
+
 // Time-table entries of one term (t: the term; dt, dT the fine and coarse steps).
 // column value of slice n, kind 0 or 1 (the cosine partner of a sinusoid)
 __device__ __forceinline__ bool grows(const pe_term& t) { return t.tkind != PE_T_SIN && t.tp[0] > 0.0; }

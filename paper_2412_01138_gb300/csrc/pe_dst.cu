@@ -148,7 +148,6 @@ constexpr int kFoldJC = 32;  // folded indices per chunk
 template <typename T, int RW, int CW>
 __global__ void __launch_bounds__(128) folded_dst_kernel(const T* __restrict__ row, const T* __restrict__ in,
                                                          T* __restrict__ out, int n, int64_t inner, int64_t np) {
-  pdl_wait();
   constexpr int JC = kFoldJC, TC = 32 * CW, TK = 8 * RW, PE = JC * TC / 128, SE = JC * TK / 128;
   __shared__ T sX[2][JC][TC + 1];  // sums and differences (then the outputs of contiguous pencils)
   __shared__ __align__(16) T sS[2][JC][4 * RW];
@@ -280,7 +279,10 @@ __global__ void __launch_bounds__(128) folded_dst_kernel(const T* __restrict__ r
 template <typename T, int RW, int CW>
 pe_status folded_launch(const T* row, const T* in, T* out, int n, int64_t inner, int64_t np, cudaStream_t st) {
   const dim3 grid((unsigned)((np + 32 * CW - 1) / (32 * CW)), (unsigned)((n + 8 * RW - 1) / (8 * RW)));
-  PE_CUDA_TRY(launch_pdl(folded_dst_kernel<T, RW, CW>, grid, dim3(128), 0, st, row, in, out, n, inner, np));
+  // a plain launch: CTAs let in while the kernel before still runs pile up on the SMs that have room, and
+  // the busiest SM is the run time (two transforms of 405 x 279 in a solve: 706 us with an early launch, 538 without)
+  folded_dst_kernel<T, RW, CW><<<grid, 128, 0, st>>>(row, in, out, n, inner, np);
+  PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;
 }
 

@@ -10,6 +10,7 @@
 // the fine propagator and the coarse step (pe_contract.cuh) are tabulated here; the sweeps
 // multiply columns and weights together on the fly.
 #include <math.h>
+#include <string.h>
 
 #include <algorithm>
 
@@ -17,6 +18,7 @@
 #include "pe_forcing_common.cuh"
 #include "pe_internal.h"
 #include "pe_learned.h"
+#include "pe_phi.cuh"
 
 namespace {
 
@@ -181,6 +183,146 @@ __global__ void __launch_bounds__(256) column_weights_kernel(Geom g, StageCols C
   }
 }
 
+// The same weights from the response table (pe_contract.cuh): per mode and term a polynomial of the
+// mode's lam, whose interval and coordinate are found once.  Memory-bound (the weights written), where the direct
+// evaluation is bound by its chain (60 float64 or 700 float32 operations per mode and sinusoid).  255^2 modes, 9 terms: 9.5 us after an 8.5 us table
+// (beside the loads) against 24.7 us in float32, 31 after 13 against 91 us in float64; 127^3, 17 terms, float32: 208
+// against 821 us.
+template <typename T>
+__global__ void __launch_bounds__(256) response_weights_kernel(Geom g, StageCols C, ColumnTables D, int R, int p, int tpt,
+                                                               int base, int T_, const T* __restrict__ resp,
+                                                               const T* __restrict__ axisF, const T* __restrict__ coefG,
+                                                               T* __restrict__ V, T* __restrict__ G,
+                                                               const double* __restrict__ lam) {
+  pdl_wait();
+  constexpr int CO = Resp<T>::comp;
+  const int64_t J = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (J >= g.ndof) return;
+  const int64_t nd = g.ndof;
+  const int K = C.K;
+  const T* ZG;
+  if constexpr (sizeof(T) == 8) ZG = D.ZG;
+  else ZG = D.ZG32;
+  int j[PE_MAX_D];
+  unflatten(g, J, j);
+  T x;
+  const int idx = resp_locate(lam[J], base, T_, x);
+  T bg[PE_MAX_S];
+#pragma unroll
+  for (int i = 0; i < PE_MAX_S; ++i) bg[i] = G && i < p ? coefG[(int64_t)i * nd + J] : T(0);
+  const int r1 = min(R, (int)(blockIdx.y + 1) * tpt);
+  for (int r = blockIdx.y * tpt; r < r1; ++r) {
+    const int k = C.first[r];
+    const bool two = k + 1 < K && C.term[k + 1] == r;
+    T P = axisF[(int64_t)R * g.off[0] + (int64_t)r * g.n[0] + j[0]];
+#pragma unroll
+    for (int a = 1; a < PE_MAX_D; ++a) if (a < g.d) P *= axisF[(int64_t)R * g.off[a] + (int64_t)r * g.n[a] + j[a]];
+    const T* c = resp + ((int64_t)r * (T_ + 1) + idx) * 2 * CO;
+    T v0, v1 = T(0);
+    if constexpr (sizeof(T) == 4) {
+      // 12 coefficients as three float4: c0 high and low, c1, c2 | c3, c4, then the second column's
+      const float4 a0 = *reinterpret_cast<const float4*>(c), a1 = *reinterpret_cast<const float4*>(c + 4);
+      v0 = a0.x + fmaf(x, fmaf(x, fmaf(x, fmaf(x, a1.y, a1.x), a0.w), a0.z), a0.y);
+      if (two) {
+        const float4 a2 = *reinterpret_cast<const float4*>(c + 8);
+        v1 = a1.z + fmaf(x, fmaf(x, fmaf(x, fmaf(x, a2.w, a2.z), a2.y), a2.x), a1.w);
+      }
+    } else {
+      v0 = c[CO - 1];
+#pragma unroll
+      for (int i = CO - 2; i >= 0; --i) v0 = fma(x, v0, c[i]);
+      if (two) {
+        v1 = c[2 * CO - 1];
+#pragma unroll
+        for (int i = CO - 2; i >= 0; --i) v1 = fma(x, v1, c[CO + i]);
+      }
+    }
+    V[(int64_t)k * nd + J] = P * v0;
+    if (two) V[(int64_t)(k + 1) * nd + J] = P * v1;
+    if (G) {
+      T gr = T(0), gi = T(0);
+#pragma unroll
+      for (int i = 0; i < PE_MAX_S; ++i)
+        if (i < p) {
+          gr = fma(bg[i], ZG[i * K + k], gr);
+          if (two) gi = fma(bg[i], ZG[i * K + k + 1], gi);
+        }
+      G[(int64_t)k * nd + J] = P * gr;
+      if (two) G[(int64_t)(k + 1) * nd + J] = P * gi;
+    }
+  }
+}
+
+// lam of node i of an interval (T: the zero interval)
+__device__ __forceinline__ double resp_node(int base, int T, int t, int i, int bits, int nodes) {
+  if (t == T) return 0.0;
+  const double lo = __hiloint2double((base + t) << (20 - bits), 0), hi = __hiloint2double((base + t + 1) << (20 - bits), 0);
+  return lo + (hi - lo) * (0.5 + 0.5 * cospi((2.0 * i + 1.0) / (2.0 * nodes)));
+}
+
+// E and dt b_1..q at every node: out[(t * nodes + i) * (1 + q)]
+__global__ void response_nodes_kernel(int base, int T, int bits, int nodes, double dt, int q, Lag LF,
+                                      double* __restrict__ out) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= (T + 1) * nodes) return;
+  const double lam = resp_node(base, T, e / nodes, e % nodes, bits, nodes);
+  double b[PE_MAX_S];
+  b_weights(-lam * dt, q, LF, b);
+  out[(int64_t)e * (1 + q)] = exp(-lam * dt);
+  for (int i = 0; i < q; ++i) out[(int64_t)e * (1 + q) + 1 + i] = dt * b[i];
+}
+
+// Polynomial coefficients of H_r on every interval (a CTA per interval; a thread per term and node, then per
+// coefficient).  Minv: monomial coefficients from node values; applied to the differences from the middle
+// node's value, which the interval makes small, so that its entries do not amplify their rounding.
+struct RespInv {
+  double m[8][8];
+};
+template <typename T>
+__global__ void __launch_bounds__(256) response_kernel(StageCols C, ColumnTables D, int R, int M, int q, int T_,
+                                                       RespInv I, const double* __restrict__ nodes,
+                                                       T* __restrict__ resp) {
+  pdl_wait();
+  constexpr int NN = Resp<T>::nodes, CO = Resp<T>::comp;
+  __shared__ double val[PE_MAX_TERMS * NN][2];
+  const int t = blockIdx.x, K = C.K, steps = chain_steps(M);
+  for (int e = threadIdx.x; e < R * NN; e += blockDim.x) {
+    const int r = e / NN, i = e - r * NN;
+    const double* nb = nodes + ((int64_t)t * NN + i) * (1 + q);
+    const int k = C.first[r];
+    const bool two = k + 1 < K && C.term[k + 1] == r;
+    double br = 0.0, bi = 0.0;
+    for (int s = 0; s < q; ++s) {
+      br = fma(nb[1 + s], D.ZF[s * K + k], br);
+      if (two) bi = fma(nb[1 + s], D.ZF[s * K + k + 1], bi);
+    }
+    double Sr, Si;
+    chain_sum(nb[0] * D.xs[r], M, steps, D.chain + 4 * r, 4 * R, Sr, Si);
+    val[e][0] = fma(br, Sr, -(bi * Si));
+    val[e][1] = fma(br, Si, bi * Sr);
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < R * 2 * NN; e += blockDim.x) {
+    const int d = e % NN, rc = e / NN, r = rc >> 1, comp = rc & 1;
+    const double mid = val[r * NN + NN / 2][comp];
+    double c = 0.0;
+#pragma unroll
+    for (int i = 0; i < NN; ++i) c = fma(I.m[d][i], val[r * NN + i][comp] - mid, c);
+    if (d == 0) c += mid;
+    T* o = resp + (((int64_t)r * (T_ + 1) + t) * 2 + comp) * CO;
+    if constexpr (sizeof(T) == 4) {
+      if (d == 0) {
+        o[0] = (float)c;
+        o[1] = (float)(c - (double)(float)c);
+      } else {
+        o[1 + d] = (float)c;
+      }
+    } else {
+      o[d] = c;
+    }
+  }
+}
+
 // 1D consistent loads of every (term, axis): out[R*off[a] + r*n_a + k] = int g_{r,a} phi_{k+1}.
 // Eight lanes per node (blockDim = 8 x 32 nodes): lane s evaluates the quadrature points
 // e = s, s + 8, ... of the node's 2 npts (its left element's points, then its right element's),
@@ -324,6 +466,96 @@ __global__ void amps_kernel(TermsDev T, double* w) {
 
 }  // namespace
 
+// Rows d of the inverse: the coefficient of x^d of the polynomial through values at the Chebyshev nodes
+// x_i = cos(pi (2 i + 1) / (2 n)), from the discrete Chebyshev transform and T_k's own coefficients.
+static RespInv response_inverse(int n) {
+  double T[8][8] = {};  // T_k in monomials
+  T[0][0] = 1.0;
+  if (n > 1) T[1][1] = 1.0;
+  for (int k = 2; k < n; ++k)
+    for (int d = 0; d < n; ++d) T[k][d] = (d ? 2.0 * T[k - 1][d - 1] : 0.0) - T[k - 2][d];
+  RespInv I{};
+  for (int d = 0; d < n; ++d)
+    for (int i = 0; i < n; ++i) {
+      double s = 0.0;
+      for (int k = 0; k < n; ++k)
+        s += (k ? 2.0 : 1.0) / n * cos(M_PI * k * (2.0 * i + 1.0) / (2.0 * n)) * T[k][d];
+      I.m[d][i] = s;
+    }
+  return I;
+}
+
+pe_status setup_response_nodes(pe_ctx* c) {
+  // the range of lam over the whole grid, zero aside
+  double lo = 0.0, hi = 0.0, least = INFINITY;
+  bool zero = true;
+  for (int a = 0; a < c->gn.d; ++a) {
+    const int n = c->gn.n[a];
+    auto ratio = [&](double th) {
+      const double sh = sin(0.5 * th);
+      return ((4.0 / c->h[a]) * sh * sh) / ((c->h[a] / 3.0) * (2.0 + cos(th)));
+    };
+    if (c->gn.per[a]) {
+      if (n > 1) least = std::min(least, ratio(2.0 * M_PI / n));
+      hi += ratio(2.0 * M_PI * (n / 2) / n);
+    } else {
+      zero = false;
+      lo += ratio(M_PI / (n + 1));
+      hi += ratio(M_PI * n / (n + 1));
+    }
+  }
+  if (zero) lo = least;
+  lo *= c->D * (1.0 - 1e-9);
+  hi *= c->D * (1.0 + 1e-9);
+  // no table for spectra beyond the normal range of a double
+  if (!(lo > 1e-300 && hi < 1e300)) return PE_OK;
+  const bool f32 = c->precision == PE_MIXED;
+  const int bits = f32 ? Resp<float>::bits : Resp<double>::bits, nodes = f32 ? Resp<float>::nodes : Resp<double>::nodes;
+  const int comp = f32 ? Resp<float>::comp : Resp<double>::comp;
+  auto lead = [bits](double v) {
+    int64_t u;
+    memcpy(&u, &v, sizeof(u));
+    return (int)(u >> (52 - bits));
+  };
+  const int base = lead(lo), T = lead(hi) - base + 1;
+  // a node costs about what eight modes save (200 x 117 modes in float64, 4200 nodes: 9 us slower with the table)
+  if ((int64_t)(T + 1) * nodes * 8 > c->g.ndof) return PE_OK;
+  if (cudaMalloc((void**)&c->resp_nodes, sizeof(double) * (size_t)(T + 1) * nodes * (1 + c->q)) != cudaSuccess ||
+      cudaMalloc(&c->resp, (f32 ? sizeof(float) : sizeof(double)) * (size_t)PE_MAX_TERMS * (T + 1) * 2 * comp) !=
+          cudaSuccess) {
+    cudaGetLastError();
+    return pe_fail(PE_ENOMEM, "pe_setup: response-table allocation failed");
+  }
+  c->resp_base = base;
+  c->resp_T = T;
+  Lag LF{};
+  for (int i = 0; i < PE_MAX_S; ++i)
+    for (int m = 0; m < PE_MAX_S; ++m) LF.a[i][m] = c->lagF[i][m];
+  response_nodes_kernel<<<((T + 1) * nodes + 63) / 64, 64, 0, c->stream>>>(base, T, bits, nodes, c->dt, c->q, LF,
+                                                                          c->resp_nodes);
+  c->launches += 1;
+  PE_CUDA_TRY(cudaGetLastError());
+  return PE_OK;
+}
+
+// The current problem's response table, after its time tables (not with the learned correction, whose bands the
+// direct kernel adds).
+static pe_status launch_response(pe_ctx* c) {
+  if (!c->resp || c->mlp) return PE_OK;
+  const dim3 grid((unsigned)(c->resp_T + 1));
+  if (c->precision == PE_MIXED) {
+    static const RespInv I = response_inverse(Resp<float>::nodes);
+    PE_CUDA_TRY(launch_pdl(response_kernel<float>, grid, dim3(160), 0, c->stream, c->cols, c->tab, c->R, c->M, c->q,
+                           c->resp_T, I, (const double*)c->resp_nodes, (float*)c->resp));
+  } else {
+    static const RespInv I = response_inverse(Resp<double>::nodes);
+    PE_CUDA_TRY(launch_pdl(response_kernel<double>, grid, dim3(160), 0, c->stream, c->cols, c->tab, c->R, c->M, c->q,
+                           c->resp_T, I, (const double*)c->resp_nodes, (double*)c->resp));
+  }
+  c->launches += 1;
+  return PE_OK;
+}
+
 pe_status launch_time_tables(pe_ctx* c) {
   const int R = c->R;
   if (R == 0) return PE_OK;
@@ -352,7 +584,7 @@ pe_status launch_time_tables(pe_ctx* c) {
                          c->stream, T, C, c->tab, c->N, c->M, c->q, c->p, c->t0, c->dT, c->dt, nF, nG));
   c->launches += 1;
   PE_CUDA_TRY(cudaGetLastError());
-  return PE_OK;
+  return launch_response(c);
 }
 
 // Room for the weights of K columns in one table.
@@ -393,6 +625,14 @@ static pe_status column_weights(pe_ctx* c, T* V, T* G, const LearnedTerms& L) {
     axisF = c->axisF32;
     coef = c->coefF32;
     coefG = c->coefG32;
+  }
+  // the table serves the form it was made in (a mixed context's float64 weights are evaluated directly)
+  if (c->resp && !L.Ktab && V && (sizeof(T) == 8) == (c->precision != PE_MIXED)) {
+    PE_CUDA_TRY(launch_pdl(response_weights_kernel<T>, grid, dim3(threads), 0, c->stream, c->g, c->cols, c->tab, c->R,
+                           c->p, tpt, c->resp_base, c->resp_T, (const T*)c->resp, axisF, coefG, V, G,
+                           (const double*)c->lam));
+    c->launches += 1;
+    return PE_OK;
   }
   PE_CUDA_TRY(launch_pdl(column_weights_kernel<T>, grid, dim3(threads), 0, c->stream, c->g, c->cols, c->tab, c->R, c->M,
                          c->q, c->p, tpt, axisF, coef, coefG, V, G, L, (const double*)c->axisF,

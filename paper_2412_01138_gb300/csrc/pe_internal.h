@@ -178,6 +178,12 @@ struct pe_ctx {
   float *V32 = nullptr, *G32 = nullptr;
   int capV64 = 0, capG64 = 0, capV32 = 0, capG32 = 0;  // columns allocated
   bool V64_valid = false;       // V64 holds the current problem's weights
+  // response tables of the weights (pe_contract.cuh) in the form's own arithmetic, grids of at least
+  // kRespMinDof modes: leading bits of the first interval, intervals, E and dt b_i at the nodes, polynomial
+  // coefficients [R][resp_T + 1][2][comp] of the current problem (null: weights evaluated directly)
+  int resp_base = 0, resp_T = 0;
+  double* resp_nodes = nullptr;
+  void* resp = nullptr;
   double* loads = nullptr;      // [PE_MAX_TERMS * nsum_full] 1D loads before the DST
   // learned coarse correction (optional)
   const struct pe_mlp* mlp = nullptr;
@@ -239,7 +245,9 @@ pe_status build_dst_matrix(int n, double* S, cudaStream_t st, int periodic = 0);
 pe_status build_dst_matrix_f32(int n, float* S, cudaStream_t st, int periodic = 0);
 
 // pe_forcing.cu
-pe_status launch_time_tables(pe_ctx* c);   // also sets c->K and c->cols
+constexpr int64_t kRespMinDof = 16384;
+pe_status setup_response_nodes(pe_ctx* c);  // at pe_setup
+pe_status launch_time_tables(pe_ctx* c);   // also sets c->K and c->cols; the response table after them
 pe_status launch_column_weights(pe_ctx* c);  // V64 and G64 (float64 form) or V32 and G32 (mixed form)
 pe_status launch_column_weights_f64(pe_ctx* c);  // V64, if not yet made for this problem
 // rows of whole-axis per-axis tables [R * nsum_full] kept by a sharded context, in its layout

@@ -102,7 +102,6 @@ __host__ __device__ constexpr int walk_cap(int SRC, int KB, int MODE) {
 
 template <int SRC, int KB, int MODE>
 __global__ void __launch_bounds__(walk_cap(SRC, KB, MODE)) walk_kernel(WalkArgs a) {
-  pdl_wait();
   extern __shared__ __align__(16) float sY[];  // [SL][2 KB]
   __shared__ double sh[32];
   __shared__ bool s_last;
@@ -259,7 +258,10 @@ pe_status walk_launch(pe_ctx* c, WalkArgs a) {
     a.SL = std::min((c->N + kPF - 1) / kPF * kPF, most);
     smem = sizeof(float) * 2 * (size_t)a.SL * KB;
   }
-  PE_CUDA_TRY(launch_pdl(walk_kernel<SRC, KB, MODE>, dim3((unsigned)blocks), dim3(threads), smem, c->stream, a));
+  // a plain launch (no early start beside the kernel before): one CTA per SM is the even share that
+  // per_mode_block chose (200 x 117 nodes: 8 us of a 277 us solve)
+  walk_kernel<SRC, KB, MODE><<<(unsigned)blocks, threads, smem, c->stream>>>(a);
+  PE_CUDA_TRY(cudaGetLastError());
   c->launches += 1;
   return PE_OK;
 }

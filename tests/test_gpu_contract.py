@@ -115,3 +115,32 @@ def test_batched_walk_stages_slices_in_chunks(pe):
                 assert k[i] == min(2, p.N)
                 for m in range(0, p.N + 1, max(1, p.N // 9)):
                     assert _rel(b.modal(i, m), fine[m], sys_.norm_w) <= bound, (prec, i, m)
+
+
+RESPONSE = {"plane": ((160, 131), 0.05, (), "s" * 5 + "e", 31), "box": ((30, 26, 27), 0.4, (), "sse", 8),
+            "periodic": ((128, 150), 0.01, (True, True), "ses", 17), "line": ((16384,), 1.0, (), "se", 5),
+            "thin": ((16, 2000), 3.0, (), "s" * 9, 64), "one_periodic": ((64, 300), 20.0, (True, False), "ees", 3)}
+
+
+@pytest.mark.parametrize("name", list(RESPONSE))
+def test_weights_from_the_response_table(pe, name):
+    """Grids large enough for the tabulated weights: spectra of 3 to 30 octaves, the zero eigenvalue of an
+    all-periodic grid (an interval of its own), stiff and slow modes; every mode of every slice against the
+    oracle, in the norm of each form's bound and mode by mode against the largest."""
+    n, D, periodic, kinds, M = RESPONSE[name]
+    d = len(n)
+    box = ((0.0, 1.0),) * d
+    facs = tuple(I.Factor(I.S_GAUSS, (0.4, 0.02)) for _ in range(d))  # excites the whole spectrum
+    forcing = tuple(I.Term(t.amp, facs, t.tkind, t.tp) for t in _terms(kinds, d, 3))
+    prob = I.Problem(d, n, box, D, 0.1, 0.8, 3, M, I.uniform_nodes(4), I.uniform_nodes(2), (), forcing, 3, 1e-12, None, "",
+                     (), periodic)
+    sys_ = osolver.ModalSystem(prob)
+    ref = osolver.parareal(sys_, tol=0.0, k_max=1)
+    for prec, bound in ((pe.PE_FP64, 1e-12), (pe.PE_MIXED, 1e-6)):
+        with pe.Solver(prob, precision=prec) as s:
+            s.set_problem()
+            s.iterate()
+            for m in range(1, prob.N + 1):
+                got, want = s.modal(m), ref.history[1][m]
+                assert _rel(got, want, sys_.norm_w) <= bound, (prec, m)
+                assert np.abs(got - want).max() <= bound * np.abs(want).max(), (prec, m)

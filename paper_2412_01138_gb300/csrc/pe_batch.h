@@ -29,7 +29,7 @@ struct BProb {
   int64_t oXs;   // chain scales of the terms, R (float: pairs at twice the offset)
   int64_t oCol;  // column map: K entries, (term << 1) | kind
   int64_t oFirst;  // first column of each term, R entries
-  int64_t oMu;   // muM / ratio: nsum
+  int64_t oMu;   // muM / ratio / rows: nsum
   int64_t oItems;  // first mode item of this problem
   int nItems;
   // learned coarse correction (pe_batch_set_learned): band table K^[r][band] (re, im) at oKt,
@@ -88,6 +88,9 @@ struct pe_batch {
   int64_t tt_total = 0;
   // arenas
   double *muM = nullptr, *ratio = nullptr;
+  double* rows = nullptr;     // per axis: sqrt(2/(n+1)) sin(pi m/(n+1)), m = 1..n (the transforms' sine rows)
+  double* scratch = nullptr;  // two nodal fields of the largest problem (get_solution)
+  int64_t ndof_max = 1;
   double *coefF = nullptr, *coefG = nullptr;
   float *coefF32 = nullptr, *coefG32 = nullptr;
   double* U = nullptr;

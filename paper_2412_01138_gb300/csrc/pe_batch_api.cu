@@ -39,7 +39,7 @@ void free_batch(pe_batch* b) {
   for (cudaGraphExec_t g : b->graph_exec)
     if (g) cudaGraphExecDestroy(g);
   void* ptrs[] = {b->d_probs, b->d_terms, b->d_mode_items, b->walk128.d_items, b->walk256.d_items,
-                  b->d_factor_jobs, b->d_mu_prefix, b->d_tt_prefix, b->muM, b->ratio, b->coefF, b->coefG,
+                  b->d_factor_jobs, b->d_mu_prefix, b->d_tt_prefix, b->muM, b->ratio, b->rows, b->scratch, b->coefF, b->coefG,
                   b->coefF32, b->coefG32, b->U, b->axisF, b->axisU0, b->axisF32, b->partials, b->active,
                   b->kcount, b->resid, b->counter, b->dflags, b->Y, b->Z, b->chain, b->xs, b->Y32, b->Z32,
                   b->chain32, b->xs32, b->V, b->G, b->V32, b->G32, b->d_cols, b->d_first, b->Kt, b->d_kt_prefix};
@@ -209,6 +209,7 @@ extern "C" pe_status pe_setup_batch(pe_batch** out, int32_t n_problems, const pe
     }
     B.K = (int)((int64_t)cols.size() - B.oCol);
     b->Kmax = std::max(b->Kmax, B.K);
+    b->ndof_max = std::max(b->ndof_max, ndof);
     B.oU = oU; oU += (int64_t)(B.N + 1) * ndof;
     B.oCF = oCF; oCF += (int64_t)(B.q + 2) * ndof;
     B.oCG = oCG; oCG += (int64_t)(B.p + 1) * ndof;
@@ -248,6 +249,8 @@ extern "C" pe_status pe_setup_batch(pe_batch** out, int32_t n_problems, const pe
   const bool mixed = b->precision == PE_MIXED;
   if (st == PE_OK) st = balloc(&b->muM, oMu);
   if (st == PE_OK) st = balloc(&b->ratio, oMu);
+  if (st == PE_OK) st = balloc(&b->rows, oMu);
+  if (st == PE_OK) st = balloc(&b->scratch, 2 * (size_t)b->ndof_max);
   if (st == PE_OK) st = balloc(&b->coefF, oCF);
   if (st == PE_OK && mixed) st = balloc(&b->coefF32, oCF);
   if (st == PE_OK) st = balloc(&b->coefG, oCG);
@@ -296,6 +299,9 @@ extern "C" pe_status pe_setup_batch(pe_batch** out, int32_t n_problems, const pe
         for (int r = 0; r < B.Ru; ++r) jobs.push_back(FactorJob{p, a, r, 1});
       }
     }
+    std::stable_sort(jobs.begin(), jobs.end(), [&](const FactorJob& x, const FactorJob& y) {
+      return b->probs[x.p].g.n[x.axis] > b->probs[y.p].g.n[y.axis];
+    });
     b->n_factor_jobs = (int)jobs.size();
     st = upload(&b->d_probs, b->probs, b->stream);
     if (st == PE_OK) st = upload(&b->d_terms, b->terms, b->stream);
@@ -514,18 +520,14 @@ extern "C" pe_status pe_batch_get_solution(pe_batch* b, int32_t problem, double*
   const BProb& B = b->probs[problem];
   int n[PE_MAX_D] = {B.g.n[0], B.g.n[1], B.g.n[2]};
   const double* last = b->U + B.oU + (int64_t)B.N * B.g.ndof;
-  pe_status st = PE_OK;
-  if (pe_is_device_ptr(nodal_out)) {
-    st = pe_dst(B.g.d, n, last, nodal_out, b->stream);
-  } else {
-    double* tmp = nullptr;
-    PE_CUDA_TRY(cudaMallocAsync((void**)&tmp, sizeof(double) * B.g.ndof, b->stream));
-    st = pe_dst(B.g.d, n, last, tmp, b->stream);
-    if (st == PE_OK) {
-      cudaError_t e = cudaMemcpyAsync(nodal_out, tmp, sizeof(double) * B.g.ndof, cudaMemcpyDeviceToHost, b->stream);
-      if (e != cudaSuccess) st = pe_cuda_fail(e, "pe_batch_get_solution");
-    }
-    cudaFreeAsync(tmp, b->stream);
+  double* rows[PE_MAX_D] = {nullptr, nullptr, nullptr};
+  for (int a = 0; a < B.g.d; ++a) rows[a] = b->rows + B.oMu + B.g.off[a];
+  const bool dev = pe_is_device_ptr(nodal_out);
+  double* out = dev ? nodal_out : b->scratch + b->ndof_max;
+  pe_status st = dst_rows_f64(B.g.d, n, rows, last, out, b->scratch, b->stream);
+  if (st == PE_OK && !dev) {
+    cudaError_t e = cudaMemcpyAsync(nodal_out, out, sizeof(double) * B.g.ndof, cudaMemcpyDeviceToHost, b->stream);
+    if (e != cudaSuccess) st = pe_cuda_fail(e, "pe_batch_get_solution");
   }
   cudaError_t e = cudaStreamSynchronize(b->stream);
   if (st == PE_OK && e != cudaSuccess) st = pe_cuda_fail(e, "pe_batch_get_solution");

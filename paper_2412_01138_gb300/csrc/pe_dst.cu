@@ -2249,6 +2249,11 @@ pe_status axis_factors_fused(pe_ctx* c, int R, const double* loads, double* fac,
   return PE_OK;
 }
 
+pe_status dst_rows_f64(int d, const int* n, double* const* rows, const double* in, double* out, double* tmp,
+                       cudaStream_t st) {
+  return dst_nd<double>(d, n, rows, in, out, tmp, st);
+}
+
 pe_status dst_nd_f64(pe_ctx* c, const double* in, double* out) {
   c->launches += c->gn.d;
   return dst_nd<double>(c->gn.d, c->gn.n, c->S, in, out, c->work1, c->stream, c->gn.per);

@@ -265,6 +265,9 @@ pe_status dst_axis_f64(const double* S, const double* in, double* out, int64_t o
 pe_status dst_axis_f32(const float* S, const float* in, float* out, int64_t outer, int n, int64_t inner,
                        cudaStream_t st, int periodic = 0);
 pe_status dst_nd_f64(pe_ctx* c, const double* in, double* out);
+// the tensor DST-I from the axes' sine rows, tmp: as many values again (in and out distinct)
+pe_status dst_rows_f64(int d, const int* n, double* const* rows, const double* in, double* out, double* tmp,
+                       cudaStream_t st);
 // float64 data transformed in float32 arithmetic through c->io32 (FFT-length axes only)
 bool dst_nd_f32_ok(const Geom& g);
 pe_status dst_nd_mixed(pe_ctx* c, const double* in, double* out);  // whole grid (c->gn); uses c->S, c->work1

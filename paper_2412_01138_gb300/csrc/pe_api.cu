@@ -129,12 +129,13 @@ void free_ctx(pe_ctx* c) {
   void* ptrs[] = {c->muM_axis, c->ratio_axis, c->S[0], c->S[1], c->S[2], c->S32[0], c->S32[1], c->S32[2],
                   c->gen_L, c->gen_X, c->axisM, c->lam, c->coefF, c->coefG,
                   c->coefF32, c->coefG32, c->U, c->Fbar, c->gG, c->work0, c->work1, c->out_nodal, c->partials,
-                  c->red, c->axisF, c->axisF32, c->axisU0, c->loads, c->tab64, c->tab32,
+                  c->axisF, c->axisF32, c->axisU0, c->loads, c->tab64, c->tab32,
                   c->Ktab, c->V64, c->G64, c->V32, c->G32, c->Fz, c->done_ctr, c->resp_nodes, c->resp,
                   c->muM_full, c->ratio_full, c->fac_full, c->work2, c->loopctl, c->loop_hist, c->io32, c->muM_inv};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->h_red) cudaFreeHost(c->h_red);
+  if (c->h_out) cudaFreeHost(c->h_out);
   if (c->h_loop) cudaFreeHost(c->h_loop);
   if (c->loop_exec) cudaGraphExecDestroy(c->loop_exec);
   if (c->setup_exec) cudaGraphExecDestroy(c->setup_exec);
@@ -146,6 +147,7 @@ void free_ctx(pe_ctx* c) {
   if (c->ev_join) cudaEventDestroy(c->ev_join);
   if (c->ev_tables) cudaEventDestroy(c->ev_tables);
   if (c->side) cudaStreamDestroy(c->side);
+  if (c->side2) cudaStreamDestroy(c->side2);
   delete c;
 }
 
@@ -352,7 +354,6 @@ extern "C" pe_status pe_setup(pe_ctx** out, int32_t d, const int32_t* n, const d
     st = dev_alloc(&c->io32, 3 * ndn + 64);
   if (st == PE_OK) st = dev_alloc(&c->out_nodal, ndn);
   if (st == PE_OK) st = dev_alloc(&c->partials, 2 * (size_t)c->max_blocks + 64);
-  if (st == PE_OK) st = dev_alloc(&c->red, 2);
   if (st == PE_OK) st = dev_alloc(&c->done_ctr, 1);
   if (st == PE_OK && cudaMemset(c->done_ctr, 0, sizeof(unsigned int)) != cudaSuccess)
     st = pe_fail(PE_ECUDA, "pe_setup: counter initialisation failed");
@@ -387,7 +388,9 @@ extern "C" pe_status pe_setup(pe_ctx** out, int32_t d, const int32_t* n, const d
     for (int a = 0; a < d && st == PE_OK && c->precision == PE_MIXED; ++a)
       st = dev_alloc(&c->S32[a], (size_t)n[a] * n[a]);
   }
-  if (st == PE_OK && cudaMallocHost((void**)&c->h_red, 4 * sizeof(double)) != cudaSuccess) {
+  if (st == PE_OK && (cudaHostAlloc((void**)&c->h_red, 2 * sizeof(double), cudaHostAllocMapped) != cudaSuccess ||
+                      cudaHostGetDevicePointer((void**)&c->red, c->h_red, 0) != cudaSuccess ||
+                      (ndn <= (size_t)kStageOut && cudaMallocHost((void**)&c->h_out, ndn * sizeof(double)) != cudaSuccess))) {
     cudaGetLastError();
     st = pe_fail(PE_ENOMEM, "pe_setup: pinned host allocation failed");
   }
@@ -402,10 +405,16 @@ extern "C" pe_status pe_setup(pe_ctx** out, int32_t d, const int32_t* n, const d
       cudaGetLastError();
       st = pe_fail(PE_ENOMEM, "pe_setup: mapped pinned host allocation failed");
     }
+    if (st == PE_OK) {
+      const LoopCtl L{0, c->max_iter, 0, (int)N, 0.0, 0.0, c->loop_hist, c->h_loop_dev};
+      if (cudaMemcpy(c->loopctl, &L, sizeof(L), cudaMemcpyHostToDevice) != cudaSuccess)
+        st = pe_cuda_fail(cudaGetLastError(), "pe_setup: loop state");
+    }
   }
   for (int i = 0; i < PE_NEV && st == PE_OK; ++i)
     if (cudaEventCreate(&c->ev[i]) != cudaSuccess) st = pe_cuda_fail(cudaGetLastError(), "cudaEventCreate");
   if (st == PE_OK && (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
+                      cudaStreamCreateWithFlags(&c->side2, cudaStreamNonBlocking) != cudaSuccess ||
                       cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
                       cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess ||
                       cudaEventCreateWithFlags(&c->ev_tables, cudaEventDisableTiming) != cudaSuccess))
@@ -481,18 +490,28 @@ static pe_status expand_dirichlet_terms(pe_ctx* c) {
 
 // out += sign * I_h g(t) in one of three forms: kind 1 the modal P_h of the interpolant,
 // kind 2 the modal V^T of its interior values, kind 3 its interior nodal values.
+struct Lift {
+  pe_term t[PE_MAX_TERMS];
+  signed char lk[PE_MAX_TERMS][PE_MAX_D];
+  int mode;
+};
+
+static Lift make_lift(const pe_ctx* c, double t, double sign, int kind) {
+  Lift L{};
+  for (int s = 0; s < c->nbd; ++s) {
+    L.t[s] = c->bterms[s];
+    L.t[s].amp = sign * c->bterms[s].amp * time_factor(c->bterms[s], t);
+    for (int a = 0; a < c->g.d; ++a) L.lk[s][a] = kind == 1 ? 1 : 3;
+  }
+  L.mode = kind == 1 ? 1 : (kind == 2 ? 2 : 0);
+  return L;
+}
+
 static pe_status add_lift(pe_ctx* c, double t, double sign, int kind, double* out) {
   if (c->nbd == 0) return PE_OK;
-  pe_term tt[PE_MAX_TERMS];
-  signed char lk[PE_MAX_TERMS][PE_MAX_D] = {};
-  for (int s = 0; s < c->nbd; ++s) {
-    tt[s] = c->bterms[s];
-    tt[s].amp = sign * c->bterms[s].amp * time_factor(c->bterms[s], t);
-    for (int a = 0; a < c->g.d; ++a) lk[s][a] = kind == 1 ? 1 : 3;
-  }
-  const int mode = kind == 1 ? 1 : (kind == 2 ? 2 : 0);
-  PE_TRY(launch_separable_factors(c, tt, c->nbd, c->axisU0, mode, lk));
-  return launch_outer_sum(c, c->axisU0, tt, c->nbd, out, 1);
+  const Lift L = make_lift(c, t, sign, kind);
+  PE_TRY(launch_separable_factors(c, L.t, c->nbd, c->axisU0, L.mode, L.lk));
+  return launch_outer_sum(c, c->axisU0, L.t, c->nbd, out, 1);
 }
 
 // The set-up and output graphs of a repeated problem (pe_options.device_loop = 2) hold the host
@@ -598,10 +617,10 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
     c->R = 1;
     memset(&c->terms[0], 0, sizeof(pe_term));
   }
-  // Two streams for grids large enough that their set-up kernels run side by side: the side
-  // stream makes the time tables, then the forward transform of nodal u0 (after its copy, for
-  // host u0); the main stream makes the per-axis forcing factors, waits for the time tables, makes
-  // the column weights, and waits for the side stream before the coarse sweep.
+  // Three streams for grids large enough that their set-up kernels run side by side: one makes the time
+  // tables, one the forward transform of nodal u0 (after its copy, for host u0); the main stream makes the
+  // per-axis forcing factors, waits for the time tables, makes the column weights, and waits for
+  // the transform before the coarse sweep.
   // (Small grids, whose kernels are launch-bound, keep everything on the main stream.)
   double* U0 = c->U;
   const bool fork_u0 = u0->kind == PE_FIELD_NODAL && u0->nodal != nullptr;
@@ -610,12 +629,13 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
   if (fork) {
     PE_CUDA_TRY(cudaEventRecord(c->ev_fork, c->stream));
     PE_CUDA_TRY(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
+    PE_CUDA_TRY(cudaStreamWaitEvent(c->side2, c->ev_fork, 0));
     cudaStream_t main_stream = c->stream;
     c->stream = c->side;
-    pe_status st = PE_OK;
-    st = launch_time_tables(c);
+    pe_status st = launch_time_tables(c);
     if (st == PE_OK && cudaEventRecord(c->ev_tables, c->side) != cudaSuccess)
       st = pe_cuda_fail(cudaGetLastError(), "pe_set_problem: event record");
+    c->stream = c->side2;
     if (st == PE_OK) {
       // device u0 is read in place by the transform; host u0 is copied in first
       const bool dev = c->u0_dev_hint >= 0 ? c->u0_dev_hint == 1 : pe_is_device_ptr(u0->nodal);
@@ -629,14 +649,30 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
       if (st == PE_OK) st = nodal_to_modal(c, src, U0);
     }
     c->stream = main_stream;
-    PE_TRY(st);
-    PE_CUDA_TRY(cudaEventRecord(c->ev_join, c->side));
+    // both streams are joined below whatever happened here
+    PE_CUDA_TRY(cudaEventRecord(c->ev_join, c->side2));
+    if (st != PE_OK) {
+      cudaStreamWaitEvent(c->stream, c->ev_join, 0);
+      return st;
+    }
   } else {
     PE_TRY(launch_time_tables(c));
   }
   // The phi/b coefficient tables depend only on lam, dt, dT and the nodes: pe_setup made them.
   // Forcing: per-axis modal factors, then the column weights.
-  PE_TRY(launch_separable_factors(c, c->terms, c->R, c->axisF, 1, c->lkind));
+  // the factors of separable u0, or of the initial lifting beside nodal u0, come along with them
+  const bool u0_terms = u0->kind == PE_FIELD_TERMS_SEPARABLE;
+  if (u0_terms) PE_TRY(pe_validate_terms(u0->n_terms, u0->terms, c->g.d, "u0"));
+  const bool lift_along = c->nbd > 0 && u0->kind == PE_FIELD_NODAL;
+  if (u0_terms) {
+    PE_TRY(launch_separable_factors_two(c, c->terms, c->R, c->axisF, c->lkind, u0->terms, u0->n_terms, c->axisU0, 1,
+                                        nullptr));
+  } else if (lift_along) {
+    const Lift L = make_lift(c, c->t0, -1.0, 2);
+    PE_TRY(launch_separable_factors_two(c, c->terms, c->R, c->axisF, c->lkind, L.t, c->nbd, c->axisU0, L.mode, L.lk));
+  } else {
+    PE_TRY(launch_separable_factors(c, c->terms, c->R, c->axisF, 1, c->lkind));
+  }
   if (general) PE_TRY(general_prepare(c));
   if (fork) PE_CUDA_TRY(cudaStreamWaitEvent(c->stream, c->ev_tables, 0));
   PE_TRY(launch_column_weights(c));
@@ -650,8 +686,7 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
     if (u0->n_terms == 0) {
       PE_CUDA_TRY(cudaMemsetAsync(U0, 0, sizeof(double) * c->g.ndof, c->stream));
     } else if (u0->kind == PE_FIELD_TERMS_SEPARABLE) {
-      PE_TRY(launch_separable_factors(c, u0->terms, u0->n_terms, c->axisU0, 1));
-      PE_TRY(launch_outer_sum(c, c->axisU0, u0->terms, u0->n_terms, U0, 0));
+      PE_TRY(launch_outer_sum(c, c->axisU0, u0->terms, u0->n_terms, U0, 0));  // factors made above
     } else {
       // nodal consistent load F = sum_t amp_t kron_a F_{t,a}, then c0 = Lambda_M^{-1} V^T F
       PE_TRY(launch_separable_factors(c, u0->terms, u0->n_terms, c->axisU0, 0));
@@ -670,9 +705,11 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
   }
   // Dirichlet lifting: w(t0) = P_h(u0 - I_h g(t0)) for descriptor data, u0 - I_h g(t0) for
   // nodal data (taken as already in V_h)
-  if (c->nbd > 0) {
-    const bool nodal = u0->kind == PE_FIELD_NODAL;
-    PE_TRY(add_lift(c, c->t0, -1.0, nodal ? 2 : 1, U0));
+  if (lift_along) {
+    const Lift L = make_lift(c, c->t0, -1.0, 2);
+    PE_TRY(launch_outer_sum(c, c->axisU0, L.t, c->nbd, U0, 1));  // factors made above
+  } else if (c->nbd > 0) {
+    PE_TRY(add_lift(c, c->t0, -1.0, 1, U0));
   }
   // k = 0: coarse sweep
   if (coarse) {
@@ -860,16 +897,16 @@ static pe_status build_loop_graph(pe_ctx* c) {
   return PE_OK;
 }
 
-// Iterations of pe_solve on the device, enqueued: a kernel arms the loop state, the graph runs
-// the loop, and the stop decision of every iteration also writes k, r and the non-finite flag
-// into the mapped pinned mirror that the host reads after the solve's wait (no copies).
+// Iterations of pe_solve on the device, enqueued: the graph runs the loop; the tolerance is read from
+// the mapped pinned mirror, into which the stop decision of every iteration also writes k, r and
+// the non-finite flag for the host to read after the solve's wait (no copies).
 static pe_status enqueue_loop_on_device(pe_ctx* c, double tol) {
   PE_TRY(build_loop_graph(c));
   volatile LoopCtl* h = c->h_loop;
   h->k = 0;
   h->nonfinite = 0;
   h->r = INFINITY;
-  PE_TRY(launch_loop_init(c, tol));
+  h->tol = tol;
   PE_CUDA_TRY(cudaGraphLaunch(c->loop_exec, c->stream));
   return PE_OK;
 }
@@ -1032,10 +1069,18 @@ static pe_status solve_begin(pe_ctx* c, const pe_field* u0, const pe_forcing* f,
   }
   PE_CUDA_TRY(cudaEventRecord(c->ev[4], c->stream));
   // the nodal solution into the caller's buffer in the same stream order
-  if (nodal_out)
-    PE_CUDA_TRY(cudaMemcpyAsync(nodal_out, c->out_nodal, sizeof(double) * c->gn.ndof,
-                                pe_is_device_ptr(nodal_out) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                                c->stream));
+  c->stage_to = nullptr;
+  if (nodal_out) {
+    // a small result for pageable host memory goes by the context's pinned buffer and is handed over by
+    // the wait (the runtime would stage it in a blocking copy of its own)
+    cudaPointerAttributes attr;
+    const bool known = cudaPointerGetAttributes(&attr, nodal_out) == cudaSuccess;
+    if (!known) cudaGetLastError();
+    const bool dev = known && (attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged);
+    if (c->h_out && (!known || attr.type == cudaMemoryTypeUnregistered)) c->stage_to = nodal_out;
+    PE_CUDA_TRY(cudaMemcpyAsync(c->stage_to ? c->h_out : nodal_out, c->out_nodal, sizeof(double) * c->gn.ndof,
+                                dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
+  }
   c->pend = true;
   c->pend_on_device = on_device;
   c->pend_tol = tol;
@@ -1048,6 +1093,8 @@ static pe_status solve_end(pe_ctx* c, pe_result* res) {
   if (!c->pend) return pe_fail(PE_ESTATE, "pe_solve_wait: no solve pending");
   c->pend = false;
   PE_CUDA_TRY(cudaStreamSynchronize(c->stream));
+  if (c->stage_to) memcpy(c->stage_to, c->h_out, sizeof(double) * c->gn.ndof);
+  c->stage_to = nullptr;
   double r = c->pend_r;
   if (c->pend_on_device) {
     PE_TRY(finish_loop_on_device(c, res, &r));

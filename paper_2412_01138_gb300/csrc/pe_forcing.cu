@@ -381,13 +381,18 @@ __global__ void __launch_bounds__(256) loads_1d_kernel(TermsDev T, Geom g, doubl
 // sum in a fixed order.  The float64 work (n FMAs per output) spreads over every SM, where a
 // half-length FFT per pencil pair runs one chain of dependent float64 latencies on a few SMs.
 constexpr int kFactorLanes = 32;
+// where the factors of one list of R terms go (muInv: 1 / mu^M, or null for none)
+struct FactorOut {
+  int R;
+  double* fac;
+  float* fac32;
+  const double* muInv;
+};
 __global__ void __launch_bounds__(256) axis_factor_matrix_kernel(Geom g, int R, const double* __restrict__ S0,
                                                                  const double* __restrict__ S1,
                                                                  const double* __restrict__ S2,
                                                                  const double* __restrict__ loads,
-                                                                 const double* __restrict__ muInv,
-                                                                 double* __restrict__ fac, float* __restrict__ fac32,
-                                                                 int64_t total) {
+                                                                 FactorOut A, FactorOut B, int64_t total) {
   pdl_wait();
   const int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kFactorLanes;
   const int sub = threadIdx.x & (kFactorLanes - 1);
@@ -406,9 +411,13 @@ __global__ void __launch_bounds__(256) axis_factor_matrix_kernel(Geom g, int R, 
 #pragma unroll
   for (int o = kFactorLanes / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
   if (sub == 0) {
-    const double v = muInv ? acc * muInv[g.off[a] + j] : acc;
-    fac[e] = v;
-    if (fac32) fac32[e] = (float)v;
+    // terms r < A.R belong to the first list, the others to the second
+    const bool second = r >= A.R;
+    const FactorOut& F = second ? B : A;
+    const int64_t o = (int64_t)F.R * g.off[a] + (int64_t)(second ? r - A.R : r) * n + j;
+    const double v = F.muInv ? acc * F.muInv[g.off[a] + j] : acc;
+    F.fac[o] = v;
+    if (F.fac32) F.fac32[o] = (float)v;
   }
 }
 
@@ -425,7 +434,10 @@ __global__ void divide_axis_mu_kernel(Geom g, int R, const double* __restrict__ 
 }
 
 // out[J] = sum_r w_r prod_a fac[R*off[a] + r*n_a + j_a]
-__global__ void outer_sum_kernel(Geom g, int R, const double* __restrict__ fac, const double* __restrict__ w,
+struct TermWeights {
+  double w[PE_MAX_TERMS];
+};
+__global__ void outer_sum_kernel(Geom g, int R, const double* __restrict__ fac, TermWeights W,
                                  double* __restrict__ out, int accumulate) {
   pdl_wait();
   const int64_t J = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -437,7 +449,7 @@ __global__ void outer_sum_kernel(Geom g, int R, const double* __restrict__ fac, 
     double P = fac[(int64_t)R * g.off[0] + (int64_t)r * g.n[0] + j[0]];
 #pragma unroll
     for (int a = 1; a < PE_MAX_D; ++a) if (a < g.d) P *= fac[(int64_t)R * g.off[a] + (int64_t)r * g.n[a] + j[a]];
-    acc += w[r] * P;
+    acc += W.w[r] * P;
   }
   out[J] = accumulate ? out[J] + acc : acc;
 }
@@ -451,17 +463,6 @@ __global__ void scale_mu_kernel(Geom g, const double* __restrict__ muM, double* 
 #pragma unroll
   for (int a = 1; a < PE_MAX_D; ++a) if (a < g.d) mu *= muM[g.off[a] + j[a]];
   x[J] = inverse ? x[J] / mu : x[J] * mu;
-}
-
-__global__ void weights_at_time_kernel(TermsDev T, double t, double* w) {
-  const int r = threadIdx.x;
-  if (r < T.n) w[r] = T.t[r].amp * eval_time(T.t[r], t);
-}
-
-__global__ void amps_kernel(TermsDev T, double* w) {
-  pdl_wait();
-  const int r = threadIdx.x;
-  if (r < T.n) w[r] = T.t[r].amp;
 }
 
 }  // namespace
@@ -723,37 +724,70 @@ pe_status launch_separable_factors(pe_ctx* c, const pe_term* terms, int nterms, 
   return compact_axis_tables(c, nterms, c->fac_full, axis_out, f32 ? c->axisF32 : nullptr);
 }
 
-static pe_status separable_factors_whole(pe_ctx* c, const pe_term* terms, int nterms, double* axis_out, int mode,
-                                         const signed char (*lk)[PE_MAX_D]) {
-  if (nterms == 0) return PE_OK;
-  TermsDev T = pack_terms(terms, nterms, lk);
-  Gauss G = make_gauss(c->quad_pts);
-  int nmax = 1;
-  for (int a = 0; a < c->g.d; ++a) nmax = c->g.n[a] > nmax ? c->g.n[a] : nmax;
-  dim3 grid((nmax + 127) / 128, nterms, c->g.d);
-  dim3 lgrid((nmax + 31) / 32, nterms, c->g.d);  // 32 nodes of eight lanes per CTA
-  double* loads = mode == 0 ? axis_out : c->loads;
-  PE_CUDA_TRY(launch_pdl(loads_1d_kernel, lgrid, dim3(32 * kLoadLanes), 0, c->stream, T, c->g, c->lo[0], c->lo[1],
-                         c->lo[2], c->h[0], c->h[1], c->h[2], G, loads));
-  c->launches += 1;
-  PE_CUDA_TRY(cudaGetLastError());
-  if (mode == 0) return PE_OK;
-  const bool f32 = (axis_out == c->axisF) && c->precision == PE_MIXED;
+static bool matrix_factors(const pe_ctx* c, int nterms) {
   // the matrix form over every SM while its float64 work stays small (R sum_a n_a^2 <= 8M FMAs)
   int64_t work = 0;
   for (int a = 0; a < c->g.d; ++a) work += (int64_t)nterms * c->g.n[a] * c->g.n[a];
-  if (c->muM_inv && work <= ((int64_t)8 << 20)) {
-    const int64_t total = (int64_t)nterms * (c->g.off[c->g.d - 1] + c->g.n[c->g.d - 1]);
-    const unsigned blocks = (unsigned)((total * kFactorLanes + 255) / 256);
-    PE_CUDA_TRY(launch_pdl(axis_factor_matrix_kernel, dim3(blocks), dim3(256), 0, c->stream, c->g, nterms,
-                           (const double*)c->S[0], (const double*)(c->g.d > 1 ? c->S[1] : c->S[0]),
-                           (const double*)(c->g.d > 2 ? c->S[2] : c->S[0]), (const double*)loads,
-                           (const double*)(mode == 1 ? c->muM_inv : nullptr), axis_out,
-                           mode == 1 && f32 ? c->axisF32 : (float*)nullptr, total));
-    c->launches += 1;
-    PE_CUDA_TRY(cudaGetLastError());
-    return PE_OK;
+  return c->muM_inv && work <= ((int64_t)8 << 20);
+}
+
+// 1D loads of the terms, then their factors in matrix form into A (and B)
+static pe_status loads_of(pe_ctx* c, const TermsDev& T, double* loads) {
+  const Gauss G = make_gauss(c->quad_pts);
+  int nmax = 1;
+  for (int a = 0; a < c->g.d; ++a) nmax = c->g.n[a] > nmax ? c->g.n[a] : nmax;
+  dim3 lgrid((nmax + 31) / 32, T.n, c->g.d);  // 32 nodes of eight lanes per CTA
+  PE_CUDA_TRY(launch_pdl(loads_1d_kernel, lgrid, dim3(32 * kLoadLanes), 0, c->stream, T, c->g, c->lo[0], c->lo[1],
+                         c->lo[2], c->h[0], c->h[1], c->h[2], G, loads));
+  c->launches += 1;
+  return PE_OK;
+}
+
+static pe_status factors_of(pe_ctx* c, const FactorOut& A, const FactorOut& B) {
+  const int nterms = A.R + B.R;
+  const int64_t total = (int64_t)nterms * (c->g.off[c->g.d - 1] + c->g.n[c->g.d - 1]);
+  const unsigned blocks = (unsigned)((total * kFactorLanes + 255) / 256);
+  PE_CUDA_TRY(launch_pdl(axis_factor_matrix_kernel, dim3(blocks), dim3(256), 0, c->stream, c->g, nterms,
+                         (const double*)c->S[0], (const double*)(c->g.d > 1 ? c->S[1] : c->S[0]),
+                         (const double*)(c->g.d > 2 ? c->S[2] : c->S[0]), (const double*)c->loads, A, B, total));
+  c->launches += 1;
+  return PE_OK;
+}
+
+static FactorOut factor_out(const pe_ctx* c, int R, double* out, int mode) {
+  return FactorOut{R, out, mode == 1 && out == c->axisF && c->precision == PE_MIXED ? c->axisF32 : nullptr,
+                   mode == 1 ? c->muM_inv : nullptr};
+}
+
+pe_status launch_separable_factors_two(pe_ctx* c, const pe_term* ta, int na, double* axis_a,
+                                       const signed char (*lka)[PE_MAX_D], const pe_term* tb, int nb, double* axis_b,
+                                       int mode_b, const signed char (*lkb)[PE_MAX_D]) {
+  if (na == 0 || nb == 0 || na + nb > PE_MAX_TERMS || c->sharded || mode_b == 0 || !matrix_factors(c, na + nb)) {
+    PE_TRY(launch_separable_factors(c, ta, na, axis_a, 1, lka));
+    return launch_separable_factors(c, tb, nb, axis_b, mode_b, lkb);
   }
+  TermsDev T = pack_terms(ta, na, lka);
+  const TermsDev U = pack_terms(tb, nb, lkb);
+  for (int i = 0; i < nb; ++i) {
+    T.t[na + i] = U.t[i];
+    for (int a = 0; a < PE_MAX_D; ++a) T.lk[na + i][a] = U.lk[i][a];
+  }
+  T.n = na + nb;
+  PE_TRY(loads_of(c, T, c->loads));
+  return factors_of(c, factor_out(c, na, axis_a, 1), factor_out(c, nb, axis_b, mode_b));
+}
+
+static pe_status separable_factors_whole(pe_ctx* c, const pe_term* terms, int nterms, double* axis_out, int mode,
+                                         const signed char (*lk)[PE_MAX_D]) {
+  if (nterms == 0) return PE_OK;
+  int nmax = 1;
+  for (int a = 0; a < c->g.d; ++a) nmax = c->g.n[a] > nmax ? c->g.n[a] : nmax;
+  dim3 grid((nmax + 127) / 128, nterms, c->g.d);
+  double* loads = mode == 0 ? axis_out : c->loads;
+  PE_TRY(loads_of(c, pack_terms(terms, nterms, lk), loads));
+  if (mode == 0) return PE_OK;
+  const bool f32 = (axis_out == c->axisF) && c->precision == PE_MIXED;
+  if (matrix_factors(c, nterms)) return factors_of(c, factor_out(c, nterms, axis_out, mode), FactorOut{});
   if (mode == 1) {
     bool done = false;
     PE_TRY(axis_factors_fused(c, nterms, loads, axis_out, f32 ? c->axisF32 : nullptr, &done));
@@ -772,31 +806,30 @@ static pe_status separable_factors_whole(pe_ctx* c, const pe_term* terms, int nt
   return PE_OK;
 }
 
+static pe_status outer_sum(pe_ctx* c, const double* fac, int R, const TermWeights& W, double* out, int accumulate) {
+  const int threads = 256;
+  PE_CUDA_TRY(launch_pdl(outer_sum_kernel, dim3((unsigned)((c->g.ndof + threads - 1) / threads)), dim3(threads), 0,
+                         c->stream, c->g, R, fac, W, out, accumulate));
+  c->launches += 1;
+  return PE_OK;
+}
+
 // out[J] = sum_r amp_r prod_a fac_{r,a}[j_a] (nodal_loads: fac are 1D loads, out a nodal load vector)
 pe_status launch_outer_sum(pe_ctx* c, const double* axis_fac, const pe_term* terms, int nterms, double* out,
                            int accumulate) {
   if (nterms == 0) return PE_OK;
-  double* w = c->partials;  // at least PE_MAX_TERMS doubles
-  TermsDev T = pack_terms(terms, nterms);
-  PE_CUDA_TRY(launch_pdl(amps_kernel, dim3(1), dim3(PE_MAX_TERMS), 0, c->stream, T, w));
-  const int threads = 256;
-  PE_CUDA_TRY(launch_pdl(outer_sum_kernel, dim3((unsigned)((c->g.ndof + threads - 1) / threads)), dim3(threads), 0,
-                         c->stream, c->g, nterms, axis_fac, (const double*)w, out, accumulate));
-  c->launches += 2;
-  PE_CUDA_TRY(cudaGetLastError());
-  return PE_OK;
+  TermWeights W{};
+  for (int r = 0; r < nterms; ++r) W.w[r] = terms[r].amp;
+  return outer_sum(c, axis_fac, nterms, W, out, accumulate);
 }
 
 pe_status launch_forcing_modal(pe_ctx* c, double t, double* out) {
-  double* w = c->partials;
-  TermsDev T = pack_terms(c->terms, c->R);
-  weights_at_time_kernel<<<1, PE_MAX_TERMS, 0, c->stream>>>(T, t, w);
-  const int threads = 256;
-  outer_sum_kernel<<<(unsigned)((c->g.ndof + threads - 1) / threads), threads, 0, c->stream>>>(c->g, c->R,
-                                                                                               c->axisF, w, out, 0);
-  c->launches += 2;
-  PE_CUDA_TRY(cudaGetLastError());
-  return PE_OK;
+  TermWeights W{};
+  for (int r = 0; r < c->R; ++r) {
+    const pe_term& T = c->terms[r];
+    W.w[r] = T.amp * (T.tkind == PE_T_SIN ? sin(T.tp[0] * t + T.tp[1]) : exp(T.tp[0] * t));
+  }
+  return outer_sum(c, c->axisF, c->R, W, out, 0);
 }
 
 pe_status launch_scale_by_muM(pe_ctx* c, double* x, int inverse) {

@@ -93,7 +93,7 @@ struct LoopCtl {
   int k, max_iter, nonfinite, hist_cap;
   double tol, r;
   double* hist;   // [hist_cap] residuals r_1 .. r_k (device)
-  LoopCtl* host;  // device address of the mapped pinned mirror that receives k, r, nonfinite
+  LoopCtl* host;  // device address of the mapped pinned mirror that gives tol and receives k, r, nonfinite
 };
 
 struct pe_ctx {
@@ -150,11 +150,15 @@ struct pe_ctx {
   double* muM_inv = nullptr;    // [nsum of the whole grid] 1 / mu^M per axis node
   double* out_nodal = nullptr;  // [gn.ndof] inverse DST of U^N after pe_solve
   double* partials = nullptr;   // [2 * max_blocks]
-  double* red = nullptr;        // [2] device
+  double* red = nullptr;        // [2] residual sums: device address of h_red
   unsigned int* done_ctr = nullptr;  // correction: CTAs finished (0 between launches)
-  cudaStream_t side = nullptr;  // second stream: the nodal u0 transform beside the forcing tables
+  // set-up of larger grids on three streams: the time tables on side, the nodal u0 transform on side2,
+  // the forcing factors on the main stream
+  cudaStream_t side = nullptr, side2 = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_tables = nullptr;
-  double* h_red = nullptr;      // [2] pinned host
+  double* h_red = nullptr;      // [2] mapped pinned host
+  double* h_out = nullptr;      // [kStageOut] pinned: small nodal results on their way to pageable memory
+  double* stage_to = nullptr;   // where pe_solve_wait copies them (null: no staged result)
   int max_blocks = 0;
   int sms = 0;                      // SMs of the context's device
   // forcing (set by pe_set_problem)
@@ -245,6 +249,7 @@ pe_status build_dst_matrix(int n, double* S, cudaStream_t st, int periodic = 0);
 pe_status build_dst_matrix_f32(int n, float* S, cudaStream_t st, int periodic = 0);
 
 // pe_forcing.cu
+constexpr int kStageOut = 8192;  // doubles
 constexpr int64_t kRespMinDof = 16384;
 pe_status setup_response_nodes(pe_ctx* c);  // at pe_setup
 pe_status launch_time_tables(pe_ctx* c);   // also sets c->K and c->cols; the response table after them
@@ -254,6 +259,11 @@ pe_status launch_column_weights_f64(pe_ctx* c);  // V64, if not yet made for thi
 pe_status compact_axis_tables(pe_ctx* c, int R, const double* in, double* out, float* out32);
 pe_status launch_separable_factors(pe_ctx* c, const pe_term* terms, int nterms, double* axis_out, int mode,
                                    const signed char (*lk)[PE_MAX_D] = nullptr);
+// Factors of two lists of terms, the second into axis_b in `mode_b`, by one set of launches where they fit
+// one (as two calls otherwise).
+pe_status launch_separable_factors_two(pe_ctx* c, const pe_term* ta, int na, double* axis_a,
+                                       const signed char (*lka)[PE_MAX_D], const pe_term* tb, int nb, double* axis_b,
+                                       int mode_b, const signed char (*lkb)[PE_MAX_D]);
 pe_status launch_outer_sum(pe_ctx* c, const double* axis_fac, const pe_term* terms, int nterms, double* out,
                            int accumulate);
 pe_status launch_forcing_modal(pe_ctx* c, double t, double* out);
@@ -287,8 +297,6 @@ pe_status launch_iteration(pe_ctx* c, int precision, bool first, LoopCtl* loop, 
 pe_status launch_forced_f64(pe_ctx* c, double* f, double* gG);
 bool first_fused(const pe_ctx* c);  // pe_solve makes the coarse iterate in the first iteration's pass
 pe_status read_sums(pe_ctx* c, double* num, double* den, cudaEvent_t after);  // waits for the stream
-// Arms the device-resident loop's state for one solve (k = 0, tol, the history, the mirror).
-pe_status launch_loop_init(pe_ctx* c, double tol);
 pe_status launch_scale_by_muM(pe_ctx* c, double* x, int inverse);
 
 // pe_general.cu: the moving terms of the general path (no-ops without any)

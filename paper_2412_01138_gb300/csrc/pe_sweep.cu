@@ -26,14 +26,12 @@ namespace {
 // Stopping decision of a device-resident loop, run by one thread after the residual sums are
 // complete: r_k appended to the history, k advanced, and the graph's while condition set to
 // continue while r > tol and k < max_iter (a non-finite sum stops the loop and is flagged).
-__device__ void loop_decide(LoopCtl* L, unsigned long long handle, double num, double den) {
+__device__ void loop_decide(LoopCtl* L, unsigned long long handle, double num, double den, bool first, double tol) {
   const bool finite = isfinite(num) && isfinite(den);
   const double r = den > 0.0 ? sqrt(num) / sqrt(den) : sqrt(num);
-  const int k = L->k;
+  const int k = first ? 0 : L->k;
   if (k < L->hist_cap) L->hist[k] = r;
   L->k = k + 1;
-  L->r = r;
-  if (!finite) L->nonfinite = 1;
   // the host reads k, r and the flag from its mapped mirror after the solve's one wait
   volatile LoopCtl* H = L->host;
   H->k = k + 1;
@@ -41,22 +39,7 @@ __device__ void loop_decide(LoopCtl* L, unsigned long long handle, double num, d
   if (!finite) H->nonfinite = 1;
   __threadfence_system();
   cudaGraphSetConditional((cudaGraphConditionalHandle)handle,
-                          (finite && r > L->tol && k + 1 < L->max_iter) ? 1u : 0u);
-}
-
-__global__ void loop_init_kernel(LoopCtl* L, int max_iter, int hist_cap, double tol, double* hist,
-                                 LoopCtl* host) {
-  pdl_wait();
-  if (threadIdx.x == 0) {
-    L->k = 0;
-    L->max_iter = max_iter;
-    L->nonfinite = 0;
-    L->hist_cap = hist_cap;
-    L->tol = tol;
-    L->r = INFINITY;
-    L->hist = hist;
-    L->host = host;
-  }
+                          (finite && r > tol && k + 1 < L->max_iter) ? 1u : 0u);
 }
 
 // The walk: one thread per mode, the slices in order.  MODE kCoarse makes the coarse iterate, MODE
@@ -89,9 +72,10 @@ struct WalkArgs {
   const double *f, *gG;     // SRC = 0: forced parts [N][ndof]
   const double *EG, *EM;    // e^{-lam dT} of the coarse step, e^{-lam M dt}
   const double* muM_axis;
-  double *U, *partials, *red;
+  double *U, *partials, *red;  // red: mapped host memory
   unsigned int* done;
   LoopCtl* loop;
+  const LoopCtl* loop_host;    // its mapped mirror, whose tol the host sets before every solve
   unsigned long long handle;
 };
 
@@ -119,6 +103,9 @@ __global__ void __launch_bounds__(walk_cap(SRC, KB, MODE)) walk_kernel(WalkArgs 
     }
   }
   double E = 0.0, EM = 0.0, o = 0.0, d = 0.0, sd = 0.0, su = 0.0, w = 0.0;
+  // the tolerance of this solve, fetched now so that the last CTA's decision does not wait for it
+  double tol = 0.0;
+  if (MODE != kCoarse && a.loop && threadIdx.x == 0) tol = reinterpret_cast<const volatile LoopCtl*>(a.loop_host)->tol;
   double* U = a.U + J;
   if (on) {
     E = a.EG[J];
@@ -218,10 +205,10 @@ __global__ void __launch_bounds__(walk_cap(SRC, KB, MODE)) walk_kernel(WalkArgs 
       td = block_sum(td, sh);
       tu = block_sum(tu, sh);
       if (threadIdx.x == 0) {
-        a.red[0] = td;
-        a.red[1] = tu;
+        reinterpret_cast<volatile double*>(a.red)[0] = td;
+        reinterpret_cast<volatile double*>(a.red)[1] = tu;
         *a.done = 0u;
-        if (a.loop) loop_decide(a.loop, a.handle, td, tu);
+        if (a.loop) loop_decide(a.loop, a.handle, td, tu, MODE == kFirst, tol);
       }
     }
   }
@@ -318,6 +305,7 @@ WalkArgs walk_args(pe_ctx* c, LoopCtl* loop, unsigned long long handle) {
   a.red = c->red;
   a.done = c->done_ctr;
   a.loop = loop;
+  a.loop_host = c->h_loop_dev;
   a.handle = handle;
   return a;
 }
@@ -380,16 +368,9 @@ pe_status launch_iteration(pe_ctx* c, int precision, bool first, LoopCtl* loop, 
 
 pe_status read_sums(pe_ctx* c, double* num, double* den, cudaEvent_t after) {
   if (after) PE_CUDA_TRY(cudaEventRecord(after, c->stream));
-  PE_CUDA_TRY(cudaMemcpyAsync(c->h_red, c->red, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   PE_CUDA_TRY(cudaStreamSynchronize(c->stream));
-  *num = c->h_red[0];
-  *den = c->h_red[1];
-  return PE_OK;
-}
-
-pe_status launch_loop_init(pe_ctx* c, double tol) {
-  PE_CUDA_TRY(launch_pdl(loop_init_kernel, dim3(1), dim3(32), 0, c->stream, c->loopctl, c->max_iter, c->N, tol,
-                         c->loop_hist, c->h_loop_dev));
-  c->launches += 1;
+  const volatile double* h = c->h_red;  // the walk's last CTA wrote the sums here
+  *num = h[0];
+  *den = h[1];
   return PE_OK;
 }

@@ -1374,110 +1374,132 @@ __global__ void __launch_bounds__(32 * W) dst512_strided_kernel(const TI* __rest
 }
 
 // Two passes at L = 1024 points (n = 511), strided pencils: radix 32 over the 32 groups of a
-// pair (a whole warp, the mirrored half of the extension from lane 32 - j), one exchange through
-// shared memory, radix 32 again, of whose outputs X[j + 32 r] the DST needs r < 16.  A CTA of W
-// warps owns blocks of 4 W consecutive pencils staged as above (511 rows, double buffered); a warp runs its two pencil pairs one after the other through one pair buffer and
-// keeps their outputs in registers until every warp is done with the stage.
+// pair (a whole warp; the mirrored half of the extension is read from the stage as well), one exchange
+// through shared memory, radix 32 again, of whose outputs X[j + 32 r] the DST needs r < 16.  A CTA of W
+// warps owns blocks of 2 W consecutive pencils, a pair per warp, staged as above (511 rows, double
+// buffered).
+//
+// Bound by issue and latency: per block of 32 pencils the transforms issue 6800 cycles per scheduler, the
+// shared-memory accesses take as many, and the block took 17600, because all warps of the one CTA an SM
+// holds are in the same phase.  So the exchange goes through a buffer of single floats, real parts first
+// (half the bytes of a complex buffer, the same number of bank cycles), and the second pass' twiddles
+// are read from a table in shared memory instead of 62 registers per lane: 16 warps per SM, not 8.  The
+// 4-byte asynchronous copies (rows of odd grids have no wider alignment) cost about ten cycles of
+// the load pipe each; a quarter of them goes out before and after each transform, where the
+// arithmetic of the other warps hides them.  511 x 511 x 255, both strided passes: 2 x 252 us with 8
+// warps and complex buffers, 2 x 245 with 16, 2 x 231 with direct mirrored reads, 2 x 215 with the
+// copies spread out (floor at 6.8 TB/s: 78 each).
+__device__ __forceinline__ int fpad5(int i) { return i + (i >> 5); }  // conflict-free for strides 1 and 32
+
 template <int W>
-__global__ void __launch_bounds__(32 * W) dst1024_strided_kernel(const float* __restrict__ in,
-                                                                 float* __restrict__ out, int64_t inner,
-                                                                 int64_t npencils, float scale,
-                                                                 const Cplx<float>* __restrict__ tw2) {
-  constexpr int L = 1024, n = 511, PS = L + L / 16 + 1, P = 4 * W, SP = P + 2;
-  pdl_wait();
+constexpr size_t strided1024_smem() {
+  return sizeof(float) * (2 * 511 * (2 * W + 2) + (size_t)W * 1056) + sizeof(Cplx<float>) * 992;
+}
+
+template <int W>
+__global__ void __launch_bounds__(32 * W, W <= 4 ? 3 : 1) dst1024_strided_kernel(const float* __restrict__ in,
+                                                                                 float* __restrict__ out, int64_t inner,
+                                                                                 int64_t npencils, float scale,
+                                                                                 const Cplx<float>* __restrict__ tw2) {
+  constexpr int n = 511, PS = 1056, P = 2 * W, SP = P + 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  float* stage[2] = {reinterpret_cast<float*>(smem_raw), reinterpret_cast<float*>(smem_raw) + n * SP};
-  Cplx<float>* a = reinterpret_cast<Cplx<float>*>(stage[1] + n * SP) + (size_t)warp * PS;
-  __shared__ int64_t offs[2][P];
+  Cplx<float>* stw = reinterpret_cast<Cplx<float>*>(smem_raw);
+  float* const stage = reinterpret_cast<float*>(stw + 992);
+  float* a = stage + 2 * n * SP + warp * PS;
   const int64_t nblk = (npencils + P - 1) / P;
-  const int src = (32 - lane) & 31;
-  // this lane's pass-2 twiddles e^{-2 pi i lane r / 1024}, the same for every pair and block
-  Cplx<float> tw[32];
-#pragma unroll
-  for (int r = 1; r < 32; ++r) tw[r] = ldg_cplx(tw2 + 32 * r + lane);
+  // pass-2 twiddles e^{-2 pi i j r / 1024}, r >= 1, at 32 (r - 1) + j (a table of the process)
+  for (int e = tid; e < 992; e += 32 * W) stw[e] = ldg_cplx(tw2 + 32 + e);
+  pdl_wait();
   const int pl = tid & (P - 1), row0 = tid / P;
-  constexpr int RSTEP = 32 * W / P;
-  auto issue = [&](int64_t blk, int b) {
-    if (tid < P) {
-      const int64_t p = blk * P + tid;
-      offs[b][tid] = p < npencils ? (p / inner) * (int64_t)n * inner + (p % inner) : -1;
+  constexpr int RSTEP = 32 * W / P, kParts = 4, PROWS = 512 / kParts;
+  // where this thread's pencil of a block starts, -1 past the end
+  auto locate = [&](int64_t blk) -> int64_t {
+    const int64_t p = blk * P + pl;
+    if (p >= npencils) return -1;
+    const int64_t q = npencils <= 0x7fffffff ? (int64_t)((uint32_t)p / (uint32_t)inner) : p / inner;
+    return q * ((n - 1) * inner) + p;
+  };
+  // part i of kParts of a block's rows, into stage b
+  auto issue = [&](int64_t o, int b, int part) {
+    float* dst = stage + b * (n * SP) + (row0 + part * PROWS) * SP + pl;
+    const float* srcp = in + o + (int64_t)(row0 + part * PROWS) * inner;
+    const int64_t step = (int64_t)RSTEP * inner;
+#pragma unroll 4
+    for (int jj = row0 + part * PROWS; jj < min(n, (part + 1) * PROWS); jj += RSTEP, dst += RSTEP * SP, srcp += step) {
+      if (o >= 0)
+        cp_async_elem(dst, srcp);
+      else
+        *dst = 0.f;
     }
-    __syncthreads();
-    const int64_t o = offs[b][pl];
-    float* dst = stage[b] + row0 * SP + pl;
-    if (o >= 0) {
-      const float* srcp = in + o + (int64_t)row0 * inner;
-      const int64_t step = (int64_t)RSTEP * inner;
-      for (int jj = row0; jj < n; jj += RSTEP, dst += RSTEP * SP, srcp += step) cp_async_elem(dst, srcp);
-    } else {
-      for (int jj = row0; jj < n; jj += RSTEP, dst += RSTEP * SP) *dst = 0.f;
-    }
-    cp_async_commit();
   };
   int cur = 0;
-  if ((int64_t)blockIdx.x < nblk) issue(blockIdx.x, 0);
+  int64_t o_cur = (int64_t)blockIdx.x < nblk ? locate(blockIdx.x) : -1;
+  if ((int64_t)blockIdx.x < nblk) {
+#pragma unroll 1
+    for (int part = 0; part < kParts; ++part) issue(o_cur, 0, part);
+  }
   for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x, cur ^= 1) {
+    cp_async_commit();
     cp_async_wait_all();
     __syncthreads();
-    const int64_t next = blk + gridDim.x;
-    if (next < nblk) issue(next, cur ^ 1);
-    float* st = stage[cur];
-    // a warp reads and writes only its own four columns of the stage: the DST values of a pair
-    // go back into the columns its inputs came from as soon as they are ready
-#pragma unroll 1
-    for (int p = 0; p < 2; ++p) {
-      const int col = 4 * warp + 2 * p;
-      Cplx<float> v[32];
+    const bool more = blk + gridDim.x < nblk;
+    const int64_t o_next = more ? locate(blk + gridDim.x) : -1;
+    float* st = stage + cur * (n * SP);
+    // a warp reads and writes only its own two columns of the stage: the DST values of the pair go
+    // back into the columns its inputs came from
+    const int col = 2 * warp;
+    Cplx<float> v[32];
 #pragma unroll
-      for (int r = 0; r < 16; ++r) {
-        const int m = lane + 32 * r;
-        if (m >= 1) {
-          const float2 z = *reinterpret_cast<const float2*>(st + (m - 1) * SP + col);
-          v[r] = Cplx<float>{z.x, z.y};
-        } else {
-          v[r] = Cplx<float>{0.f, 0.f};
-        }
+    for (int r = 0; r < 16; ++r) {
+      const int m = lane + 32 * r;
+      if (m >= 1) {
+        const float2 z = *reinterpret_cast<const float2*>(st + (m - 1) * SP + col);
+        v[r] = Cplx<float>{z.x, z.y};
+      } else {
+        v[r] = Cplx<float>{0.f, 0.f};
       }
+    }
 #pragma unroll
-      for (int r = 16; r < 32; ++r) {
-        // 1024 - m = 32 (31 - r) + (32 - j) for j >= 1; 32 (32 - r) for j = 0 (lane 0's own row)
-        float re = __shfl_sync(0xffffffffu, v[31 - r].re, src);
-        float im = __shfl_sync(0xffffffffu, v[31 - r].im, src);
-        if (lane == 0) {
-          re = r == 16 ? 0.f : v[32 - r].re;
-          im = r == 16 ? 0.f : v[32 - r].im;
-        }
-        v[r] = Cplx<float>{-re, -im};
-      }
-      dft_regs<float, 32>(v);
-      __syncwarp();  // the previous pair's reads of the pair buffer are done
+    for (int r = 16; r < 32; ++r) {  // the mirrored half, x[1024 - m] = -x[m]
+      const int m = 1024 - lane - 32 * r;
+      const float2 z = *reinterpret_cast<const float2*>(st + (min(m, n) - 1) * SP + col);
+      v[r] = Cplx<float>{m <= n ? -z.x : 0.f, m <= n ? -z.y : 0.f};
+    }
+    if (more) issue(o_next, cur ^ 1, 0);
+    dft_regs<float, 32>(v);
+    if (more) issue(o_next, cur ^ 1, 1);
+    __syncwarp();  // the previous block's reads of the exchange buffer are done
 #pragma unroll
-      for (int r = 0; r < 32; ++r) a[fpad(32 * lane + r)] = v[brevc(r, 5)];
-      __syncwarp();
+    for (int r = 0; r < 32; ++r) a[fpad5(32 * lane + r)] = v[brevc(r, 5)].re;
+    __syncwarp();
 #pragma unroll
-      for (int r = 0; r < 32; ++r) v[r] = a[fpad(lane + 32 * r)];
+    for (int r = 0; r < 32; ++r) v[r].re = a[fpad5(lane + 32 * r)];
+    __syncwarp();
 #pragma unroll
-      for (int r = 1; r < 32; ++r) v[r] = cmul(v[r], tw[r]);
-      dft_regs<float, 32>(v);
+    for (int r = 0; r < 32; ++r) a[fpad5(32 * lane + r)] = v[brevc(r, 5)].im;
+    __syncwarp();
 #pragma unroll
-      for (int r = 0; r < 16; ++r) {
-        const int m = lane + 32 * r;
-        const Cplx<float> X = v[brevc(r, 5)];
-        if (m >= 1) *reinterpret_cast<float2*>(st + (m - 1) * SP + col) = make_float2(-X.im * scale, X.re * scale);
-      }
+    for (int r = 0; r < 32; ++r) v[r].im = a[fpad5(lane + 32 * r)];
+#pragma unroll
+    for (int r = 1; r < 32; ++r) v[r] = cmul(v[r], stw[32 * (r - 1) + lane]);
+    if (more) issue(o_next, cur ^ 1, 2);
+    dft_regs<float, 32>(v);
+    if (more) issue(o_next, cur ^ 1, 3);
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      const int m = lane + 32 * r;
+      const Cplx<float> X = v[brevc(r, 5)];
+      if (m >= 1) *reinterpret_cast<float2*>(st + (m - 1) * SP + col) = make_float2(-X.im * scale, X.re * scale);
     }
     __syncthreads();
-    const float* ost = st;
-    {
-      const int64_t o = offs[cur][pl];
-      if (o >= 0) {
-        float* dstp = out + o + (int64_t)row0 * inner;
-        const float* sp = ost + row0 * SP + pl;
-        const int64_t step = (int64_t)RSTEP * inner;
-        for (int k = row0; k < n; k += RSTEP, sp += RSTEP * SP, dstp += step) *dstp = *sp;
-      }
+    if (o_cur >= 0) {
+      float* dstp = out + o_cur + (int64_t)row0 * inner;
+      const float* sp = st + row0 * SP + pl;
+      const int64_t step = (int64_t)RSTEP * inner;
+      for (int r = row0; r < n; r += RSTEP, sp += RSTEP * SP, dstp += step) *dstp = *sp;
     }
+    o_cur = o_next;
   }
   cp_async_wait_all();
 }
@@ -1948,13 +1970,13 @@ pe_status fft512_strided_launch(const TI* in, TO* out, int64_t inner, int64_t np
 }
 
 // the two-pass float32 kernel: strided pencils of n = 511 (L = 1024)
-pe_status fft1024_strided_launch(const float* in, float* out, int64_t inner, int64_t npencils, float scale,
-                                 cudaStream_t st) {
-  constexpr int PS = 1024 + 1024 / 16 + 1, W = kStridedWarps, P = 4 * W;
-  const size_t smem = sizeof(float) * 2 * 511 * (P + 2) + sizeof(Cplx<float>) * PS * W;
+template <int W>
+pe_status fft1024_strided_w(const float* in, float* out, int64_t inner, int64_t npencils, float scale,
+                            cudaStream_t st) {
+  constexpr size_t smem = strided1024_smem<W>();
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [smem] {
+  std::call_once(once, [] {
     attr = cudaFuncSetAttribute(dst1024_strided_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   });
   if (attr != cudaSuccess) return pe_cuda_fail(attr, "dst: shared-memory attribute");
@@ -1965,12 +1987,21 @@ pe_status fft1024_strided_launch(const float* in, float* out, int64_t inner, int
   PE_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   PE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, dst1024_strided_kernel<W>, 32 * W, smem));
   if (per_sm < 1) return pe_fail(PE_ECUDA, "dst: the 1024-point strided kernel does not fit an SM");
-  const int64_t nblk = (npencils + P - 1) / P;
+  const int64_t nblk = (npencils + 2 * W - 1) / (2 * W);
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(nblk, (int64_t)sms * per_sm));
   PE_CUDA_TRY(launch_pdl(dst1024_strided_kernel<W>, dim3((unsigned)grid), dim3(32 * W), smem, st, in, out, inner,
                          npencils, scale, tw2));
-  PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;
+}
+
+// Blocks of 32 pencils (128-byte rows); of eight, three CTAs per SM, up to the one wave of blocks that
+// makes of the 152 SMs, where more SMs at work count for more than long rows (961 pencils: 24.7
+// against 28.2 us with the two short axes, 511: 14.5 against 16.6; 8001: 72.3 against 71.9; 130305 per
+// pass: 310 against 215).
+pe_status fft1024_strided_launch(const float* in, float* out, int64_t inner, int64_t npencils, float scale,
+                                 cudaStream_t st) {
+  if (npencils <= 152 * 3 * 8) return fft1024_strided_w<4>(in, out, inner, npencils, scale, st);
+  return fft1024_strided_w<16>(in, out, inner, npencils, scale, st);
 }
 
 template <typename T>

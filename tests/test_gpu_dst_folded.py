@@ -74,3 +74,23 @@ def test_few_float64_pencils(env, m, pencils, strided):
     if pencils > 1:  # the other axis in the matrix form
         bound += (pencils / 2 + 3) * 2.0 ** -53 * math.sqrt(pencils)
     assert err <= bound, (err, bound)
+
+
+@pytest.mark.parametrize("n", [(511, 305), (511, 3648), (511, 3649), (2, 511, 3500)],
+                         ids=["511x305", "511x3648", "511x3649", "2x511x3500"])
+def test_strided_511_float32(env, n):
+    """The two-pass kernel of 511 strided float32 values: in its blocks of 8 pencils, at the last and the first count
+    of the two block sizes, with ragged tails and several blocks to a CTA, and with blocks that cross a plane.
+    Ten butterfly stages: 10 sqrt(10) u relative, and the other axes in the matrix form."""
+    pe, torch = env
+    x = np.random.default_rng(sum(n)).standard_normal(n).astype(np.float32)
+    d = torch.tensor(x.reshape(-1), device="cuda")
+    out = torch.empty_like(d)
+    pe.dst(len(n), n, d, out, f32=True)
+    pe.dst(len(n), n, d, d, f32=True)
+    ref = _dense(x.astype(np.float64))
+    u = 2.0 ** -24
+    bound = 10 * math.sqrt(10) * u + sum((v / 2 + 3) * u * math.sqrt(v) for v in n if v != 511)
+    for got in (out, d):
+        err = np.linalg.norm(got.cpu().numpy().astype(np.float64).reshape(n) - ref) / np.linalg.norm(ref)
+        assert err <= bound, (err, bound)

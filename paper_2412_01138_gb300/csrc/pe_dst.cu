@@ -896,13 +896,12 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && LOGL <= 9) ? 2 : 1) ds
   // strided pencils: blocks of P consecutive pencils, each row j one contiguous run of P
   // values; the next block's rows are staged (cp.async) while this block is transformed
   const int64_t nblk = (npencils + P - 1) / P;
-  int64_t* offs[2] = {off, off + P};
   T* stage = reinterpret_cast<T*>(off + 2 * P);
   int cur = 0;
   if ((int64_t)blockIdx.x < nblk) {
-    block_offsets(blockIdx.x, P, n, inner, npencils, offs[0]);
+    block_offsets(blockIdx.x, P, n, inner, npencils, off);
     __syncthreads();
-    stage_block_async(in, offs[0], P, logP, n, inner, stage);
+    stage_block_async(in, off, P, logP, n, inner, stage);
   }
   for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x, cur ^= 1) {
     cp_async_wait_all();
@@ -922,9 +921,9 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && LOGL <= 9) ? 2 : 1) ds
     __syncthreads();
     const int64_t next = blk + gridDim.x;
     if (next < nblk) {
-      block_offsets(next, P, n, inner, npencils, offs[cur ^ 1]);
+      block_offsets(next, P, n, inner, npencils, off + (cur ^ 1) * P);
       __syncthreads();
-      stage_block_async(in, offs[cur ^ 1], P, logP, n, inner, stage);
+      stage_block_async(in, off + (cur ^ 1) * P, P, logP, n, inner, stage);
     }
     StockhamPasses<T, LOGL, LOGL, 1>::run(bufs + (size_t)warp * PS, ptw, lane);
     __syncthreads();
@@ -933,7 +932,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && LOGL <= 9) ? 2 : 1) ds
       const int pl = e & (P - 1), k = e >> logP;
       const Cplx<T> Z = bufs[(size_t)(pl >> 1) * PS + fpad(k + 1)];
       const T val = (pl & 1) ? Z.re * scale : -Z.im * scale;
-      const int64_t o = offs[cur][pl];
+      const int64_t o = off[cur * P + pl];
       if (o >= 0) out[o + (int64_t)k * inner] = val;
     }
   }
@@ -1130,13 +1129,12 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && LOGN <= 9) ? 2 : 1)
   }
   // strided pencils: as in dst_fft_warp_kernel, the next block is staged while this one runs
   const int64_t nblk = (npencils + P - 1) / P;
-  int64_t* offs[2] = {off, off + P};
   T* stage = reinterpret_cast<T*>(off + 2 * P);
   int cur = 0;
   if ((int64_t)blockIdx.x < nblk) {
-    block_offsets(blockIdx.x, P, n, inner, npencils, offs[0]);
+    block_offsets(blockIdx.x, P, n, inner, npencils, off);
     __syncthreads();
-    stage_block_async(in, offs[0], P, logP, n, inner, stage);
+    stage_block_async(in, off, P, logP, n, inner, stage);
   }
   for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x, cur ^= 1) {
     cp_async_wait_all();
@@ -1149,9 +1147,9 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && LOGN <= 9) ? 2 : 1)
     __syncthreads();
     const int64_t next = blk + gridDim.x;
     if (next < nblk) {
-      block_offsets(next, P, n, inner, npencils, offs[cur ^ 1]);
+      block_offsets(next, P, n, inner, npencils, off + (cur ^ 1) * P);
       __syncthreads();
-      stage_block_async(in, offs[cur ^ 1], P, logP, n, inner, stage);
+      stage_block_async(in, off + (cur ^ 1) * P, P, logP, n, inner, stage);
     }
     if constexpr (DHT) dht_pair<T, LOGN>(a, ptw, lane);
     else half_dst_pair<T, LOGN>(a, ptw, fold, lane);
@@ -1159,7 +1157,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4 && LOGN <= 9) ? 2 : 1)
     for (int e = tid; e < P * n; e += B) {
       const int pl = e & (P - 1), k = e >> logP;
       const Cplx<T> F = bufs[(size_t)(pl >> 1) * PS + fpad(k + SH)];
-      const int64_t o = offs[cur][pl];
+      const int64_t o = off[cur * P + pl];
       if (o >= 0) out[o + (int64_t)k * inner] = ((pl & 1) ? F.im : F.re) * scale;
     }
   }
@@ -1261,8 +1259,8 @@ __global__ void __launch_bounds__(32 * W) dst512_strided_kernel(const TI* __rest
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int h = lane >> 4, j = lane & 15;
-  float* stage[2] = {reinterpret_cast<float*>(smem_raw), reinterpret_cast<float*>(smem_raw) + n * SP};
-  Cplx<float>* buf = reinterpret_cast<Cplx<float>*>(stage[1] + n * SP) + (size_t)warp * 2 * PS;
+  float* const stage = reinterpret_cast<float*>(smem_raw);
+  Cplx<float>* buf = reinterpret_cast<Cplx<float>*>(stage + 2 * n * SP) + (size_t)warp * 2 * PS;
   __shared__ int64_t offs[2][P];
   const int64_t nblk = (npencils + P - 1) / P;
   const int src = ((16 - j) & 15) | (h << 4);
@@ -1280,7 +1278,7 @@ __global__ void __launch_bounds__(32 * W) dst512_strided_kernel(const TI* __rest
     }
     __syncthreads();
     const int64_t o = offs[b][pl];
-    float* dst = stage[b] + row0 * SP + pl;
+    float* dst = stage + b * (n * SP) + row0 * SP + pl;
     if (o >= 0) {
       const TI* srcp = in + o + (int64_t)row0 * inner;
       const int64_t step = (int64_t)RSTEP * inner;
@@ -1308,7 +1306,7 @@ __global__ void __launch_bounds__(32 * W) dst512_strided_kernel(const TI* __rest
     __syncthreads();
     const int64_t next = blk + gridDim.x;
     if (next < nblk) issue(next, cur ^ 1);
-    const float* st = stage[cur];
+    const float* st = stage + cur * (n * SP);
     // pass 1 on this warp's pencil pair h: columns 4 warp + 2 h, + 1 of the stage rows
     const int col = 4 * warp + 2 * h;
     Cplx<float> v[32];
@@ -1339,7 +1337,7 @@ __global__ void __launch_bounds__(32 * W) dst512_strided_kernel(const TI* __rest
     // a warp reads and writes only its own four columns of the stage, so its DST values go back
     // into them once its own lanes are done (the pair buffers are per warp too)
     __syncwarp();
-    float* ost = stage[cur];
+    float* ost = stage + cur * (n * SP);
 #pragma unroll 1
     for (int p = 0; p < 2; ++p) {
       const Cplx<float>* b = buf + p * PS;
@@ -1625,13 +1623,12 @@ __global__ void __launch_bounds__(kTeamThreads) dst_fft_team_kernel(const T* __r
   // strided pencils: blocks of P consecutive pencils staged row by row (cp.async), the next block
   // staged while this one is transformed
   const int64_t nblk = (npencils + P - 1) / P;
-  int64_t* offs[2] = {off, off + P};
   T* stage = reinterpret_cast<T*>(off + 2 * P);
   int cur = 0;
   if ((int64_t)blockIdx.x < nblk) {
-    block_offsets(blockIdx.x, P, n, inner, npencils, offs[0]);
+    block_offsets(blockIdx.x, P, n, inner, npencils, off);
     __syncthreads();
-    stage_block_async(in, offs[0], P, logP, n, inner, stage);
+    stage_block_async(in, off, P, logP, n, inner, stage);
   }
   for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x, cur ^= 1) {
     cp_async_wait_all();
@@ -1650,9 +1647,9 @@ __global__ void __launch_bounds__(kTeamThreads) dst_fft_team_kernel(const T* __r
     __syncthreads();
     const int64_t next = blk + gridDim.x;
     if (next < nblk) {
-      block_offsets(next, P, n, inner, npencils, offs[cur ^ 1]);
+      block_offsets(next, P, n, inner, npencils, off + (cur ^ 1) * P);
       __syncthreads();
-      stage_block_async(in, offs[cur ^ 1], P, logP, n, inner, stage);
+      stage_block_async(in, off + (cur ^ 1) * P, P, logP, n, inner, stage);
     }
     TeamPasses<T, LOGL, LOGL, 1, TS>::run(a, ptw, tl, bar);
     __syncthreads();
@@ -1660,7 +1657,7 @@ __global__ void __launch_bounds__(kTeamThreads) dst_fft_team_kernel(const T* __r
       const int pl = e & (P - 1), k = e >> logP;
       const Cplx<T> Z = bufs[(size_t)(pl >> 1) * PS + fpad(k + 1)];
       const T val = (pl & 1) ? Z.re * scale : -Z.im * scale;
-      const int64_t o = offs[cur][pl];
+      const int64_t o = off[cur * P + pl];
       if (o >= 0) out[o + (int64_t)k * inner] = val;
     }
   }

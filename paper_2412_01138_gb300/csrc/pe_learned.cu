@@ -104,6 +104,10 @@ __global__ void samples_kernel(int n, const double* __restrict__ lam, const doub
 //      adds their G partials in a fixed order (deterministic), then applies Adam (or, for a
 //      gradient evaluation, writes the gradient);
 //   4. grid barrier (the next step reads the updated parameters).
+// A step is a chain of trips to L2, not work (4096 samples are one round of 27 per CTA): so a thread issues all
+// its parameter loads, and all its partial-gradient loads, before it uses the first, the barriers arrive
+// with a release and poll with an acquire instead of two full fences, and the Adam scalars are made
+// while the parameters travel: 13.3 to 11.8 us a step of 4096 samples on 152 SMs.
 // Barriers are bounded waits: on expiry the CTA records an error and returns (every other
 // CTA then expires at its next wait); the host reports PE_ETIMEOUT.
 // ---------------------------------------------------------------------------
@@ -113,6 +117,8 @@ constexpr int TR_ROUND = 32;            // samples per CTA per round: the M of t
 constexpr int AP = H + 4;               // padded row stride of W2 and the activations in shared memory
 constexpr int NPARAM_L = NPARAM + 1;    // the gradient slots plus one slot for the loss
 constexpr int NSIMT = NPARAM_L - H * H;  // slots summed on the CUDA cores: all but W2
+constexpr int NOTHER = NPARAM - H * H;  // the parameters but W2
+static_assert(2 * 4 * TR_THREADS == H * H && OW2 % 4 == 0, "two float4 of W2 per thread");
 static_assert(NSIMT <= TR_THREADS, "one CUDA-core gradient slot per thread");
 static_assert(TR_WARPS == 16 && TR_ROUND == 32 && H == 64, "MMA tile assignment below");
 constexpr long long kGridWaitCycles = 2000000000LL;  // about a second
@@ -148,17 +154,20 @@ __device__ bool grid_barrier(const TrainArgs& a, unsigned target, int* s_ok) {
   __syncthreads();
   if (threadIdx.x == 0) {
     int ok = 1;
-    __threadfence();
-    atomicAdd(a.bar_count, 1u);
+    unsigned* count = (unsigned*)__cvta_generic_to_global(a.bar_count);
+    // release: what this CTA's threads wrote before the __syncthreads above; acquire: what the others wrote
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
     const long long t0 = clock64();
-    while (*(volatile unsigned*)a.bar_count < target) {
-      if (*(volatile int*)a.err || clock64() - t0 > kGridWaitCycles) {
+    for (;;) {
+      unsigned seen;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
+      if (seen >= target) break;
+      if (clock64() - t0 > kGridWaitCycles || *(volatile int*)a.err) {
         atomicExch(a.err, 1);
         ok = 0;
         break;
       }
     }
-    __threadfence();
     *s_ok = ok;
   }
   __syncthreads();
@@ -240,10 +249,12 @@ __global__ void __launch_bounds__(TR_THREADS) train_kernel(TrainArgs a) {
     if (tid < TR_ROUND) {
       const bool live = tid < cnt;
       const int smp = r0 + tid;
-      S.X[tid][0] = live ? a.x[2 * smp] : 0.f;
-      S.X[tid][1] = live ? a.x[2 * smp + 1] : 0.f;
-      S.TG[tid][0] = live ? a.t[2 * smp] : 0.f;
-      S.TG[tid][1] = live ? a.t[2 * smp + 1] : 0.f;
+      const float x0 = live ? a.x[2 * smp] : 0.f, x1 = live ? a.x[2 * smp + 1] : 0.f;
+      const float t0 = live ? a.t[2 * smp] : 0.f, t1 = live ? a.t[2 * smp + 1] : 0.f;
+      S.X[tid][0] = x0;
+      S.X[tid][1] = x1;
+      S.TG[tid][0] = t0;
+      S.TG[tid][1] = t1;
     }
   };
   for (int s = 0; s < a.nsteps; ++s) {
@@ -255,18 +266,30 @@ __global__ void __launch_bounds__(TR_THREADS) train_kernel(TrainArgs a) {
     // this CTA's samples of the batch
     const int s0 = off + (int)((int64_t)c * nb / G), s1 = off + (int)((int64_t)(c + 1) * nb / G);
     // 1. the first round's samples and the parameters into shared memory (parameters from L2:
-    //    other CTAs updated them in the last step)
-    load_round(s0, min(TR_ROUND, s1 - s0));
-    for (int i = tid; i < 2 * H; i += TR_THREADS) {
-      S.W1[i] = __ldcg(a.params + OW1 + i);
-      S.W3[i] = __ldcg(a.params + OW3 + i);
+    //    other CTAs updated them in the last step), every load of a thread before its first store
+    {
+      const float4* w2 = reinterpret_cast<const float4*>(a.params + OW2);
+      const float4 wa = __ldcg(w2 + tid), wb = __ldcg(w2 + TR_THREADS + tid);
+      float other = 0.f;
+      if (tid < NOTHER) other = __ldcg(a.params + (tid < OW2 ? tid : tid + H * H));
+      load_round(s0, min(TR_ROUND, s1 - s0));
+      const int i0 = 4 * tid, i1 = 4 * (TR_THREADS + tid);
+      *reinterpret_cast<float4*>(S.W2 + (i0 >> 6) * AP + (i0 & (H - 1))) = wa;
+      *reinterpret_cast<float4*>(S.W2 + (i1 >> 6) * AP + (i1 & (H - 1))) = wb;
+      if (tid < NOTHER) {
+        const int k = tid < OW2 ? tid : tid + H * H;
+        if (k < OB1) S.W1[k - OW1] = other;
+        else if (k < OW2) S.b1[k - OB1] = other;
+        else if (k < OW3) S.b2[k - OB2] = other;
+        else if (k < OB3) S.W3[k - OW3] = other;
+        else S.b3[k - OB3] = other;
+      }
     }
-    for (int i = tid; i < H; i += TR_THREADS) {
-      S.b1[i] = __ldcg(a.params + OB1 + i);
-      S.b2[i] = __ldcg(a.params + OB2 + i);
-    }
-    for (int i = tid; i < H * H; i += TR_THREADS) S.W2[(i >> 6) * AP + (i & (H - 1))] = __ldcg(a.params + OW2 + i);
-    if (tid < 2) S.b3[tid] = __ldcg(a.params + OB3 + tid);
+    // the step's Adam scalars, ready before the first barrier
+    const long long step = a.adam_step0 + s + 1;
+    const float bc1 = 1.f - powf(a.b1, (float)step), bc2 = 1.f - powf(a.b2, (float)step);
+    const float cosv = 0.5f * (1.f + cospif((float)it / (float)a.total));
+    const float lr_t = a.lr * (0.01f + 0.99f * cosv);
     __syncthreads();
     float gw[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};  // dW2 tiles of this warp
     float gs = 0.f;                                                 // CUDA-core slot ks
@@ -382,10 +405,6 @@ __global__ void __launch_bounds__(TR_THREADS) train_kernel(TrainArgs a) {
     // 3. this CTA's parameters: lane l of warp w adds the partials of parameter kb + l of the
     //    CTAs w, w + 16, ...; warp 0 adds the 16 warp sums in warp order, then Adam (or the
     //    gradient out)
-    const long long step = a.adam_step0 + s + 1;
-    const float bc1 = 1.f - powf(a.b1, (float)step), bc2 = 1.f - powf(a.b2, (float)step);
-    const float cosv = 0.5f * (1.f + cospif((float)it / (float)a.total));
-    const float lr_t = a.lr * (0.01f + 0.99f * cosv);
     auto apply = [&](int k, float g) {
       if (!adam) {
         a.grad_out[k] = g;
@@ -405,8 +424,18 @@ __global__ void __launch_bounds__(TR_THREADS) train_kernel(TrainArgs a) {
       const int k = kb + lane;
       float g = 0.f;
       if (k < k1) {
-#pragma unroll 4
-        for (int cc = warp; cc < G; cc += TR_WARPS) g += __ldcg(a.partial + (int64_t)cc * NPARAM_L + k);
+        // (ten rows at a time, all of them in flight: one trip to L2 for 152 CTAs)
+        for (int c0 = warp; c0 < G; c0 += 10 * TR_WARPS) {
+          float v[10];
+#pragma unroll
+          for (int u = 0; u < 10; ++u) {
+            const int cc = c0 + u * TR_WARPS;
+            v[u] = cc < G ? __ldcg(a.partial + (int64_t)cc * NPARAM_L + k) : 0.f;
+          }
+#pragma unroll
+          for (int u = 0; u < 10; ++u)
+            if (c0 + u * TR_WARPS < G) g += v[u];
+        }
       }
       wsum[warp * 32 + lane] = g;
       __syncthreads();

@@ -13,9 +13,10 @@
 //    pencils transform the full odd extension with one warp per
 //    pencil pair (dst_fft_warp_kernel); both run self-sorting radix-4..32 passes.
 //    Pencils with n + 1 < 16 use a block-wide radix-2 kernel (dst_fft_kernel).
-//  * any other n, and many short float64 pencils (takes_folded): the matrix form, folded by its symmetry to half the multiplications
-//    (folded_dst_kernel).  A periodic axis without an FFT form keeps the plain product with its
-//    Hartley matrix (strided_gemm_kernel).
+//  * any other n, and many short float64 pencils (takes_folded): the matrix form, folded by its
+//    symmetry to half the multiplications (folded_dst_kernel); up to eight pencils, in sums shared by
+//    the lanes of a warp (few_matrix_kernel).  A periodic axis without an FFT form keeps the plain
+//    product with its Hartley matrix (strided_gemm_kernel, few_matrix_kernel).
 #include <algorithm>
 #include <mutex>
 
@@ -2104,6 +2105,144 @@ pe_status fft_axis(const T* in, T* out, int64_t outer, int n, int64_t inner, int
   return PE_OK;
 }
 
+// ---------------------------------------------------------------------------
+// Matrix form for few pencils (a line; its sources' factors): a warp makes KO outputs of up to NP pencils,
+// its lanes a share of the sum each.  The tiles above compute 32 pencils or columns whether there
+// are that many or not.
+// FOLD: m is the sine row, kept in shared memory with the zeros of sin 0 and sin pi at its ends; the even
+// outputs sum S x over x_j + x_{n-1-j}, the odd ones over the differences, j < (n + 1) / 2.  Bound by the
+// float64 pipe: n^2 / 2 multiply-adds a pencil, half as many additions for the fold.
+// Else m is a symmetric n x n matrix (Hartley), of which a warp streams KO rows: bound by reading
+// it (n = 7353 float64: 433 MB, 64 us at 6.8 TB/s), and by the float64 pipe.
+// One pencil of 7353, folded: float64 2094 to 180 us, float32 209 to 35; of 300: 28 to 14 and 14 to 10.
+constexpr int kFewKO = 4;
+
+template <typename T, int NP, bool FOLD>
+__global__ void __launch_bounds__(256) few_matrix_kernel(const T* __restrict__ m, const T* __restrict__ in,
+                                                         T* __restrict__ out, int n, int64_t inner, int np) {
+  constexpr int KO = kFewKO;
+  extern __shared__ __align__(16) unsigned char few_smem[];
+  T* row = reinterpret_cast<T*>(few_smem);  // row[q] = sqrt(2/(n+1)) sin(pi q/(n+1)), q = 0..n+1
+  const int tid = threadIdx.x, lane = tid & 31;
+  if constexpr (FOLD) {
+    for (int q = tid; q < n + 2; q += 256) row[q] = q >= 1 && q <= n ? m[q - 1] : T(0);
+    __syncthreads();
+  }
+  const int k0 = (blockIdx.x * 8 + (tid >> 5)) * KO, p0 = blockIdx.y * NP;
+  if (k0 >= n) return;
+  const T* x[NP];
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    const int64_t c = min(p0 + p, np - 1);
+    x[p] = in + (c / inner) * n * inner + c % inner;
+  }
+  T acc[KO][NP];
+#pragma unroll
+  for (int o = 0; o < KO; ++o)
+#pragma unroll
+    for (int p = 0; p < NP; ++p) acc[o][p] = T(0);
+  if constexpr (FOLD) {
+    const int h = (n + 1) / 2;
+    const unsigned half = (unsigned)n + 1u, period = 2u * half;
+    unsigned q[KO], step[KO];  // (j+1)(k+1) mod 2(n+1) and its advance over 32 indices
+#pragma unroll
+    for (int o = 0; o < KO; ++o) {
+      const unsigned kk = (unsigned)(k0 + o + 1) % period;
+      q[o] = (unsigned)(lane + 1) * kk % period;
+      step[o] = 32u * kk % period;
+    }
+    for (int j = lane; j < h; j += 32) {
+      T sum[NP], dif[NP];
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const T a = x[p][(int64_t)j * inner];
+        const bool mid = 2 * j == n - 1;  // its own mirror: it enters the even outputs alone
+        const T b = mid ? T(0) : x[p][(int64_t)(n - 1 - j) * inner];
+        sum[p] = a + b;
+        dif[p] = mid ? T(0) : a - b;
+      }
+#pragma unroll
+      for (int o = 0; o < KO; ++o) {  // k0 is even
+        const bool neg = q[o] > half;
+        const T e = row[neg ? q[o] - half : q[o]], v = neg ? -e : e;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) acc[o][p] = fma(v, (o & 1) ? dif[p] : sum[p], acc[o][p]);
+        q[o] += step[o];
+        if (q[o] >= period) q[o] -= period;
+      }
+    }
+  } else {
+    const T* r[KO];
+#pragma unroll
+    for (int o = 0; o < KO; ++o) r[o] = m + (int64_t)min(k0 + o, n - 1) * n;
+#pragma unroll 4
+    for (int j = lane; j < n; j += 32) {
+      T v[KO];
+#pragma unroll
+      for (int o = 0; o < KO; ++o) v[o] = __ldg(r[o] + j);
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const T a = x[p][(int64_t)j * inner];
+#pragma unroll
+        for (int o = 0; o < KO; ++o) acc[o][p] = fma(v[o], a, acc[o][p]);
+      }
+    }
+  }
+  // the KO NP sums over the lanes: halving steps leave lane l with value l mod KO NP (one addition
+  // per value instead of five), plain ones add what is left
+  constexpr int NV = KO * NP;
+  T v[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) v[i] = acc[i / NP][i % NP];
+#pragma unroll
+  for (int w = NV / 2; w > 0; w >>= 1) {
+    const bool up = lane & w;
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      const T give = up ? v[i] : v[i + w], keep = up ? v[i + w] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, w);
+    }
+  }
+#pragma unroll
+  for (int w = NV; w < 32; w <<= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], w);
+  const int o = lane / NP, p = lane % NP;
+  if (lane < NV && k0 + o < n && p0 + p < np) {
+    const int64_t c = p0 + p;
+    out[(c / inner) * n * inner + c % inner + (int64_t)(k0 + o) * inner] = v[0];
+  }
+}
+
+template <typename T, int NP, bool FOLD>
+pe_status few_matrix_launch(const T* m, const T* in, T* out, int n, int64_t inner, int np, cudaStream_t st) {
+  const size_t smem = FOLD ? sizeof(T) * (size_t)(n + 2) : 0;
+  if constexpr (FOLD) {
+    static std::once_flag once;
+    static cudaError_t attr = cudaSuccess;
+    std::call_once(once, [] {
+      attr = cudaFuncSetAttribute(few_matrix_kernel<T, NP, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(T) * (16384 + 2));
+    });
+    if (attr != cudaSuccess) return pe_cuda_fail(attr, "dst: shared-memory attribute");
+  }
+  const dim3 grid((unsigned)((n + 8 * kFewKO - 1) / (8 * kFewKO)), (unsigned)((np + NP - 1) / NP));
+  few_matrix_kernel<T, NP, FOLD><<<grid, 256, smem, st>>>(m, in, out, n, inner, np);
+  PE_CUDA_TRY(cudaGetLastError());
+  return PE_OK;
+}
+
+// Where the kernel above is ahead of the tiles: its sums over the lanes and its bookkeeping cost an output about as
+// much as 64 indices of the sum, for every pencil (float64, the other axis included: 4 x 100, 25.3 against
+// 27.4 us; 8 x 300, 41.9 against 40.4; 8 x 700, 63 against 67; 16 x 7353 float32, 508 against 264).
+inline bool few_matrix_takes(int n, int64_t np) { return n <= 16384 && (np <= 2 || (np <= 8 && n >= 64 * np)); }
+
+template <typename T, bool FOLD>
+pe_status few_matrix_axis(const T* m, const T* in, T* out, int n, int64_t inner, int np, cudaStream_t st) {
+  if (np == 1) return few_matrix_launch<T, 1, FOLD>(m, in, out, n, inner, np, st);
+  if (np == 2) return few_matrix_launch<T, 2, FOLD>(m, in, out, n, inner, np, st);
+  if (np <= 4) return few_matrix_launch<T, 4, FOLD>(m, in, out, n, inner, np, st);
+  return few_matrix_launch<T, 8, FOLD>(m, in, out, n, inner, np, st);
+}
+
 // Whether a Dirichlet axis takes the folded matrix form (and so needs its sine row): without an FFT form
 // always; in float64 also up to n = 63 for more pencils than the block-wide FFT serves, where n/2 + 1
 // multiplications per value cost less than the FFT of the short odd extension (255 x 255 x n: 460 us
@@ -2119,12 +2258,17 @@ template <typename T>
 pe_status dst_axis(const T* S, const T* in, T* out, int64_t outer, int n, int64_t inner, cudaStream_t st,
                    int periodic = 0) {
   int logL = 0;
-  if (!periodic && takes_folded<T>(n, outer * inner)) return folded_axis<T>(S, in, out, outer, n, inner, st);
+  const int64_t np = outer * inner;
+  if (!periodic && takes_folded<T>(n, np)) {
+    if (few_matrix_takes(n, np)) return few_matrix_axis<T, true>(S, in, out, n, inner, (int)np, st);
+    return folded_axis<T>(S, in, out, outer, n, inner, st);
+  }
   if (!periodic && fft_size_ok(n, &logL)) return fft_axis<T>(in, out, outer, n, inner, logL, st);
   if (periodic) {
     bool done = false;
     PE_TRY(dht_fft_axis<T>(in, out, outer, n, inner, st, &done));
     if (done) return PE_OK;
+    if (few_matrix_takes(n, np)) return few_matrix_axis<T, false>(S, in, out, n, inner, (int)np, st);
   }
   // Hartley matrix: large tiles when they still give >= 2 CTAs per SM, else small ones
   const int64_t rows = inner == 1 ? outer : n;

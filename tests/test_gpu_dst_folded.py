@@ -94,3 +94,41 @@ def test_strided_511_float32(env, n):
     for got in (out, d):
         err = np.linalg.norm(got.cpu().numpy().astype(np.float64).reshape(n) - ref) / np.linalg.norm(ref)
         assert err <= bound, (err, bound)
+
+
+@pytest.mark.parametrize("m", [2, 5, 36, 301, 1030])
+@pytest.mark.parametrize("pencils", [1, 2, 3, 7, 8, 9])
+@pytest.mark.parametrize("strided", [False, True], ids=["contiguous", "strided"])
+@pytest.mark.parametrize("f32", [False, True], ids=["float64", "float32"])
+def test_few_pencils_in_the_matrix_form(env, m, pencils, strided, f32):
+    """A warp's share of every sum, at both parities of the length, fewer outputs than a warp makes, every group size,
+    a ragged last group and the first count that goes to the tiles at any length.  Sums of n/2 products and a tree, as above."""
+    pe, torch = env
+    n = (m,) if pencils == 1 else ((m, pencils) if strided else (pencils, m))
+    x = np.random.default_rng(m + pencils).standard_normal(n)
+    x = x.astype(np.float32) if f32 else x
+    d = torch.tensor(x.reshape(-1), device="cuda")
+    pe.dst(len(n), n, d, d, f32=f32)
+    ref = _dense(x.astype(np.float64))
+    u = 2.0 ** (-24 if f32 else -53)
+    bound = sum((v / 2 + 3) * u * math.sqrt(v) for v in n)
+    err = np.linalg.norm(d.cpu().numpy().astype(np.float64).reshape(n) - ref) / np.linalg.norm(ref)
+    assert err <= bound, (err, bound)
+
+
+@pytest.mark.parametrize("n,periodic", [((517,), (True,)), ((517, 8), (True, False)), ((45, 2), (True, True))],
+                         ids=["517", "517x8", "45x2"])
+def test_few_periodic_pencils(env, n, periodic):
+    """A periodic line and thin grids whose Hartley transforms have few pencils, against the oracle at the
+    periodic tests' bounds."""
+    from oracle import solver as osolver
+    from test_gpu_periodic import _problem, _rel
+
+    pe, _ = env
+    prob = _problem(n, periodic, N=3, M=4)
+    sys_ = osolver.ModalSystem(prob)
+    fine = osolver.sequential_fine(sys_)
+    for precision, tol in ((pe.PE_FP64, 1e-12), (pe.PE_MIXED, 1e-6)):
+        with pe.Solver(prob, precision=precision) as s:
+            s.solve(tol=0.1 * tol)
+            assert _rel(s.solution(prob.N).reshape(prob.n), sys_.to_nodal(fine[-1])) <= tol

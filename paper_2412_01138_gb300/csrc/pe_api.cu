@@ -612,6 +612,7 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
     else c->terms[c->R++] = f->terms[i];
   }
   if (c->nbd > 0) PE_TRY(expand_dirichlet_terms(c));
+  c->only_moving = c->R == 0 && c->Rm > 0;
   if (c->R == 0) {
     // no (fixed) source: one zero term keeps every kernel shape valid
     c->R = 1;
@@ -632,7 +633,7 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
     PE_CUDA_TRY(cudaStreamWaitEvent(c->side2, c->ev_fork, 0));
     cudaStream_t main_stream = c->stream;
     c->stream = c->side;
-    pe_status st = launch_time_tables(c);
+    pe_status st = c->only_moving ? PE_OK : launch_time_tables(c);
     if (st == PE_OK && cudaEventRecord(c->ev_tables, c->side) != cudaSuccess)
       st = pe_cuda_fail(cudaGetLastError(), "pe_set_problem: event record");
     c->stream = c->side2;
@@ -655,7 +656,7 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
       cudaStreamWaitEvent(c->stream, c->ev_join, 0);
       return st;
     }
-  } else {
+  } else if (!c->only_moving) {
     PE_TRY(launch_time_tables(c));
   }
   // The phi/b coefficient tables depend only on lam, dt, dT and the nodes: pe_setup made them.
@@ -675,7 +676,7 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
   }
   if (general) PE_TRY(general_prepare(c));
   if (fork) PE_CUDA_TRY(cudaStreamWaitEvent(c->stream, c->ev_tables, 0));
-  PE_TRY(launch_column_weights(c));
+  if (!c->only_moving) PE_TRY(launch_column_weights(c));
   if (fork) PE_CUDA_TRY(cudaStreamWaitEvent(c->stream, c->ev_join, 0));
   PE_CUDA_TRY(record_timing(c, c->ev[1]));
   // U^0 = P_h u0

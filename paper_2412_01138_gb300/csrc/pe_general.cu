@@ -172,7 +172,7 @@ template <typename T, int Q>
 __global__ void __launch_bounds__(256) gen_fine_kernel(TermsDev D, MovingPairs P, Geom g, int n0, int M, int q,
                                                        int64_t stages, const double* __restrict__ axisM,
                                                        const double* __restrict__ muM, const T* __restrict__ coef,
-                                                       const T* __restrict__ X, double* __restrict__ Fbar) {
+                                                       const T* __restrict__ X, double* __restrict__ Fbar, int add) {
   pdl_wait();
   constexpr bool F64 = sizeof(T) == 8;
   const int64_t nd = g.ndof;
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(256) gen_fine_kernel(TermsDev D, MovingPairs P
     sum = fma(static_factor(g, j, r, D.n, D.t[r], axisM, muM), (double)c, sum);
   }
   double* out = Fbar + (int64_t)(n0 + blockIdx.y) * nd + J;
-  *out += sum;
+  *out = add ? *out + sum : sum;
 }
 
 // The moving terms' part of the coarse forcing, added to gG: sum_r C_r sum_i dT b_i prod X_{r,a}[n p + i][j_a].
@@ -245,7 +245,8 @@ __global__ void __launch_bounds__(256) gen_coarse_kernel(TermsDev D, MovingPairs
                                                          const double* __restrict__ axisM,
                                                          const double* __restrict__ muM,
                                                          const double* __restrict__ coefG,
-                                                         const double* __restrict__ X, double* __restrict__ gG) {
+                                                         const double* __restrict__ X, double* __restrict__ gG,
+                                                         int add) {
   pdl_wait();
   const int64_t nd = g.ndof;
   const int64_t J = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -268,7 +269,8 @@ __global__ void __launch_bounds__(256) gen_coarse_kernel(TermsDev D, MovingPairs
     }
     sum = fma(static_factor(g, j, r, D.n, D.t[r], axisM, muM), acc, sum);
   }
-  gG[(int64_t)n * nd + J] += sum;
+  double* out = gG + (int64_t)n * nd + J;
+  *out = add ? *out + sum : sum;
 }
 
 StageGen make_gen(const pe_ctx* c, int coarse, int n0) {
@@ -344,7 +346,8 @@ pe_status general_prepare(pe_ctx* c) {
     }
     c->gen_cap = need;
   }
-  return launch_separable_factors(c, c->mterms, c->Rm, c->axisM, 1);
+  // (on a line every factor moves: none is static)
+  return P.n == c->Rm * c->g.d ? PE_OK : launch_separable_factors(c, c->mterms, c->Rm, c->axisM, 1);
 }
 
 pe_status general_add_coarse(pe_ctx* c) {
@@ -355,7 +358,8 @@ pe_status general_add_coarse(pe_ctx* c) {
   PE_TRY(stage_tables<double>(c, P, make_gen(c, 1, 0), stages, &X));
   PE_CUDA_TRY(launch_pdl(gen_coarse_kernel, dim3((unsigned)((c->g.ndof + 255) / 256), c->N), dim3(256), 0, c->stream,
                          pack_terms(c->mterms, c->Rm), P, c->g, c->p, stages, (const double*)c->axisM,
-                         (const double*)c->muM_axis, (const double*)c->coefG, (const double*)X, c->gG));
+                         (const double*)c->muM_axis, (const double*)c->coefG, (const double*)X, c->gG,
+                         c->only_moving ? 0 : 1));
   c->launches += 1;
   return PE_OK;
 }
@@ -377,7 +381,7 @@ static pe_status add_fine(pe_ctx* c, const T* coef) {
     PE_TRY(stage_tables<T>(c, P, make_gen(c, 0, n0), stages, &X));
     PE_CUDA_TRY(launch_pdl(kern, dim3((unsigned)((c->g.ndof + 255) / 256), ns), dim3(256), 0, c->stream, TD, P, c->g, n0,
                            c->M, c->q, stages, (const double*)c->axisM, (const double*)c->muM_axis, coef, (const T*)X,
-                           c->Fbar));
+                           c->Fbar, c->only_moving ? 0 : 1));
     c->launches += 1;
   }
   return PE_OK;

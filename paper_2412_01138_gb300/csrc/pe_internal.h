@@ -129,6 +129,7 @@ struct pe_ctx {
   // factors, and the stage tables of a chunk of slices (1D loads, their transforms; float in the
   // mixed fine sweep), grown on demand
   int Rm = 0;
+  bool only_moving = false;   // no fixed source: no columns, the moving terms alone make the forced parts
   pe_term mterms[PE_MAX_TERMS];
   double* axisM = nullptr;      // [PE_MAX_TERMS * nsum]
   double *gen_L = nullptr, *gen_X = nullptr;

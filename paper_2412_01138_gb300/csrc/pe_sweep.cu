@@ -318,7 +318,10 @@ bool mixed_columns(const pe_ctx* c, int precision) {
 // Forced parts in memory: F^M(0) into f, the coarse forcing (float64 here in either form) into gG,
 // where not null.
 pe_status forced_parts(pe_ctx* c, int precision, double* f, double* gG) {
-  if (precision == PE_MIXED) {
+  // Without a fixed source there are no column sums and the moving terms store theirs (the moving hat on a line
+  // of 1023, set-up and four iterations, mixed: one kernel an iteration and six of the set-up fewer, 492 to 460 us)
+  if (c->only_moving) {
+  } else if (precision == PE_MIXED) {
     if (f) PE_TRY(forced_f32(c, f));
     if (gG) PE_TRY(launch_forced_f64(c, nullptr, gG));
   } else {

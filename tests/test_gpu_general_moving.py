@@ -67,3 +67,28 @@ def test_moving_terms_match_full_quadrature(pe, name):
             s.solve(tol=1e-10)
             for m in range(1, prob.N + 1, max(1, prob.N // 9)):
                 assert _rel(s.modal(m), ref[m], sys_.norm_w) <= bound, (prec, m)
+
+
+@pytest.mark.parametrize("n,axes", [((37,), [(0,), (0,)]), ((17, 12), [(0,), (0, 1)])], ids=["line", "plane"])
+def test_one_context_with_and_without_fixed_terms(pe, n, axes):
+    """Problems with fixed terms, without, and with them again on one context give what a fresh context gives, bit for bit,
+    and a float64 refinement of the one without reaches the oracle."""
+    probs = [_prob(n, axes, 3), _prob(n, axes, 3, fixed=0), _prob(n, axes, 3)]
+    with pe.Solver(probs[0], precision=pe.PE_MIXED, forcing_path=pe.PE_FORCING_GENERAL) as s:
+        for prob in probs:
+            s.prob, s._f_struct = prob, None  # (the binding marshals its terms once)
+            s.set_problem()
+            s.iterate()
+            s.refine()
+            s.refine()
+            s.refine()
+            with pe.Solver(prob, precision=pe.PE_MIXED, forcing_path=pe.PE_FORCING_GENERAL) as fresh:
+                fresh.set_problem()
+                fresh.iterate()
+                fresh.refine()
+                fresh.refine()
+                fresh.refine()
+                for m in range(prob.N + 1):
+                    assert np.array_equal(s.modal(m), fresh.modal(m)), m
+            sys_ = osolver.ModalSystem(prob, forcing_route="full")
+            assert _rel(s.modal(prob.N), osolver.sequential_fine(sys_)[prob.N], sys_.norm_w) <= 1e-12

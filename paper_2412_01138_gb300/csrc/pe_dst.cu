@@ -14,7 +14,7 @@
 //    pencil pair (dst_fft_warp_kernel); both run self-sorting radix-4..32 passes.
 //    Pencils with n + 1 < 16 use a block-wide radix-2 kernel (dst_fft_kernel).
 //  * any other n, and many short float64 pencils (takes_folded): the matrix form, folded by its
-//    symmetry to half the multiplications (folded_dst_kernel); up to eight pencils, in sums shared by
+//    symmetry to half the multiplications (folded_dst_kernel); a few pencils, in sums shared by
 //    the lanes of a warp (few_matrix_kernel).  A periodic axis without an FFT form keeps the plain
 //    product with its Hartley matrix (strided_gemm_kernel, few_matrix_kernel).
 #include <algorithm>
@@ -2119,7 +2119,7 @@ constexpr int kFewKO = 4;
 
 template <typename T, int NP, bool FOLD>
 __global__ void __launch_bounds__(256) few_matrix_kernel(const T* __restrict__ m, const T* __restrict__ in,
-                                                         T* __restrict__ out, int n, int64_t inner, int np) {
+                                                         T* __restrict__ out, int n, int64_t inner, int first, int np) {
   constexpr int KO = kFewKO;
   extern __shared__ __align__(16) unsigned char few_smem[];
   T* row = reinterpret_cast<T*>(few_smem);  // row[q] = sqrt(2/(n+1)) sin(pi q/(n+1)), q = 0..n+1
@@ -2128,7 +2128,7 @@ __global__ void __launch_bounds__(256) few_matrix_kernel(const T* __restrict__ m
     for (int q = tid; q < n + 2; q += 256) row[q] = q >= 1 && q <= n ? m[q - 1] : T(0);
     __syncthreads();
   }
-  const int k0 = (blockIdx.x * 8 + (tid >> 5)) * KO, p0 = blockIdx.y * NP;
+  const int k0 = (blockIdx.x * 8 + (tid >> 5)) * KO, p0 = first + blockIdx.y * NP;
   if (k0 >= n) return;
   const T* x[NP];
 #pragma unroll
@@ -2213,7 +2213,8 @@ __global__ void __launch_bounds__(256) few_matrix_kernel(const T* __restrict__ m
 }
 
 template <typename T, int NP, bool FOLD>
-pe_status few_matrix_launch(const T* m, const T* in, T* out, int n, int64_t inner, int np, cudaStream_t st) {
+pe_status few_matrix_launch(const T* m, const T* in, T* out, int n, int64_t inner, int first, int np,
+                            cudaStream_t st) {
   const size_t smem = FOLD ? sizeof(T) * (size_t)(n + 2) : 0;
   if constexpr (FOLD) {
     static std::once_flag once;
@@ -2224,23 +2225,35 @@ pe_status few_matrix_launch(const T* m, const T* in, T* out, int n, int64_t inne
     });
     if (attr != cudaSuccess) return pe_cuda_fail(attr, "dst: shared-memory attribute");
   }
-  const dim3 grid((unsigned)((n + 8 * kFewKO - 1) / (8 * kFewKO)), (unsigned)((np + NP - 1) / NP));
-  few_matrix_kernel<T, NP, FOLD><<<grid, 256, smem, st>>>(m, in, out, n, inner, np);
+  const dim3 grid((unsigned)((n + 8 * kFewKO - 1) / (8 * kFewKO)), (unsigned)((np - first + NP - 1) / NP));
+  few_matrix_kernel<T, NP, FOLD><<<grid, 256, smem, st>>>(m, in, out, n, inner, first, np);
   PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;
 }
 
 // Where the kernel above is ahead of the tiles: its sums over the lanes and its bookkeeping cost an output about as
 // much as 64 indices of the sum, for every pencil (float64, the other axis included: 4 x 100, 25.3 against
-// 27.4 us; 8 x 300, 41.9 against 40.4; 8 x 700, 63 against 67; 16 x 7353 float32, 508 against 264).
-inline bool few_matrix_takes(int n, int64_t np) { return n <= 16384 && (np <= 2 || (np <= 8 && n >= 64 * np)); }
+// 27.4 us; 8 x 300, 41.9 against 40.4; 8 x 700, 63 against 67; 16 x 1100, 91.6 against 95.6;
+// 16 x 7353, 1668 against 2165, but float32 508 against 264).  In float64 up to sixteen: the tiles of nine pencils are
+// a few heavy CTAs, which also pile up beside another stream's (a line of 8191 with nine terms: 5.16 to
+// 1.66 ms a solve).
+template <typename T>
+bool few_matrix_takes(int n, int64_t np) {
+  return n <= 16384 &&
+         (np <= 2 || (np <= 8 && n >= 64 * np) || (sizeof(T) == 8 && np <= 16 && n >= 1024));
+}
 
+// Eight pencils a launch row; the rest in a launch of their own size where the work, not the latency of one more launch,
+// counts (9 x 7353: 1016 us, 1668 in two full rows; 12 x 1100: 131 us in two launches, 92 in one).
 template <typename T, bool FOLD>
 pe_status few_matrix_axis(const T* m, const T* in, T* out, int n, int64_t inner, int np, cudaStream_t st) {
-  if (np == 1) return few_matrix_launch<T, 1, FOLD>(m, in, out, n, inner, np, st);
-  if (np == 2) return few_matrix_launch<T, 2, FOLD>(m, in, out, n, inner, np, st);
-  if (np <= 4) return few_matrix_launch<T, 4, FOLD>(m, in, out, n, inner, np, st);
-  return few_matrix_launch<T, 8, FOLD>(m, in, out, n, inner, np, st);
+  const int whole = n < 4096 && np > 8 ? np : np / 8 * 8, rest = np - whole;
+  if (whole) PE_TRY((few_matrix_launch<T, 8, FOLD>(m, in, out, n, inner, 0, whole, st)));
+  if (rest == 0) return PE_OK;
+  if (rest == 1) return few_matrix_launch<T, 1, FOLD>(m, in, out, n, inner, whole, np, st);
+  if (rest == 2) return few_matrix_launch<T, 2, FOLD>(m, in, out, n, inner, whole, np, st);
+  if (rest <= 4) return few_matrix_launch<T, 4, FOLD>(m, in, out, n, inner, whole, np, st);
+  return few_matrix_launch<T, 8, FOLD>(m, in, out, n, inner, whole, np, st);
 }
 
 // Whether a Dirichlet axis takes the folded matrix form (and so needs its sine row): without an FFT form
@@ -2260,7 +2273,7 @@ pe_status dst_axis(const T* S, const T* in, T* out, int64_t outer, int n, int64_
   int logL = 0;
   const int64_t np = outer * inner;
   if (!periodic && takes_folded<T>(n, np)) {
-    if (few_matrix_takes(n, np)) return few_matrix_axis<T, true>(S, in, out, n, inner, (int)np, st);
+    if (few_matrix_takes<T>(n, np)) return few_matrix_axis<T, true>(S, in, out, n, inner, (int)np, st);
     return folded_axis<T>(S, in, out, outer, n, inner, st);
   }
   if (!periodic && fft_size_ok(n, &logL)) return fft_axis<T>(in, out, outer, n, inner, logL, st);
@@ -2268,7 +2281,7 @@ pe_status dst_axis(const T* S, const T* in, T* out, int64_t outer, int n, int64_
     bool done = false;
     PE_TRY(dht_fft_axis<T>(in, out, outer, n, inner, st, &done));
     if (done) return PE_OK;
-    if (few_matrix_takes(n, np)) return few_matrix_axis<T, false>(S, in, out, n, inner, (int)np, st);
+    if (few_matrix_takes<T>(n, np)) return few_matrix_axis<T, false>(S, in, out, n, inner, (int)np, st);
   }
   // Hartley matrix: large tiles when they still give >= 2 CTAs per SM, else small ones
   const int64_t rows = inner == 1 ? outer : n;

@@ -12,8 +12,8 @@ u0 = nodal values of sin(pi x) sin(pi y), f = manufactured term + 8 seeded
 Gaussian bumps modulated by sin(w t + phi), 32 slices x 64 substeps, RK4 fine
 (c = 0, 1/4, 1/2, 3/4), 2-stage coarse with seeded random nodes.  The main
 line is the float64 path; "chosen" reports the mixed-precision form on the
-same workload with its stage contraction on the tensor cores ("mixed_simt": the
-same form on the CUDA cores).  --impl reference times the CPU oracle instead.
+same workload with the loop on the device and its phases replayed as graphs ("mixed_simt": the
+same kernels under the host-driven loop).  --impl reference times the CPU oracle instead.
 
 Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
        (N > 1: launch with torch.distributed.run; ranks solve independent
@@ -41,9 +41,6 @@ METRIC = "time to rel-L2 1e-6 & fine DoF·substeps/s: chosen form vs plain FP64,
 UNIT = "fine DoF*substeps/s"
 TOL = 1e-6
 L2_BYTES = 129 * 1024 * 1024
-
-
-TC_MIN_DOF = 4096  # below this the split operand images cost more than the tensor cores save
 
 
 _FLUSH = None
@@ -83,15 +80,12 @@ def cur_stream():
     return torch.cuda.current_stream()
 
 
-def chosen_kw(pe, prec, prob=None):
-    """Solver options of a separable-path solve: the mixed form (the chosen form) runs its stage
-    contraction on the tensor cores (on the CUDA cores for grids under TC_MIN_DOF nodes, which are
-    launch-bound) and its Parareal loop on the device, with the set-up and output phases of a
-    repeated solve replayed as graphs; float64 is the plain form (SIMT kernel, host-driven loop
-    of Algorithm 1)."""
+def chosen_kw(pe, prec):
+    """Solver options of a separable-path solve: the mixed form (the chosen form) runs its Parareal
+    loop on the device, with the set-up and output phases of a repeated solve replayed as graphs;
+    float64 is the plain form (host-driven loop of Algorithm 1).  Both fine engines run the same kernels."""
     if prec == pe.PE_MIXED:
-        small = prob is not None and prob.ndof < TC_MIN_DOF
-        return {"fine_engine": pe.PE_FINE_SIMT if small else pe.PE_FINE_TC, "device_loop": 2}
+        return {"fine_engine": pe.PE_FINE_SIMT, "device_loop": 2}
     return {"fine_engine": pe.PE_FINE_SIMT}
 
 
@@ -290,7 +284,7 @@ def run_batch_learned(pe, args, barrier, probs):
         barrier()
         dt = (time.perf_counter() - t0) / args.steps
         r, k = b.status()
-    out.update({"form": "batched, tensor-core fine engine, learned coarse correction", "time_to_tol_ms": 1e3 * dt,
+    out.update({"form": "batched, learned coarse correction", "time_to_tol_ms": 1e3 * dt,
                 "value": infos[-1]["fine_dof_substeps"] / dt, "unit": UNIT,
                 "iterations_histogram": {int(v): int((k == v).sum()) for v in np.unique(k)},
                 "max_residual": float(r.max()), "graph_replays": infos[-1]["graph_replays"],
@@ -303,11 +297,9 @@ def run_batch(pe, args, barrier):
     """512 uneven 2D problems: batched persistent mixed form vs a per-problem float64 loop."""
     probs = I.config4(count=args.batch_count)
     out = {"workload": f"{len(probs)} uneven 2D problems (n 31..511, 16-64 slices x 32 substeps, RK4/RK2)"}
-    for name, eng, form in (("chosen", pe.PE_FINE_TC, "batched persistent launches, CUDA graph per iteration, "
-                                                      "stage contraction on the tensor cores (problem x slice group x "
-                                                      "128-mode tile items), float32 recurrence, float64 residual"),
-                            ("simt", pe.PE_FINE_SIMT, "batched persistent launch, CUDA graph per iteration, float32 "
-                                                      "fine stages on the CUDA cores")):
+    for name, eng, form in (("chosen", pe.PE_FINE_TC, "batched launches over (problem, mode block) items, CUDA graph per "
+                                                      "iteration, float32 column sums, float64 recurrence and residual"),
+                            ("simt", pe.PE_FINE_SIMT, "the same kernels through fine_engine = PE_FINE_SIMT")):
         with pe.BatchSolver(probs, precision=pe.PE_MIXED, fine_engine=eng) as b:
             b.autotune(None)
             for _ in range(max(1, args.warmup)):
@@ -351,8 +343,8 @@ def run_batch(pe, args, barrier):
 
 def run_config1(pe, args, barrier):
     """The 1D workload (63 interior nodes, 8 x 16, RK2/RK2, manufactured e^{-t} sin(pi x)): float64 to
-    its own residual tolerance 1e-12 and to 1e-6, and the chosen mixed form (tensor-core stage
-    contraction) to 1e-6; every mode checked against the oracle (a launch- and latency-bound size)."""
+    its own residual tolerance 1e-12 and to 1e-6, and the chosen mixed form
+    to 1e-6; every mode checked against the oracle (a launch- and latency-bound size)."""
     from oracle import solver as osolver
 
     prob = I.config1()
@@ -360,7 +352,7 @@ def run_config1(pe, args, barrier):
     out = {"workload": prob.label}
     for name, prec, tol in (("fp64_tol1e-12", pe.PE_FP64, 1e-12), ("fp64", pe.PE_FP64, TOL),
                             ("chosen", pe.PE_MIXED, TOL)):
-        with pe.Solver(prob, precision=prec, stream=cur_stream(), **chosen_kw(pe, prec, prob)) as s:
+        with pe.Solver(prob, precision=prec, stream=cur_stream(), **chosen_kw(pe, prec)) as s:
             ms, infos = timed_solves(s, max(10, args.steps), max(3, args.warmup), barrier, tol=tol)
             dt = ms / 1e3
             modal = s.modal(prob.N)
@@ -371,7 +363,7 @@ def run_config1(pe, args, barrier):
                      "gpu_launches": infos[-1]["kernel_launches"],
                      "phases_ms": {k: infos[-1][k] for k in ("ms_tables", "ms_prepare", "ms_iterations",
                                                              "ms_output")},
-                     "options": {k: v for k, v in chosen_kw(pe, prec, prob).items()}}
+                     "options": {k: v for k, v in chosen_kw(pe, prec).items()}}
     out["speedup_time_to_tol"] = out["fp64"]["time_to_tol_ms"] / out["chosen"]["time_to_tol_ms"]
     return out
 
@@ -431,7 +423,7 @@ def run_learned(pe, args, barrier):
                          "value": prob.ndof * prob.N * prob.M * infos[-1]["fine_sweeps"] / dt, "unit": UNIT,
                          "residual": infos[-1]["residual"], "modal": modal}
         s.set_learned(None)
-    # the plain float64 form on the same workload (plain G, SIMT float64 fine kernel)
+    # the plain float64 form on the same workload (plain G)
     with pe.Solver(prob, precision=pe.PE_FP64, stream=cur_stream()) as s:
         ms, infos = timed_solves(s, max(1, min(args.steps, 3)), max(1, args.warmup), barrier, tol=TOL)
         dt = ms / 1e3
@@ -644,12 +636,12 @@ def run_dst(pe, args, barrier):
 
 
 def run_general(pe, args, barrier, u0_dev, u0_host):
-    """The 255^2 workload through the general forcing path: consistent load + tensor DST-I at
-    every one of the 32 x 64 x 4 fine stage times, per sweep.  Parity against the oracle on
+    """The 255^2 workload through the general forcing path: the source at every one of the
+    32 x 64 x 4 fine stage times, per sweep (products of transformed axis factors).  Parity against the oracle on
     1024 sampled modes (the source is separable: the oracle's element quadrature of it equals
     its per-axis route, which runs on a mode subset)."""
     prob = workload()
-    out = {"workload": prob.label + " general forcing path (DST per stage time)"}
+    out = {"workload": prob.label + " general forcing path (source at every stage time)"}
     rate, dtc, nm, k_or, sys_, ref, idx = oracle_sample(prob, 1024, seed=23, u0_nodal=u0_host)
     w = sys_.norm_w
     for name, prec in (("fp64", pe.PE_FP64), ("mixed", pe.PE_MIXED)):
@@ -661,7 +653,7 @@ def run_general(pe, args, barrier, u0_dev, u0_host):
         sweeps = infos[-1]["fine_sweeps"]
         out[name] = {"time_to_tol_ms": 1e3 * dt, "iterations": infos[-1]["k"],
                      "value": prob.ndof * prob.N * prob.M * sweeps / dt, "unit": UNIT,
-                     "dst_transforms_per_step": sweeps * prob.N * prob.M * prob.q + prob.N * prob.p + 2,
+                     "source_evaluations_per_step": sweeps * prob.N * prob.M * prob.q + prob.N * prob.p,
                      "rel_l2_vs_oracle": float(np.sqrt(np.sum(w * (m[idx] - ref.U[-1]) ** 2)) /
                                                np.sqrt(np.sum(w * ref.U[-1] ** 2)))}
     return out

@@ -524,6 +524,14 @@ void drop_solve_graphs(pe_ctx* c) {
   c->graph_key_seen = 0;
 }
 
+// The loop graph holds the addresses of the column weights and the number of columns; whoever frees a weight
+// table drops it.
+void drop_loop_graph(pe_ctx* c) {
+  if (c->loop_exec) cudaGraphExecDestroy(c->loop_exec);
+  c->loop_exec = nullptr;
+  c->loop_K = c->loop_prec = -1;
+}
+
 extern "C" pe_status pe_set_dirichlet(pe_ctx* c, int32_t n_terms, const pe_term* g) {
   if (c && c->pend) return pe_fail(PE_ESTATE, "pe_set_dirichlet: a solve is pending (pe_solve_wait first)");
   if (!c) return pe_fail(PE_EINVAL, "pe_set_dirichlet: ctx is NULL");
@@ -823,10 +831,7 @@ static bool loop_on_device(const pe_ctx* c) {
 
 static pe_status build_loop_graph(pe_ctx* c) {
   if (c->loop_exec && c->loop_K == c->K && c->loop_prec == c->precision) return PE_OK;
-  if (c->loop_exec) {
-    PE_CUDA_TRY(cudaGraphExecDestroy(c->loop_exec));
-    c->loop_exec = nullptr;
-  }
+  drop_loop_graph(c);
   cudaGraph_t graph = nullptr;
   PE_CUDA_TRY(cudaGraphCreate(&graph, 0));
   cudaGraphConditionalHandle handle;

@@ -594,6 +594,7 @@ static pe_status grow_weights(pe_ctx* c, T** W, int* cap) {
   const int K = c->K;
   if (K <= *cap) return PE_OK;
   PE_CUDA_TRY(cudaStreamSynchronize(c->stream));
+  drop_loop_graph(c);  // it was captured with the address given back here
   if (*W) cudaFree(*W);
   *W = nullptr;
   *cap = 0;

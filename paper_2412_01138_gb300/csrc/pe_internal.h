@@ -360,3 +360,5 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
 
 // Drops the cached set-up and output graphs of a repeated problem (pe_api.cu).
 void drop_solve_graphs(pe_ctx* c);
+// Drops the device-resident loop's graph (pe_api.cu); the next solve builds it anew.
+void drop_loop_graph(pe_ctx* c);

@@ -1,0 +1,129 @@
+"""Host code of the library over a CUDA runtime without a GPU (tests/fake/cudart.cpp): the order of allocations,
+streams, events and graph launches, and what a failing allocation leaves behind.
+
+The library's own objects are linked with that runtime in place of NVIDIA's.  Kernels do nothing there, so nothing is
+said about values; each test reads the log of the calls that the library made.
+"""
+import contextlib
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2412_01138_gb300 import inputs as I
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+class Runtime:
+    def __init__(self, path):
+        from paper_2412_01138_gb300 import pe
+
+        self.lib = pe.load_library(path)
+        self.lib.fake_line.restype = C.c_char_p
+        self.lib.fake_malloc.restype = C.c_void_p
+        self.lib.fake_malloc.argtypes = [C.c_size_t]
+
+    def clear(self):
+        self.lib.fake_clear()
+
+    def log(self):
+        return [self.lib.fake_line(i).decode().split() for i in range(self.lib.fake_count())]
+
+    @contextlib.contextmanager
+    def allocation_fails(self, after):
+        self.lib.fake_fail_in(after)
+        try:
+            yield
+        finally:
+            self.lib.fake_fail_in(-1)
+
+
+@pytest.fixture(scope="module")
+def linked(tmp_path_factory):
+    from paper_2412_01138_gb300 import build
+
+    build.build()
+    out = tmp_path_factory.mktemp("fake")
+    obj, lib = str(out / "cudart.o"), str(out / "libpe.so")
+    include = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc()))), "include")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-I", include, "-c",
+                    os.path.join(HERE, "fake", "cudart.cpp"), "-o", obj], check=True)
+    objs = [os.path.join(build.OUT, f[:-3] + ".o") for f in sorted(os.listdir(build.CSRC)) if f.endswith(".cu")]
+    # -Bsymbolic: a runtime that another package has loaded into the process does not take the calls
+    subprocess.run(["g++", "-shared", "-Wl,-Bsymbolic", "-o", lib] + objs + [obj], check=True)
+    return Runtime(lib)
+
+
+@pytest.fixture
+def rt(linked, monkeypatch):
+    from paper_2412_01138_gb300 import pe
+
+    monkeypatch.setattr(pe, "_lib", linked.lib)
+    linked.clear()
+    linked.lib.fake_set_device(0)
+    return linked
+
+
+def _prob(columns, n=(40, 33), N=4, M=16):
+    """`columns` exponential terms: as many source columns."""
+    box = ((0.0, 1.0),) * len(n)
+    u0, _, _ = I.sin_mode(len(n), box, 0.05)
+    facs = tuple(I.Factor(I.S_SIN, (3.0, 0.1)) for _ in n)
+    f = tuple(I.Term(1.0, facs, I.T_EXP, (-0.1 * i, 0.0)) for i in range(columns))
+    return I.Problem(len(n), n, box, 0.05, 0.0, 1.0, N, M, I.uniform_nodes(3), I.uniform_nodes(2), u0, f, 3, 1e-6)
+
+
+def _with(s, prob):
+    s.prob, s._f_struct = prob, None  # (the binding marshals its terms once)
+
+
+def _solve(s, **kw):
+    from paper_2412_01138_gb300 import pe
+
+    try:
+        s.solve(**kw)
+    except pe.PEError as e:  # no kernel ran, so no residual was written
+        assert e.status == pe.PE_ENOCONV
+
+
+def _stale_launches(log):
+    """Launches of graphs that were made before some device memory was freed."""
+    made, last_free = {}, -1
+    out = []
+    for i, l in enumerate(log):
+        if l[0] == "exec_new":
+            made[l[1]] = i
+        elif l[0] == "free":
+            last_free = i
+        elif l[0] == "exec_launch" and made[l[2]] < last_free:
+            out.append(i)
+    return out
+
+
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "mixed"])
+@pytest.mark.parametrize("between", ["set_problem", "solve", "out_of_memory"])
+def test_loop_graph_does_not_outlive_the_weights_it_reads(rt, precision, between):
+    """Few columns, a problem with more (whose weight tables are allocated anew), the first one again."""
+    from paper_2412_01138_gb300 import pe
+
+    few, more = _prob(5), _prob(9)
+    with pe.Solver(few, precision=precision, device_loop=1) as s:
+        _solve(s)
+        _with(s, more)
+        if between == "set_problem":
+            s.set_problem()
+        elif between == "solve":
+            _solve(s)
+        else:
+            with rt.allocation_fails(1):  # the second of the two tables
+                with pytest.raises(pe.PEError) as ei:
+                    s.solve()
+            assert ei.value.status == pe.PE_ENOMEM
+        _with(s, few)
+        _solve(s)
+        log = rt.log()
+    assert sum(l[0] == "exec_launch" for l in log) >= 2 and any(l[0] == "free" for l in log)
+    assert not _stale_launches(log)

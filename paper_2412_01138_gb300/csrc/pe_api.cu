@@ -1021,7 +1021,9 @@ static pe_status solve_begin(pe_ctx* c, const pe_field* u0, const pe_forcing* f,
   c->u0_dev_hint = -1;
   if (c->device_loop == 2 && loop_on_device(c) && u0) {
     const bool host_u0 = u0->kind == PE_FIELD_NODAL && u0->nodal && !pe_is_device_ptr(u0->nodal);
-    if (!host_u0) {
+    if (host_u0) {
+      drop_solve_graphs(c);  // this solve's set-up replaces the host state that a replay relies on
+    } else {
       if (u0->kind == PE_FIELD_NODAL) c->u0_dev_hint = 1;
       const uint64_t key = problem_key(c, u0, f);
       if (key != c->graph_key) {

@@ -60,3 +60,33 @@ def test_more_columns_between_two_solves(pe, precision, loop):
         _with(s, few)
         for _ in range(3):
             _same(_state(s, s.solve()), want)
+
+
+@pytest.mark.parametrize("columns", [3, 19], ids=["fewer", "more"])
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "mixed"])
+def test_host_u0_between_two_replays(pe, precision, columns):
+    """device_loop = 2: a solve with initial data in host memory runs its set-up directly and so changes the host state
+    that the replayed set-up of the problem before relies on (columns, terms, tables)."""
+    import torch
+
+    first, other = _prob(9), _prob(columns)
+    u0 = np.random.default_rng(1).standard_normal(first.ndof)
+    dev = torch.from_numpy(u0).cuda()
+
+    def full(s, nodal):
+        info = s.solve(u0_kind=pe.PE_FIELD_NODAL, nodal=nodal)
+        s.refine()
+        return _state(s, info)
+
+    want = {}
+    for name, prob, nodal in (("first", first, dev), ("other", other, u0)):
+        with pe.Solver(prob, precision=precision) as s:
+            want[name] = full(s, nodal)
+    with pe.Solver(first, precision=precision, device_loop=2) as s:
+        for _ in range(3):
+            _same(full(s, dev), want["first"])
+        _with(s, other)
+        _same(full(s, u0), want["other"])
+        _with(s, first)
+        for _ in range(3):
+            _same(full(s, dev), want["first"])

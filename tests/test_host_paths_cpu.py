@@ -127,3 +127,36 @@ def test_loop_graph_does_not_outlive_the_weights_it_reads(rt, precision, between
         log = rt.log()
     assert sum(l[0] == "exec_launch" for l in log) >= 2 and any(l[0] == "free" for l in log)
     assert not _stale_launches(log)
+
+
+@pytest.mark.parametrize("columns", [3, 9, 14], ids=["fewer", "as_many", "more"])
+def test_replayed_set_up_is_dropped_by_a_solve_from_host_memory(rt, columns):
+    """device_loop = 2: the replayed set-up relies on the host state (terms, columns, weight tables) of its own problem;
+    a solve in between with u0 in host memory, which runs its set-up directly, replaces that state."""
+    from paper_2412_01138_gb300 import pe
+
+    first, other = _prob(9), _prob(columns)
+    host = np.zeros(first.ndof)
+
+    def dev(s):  # u0 in (what this runtime takes for) device memory
+        f = pe.pe_field(pe.PE_FIELD_NODAL, 0, None, u0)
+        st = rt.lib.pe_solve(s.ctx, C.byref(f), C.byref(s._forcing()), 1e-6, None)
+        assert st == pe.PE_ENOCONV
+
+    u0 = rt.lib.fake_malloc(8 * first.ndof)
+    with pe.Solver(first, device_loop=2) as s:
+        dev(s)
+        dev(s)  # captures the set-up and output phases
+        held = {l[1] for l in rt.log() if l[0] == "exec_new"}
+        assert len(held) == 3
+        _with(s, other)
+        rt.clear()
+        _solve(s, u0_kind=pe.PE_FIELD_NODAL, nodal=host)
+        dropped = {l[1] for l in rt.log() if l[0] == "exec_del"}
+        _with(s, first)
+        rt.clear()
+        dev(s)
+        launched = {l[2] for l in rt.log() if l[0] == "exec_launch"}
+    assert len(dropped & held) >= 2 and not launched & dropped
+    # the first problem's set-up ran directly again
+    assert any(l[0] == "launch" and "time_tables" in l[2] for l in rt.log())

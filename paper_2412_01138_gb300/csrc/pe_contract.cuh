@@ -105,7 +105,8 @@ __device__ __forceinline__ void chain_sum(F2 x, int M, int steps, const float* _
 // Response tables.  The weight of a term's columns is P times a function of lam alone,
 //   H_r(lam) = (sum_i dt b_i(-lam dt) Z(c_i dt)) S_M(lam)   (complex for a sinusoid),
 // smooth over scales of lam itself: on an interval of relative width w the interpolation at n Chebyshev
-// nodes is off by 2 (w/4)^n at most (in units of int e^{-lam s} ds times the term's size).  Where a grid has many
+// nodes is off by 2 (w/4)^n at most (in units of int e^{-lam s} ds times the term's size; a term that decays over a
+// slice has a far smaller weight than that, and is left to the direct evaluation: response_exact).  Where a grid has many
 // more modes than an interval table has nodes, H is tabulated per problem and a mode evaluates a
 // polynomial instead of the q stages and the chain.  Intervals split each octave of lam evenly into 2^bits
 // (index and local coordinate are bits of lam): float 16 per octave and 5 nodes (2e-9 of the scale, a

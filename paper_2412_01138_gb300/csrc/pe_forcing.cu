@@ -529,6 +529,8 @@ pe_status setup_response_nodes(pe_ctx* c) {
   }
   c->resp_base = base;
   c->resp_T = T;
+  c->resp_lo = lo;
+  c->resp_hi = hi;
   Lag LF{};
   for (int i = 0; i < PE_MAX_S; ++i)
     for (int m = 0; m < PE_MAX_S; ++m) LF.a[i][m] = c->lagF[i][m];
@@ -539,10 +541,31 @@ pe_status setup_response_nodes(pe_ctx* c) {
   return PE_OK;
 }
 
-// The current problem's response table, after its time tables (not with the learned correction, whose bands the
-// direct kernel adds).
+// Whether the tabulated weights of a term are as exact as the form rounds, relative to the weight itself on every
+// mode.  A term that persists, or grows and is counted from the slice's end, has weights of the size of int e^{-lam s} ds, in
+// which the table's error is bounded.  For e^{-alpha t} the weight is int_0^dT e^{-lam s} e^{-alpha (dT - s)} ds:
+// its n-th derivative in lam is the weight times a mean of s^n, at most dT^n and, where lam > alpha, n! / (lam - alpha)^n.  With
+// n! >= (n/e)^n the interpolation error on an interval of width w lam, 2 (w lam / 4)^n max |H^(n)| / n!, is at most
+//   2 ((w lam / 4) min(e dT / n, 1 / (lam - alpha)))^n H,
+// largest where the two meet, lam = alpha + n / (e dT), or at the end of the spectrum next to it.  (160^2 modes, one
+// source, mixed: dT = 3, alpha = 30, lam_min = 20 gave 7e-5 in the solution by the table; float64 5e-11 on 208^2.)
+static bool response_exact(const pe_ctx* c, const pe_term& t) {
+  if (t.tkind == PE_T_SIN || !(t.tp[0] < 0.0)) return true;
+  const bool f32 = c->precision == PE_MIXED;
+  const double n = f32 ? Resp<float>::nodes : Resp<double>::nodes, w = ldexp(1.0, -(f32 ? Resp<float>::bits : Resp<double>::bits));
+  const double alpha = -t.tp[0], reach = n / (M_E * c->dT);
+  const double lam = std::min(std::max(alpha + reach, c->resp_lo), c->resp_hi);
+  const double f = 0.25 * w * lam / std::max(reach, lam - alpha);
+  return 2.0 * pow(f, n) <= (f32 ? 0x1p-24 : 0x1p-53);
+}
+
+// The current problem's weights come from the table (not with the learned correction, whose bands the
+// direct kernel adds).  All of them or none: one term beyond the table's reach takes the problem to the direct kernel.
+static bool uses_response(const pe_ctx* c) { return c->resp && c->resp_on && !c->mlp; }
+
+// The current problem's response table, after its time tables.
 static pe_status launch_response(pe_ctx* c) {
-  if (!c->resp || c->mlp) return PE_OK;
+  if (!uses_response(c)) return PE_OK;
   const dim3 grid((unsigned)(c->resp_T + 1));
   if (c->precision == PE_MIXED) {
     static const RespInv I = response_inverse(Resp<float>::nodes);
@@ -579,6 +602,7 @@ pe_status launch_time_tables(pe_ctx* c) {
   }
   c->cols = C;
   c->K = C.K;
+  c->resp_on = c->resp && std::all_of(c->terms, c->terms + R, [c](const pe_term& t) { return response_exact(c, t); });
   const int total = c->N * C.K + (c->q + c->p) * C.K + R * (chain_steps(c->M) + 1);
   const int threads = 128;
   PE_CUDA_TRY(launch_pdl(time_tables_kernel, dim3((unsigned)((total + threads - 1) / threads)), dim3(threads), 0,
@@ -629,7 +653,7 @@ static pe_status column_weights(pe_ctx* c, T* V, T* G, const LearnedTerms& L) {
     coefG = c->coefG32;
   }
   // the table serves the form it was made in (a mixed context's float64 weights are evaluated directly)
-  if (c->resp && !L.Ktab && V && (sizeof(T) == 8) == (c->precision != PE_MIXED)) {
+  if (uses_response(c) && V && (sizeof(T) == 8) == (c->precision != PE_MIXED)) {
     PE_CUDA_TRY(launch_pdl(response_weights_kernel<T>, grid, dim3(threads), 0, c->stream, c->g, c->cols, c->tab, c->R,
                            c->p, tpt, c->resp_base, c->resp_T, (const T*)c->resp, axisF, coefG, V, G,
                            (const double*)c->lam));

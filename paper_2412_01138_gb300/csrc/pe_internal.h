@@ -187,6 +187,8 @@ struct pe_ctx {
   // kRespMinDof modes: leading bits of the first interval, intervals, E and dt b_i at the nodes, polynomial
   // coefficients [R][resp_T + 1][2][comp] of the current problem (null: weights evaluated directly)
   int resp_base = 0, resp_T = 0;
+  double resp_lo = 0.0, resp_hi = 0.0;  // the spectrum it spans (zero aside)
+  bool resp_on = false;                 // the current problem's weights are within its reach (response_exact)
   double* resp_nodes = nullptr;
   void* resp = nullptr;
   double* loads = nullptr;      // [PE_MAX_TERMS * nsum_full] 1D loads before the DST

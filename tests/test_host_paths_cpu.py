@@ -160,3 +160,24 @@ def test_replayed_set_up_is_dropped_by_a_solve_from_host_memory(rt, columns):
     assert len(dropped & held) >= 2 and not launched & dropped
     # the first problem's set-up ran directly again
     assert any(l[0] == "launch" and "time_tables" in l[2] for l in rt.log())
+
+
+@pytest.mark.parametrize("precision,n", [(0, (208, 208)), (1, (160, 160))], ids=["fp64", "mixed"])
+@pytest.mark.parametrize("D,T,rates", [(0.1, 4.0, (-0.5,)), (0.1, 4.0, (-1.0, 2.0, 0.0)), (1.0, 4.0, (5.0,)),
+                                       (1.0, 4.0, (-0.5, -20.0)), (1.0, 4.0, (-40.0,)), (1e-4, 4.0, (-1e4,))])
+def test_weights_are_tabulated_only_within_the_tables_reach(rt, precision, n, D, T, rates):
+    """The table where every term persists, grows or decays little over a slice (here of length 1), the direct evaluation where
+    the table's error, relative to the weight of some mode, could pass the form's rounding."""
+    from paper_2412_01138_gb300 import pe
+
+    prob = _prob(1, n=n, N=int(T))
+    f = tuple(I.Term(1.0, prob.forcing[0].factors, I.T_EXP, (r, 0.0)) for r in rates)
+    f += (I.Term(1.0, prob.forcing[0].factors, I.T_SIN, (30.0, 0.0)),)
+    prob = I.Problem(2, n, prob.box, D, 0.0, T, prob.N, prob.M, prob.fine_nodes, prob.coarse_nodes, prob.u0, f, 3, 1e-6)
+    with pe.Solver(prob, precision=precision) as s:
+        rt.clear()
+        s.set_problem()
+        names = " ".join(l[2] for l in rt.log() if l[0] == "launch")
+    decays = max(-min(rates), 0.0)  # over a slice
+    limit = 1.84 if precision else 0.55
+    assert ("response_weights" in names) == (decays < limit) and ("column_weights" in names) == (decays > limit)

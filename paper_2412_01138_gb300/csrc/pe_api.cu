@@ -424,7 +424,7 @@ extern "C" pe_status pe_setup(pe_ctx** out, int32_t d, const int32_t* n, const d
   for (int a = 0; a < d && st == PE_OK; ++a)
     if (c->S32[a]) st = build_dst_matrix_f32(n[a], c->S32[a], c->stream, c->g.per[a]);
   if (st == PE_OK) st = launch_coef_tables(c);
-  if (st == PE_OK && c->g.ndof >= kRespMinDof) st = setup_response_nodes(c);
+  if (st == PE_OK && c->gn.ndof >= kRespMinDof) st = setup_response_nodes(c);
   if (st == PE_OK) {
     cudaError_t e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) st = pe_cuda_fail(e, "pe_setup");

@@ -520,7 +520,8 @@ pe_status setup_response_nodes(pe_ctx* c) {
   };
   const int base = lead(lo), T = lead(hi) - base + 1;
   // a node costs about what eight modes save (200 x 117 modes in float64, 4200 nodes: 9 us slower with the table)
-  if ((int64_t)(T + 1) * nodes * 8 > c->g.ndof) return PE_OK;
+  // (the whole grid decides, for a shard too: its weights are the unsharded solve's, bit for bit)
+  if ((int64_t)(T + 1) * nodes * 8 > c->gn.ndof) return PE_OK;
   if (cudaMalloc((void**)&c->resp_nodes, sizeof(double) * (size_t)(T + 1) * nodes * (1 + c->q)) != cudaSuccess ||
       cudaMalloc(&c->resp, (f32 ? sizeof(float) : sizeof(double)) * (size_t)PE_MAX_TERMS * (T + 1) * 2 * comp) !=
           cudaSuccess) {

@@ -1005,7 +1005,9 @@ static pe_status output_phase(pe_ctx* c) {
 // The solve in two halves: solve_begin enqueues the whole solve on the context's stream (with
 // the loop on the device nothing in it waits for the GPU; the host-driven loop waits for every
 // residual), solve_end waits for the stream and reports.
-static pe_status solve_begin(pe_ctx* c, const pe_field* u0, const pe_forcing* f, double tol, double* nodal_out) {
+// staged: a small result for pageable host memory may be handed over by solve_end.
+static pe_status solve_begin(pe_ctx* c, const pe_field* u0, const pe_forcing* f, double tol, double* nodal_out,
+                             bool staged) {
   if (!c) return pe_fail(PE_EINVAL, "pe_solve: ctx is NULL");
   if (c->pend) return pe_fail(PE_ESTATE, "pe_solve: a solve is pending (pe_solve_wait first)");
   if (!(tol >= 0.0)) return pe_fail(PE_EINVAL, "pe_solve: tol must be >= 0");
@@ -1079,13 +1081,13 @@ static pe_status solve_begin(pe_ctx* c, const pe_field* u0, const pe_forcing* f,
   // the nodal solution into the caller's buffer in the same stream order
   c->stage_to = nullptr;
   if (nodal_out) {
-    // a small result for pageable host memory goes by the context's pinned buffer and is handed over by
-    // the wait (the runtime would stage it in a blocking copy of its own)
+    // a small result for pageable host memory goes by the context's pinned buffer and is handed over after the wait
+    // of the same call (the runtime would stage it in a blocking copy of its own)
     cudaPointerAttributes attr;
     const bool known = cudaPointerGetAttributes(&attr, nodal_out) == cudaSuccess;
     if (!known) cudaGetLastError();
     const bool dev = known && (attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged);
-    if (c->h_out && (!known || attr.type == cudaMemoryTypeUnregistered)) c->stage_to = nodal_out;
+    if (staged && c->h_out && (!known || attr.type == cudaMemoryTypeUnregistered)) c->stage_to = nodal_out;
     PE_CUDA_TRY(cudaMemcpyAsync(c->stage_to ? c->h_out : nodal_out, c->out_nodal, sizeof(double) * c->gn.ndof,
                                 dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
   }
@@ -1130,20 +1132,20 @@ static pe_status solve_end(pe_ctx* c, pe_result* res) {
 }
 
 extern "C" pe_status pe_solve(pe_ctx* c, const pe_field* u0, const pe_forcing* f, double tol, pe_result* res) {
-  PE_TRY(solve_begin(c, u0, f, tol, nullptr));
+  PE_TRY(solve_begin(c, u0, f, tol, nullptr, false));
   return solve_end(c, res);
 }
 
 extern "C" pe_status pe_solve_out(pe_ctx* c, const pe_field* u0, const pe_forcing* f, double tol, double* nodal_out,
                                   pe_result* res) {
   if (!nodal_out) return pe_fail(PE_EINVAL, "pe_solve_out: nodal_out is NULL");
-  PE_TRY(solve_begin(c, u0, f, tol, nodal_out));
+  PE_TRY(solve_begin(c, u0, f, tol, nodal_out, true));
   return solve_end(c, res);
 }
 
 extern "C" pe_status pe_solve_async(pe_ctx* c, const pe_field* u0, const pe_forcing* f, double tol,
                                     double* nodal_out) {
-  return solve_begin(c, u0, f, tol, nodal_out);
+  return solve_begin(c, u0, f, tol, nodal_out, false);
 }
 
 extern "C" pe_status pe_solve_wait(pe_ctx* c, pe_result* res) { return solve_end(c, res); }

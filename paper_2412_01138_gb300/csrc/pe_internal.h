@@ -159,7 +159,7 @@ struct pe_ctx {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_tables = nullptr;
   double* h_red = nullptr;      // [2] mapped pinned host
   double* h_out = nullptr;      // [kStageOut] pinned: small nodal results on their way to pageable memory
-  double* stage_to = nullptr;   // where pe_solve_wait copies them (null: no staged result)
+  double* stage_to = nullptr;   // where pe_solve_out copies them after its wait (null: no staged result)
   int max_blocks = 0;
   int sms = 0;                      // SMs of the context's device
   // forcing (set by pe_set_problem)

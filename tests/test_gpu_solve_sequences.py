@@ -90,3 +90,18 @@ def test_host_u0_between_two_replays(pe, precision, columns):
         _with(s, first)
         for _ in range(3):
             _same(full(s, dev), want["first"])
+
+
+@pytest.mark.parametrize("n", [(63,), (40, 33), (120, 90)], ids=["line", "small", "large"])
+def test_async_result_in_pageable_memory_is_there_on_return(pe, n):
+    """pe_solve_async waits for a copy to pageable memory of any size; pe_solve_wait only reports."""
+    prob = _prob(5, n=n)
+    with pe.Solver(prob) as s:
+        s.solve()
+        want = s.solution(prob.N)
+    with pe.Solver(prob, device_loop=1) as s:
+        out = np.full(prob.ndof, np.nan)
+        s.solve_async(out=out)
+        got = out.copy()
+        s.wait()
+    assert np.array_equal(got, want) and np.array_equal(out, want)

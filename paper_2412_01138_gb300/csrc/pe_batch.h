@@ -124,7 +124,8 @@ struct pe_batch {
   int fine_engine = PE_FINE_SIMT;  // (both run the same kernels)
   // launch shape of the persistent walk kernel
   int tune_threads = 128, tune_ctas = 4;
-  cudaEvent_t ev[3] = {};
+  cudaEvent_t ev[3] = {};          // timing of a solve
+  cudaEvent_t ev_order = nullptr;  // between the caller's stream and the batch's
   bool tuned = false;
   bool have_problem = false;
   int64_t launches = 0;

@@ -48,6 +48,7 @@ void free_batch(pe_batch* b) {
   if (b->h_flags) cudaFreeHost(b->h_flags);
   for (cudaEvent_t e : b->ev)
     if (e) cudaEventDestroy(e);
+  if (b->ev_order) cudaEventDestroy(b->ev_order);
   if (b->stream) cudaStreamDestroy(b->stream);
   delete b;
 }
@@ -274,6 +275,8 @@ extern "C" pe_status pe_setup_batch(pe_batch** out, int32_t n_problems, const pe
   if (st == PE_OK) st = balloc(&b->dflags, 2);
   for (cudaEvent_t& e : b->ev)
     if (st == PE_OK && cudaEventCreate(&e) != cudaSuccess) st = pe_cuda_fail(cudaGetLastError(), "pe_setup_batch: event");
+  if (st == PE_OK && cudaEventCreateWithFlags(&b->ev_order, cudaEventDisableTiming) != cudaSuccess)
+    st = pe_cuda_fail(cudaGetLastError(), "pe_setup_batch: event");
   if (st == PE_OK && cudaMallocHost((void**)&b->h_flags, 2 * sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
     st = pe_fail(PE_ENOMEM, "pe_setup_batch: pinned allocation failed");
@@ -446,8 +449,8 @@ extern "C" pe_status pe_batch_solve(pe_batch* b, double tol, pe_batch_result* re
   if (!(tol >= 0.0)) return pe_fail(PE_EINVAL, "pe_batch_solve: tol must be >= 0");
   cudaEvent_t* ev = b->ev;
   if (b->user_stream) {
-    PE_CUDA_TRY(cudaEventRecord(ev[0], b->user_stream));
-    PE_CUDA_TRY(cudaStreamWaitEvent(b->stream, ev[0], 0));
+    PE_CUDA_TRY(cudaEventRecord(b->ev_order, b->user_stream));
+    PE_CUDA_TRY(cudaStreamWaitEvent(b->stream, b->ev_order, 0));
   }
   b->launches = 0;
   PE_TRY(reset_iteration_state(b));
@@ -473,8 +476,8 @@ extern "C" pe_status pe_batch_solve(pe_batch* b, double tol, pe_batch_result* re
   PE_CUDA_TRY(cudaEventSynchronize(ev[2]));
   b->have_problem = true;
   if (b->user_stream) {
-    PE_CUDA_TRY(cudaEventRecord(ev[0], b->stream));
-    PE_CUDA_TRY(cudaStreamWaitEvent(b->user_stream, ev[0], 0));
+    PE_CUDA_TRY(cudaEventRecord(b->ev_order, b->stream));
+    PE_CUDA_TRY(cudaStreamWaitEvent(b->user_stream, b->ev_order, 0));
   }
   if (res) {
     std::vector<int> k((size_t)b->P);

@@ -181,3 +181,27 @@ def test_weights_are_tabulated_only_within_the_tables_reach(rt, precision, n, D,
     decays = max(-min(rates), 0.0)  # over a slice
     limit = 1.84 if precision else 0.55
     assert ("response_weights" in names) == (decays < limit) and ("column_weights" in names) == (decays > limit)
+
+
+def _batch_probs(count=3):
+    return [_prob(3 + i, n=(17 + i, 9), N=3) for i in range(count)]
+
+
+def _recorded(log, upto, event):
+    return max(i for i in range(upto) if log[i][0] == "record" and log[i][2] == event)
+
+
+@pytest.mark.parametrize("stream", [None, 48], ids=["default", "callers"])
+def test_batch_times_run_forward(rt, stream):
+    """Both ends of every reported time were recorded in order (the event of one was once recorded again to order the
+    caller's stream)."""
+    from paper_2412_01138_gb300 import pe
+
+    with pe.BatchSolver(_batch_probs(), stream=stream) as b:
+        rt.clear()
+        b.solve(tol=1e-6)
+        log = rt.log()
+    pairs = [(i, l) for i, l in enumerate(log) if l[0] == "elapsed"]
+    assert len(pairs) == 2
+    for i, l in pairs:
+        assert _recorded(log, i, l[1]) < _recorded(log, i, l[2])

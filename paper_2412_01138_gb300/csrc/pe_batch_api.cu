@@ -444,14 +444,19 @@ extern "C" pe_status pe_batch_autotune(pe_batch* b, const char* cache_path) {
   return PE_OK;
 }
 
+// What the caller's stream (the legacy default stream where the batch was given none) still has to do with a buffer or
+// a network it hands over comes before the work on the batch's own stream, which waits for no other by itself.
+static pe_status after_caller(pe_batch* b) {
+  PE_CUDA_TRY(cudaEventRecord(b->ev_order, b->user_stream));
+  PE_CUDA_TRY(cudaStreamWaitEvent(b->stream, b->ev_order, 0));
+  return PE_OK;
+}
+
 extern "C" pe_status pe_batch_solve(pe_batch* b, double tol, pe_batch_result* res) {
   if (!b) return pe_fail(PE_EINVAL, "pe_batch_solve: NULL batch");
   if (!(tol >= 0.0)) return pe_fail(PE_EINVAL, "pe_batch_solve: tol must be >= 0");
   cudaEvent_t* ev = b->ev;
-  if (b->user_stream) {
-    PE_CUDA_TRY(cudaEventRecord(b->ev_order, b->user_stream));
-    PE_CUDA_TRY(cudaStreamWaitEvent(b->stream, b->ev_order, 0));
-  }
+  PE_TRY(after_caller(b));
   b->launches = 0;
   PE_TRY(reset_iteration_state(b));
   PE_TRY(ensure_graphs(b, tol));
@@ -510,6 +515,7 @@ extern "C" pe_status pe_batch_get_modal(pe_batch* b, int32_t problem, int32_t sl
   if (slice < 0 || slice > B.N) return pe_fail(PE_EINVAL, "pe_batch_get_modal: slice out of range");
   if (!b->have_problem) return pe_fail(PE_ESTATE, "pe_batch_get_modal: no solve has completed");
   const bool dev = pe_is_device_ptr(out);
+  PE_TRY(after_caller(b));
   PE_CUDA_TRY(cudaMemcpyAsync(out, b->U + B.oU + (int64_t)slice * B.g.ndof, sizeof(double) * B.g.ndof,
                               dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, b->stream));
   PE_CUDA_TRY(cudaStreamSynchronize(b->stream));
@@ -527,6 +533,7 @@ extern "C" pe_status pe_batch_get_solution(pe_batch* b, int32_t problem, double*
   for (int a = 0; a < B.g.d; ++a) rows[a] = b->rows + B.oMu + B.g.off[a];
   const bool dev = pe_is_device_ptr(nodal_out);
   double* out = dev ? nodal_out : b->scratch + b->ndof_max;
+  PE_TRY(after_caller(b));
   pe_status st = dst_rows_f64(B.g.d, n, rows, last, out, b->scratch, b->stream);
   if (st == PE_OK && !dev) {
     cudaError_t e = cudaMemcpyAsync(nodal_out, out, sizeof(double) * B.g.ndof, cudaMemcpyDeviceToHost, b->stream);

@@ -29,3 +29,26 @@ def test_times_are_those_of_the_solve_with_a_callers_stream(pe):
             info = b.solve(tol=1e-6)
             assert info["ms_prepare"] > 0.0 and info["ms_iterations"] > 0.0
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("own_stream", [False, True], ids=["default", "callers"])
+def test_a_buffer_is_written_after_its_last_reader(pe, own_stream):
+    """One device buffer for every solution, read by work of the caller's stream that has not run yet when the next call
+    is made."""
+    import torch
+
+    probs = I.config4(count=4)
+    stream = torch.cuda.Stream() if own_stream else None
+    with pe.BatchSolver(probs, stream=stream) as b, torch.cuda.stream(stream):
+        b.solve(tol=1e-6)
+        want = [b.solution(i) for i in range(4)]
+        modal = [b.modal(i, 1) for i in range(4)]
+        buf = torch.empty(max(p.ndof for p in probs), dtype=torch.float64, device="cuda")
+        for fetch, ref in ((lambda i: b.solution(i, out=buf), want), (lambda i: b.modal(i, 1, out=buf), modal)):
+            kept = []
+            for i, p in enumerate(probs):
+                fetch(i)
+                torch.cuda._sleep(20000000)  # about 10 ms of another kernel
+                kept.append(buf[:p.ndof].clone())
+            for i, k in enumerate(kept):
+                assert np.array_equal(k.cpu().numpy(), ref[i]), i

@@ -205,3 +205,27 @@ def test_batch_times_run_forward(rt, stream):
     assert len(pairs) == 2
     for i, l in pairs:
         assert _recorded(log, i, l[1]) < _recorded(log, i, l[2])
+
+
+@pytest.mark.parametrize("stream", [None, 48], ids=["default", "callers"])
+@pytest.mark.parametrize("call", ["solve", "solution", "modal"])
+def test_batch_works_after_the_callers_stream(rt, stream, call):
+    """The batch's own stream waits for nothing by itself: before it writes a buffer of the caller's (or reads a network)
+    it is ordered after the caller's stream, the legacy default stream where none was given."""
+    from paper_2412_01138_gb300 import pe
+
+    with pe.BatchSolver(_batch_probs(), stream=stream) as b:
+        b.solve(tol=1e-6)
+        rt.clear()
+        if call == "solve":
+            b.solve(tol=1e-6)
+        elif call == "solution":
+            b.solution(1)
+        else:
+            b.modal(1, 0)
+        log = rt.log()
+    works = next(i for i, l in enumerate(log) if l[0] in ("launch", "copy", "exec_launch"))
+    wait = next((i for i, l in enumerate(log) if l[0] == "wait" and l[1] == log[works][1]), len(log))
+    assert wait < works
+    recorded = [l for l in log[:wait] if l[0] == "record" and l[2] == log[wait][2]]
+    assert recorded and recorded[-1][1] == str(stream or 0)

@@ -1,6 +1,7 @@
 // Internal layout of the batched solver (pe_batch): per-problem records,
 // work items and arenas.  Not part of the ABI.
 #pragma once
+#include <mutex>
 #include <vector>
 
 #include "pe_forcing_common.cuh"
@@ -126,6 +127,7 @@ struct pe_batch {
   int tune_threads = 128, tune_ctas = 4;
   cudaEvent_t ev[3] = {};          // timing of a solve
   cudaEvent_t ev_order = nullptr;  // between the caller's stream and the batch's
+  std::mutex fetch;                // one fetch at a time: it owns scratch and ev_order until it has waited
   bool tuned = false;
   bool have_problem = false;
   int64_t launches = 0;

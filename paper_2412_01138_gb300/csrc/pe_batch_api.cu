@@ -515,6 +515,7 @@ extern "C" pe_status pe_batch_get_modal(pe_batch* b, int32_t problem, int32_t sl
   if (slice < 0 || slice > B.N) return pe_fail(PE_EINVAL, "pe_batch_get_modal: slice out of range");
   if (!b->have_problem) return pe_fail(PE_ESTATE, "pe_batch_get_modal: no solve has completed");
   const bool dev = pe_is_device_ptr(out);
+  std::lock_guard<std::mutex> lock(b->fetch);
   PE_TRY(after_caller(b));
   PE_CUDA_TRY(cudaMemcpyAsync(out, b->U + B.oU + (int64_t)slice * B.g.ndof, sizeof(double) * B.g.ndof,
                               dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, b->stream));
@@ -533,6 +534,7 @@ extern "C" pe_status pe_batch_get_solution(pe_batch* b, int32_t problem, double*
   for (int a = 0; a < B.g.d; ++a) rows[a] = b->rows + B.oMu + B.g.off[a];
   const bool dev = pe_is_device_ptr(nodal_out);
   double* out = dev ? nodal_out : b->scratch + b->ndof_max;
+  std::lock_guard<std::mutex> lock(b->fetch);
   PE_TRY(after_caller(b));
   pe_status st = dst_rows_f64(B.g.d, n, rows, last, out, b->scratch, b->stream);
   if (st == PE_OK && !dev) {

@@ -3,6 +3,7 @@
 // allocations down to the one that returns cudaErrorMemoryAllocation.
 #include <cuda_runtime.h>
 #include <string.h>
+#include <unistd.h>
 
 #include <map>
 #include <mutex>
@@ -22,7 +23,7 @@ std::string name_of(const void* f) {
   return it == names().end() ? "?" : it->second;
 }
 std::map<const void*, size_t> device;  // allocations, by address
-int fail_in = -1, current_device = 0;
+int fail_in = -1, current_device = 0, slow = 0;
 long next_id = 1;
 
 std::string id(const void* p) { return std::to_string((unsigned long long)p); }
@@ -72,6 +73,7 @@ struct Call {
 };
 thread_local std::vector<Call> calls;
 cudaError_t launched(const void* f, cudaStream_t st, size_t smem) {
+  if (slow) usleep(slow);
   note("launch " + id(st) + " " + name_of(f) + " " + std::to_string(smem));
   return cudaSuccess;
 }
@@ -86,6 +88,7 @@ void fake_clear() {
 int fake_count() { return (int)lines.size(); }
 const char* fake_line(int i) { return lines[(size_t)i].c_str(); }
 void fake_fail_in(int n) { fail_in = n; }  // the (n + 1)-th allocation from now fails
+void fake_slow(int us) { slow = us; }  // microseconds a launch takes
 void fake_set_device(int d) { current_device = d; }
 void* fake_malloc(size_t n) {
   void* p = nullptr;

@@ -52,3 +52,36 @@ def test_a_buffer_is_written_after_its_last_reader(pe, own_stream):
                 kept.append(buf[:p.ndof].clone())
             for i, k in enumerate(kept):
                 assert np.array_equal(k.cpu().numpy(), ref[i]), i
+
+
+@pytest.mark.parametrize("device", [False, True], ids=["host", "device"])
+def test_threads_fetch_from_one_batch(pe, device):
+    """Several threads fetch solutions of one batch at once (the calls release the interpreter's lock): the transforms
+    share the batch's scratch."""
+    import threading
+
+    import torch
+
+    probs = I.config4(count=5)
+    with pe.BatchSolver(probs) as b:
+        b.solve(tol=1e-6)
+        want = [b.solution(i) for i in range(5)]
+        wrong = []
+
+        def fetch(seed):
+            rng = np.random.default_rng(seed)
+            for i in rng.integers(0, 5, 40):
+                if device:
+                    out = torch.empty(probs[i].ndof, dtype=torch.float64, device="cuda")
+                    got = b.solution(int(i), out=out).cpu().numpy()
+                else:
+                    got = b.solution(int(i))
+                if not np.array_equal(got, want[i]):
+                    wrong.append(int(i))
+
+        ts = [threading.Thread(target=fetch, args=(s,)) for s in range(6)]
+        for t in ts:
+            t.start()
+        for t in ts:
+            t.join()
+        assert not wrong

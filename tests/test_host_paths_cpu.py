@@ -229,3 +229,31 @@ def test_batch_works_after_the_callers_stream(rt, stream, call):
     assert wait < works
     recorded = [l for l in log[:wait] if l[0] == "record" and l[2] == log[wait][2]]
     assert recorded and recorded[-1][1] == str(stream or 0)
+
+
+def test_two_threads_fetch_from_one_batch_one_after_the_other(rt):
+    """A fetch transforms through the batch's scratch on the batch's stream and waits: until then no other fetch may
+    enqueue anything."""
+    import threading
+
+    from paper_2412_01138_gb300 import pe
+
+    probs = [_prob(3, n=(17, 9, 8), N=3) for _ in range(3)]
+    with pe.BatchSolver(probs) as b:
+        b.solve(tol=1e-6)
+        b.solution(0)
+        rt.clear()
+        b.solution(0)
+        one = [l[0] for l in rt.log()]
+        rt.clear()
+        rt.lib.fake_slow(200)  # microseconds a launch: the calls of two threads meet
+        try:
+            ts = [threading.Thread(target=lambda: [b.solution(i % 3) for i in range(20)]) for _ in range(4)]
+            for t in ts:
+                t.start()
+            for t in ts:
+                t.join()
+        finally:
+            rt.lib.fake_slow(0)
+        log = [l[0] for l in rt.log()]
+    assert log == one * 80

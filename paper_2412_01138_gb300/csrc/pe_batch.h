@@ -95,6 +95,7 @@ struct pe_batch {
   double *coefF = nullptr, *coefG = nullptr;
   float *coefF32 = nullptr, *coefG32 = nullptr;
   double* U = nullptr;
+  size_t u_total = 0;         // its length
   double *axisF = nullptr, *axisU0 = nullptr;
   float* axisF32 = nullptr;
   // time tables and column weights (pe_contract.cuh); float forms in the mixed form
@@ -128,7 +129,6 @@ struct pe_batch {
   cudaEvent_t ev[3] = {};          // timing of a solve
   cudaEvent_t ev_order = nullptr;  // between the caller's stream and the batch's
   std::mutex fetch;                // one fetch at a time: it owns scratch and ev_order until it has waited
-  bool tuned = false;
   bool have_problem = false;
   int64_t launches = 0;
   uint64_t signature = 0;

@@ -248,6 +248,7 @@ extern "C" pe_status pe_setup_batch(pe_batch** out, int32_t n_problems, const pe
 
   // ---- arenas --------------------------------------------------------------
   const bool mixed = b->precision == PE_MIXED;
+  b->u_total = (size_t)oU;
   if (st == PE_OK) st = balloc(&b->muM, oMu);
   if (st == PE_OK) st = balloc(&b->ratio, oMu);
   if (st == PE_OK) st = balloc(&b->rows, oMu);
@@ -388,6 +389,54 @@ float ms_between(cudaEvent_t a, cudaEvent_t b) {
 
 }  // namespace
 
+// What the caller's stream (the legacy default stream where the batch was given none) still has to do with a buffer or
+// a network it hands over comes before the work on the batch's own stream, which waits for no other by itself.
+static pe_status after_caller(pe_batch* b) {
+  PE_CUDA_TRY(cudaEventRecord(b->ev_order, b->user_stream));
+  PE_CUDA_TRY(cudaStreamWaitEvent(b->stream, b->ev_order, 0));
+  return PE_OK;
+}
+
+namespace {
+
+// The fastest launch shape of the walk on a prepared state; the timed walks write iterates.
+pe_status time_shapes(pe_batch* b, int* threads, int* ctas) {
+  PE_TRY(reset_iteration_state(b));
+  PE_TRY(batch_launch_prepare(b));
+  const int cand_threads[2] = {128, 256};
+  float best = 1e30f;
+  for (int ti = 0; ti < 2; ++ti) {
+    for (int ct = 1; ct <= 4; ++ct) {
+      float ms = 0.f, tot = 0.f;
+      PE_TRY(batch_time_walk(b, cand_threads[ti], ct, &ms));  // warm
+      for (int rep = 0; rep < 2; ++rep) {
+        PE_TRY(batch_time_walk(b, cand_threads[ti], ct, &ms));
+        tot += ms;
+      }
+      if (tot < best) {
+        best = tot;
+        *threads = cand_threads[ti];
+        *ctas = ct;
+      }
+    }
+  }
+  return PE_OK;
+}
+
+// What a finished solve can still be asked for (iterates, k, residuals), kept in `buf` or put back from it.
+size_t result_bytes(const pe_batch* b) { return sizeof(double) * (b->u_total + b->P) + sizeof(int) * b->P; }
+pe_status copy_result(pe_batch* b, double* buf, bool back) {
+  const auto part = [&](void* own, void* kept, size_t bytes) {
+    return cudaMemcpyAsync(back ? own : kept, back ? kept : own, bytes, cudaMemcpyDeviceToDevice, b->stream);
+  };
+  PE_CUDA_TRY(part(b->U, buf, sizeof(double) * b->u_total));
+  PE_CUDA_TRY(part(b->resid, buf + b->u_total, sizeof(double) * b->P));
+  PE_CUDA_TRY(part(b->kcount, buf + b->u_total + b->P, sizeof(int) * b->P));
+  return PE_OK;
+}
+
+}  // namespace
+
 extern "C" pe_status pe_batch_autotune(pe_batch* b, const char* cache_path) {
   if (!b) return pe_fail(PE_EINVAL, "pe_batch_autotune: NULL batch");
   cudaDeviceProp prop;
@@ -408,47 +457,39 @@ extern "C" pe_status pe_batch_autotune(pe_batch* b, const char* cache_path) {
       if (ss >> k >> th >> ct && k == key && (th == 128 || th == 256) && ct >= 1 && ct <= 8) {
         b->tune_threads = th;
         b->tune_ctas = ct;
-        b->tuned = true;
         return PE_OK;
       }
     }
   }
-  // time every candidate on a prepared state (the walks write iterates that the next solve makes anew)
-  PE_TRY(reset_iteration_state(b));
-  PE_TRY(batch_launch_prepare(b));
-  const int cand_threads[2] = {128, 256};
-  float best = 1e30f;
-  int best_t = 128, best_c = 4;
-  for (int ti = 0; ti < 2; ++ti) {
-    for (int ct = 1; ct <= 4; ++ct) {
-      float ms = 0.f, tot = 0.f;
-      PE_TRY(batch_time_walk(b, cand_threads[ti], ct, &ms));  // warm
-      for (int rep = 0; rep < 2; ++rep) {
-        PE_TRY(batch_time_walk(b, cand_threads[ti], ct, &ms));
-        tot += ms;
-      }
-      if (tot < best) {
-        best = tot;
-        best_t = cand_threads[ti];
-        best_c = ct;
-      }
+  PE_TRY(after_caller(b));
+  // a finished solve stays as it is; without room to keep it the launch shape stays as it is
+  double* kept = nullptr;
+  if (b->have_problem) {
+    if (cudaMalloc((void**)&kept, result_bytes(b)) != cudaSuccess) {
+      cudaGetLastError();
+      return PE_OK;
+    }
+    const pe_status st = copy_result(b, kept, false);
+    if (st != PE_OK) {
+      cudaFree(kept);
+      return st;
     }
   }
+  int best_t = 128, best_c = 4;
+  pe_status st = time_shapes(b, &best_t, &best_c);
+  if (kept) {
+    const pe_status back = copy_result(b, kept, true);
+    cudaStreamSynchronize(b->stream);
+    cudaFree(kept);
+    if (st == PE_OK) st = back;
+  }
+  PE_TRY(st);
   b->tune_threads = best_t;
   b->tune_ctas = best_c;
-  b->tuned = true;
   if (cache_path) {
     std::ofstream outf(cache_path, std::ios::app);
     if (outf) outf << key << " " << best_t << " " << best_c << "\n";
   }
-  return PE_OK;
-}
-
-// What the caller's stream (the legacy default stream where the batch was given none) still has to do with a buffer or
-// a network it hands over comes before the work on the batch's own stream, which waits for no other by itself.
-static pe_status after_caller(pe_batch* b) {
-  PE_CUDA_TRY(cudaEventRecord(b->ev_order, b->user_stream));
-  PE_CUDA_TRY(cudaStreamWaitEvent(b->stream, b->ev_order, 0));
   return PE_OK;
 }
 

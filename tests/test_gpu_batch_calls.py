@@ -85,3 +85,23 @@ def test_threads_fetch_from_one_batch(pe, device):
         for t in ts:
             t.join()
         assert not wrong
+
+
+@pytest.mark.parametrize("engine", [0, 1], ids=["simt", "tc"])
+def test_autotune_leaves_a_finished_solve_as_it_is(pe, engine):
+    probs = I.config4(count=5)
+    with pe.BatchSolver(probs, fine_engine=engine) as b:
+        b.solve(tol=1e-6)
+
+        def results():
+            r, k = b.status()
+            return [r, k] + [b.modal(i, m) for i, p in enumerate(probs) for m in (0, 1, p.N)] + \
+                [b.solution(i) for i in range(len(probs))]
+
+        before = results()
+        b.autotune(None)
+        for x, y in zip(before, results()):
+            assert np.array_equal(x, y)
+        b.solve(tol=1e-6)
+        for x, y in zip(before[1:], results()[1:]):  # (the residual sums follow the launch shape's items)
+            assert np.array_equal(x, y)

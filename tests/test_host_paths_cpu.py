@@ -257,3 +257,22 @@ def test_two_threads_fetch_from_one_batch_one_after_the_other(rt):
             rt.lib.fake_slow(0)
         log = [l[0] for l in rt.log()]
     assert log == one * 80
+
+
+def test_autotune_without_room_for_the_results_changes_nothing(rt):
+    from paper_2412_01138_gb300 import pe
+
+    with pe.BatchSolver(_batch_probs()) as b:
+        b.solve(tol=1e-6)
+        rt.clear()
+        with rt.allocation_fails(0):
+            b.autotune(None)
+        assert not any(l[0] in ("launch", "copy", "exec_launch") for l in rt.log())
+        rt.clear()
+        b.autotune(None)
+        log = rt.log()
+    # kept aside, timed, put back
+    copies = [i for i, l in enumerate(log) if l[0] == "copy"]
+    walks = [i for i, l in enumerate(log) if l[0] == "launch" and "b_walk" in l[2]]
+    assert len(copies) == 6 and copies[2] < walks[0] and walks[-1] < copies[3]
+    assert [l for l in log if l[0] == "malloc"][0][1] == [l for l in log if l[0] == "free"][0][1]

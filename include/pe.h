@@ -414,7 +414,7 @@ pe_status pe_setup_batch(pe_batch** out, int32_t n_problems, const pe_problem* p
 
 /* Pick the persistent walk kernel's launch shape (threads per CTA x CTAs per SM)
  * by timing the candidates on this batch; cache_path (may be NULL) is a text file
- * of previous choices keyed by device and batch signature, read and appended.  The
+ * of previous choices keyed by device, kernel and batch signature, read and appended.  The
  * results of a finished solve stay as they are (kept aside meanwhile; where the device
  * has no room for that, the launch shape stays as it is instead). */
 pe_status pe_batch_autotune(pe_batch* b, const char* cache_path);

@@ -444,7 +444,8 @@ extern "C" pe_status pe_batch_autotune(pe_batch* b, const char* cache_path) {
   PE_CUDA_TRY(cudaGetDevice(&dev));
   PE_CUDA_TRY(cudaGetDeviceProperties(&prop, dev));
   char key[320];
-  snprintf(key, sizeof(key), "%s|%016llx", prop.name, (unsigned long long)b->signature);
+  // (the kernel whose shape was timed is part of the key: a file of another one's choices is left alone)
+  snprintf(key, sizeof(key), "%s|walk|%016llx", prop.name, (unsigned long long)b->signature);
   for (char* c = key; *c; ++c)
     if (*c == ' ') *c = '_';
   if (cache_path) {

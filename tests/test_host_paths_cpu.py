@@ -276,3 +276,24 @@ def test_autotune_without_room_for_the_results_changes_nothing(rt):
     walks = [i for i, l in enumerate(log) if l[0] == "launch" and "b_walk" in l[2]]
     assert len(copies) == 6 and copies[2] < walks[0] and walks[-1] < copies[3]
     assert [l for l in log if l[0] == "malloc"][0][1] == [l for l in log if l[0] == "free"][0][1]
+
+
+def test_tuning_files_of_another_kernel_are_not_taken(rt, tmp_path):
+    """A tuning file from before the walk holds shapes that were timed on the per-substep kernel, keyed by device and
+    signature alone: they are left in place and the walk is timed."""
+    from paper_2412_01138_gb300 import pe
+
+    cache = tmp_path / "tune.txt"
+    with pe.BatchSolver(_batch_probs()) as b:
+        b.autotune(str(cache))
+    device, kernel, signature = cache.read_text().split()[0].split("|")
+    cache.write_text(f"{device}|{signature} 256 2\n")
+    with pe.BatchSolver(_batch_probs()) as b:
+        rt.clear()
+        b.autotune(str(cache))
+        assert any("b_walk" in l[2] for l in rt.log() if l[0] == "launch")
+        lines = cache.read_text().splitlines()
+        assert len(lines) == 2 and lines[0] == f"{device}|{signature} 256 2"
+        rt.clear()
+        b.autotune(str(cache))  # the new line is taken
+        assert not any(l[0] == "launch" for l in rt.log())

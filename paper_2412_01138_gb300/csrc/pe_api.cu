@@ -597,7 +597,8 @@ static cudaError_t record_timing(pe_ctx* c, cudaEvent_t e) {
 
 // Algorithm 1 up to its loop; the coarse sweep only where `coarse` (pe_solve makes it in the same
 // pass as the first iteration, launch_iteration).
-static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcing* f, bool coarse) {
+// *forked: work has been given to the side streams.
+static pe_status set_problem_phases(pe_ctx* c, const pe_field* u0, const pe_forcing* f, bool coarse, bool* forked) {
   if (!u0) return pe_fail(PE_EINVAL, "pe_set_problem: u0 is NULL");
   const int nf = f ? f->n_terms : 0;
   const bool general = c->forcing_path == PE_FORCING_GENERAL;
@@ -636,6 +637,7 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
   const bool fork = fork_u0 && c->gn.ndof >= kForkMinDof;
   const bool inline_u0 = fork_u0 && !fork;  // nodal u0, transformed below on the main stream
   if (fork) {
+    *forked = true;
     PE_CUDA_TRY(cudaEventRecord(c->ev_fork, c->stream));
     PE_CUDA_TRY(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
     PE_CUDA_TRY(cudaStreamWaitEvent(c->side2, c->ev_fork, 0));
@@ -658,12 +660,8 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
       if (st == PE_OK) st = nodal_to_modal(c, src, U0);
     }
     c->stream = main_stream;
-    // both streams are joined below whatever happened here
+    PE_TRY(st);
     PE_CUDA_TRY(cudaEventRecord(c->ev_join, c->side2));
-    if (st != PE_OK) {
-      cudaStreamWaitEvent(c->stream, c->ev_join, 0);
-      return st;
-    }
   } else if (!c->only_moving) {
     PE_TRY(launch_time_tables(c));
   }
@@ -731,6 +729,26 @@ static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcin
   c->have_problem = true;
   c->have_output = false;
   return PE_OK;
+}
+
+static pe_status set_problem_impl(pe_ctx* c, const pe_field* u0, const pe_forcing* f, bool coarse) {
+  bool forked = false;
+  const pe_status st = set_problem_phases(c, u0, f, coarse, &forked);
+  if (st != PE_OK && forked) {
+    // a failure between the fork and its join: nothing is left running that reads the caller's u0 (or, in a capture,
+    // unjoined)
+    if (c->capturing) {
+      cudaEventRecord(c->ev_tables, c->side);
+      cudaEventRecord(c->ev_join, c->side2);
+      cudaStreamWaitEvent(c->stream, c->ev_tables, 0);
+      cudaStreamWaitEvent(c->stream, c->ev_join, 0);
+    } else {
+      cudaStreamSynchronize(c->side);
+      cudaStreamSynchronize(c->side2);
+    }
+    cudaGetLastError();
+  }
+  return st;
 }
 
 extern "C" pe_status pe_set_problem(pe_ctx* c, const pe_field* u0, const pe_forcing* f) {

@@ -297,3 +297,32 @@ def test_tuning_files_of_another_kernel_are_not_taken(rt, tmp_path):
         rt.clear()
         b.autotune(str(cache))  # the new line is taken
         assert not any(l[0] == "launch" for l in rt.log())
+
+
+@pytest.mark.parametrize("call", ["set_problem", "solve"])
+@pytest.mark.parametrize("fails", [0, 1, "general"])
+def test_a_failing_set_up_leaves_nothing_running(rt, call, fails):
+    """Grids large enough for set-up on three streams: where an allocation fails beside the transform of the caller's u0
+    (a weight table, or the moving terms' stage tables), the call waits for the other streams before it returns."""
+    from paper_2412_01138_gb300 import pe
+
+    prob = _prob(5, n=(71, 65))
+    kw = {}
+    if fails == "general":
+        hat = I.Term(1.0, (I.Factor(I.S_MOVING_HAT, (0.5, 0.2, 1.0, 0.1)), prob.forcing[0].factors[1]))
+        prob = I.Problem(2, prob.n, prob.box, prob.D, 0.0, 1.0, prob.N, prob.M, prob.fine_nodes, prob.coarse_nodes, prob.u0,
+                         prob.forcing + (hat,), 3, 1e-6)
+        kw = {"forcing_path": pe.PE_FORCING_GENERAL}
+    with pe.Solver(prob, **kw) as s:
+        rt.clear()
+        with rt.allocation_fails(0 if fails == "general" else fails):
+            with pytest.raises(pe.PEError) as ei:
+                getattr(s, call)(u0_kind=pe.PE_FIELD_NODAL, nodal=np.zeros(prob.ndof))
+        assert ei.value.status == pe.PE_ENOMEM
+        log = rt.log()
+    main = "0"
+    used = {l[1] for l in log if l[0] in ("launch", "copy")} - {main}
+    assert len(used) == 2
+    for stream in used:
+        last = max(i for i, l in enumerate(log) if l[0] in ("launch", "copy") and l[1] == stream)
+        assert ["sync", stream] in log[last:]

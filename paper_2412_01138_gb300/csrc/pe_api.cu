@@ -9,8 +9,11 @@
 
 #include <algorithm>
 #include <climits>
+#include <map>
+#include <mutex>
 #include <new>
 #include <string>
+#include <utility>
 
 #include "pe_contract.cuh"
 #include "pe_internal.h"
@@ -100,6 +103,20 @@ void pe_lagrange_coeffs(int s, const double* c, double a[PE_MAX_S][PE_MAX_S]) {
     }
     for (int k = 0; k < s; ++k) a[i][k] = poly[k];
   }
+}
+
+pe_status allow_smem(const void* kern, size_t bytes) {
+  if (bytes <= 40 * 1024) return PE_OK;  // (48 KB without asking, a kernel's static shared memory included)
+  static std::map<std::pair<const void*, int>, size_t> allowed;
+  static std::mutex mu;
+  int dev = 0;
+  PE_CUDA_TRY(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lock(mu);
+  size_t& have = allowed[{kern, dev}];
+  if (bytes <= have) return PE_OK;
+  PE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  have = bytes;
+  return PE_OK;
 }
 
 bool pe_is_device_ptr(const void* p) {

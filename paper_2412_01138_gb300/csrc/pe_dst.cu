@@ -1798,7 +1798,7 @@ pe_status fft_grid(const void* kern, int64_t npencils, size_t smem_per_warp, siz
   const int P = 2 * warps;
   // pair buffers, two offset lists, and (strided launches) the staged rows of one block
   const size_t smem = smem_per_warp * (size_t)warps + 2 * sizeof(int64_t) * P + stage_per_pencil * P;
-  if (smem > 48 * 1024) PE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PE_TRY(allow_smem(kern, smem));
   int per_sm = 0;
   PE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, smem));
   const int64_t nblk = (npencils + P - 1) / P;
@@ -1888,7 +1888,7 @@ pe_status fft_team_launch(const T* in, T* out, int n, int64_t inner, int64_t npe
   auto kern = dst_fft_team_kernel<T, LOGL, TW>;
   const size_t smem = sizeof(Cplx<T>) * (size_t)TEAMS * (PADL + 1) + 2 * sizeof(int64_t) * P +
                       (inner > 1 ? sizeof(T) * (size_t)P * n : 0);
-  if (smem > 48 * 1024) PE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PE_TRY(allow_smem((const void*)kern, smem));
   int dev = 0, sms = 0, per_sm = 0;
   PE_CUDA_TRY(cudaGetDevice(&dev));
   PE_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1905,14 +1905,6 @@ pe_status fft_team_launch(const T* in, T* out, int n, int64_t inner, int64_t npe
 template <typename TI, typename TO>
 pe_status fft512_contig_launch(const TI* in, TO* out, int64_t npencils, float scale, cudaStream_t st) {
   constexpr int PS = 512 + 512 / 16 + 1;
-  const size_t smem8 = sizeof(Cplx<float>) * 2 * PS * 8;
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [smem8] {
-    attr = cudaFuncSetAttribute(dst512_contig_kernel<TI, TO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem8);
-  });
-  if (attr != cudaSuccess) return pe_cuda_fail(attr, "dst: shared-memory attribute");
   const Cplx<float>* tw2 = pass_twiddles<float, kPlanTwo>(9, 16 * 32, st);
   if (!tw2) return pe_fail(PE_ECUDA, "dst: twiddle table allocation failed");
   int dev = 0, sms = 0, per_sm = 0;
@@ -1921,6 +1913,7 @@ pe_status fft512_contig_launch(const TI* in, TO* out, int64_t npencils, float sc
   const int64_t nquads = ((npencils + 1) / 2 + 1) / 2;
   const int warps = nquads < 8 * (int64_t)sms ? 1 : 8;
   const size_t smem = sizeof(Cplx<float>) * 2 * PS * warps;
+  PE_TRY(allow_smem((const void*)dst512_contig_kernel<TI, TO>, smem));
   PE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, dst512_contig_kernel<TI, TO>, 32 * warps, smem));
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((nquads + warps - 1) / warps,
                                                               (int64_t)sms * std::max(per_sm, 1)));
@@ -1936,13 +1929,7 @@ pe_status fft512_strided_launch_w(const TI* in, TO* out, int64_t inner, int64_t 
                                   cudaStream_t st) {
   constexpr int PS = 512 + 512 / 16 + 1, P = 4 * W;
   const size_t smem = sizeof(float) * 2 * 255 * (P + 2) + sizeof(Cplx<float>) * 2 * PS * W;
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [smem] {
-    attr = cudaFuncSetAttribute(dst512_strided_kernel<W, TI, TO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem);
-  });
-  if (attr != cudaSuccess) return pe_cuda_fail(attr, "dst: shared-memory attribute");
+  PE_TRY(allow_smem((const void*)dst512_strided_kernel<W, TI, TO>, smem));
   const Cplx<float>* tw2 = pass_twiddles<float, kPlanTwo>(9, 16 * 32, st);
   if (!tw2) return pe_fail(PE_ECUDA, "dst: twiddle table allocation failed");
   int dev = 0, sms = 0, per_sm = 0;
@@ -1972,12 +1959,7 @@ template <int W>
 pe_status fft1024_strided_w(const float* in, float* out, int64_t inner, int64_t npencils, float scale,
                             cudaStream_t st) {
   constexpr size_t smem = strided1024_smem<W>();
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(dst1024_strided_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  });
-  if (attr != cudaSuccess) return pe_cuda_fail(attr, "dst: shared-memory attribute");
+  PE_TRY(allow_smem((const void*)dst1024_strided_kernel<W>, smem));
   const Cplx<float>* tw2 = pass_twiddles<float, kPlanTwo>(10, 32 * 32, st);
   if (!tw2) return pe_fail(PE_ECUDA, "dst: twiddle table allocation failed");
   int dev = 0, sms = 0, per_sm = 0;
@@ -2094,9 +2076,7 @@ pe_status fft_axis(const T* in, T* out, int64_t outer, int n, int64_t inner, int
   int pairs = (int)(pairs64 < 1 ? 1 : (pairs64 > max_pairs ? max_pairs : pairs64));
   const int64_t want_ctas = (npencils + 2 * pairs - 1) / (2 * pairs);
   const size_t smem = sizeof(Cplx<T>) * ((size_t)pairs * L + L / 2);
-  if (smem > 48 * 1024) {
-    PE_CUDA_TRY(cudaFuncSetAttribute(dst_fft_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  }
+  PE_TRY(allow_smem((const void*)dst_fft_kernel<T>, smem));
   const T scale = (T)(0.5 * sqrt(2.0 / (double)(n + 1)));
   const int threads = L / 2 * pairs >= 256 ? 256 : (L / 2 * pairs >= 128 ? 128 : 64);
   PE_CUDA_TRY(launch_pdl(dst_fft_kernel<T>, dim3((unsigned)want_ctas), dim3(threads), smem, st, in, out, n, logL, inner,
@@ -2216,15 +2196,7 @@ template <typename T, int NP, bool FOLD>
 pe_status few_matrix_launch(const T* m, const T* in, T* out, int n, int64_t inner, int first, int np,
                             cudaStream_t st) {
   const size_t smem = FOLD ? sizeof(T) * (size_t)(n + 2) : 0;
-  if constexpr (FOLD) {
-    static std::once_flag once;
-    static cudaError_t attr = cudaSuccess;
-    std::call_once(once, [] {
-      attr = cudaFuncSetAttribute(few_matrix_kernel<T, NP, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)sizeof(T) * (16384 + 2));
-    });
-    if (attr != cudaSuccess) return pe_cuda_fail(attr, "dst: shared-memory attribute");
-  }
+  PE_TRY(allow_smem((const void*)few_matrix_kernel<T, NP, FOLD>, smem));
   const dim3 grid((unsigned)((n + 8 * kFewKO - 1) / (8 * kFewKO)), (unsigned)((np - first + NP - 1) / NP));
   few_matrix_kernel<T, NP, FOLD><<<grid, 256, smem, st>>>(m, in, out, n, inner, first, np);
   PE_CUDA_TRY(cudaGetLastError());
@@ -2574,9 +2546,7 @@ pe_status fft_axis_tw(const double* in, double* out, int64_t outer, int n, int64
   const int pairs = (int)(pairs64 < 1 ? 1 : (pairs64 > max_pairs ? max_pairs : pairs64));
   const int64_t ctas = (npencils + 2 * pairs - 1) / (2 * pairs);
   const size_t smem = sizeof(Cplx<double>) * ((size_t)pairs * L + L / 2);
-  if (smem > 48 * 1024)
-    PE_CUDA_TRY(cudaFuncSetAttribute(dst_fft_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
+  PE_TRY(allow_smem((const void*)dst_fft_kernel<double>, smem));
   const int threads = L / 2 * pairs >= 256 ? 256 : (L / 2 * pairs >= 128 ? 128 : 64);
   dst_fft_kernel<double><<<(unsigned)ctas, threads, smem, st>>>(in, out, n, logL, inner, npencils, pairs,
                                                                 0.5 * sqrt(2.0 / (double)(n + 1)), tw);

@@ -360,6 +360,10 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
+// Lets `kern` be launched with `bytes` of dynamic shared memory on the current device, whatever other threads and devices
+// of the process use it with: function attributes belong to a device, and the largest size asked for there stays set.
+pe_status allow_smem(const void* kern, size_t bytes);
+
 // Drops the cached set-up and output graphs of a repeated problem (pe_api.cu).
 void drop_solve_graphs(pe_ctx* c);
 // Drops the device-resident loop's graph (pe_api.cu); the next solve builds it anew.

@@ -23,7 +23,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <mutex>
 #include <vector>
 
 #include "pe_batch.h"
@@ -658,12 +657,7 @@ static pe_status run_train(pe_mlp* m, const float* x, const float* t, int n, int
   const int own_cap = (NPARAM_L + sms - 1) / sms + 1;
   const size_t smem = sizeof(TrainSmem) + 3 * sizeof(float) * (size_t)own_cap;
   if (smem > 200 * 1024) return pe_fail(PE_ECUDA, "pe_mlp: too few SMs for the training kernel");
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  });
-  if (attr != cudaSuccess) return pe_cuda_fail(attr, "pe_mlp: shared-memory attribute");
+  PE_TRY(allow_smem((const void*)train_kernel, smem));
   int per_sm = 0;
   PE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, train_kernel, TR_THREADS, smem));
   if (per_sm < 1) return pe_fail(PE_ECUDA, "pe_mlp: the training kernel does not fit an SM");

@@ -389,12 +389,7 @@ inline int64_t rup(int64_t a, int64_t b) { return (a + b - 1) / b * b; }
 
 template <int NSPLIT>
 pe_status tc_launch(const CUtensorMap& mB, const TcPass& P, dim3 grid, int* err, cudaStream_t st) {
-  static bool attr_set = false;  // the same value for every device and call
-  if (!attr_set) {
-    PE_CUDA_TRY(cudaFuncSetAttribute(tc_dst_kernel<NSPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     tc_smem_bytes<NSPLIT>()));
-    attr_set = true;
-  }
+  PE_TRY(allow_smem((const void*)tc_dst_kernel<NSPLIT>, tc_smem_bytes<NSPLIT>()));
   tc_dst_kernel<NSPLIT><<<grid, TC_THREADS, tc_smem_bytes<NSPLIT>(), st>>>(mB, P, err);
   PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;

@@ -74,7 +74,7 @@ struct Call {
 thread_local std::vector<Call> calls;
 cudaError_t launched(const void* f, cudaStream_t st, size_t smem) {
   if (slow) usleep(slow);
-  note("launch " + id(st) + " " + name_of(f) + " " + std::to_string(smem));
+  note("launch " + id(st) + " " + name_of(f) + " " + std::to_string(smem) + " " + std::to_string(current_device));
   return cudaSuccess;
 }
 }  // namespace

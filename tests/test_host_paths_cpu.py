@@ -326,3 +326,33 @@ def test_a_failing_set_up_leaves_nothing_running(rt, call, fails):
     for stream in used:
         last = max(i for i, l in enumerate(log) if l[0] in ("launch", "copy") and l[1] == stream)
         assert ["sync", stream] in log[last:]
+
+
+def test_shared_memory_limits_are_raised_on_every_device(rt):
+    """Function attributes belong to a device: kernels that take more than 48 KB have them raised on each one, and never
+    lowered where a call with less follows."""
+    from paper_2412_01138_gb300 import pe
+
+    def transforms():
+        for f32, n in ((0, (7000,)), (1, (13000,)), (0, (255, 255, 9)), (0, (1023, 700)), (1, (255, 255, 3)), (1, (511, 511)),
+                       (1, (511, 63, 500)), (1, (1023, 1023)), (0, (127, 127, 127)), (0, (511, 1023)), (0, (7000,))):
+            size = int(np.prod(n)) * (4 if f32 else 8)
+            a, b = rt.lib.fake_malloc(size), rt.lib.fake_malloc(size)
+            fn = rt.lib.pe_dst_f32 if f32 else rt.lib.pe_dst
+            assert fn(len(n), (C.c_int32 * len(n))(*n), a, b, None) == pe.PE_OK
+        net = pe.MLP()
+        x = np.zeros((64, 2), dtype=np.float32)
+        net.train(x, x, epochs=1, batch=32)
+        net.close()
+
+    for device in (0, 1):
+        rt.lib.fake_set_device(device)
+        transforms()
+    limit, big = {}, set()
+    for l in rt.log():
+        if l[0] == "attribute":
+            limit[l[1], l[2]] = int(l[3])
+        elif l[0] == "launch" and int(l[3]) > 48 * 1024:
+            big.add((l[4], l[2]))
+            assert limit.get((l[4], l[2]), 0) >= int(l[3]), l
+    assert len({k for d, k in big}) >= 5 and len(big) == 2 * len({k for d, k in big})

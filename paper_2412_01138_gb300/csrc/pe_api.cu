@@ -360,9 +360,12 @@ extern "C" pe_status pe_setup(pe_ctx** out, int32_t d, const int32_t* n, const d
   if (st == PE_OK && c->precision == PE_MIXED) st = dev_alloc(&c->coefF32, (size_t)(c->q + 2) * nd);
   if (st == PE_OK && c->precision == PE_MIXED) st = dev_alloc(&c->coefG32, (size_t)c->p * nd);
   if (st == PE_OK) st = dev_alloc(&c->U, (N + 1) * nd);
-  if (st == PE_OK) st = dev_alloc(&c->Fbar, N * nd);
+  // (the mixed separable form makes its forced parts inside the walk: only pe_refine stores some there, in a table
+  // it allocates)
+  const bool in_walk = c->precision == PE_MIXED && c->forcing_path == PE_FORCING_SEPARABLE;
+  if (st == PE_OK && !in_walk && !c->cache_forced) st = dev_alloc(&c->Fbar, N * nd);
   if (st == PE_OK && c->cache_forced) st = dev_alloc(&c->Fz, N * nd);
-  if (st == PE_OK) st = dev_alloc(&c->gG, N * nd);
+  if (st == PE_OK && !in_walk) st = dev_alloc(&c->gG, N * nd);
   if (st == PE_OK) st = dev_alloc(&c->work0, ndn + 64);
   if (st == PE_OK) st = dev_alloc(&c->work1, ndn + 64);
   // the mixed form transforms u0 and the solution in float32 (grids of at least 4096 nodes whose

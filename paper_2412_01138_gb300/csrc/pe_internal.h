@@ -143,8 +143,9 @@ struct pe_ctx {
   double* Fz = nullptr;         // [N * ndof] cached F^M(0) per slice (cache_forced)
   int fz_prec = -1;             // precision Fz was computed in, -1: none for this problem
   int64_t sweeps = 0;           // fine sweeps executed since the last reset
-  double* Fbar = nullptr;       // [N * ndof] F^M(0) of each slice (float64 and general sweeps)
-  double* gG = nullptr;         // [N * ndof] coarse forcing of each slice (float64 and general)
+  double* Fbar = nullptr;       // [N * ndof] F^M(0) of each slice (float64 and general sweeps; mixed separable: from
+                                // the first pe_refine on)
+  double* gG = nullptr;         // [N * ndof] coarse forcing of each slice (float64 and general; else null)
   double* work0 = nullptr;      // [gn.ndof] nodal / DST scratch
   double* work1 = nullptr;      // [gn.ndof]
   float* io32 = nullptr;        // [3 gn.ndof] float32 transform scratch of the mixed form (null: float64 transforms)

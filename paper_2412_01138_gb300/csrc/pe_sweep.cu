@@ -362,6 +362,12 @@ pe_status launch_iteration(pe_ctx* c, int precision, bool first, LoopCtl* loop, 
     }
     a.f = c->Fz;
   } else {
+    if (!c->Fbar && cudaMalloc((void**)&c->Fbar, sizeof(double) * (size_t)c->N * c->g.ndof) != cudaSuccess) {
+      cudaGetLastError();
+      c->Fbar = nullptr;
+      return pe_fail(PE_ENOMEM, "pe_refine: allocation of the forced parts failed");
+    }
+    a.f = c->Fbar;
     c->sweeps += 1;
     PE_TRY(forced_parts(c, precision, c->Fbar, first ? c->gG : nullptr));
   }

@@ -53,7 +53,7 @@ cudaError_t allocate(void** p, size_t bytes, const char* what) {
     *p = calloc(bytes ? bytes : 1, 1);
     device[*p] = bytes ? bytes : 1;
   }
-  note(std::string(what) + " " + id(*p));
+  note(std::string(what) + " " + id(*p) + " " + std::to_string(bytes));
   return cudaSuccess;
 }
 cudaError_t release(void* p) {

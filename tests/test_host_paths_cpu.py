@@ -356,3 +356,29 @@ def test_shared_memory_limits_are_raised_on_every_device(rt):
             big.add((l[4], l[2]))
             assert limit.get((l[4], l[2]), 0) >= int(l[3]), l
     assert len({k for d, k in big}) >= 5 and len(big) == 2 * len({k for d, k in big})
+
+
+@pytest.mark.parametrize("form,at_setup,by_refine", [("fp64", 2, 0), ("mixed", 0, 1), ("mixed_general", 2, 0),
+                                                     ("mixed_cached", 1, 0), ("fp64_cached", 2, 0)])
+def test_forced_parts_are_allocated_where_something_fills_them(rt, form, at_setup, by_refine):
+    """Arrays of a value per mode and slice beside the iterate: the forced parts of the fine and the coarse step (cached: of
+    the fine step, kept) where kernels store them; none in the mixed separable form until a refinement."""
+    from paper_2412_01138_gb300 import pe
+
+    prob = _prob(5, n=(37, 29), N=11)
+    size = str(8 * prob.N * prob.ndof)
+    kw = {"precision": int(form.startswith("mixed")), "cache_forced": form.endswith("cached")}
+    if form.endswith("general"):
+        kw["forcing_path"] = pe.PE_FORCING_GENERAL
+
+    def count():
+        return sum(l[0] == "malloc" and l[2] == size for l in rt.log())
+
+    with pe.Solver(prob, **kw) as s:
+        assert count() == at_setup
+        s.set_problem()
+        s.iterate()
+        assert count() == at_setup
+        s.refine()
+        s.refine()
+        assert count() == at_setup + by_refine

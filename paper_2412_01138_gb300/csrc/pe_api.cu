@@ -332,7 +332,6 @@ extern "C" pe_status pe_setup(pe_ctx** out, int32_t d, const int32_t* n, const d
   c->max_iter = o.max_iter == 0 ? n_slices : std::min(o.max_iter, n_slices);
   c->stream = (cudaStream_t)o.cuda_stream;
 
-  const int threads = 256;
   // modal arrays hold this context's modes (nd); nodal arrays and per-axis loads the whole grid
   const size_t N = (size_t)n_slices, nd = (size_t)c->g.ndof, ndn = (size_t)ndof, MT = PE_MAX_TERMS;
   const int nsl = c->nsum;

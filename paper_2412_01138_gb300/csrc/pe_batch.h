@@ -31,8 +31,7 @@ struct BProb {
   int64_t oCol;  // column map: K entries, (term << 1) | kind
   int64_t oFirst;  // first column of each term, R entries
   int64_t oMu;   // muM / ratio / rows: nsum
-  int64_t oItems;  // first mode item of this problem
-  int nItems;
+  int64_t oItems;  // first residual slot of this problem
   // learned coarse correction (pe_batch_set_learned): band table K^[r][band] (re, im) at oKt,
   // bands log-spaced in log(lam dT) from lloglo by lstep
   int64_t oKt;

@@ -229,14 +229,6 @@ struct pe_ctx {
   int capturing = 0;                // the phase being run is captured (timing events become graph nodes)
 };
 
-// Substeps of time factors (per_m values each) staged per shared-memory fill.
-inline int pick_mchunk(int M, int per_m, size_t elem) {
-  const size_t budget = 48 * 1024;
-  int mc = (int)(budget / (elem * (size_t)per_m));
-  if (mc < 1) mc = 1;
-  return mc < M ? mc : M;
-}
-
 // ---------------------------------------------------------------------------
 // launchers (each returns a pe_status and reports errors through pe_set_error)
 // ---------------------------------------------------------------------------

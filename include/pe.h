@@ -356,8 +356,8 @@ pe_status pe_dst_f32(int32_t d, const int32_t* n, const float* in, float* out, v
  * can synchronise the device).  The
  * paper has no counterpart: this is an interface variant, not a step of the method.
  * It calls no cudaMalloc, cudaFree or other allocating routine; its scratch (ping-pong
- * array, sine rows, FFT twiddles) is one file-scope device array of 1,835,008
- * doubles (about 14.7 MB) that every GPU loading the library holds until the process
+ * array, sine rows, FFT twiddles) is one file-scope device array of 1,054,720
+ * doubles (about 8.4 MB) that every GPU loading the library holds until the process
  * exits.  Limits: at most 1,048,576 values in total; an axis whose n+1 is not a power
  * of two must have n <= 512.  Larger sizes return PE_EINVAL with a message.
  * The first call on a device looks up the array's device address (cudaGetSymbolAddress)

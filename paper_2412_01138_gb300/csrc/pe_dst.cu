@@ -2506,13 +2506,14 @@ extern "C" pe_status pe_dst_f32(int32_t d, const int32_t* n, const float* in, fl
 // can synchronise the device).  This entry point keeps every scratch
 // buffer of the transform (the ping-pong array, the sine rows of axes without an FFT
 // length, the FFT twiddles) in one file-scope device array.  Every GPU that
-// loads the library holds that array (about 14.7 MB) until the process exits.
+// loads the library holds that array (about 8.4 MB) until the process exits.
 // ---------------------------------------------------------------------------
 namespace {
 
 constexpr int64_t kNoallocMaxNdof = (int64_t)1 << 20;     // ping-pong capacity (doubles)
 constexpr int kNoallocMaxMatrixN = 512;                   // axes on the matrix path
-constexpr int64_t kNoallocSlot = (int64_t)kNoallocMaxMatrixN * kNoallocMaxMatrixN;  // per axis
+constexpr int64_t kNoallocSlot = 2048;  // per axis: a row of n <= 512 sines, or 1024 twiddles of n + 1 <= 1024
+static_assert(kNoallocSlot >= kNoallocMaxMatrixN && kNoallocSlot >= 2 * 1024, "a slot holds either");
 constexpr int64_t kNoallocDoubles = kNoallocMaxNdof + PE_MAX_D * kNoallocSlot;
 
 static __device__ __align__(256) double g_dst_scratch[kNoallocDoubles];
@@ -2565,8 +2566,7 @@ extern "C" pe_status pe_dst_noalloc(int32_t d, const int32_t* n, const double* i
     if (n[a] < 1) return pe_fail(PE_EINVAL, "pe_dst_noalloc: n_a must be >= 1");
     fft[a] = fft_size_ok(n[a], &logL[a]);
     if (!fft[a] && n[a] > kNoallocMaxMatrixN)
-      return pe_fail(PE_EINVAL, "pe_dst_noalloc: an axis with n+1 not a power of two must have n <= 512 "
-                                "(its DST-I matrix must fit the built-in scratch array)");
+      return pe_fail(PE_EINVAL, "pe_dst_noalloc: an axis with n+1 not a power of two must have n <= 512");
     ndof *= n[a];
     if (ndof > kNoallocMaxNdof)
       return pe_fail(PE_EINVAL, "pe_dst_noalloc: at most 1048576 values (the built-in scratch array's capacity)");

@@ -127,7 +127,7 @@ struct pe_batch {
   int tune_threads = 128, tune_ctas = 4;
   cudaEvent_t ev[3] = {};          // timing of a solve
   cudaEvent_t ev_order = nullptr;  // between the caller's stream and the batch's
-  std::mutex fetch;                // one fetch at a time: it owns scratch and ev_order until it has waited
+  std::mutex fetch;                // one fetch at a time: it owns scratch until it has waited
   bool have_problem = false;
   int64_t launches = 0;
   uint64_t signature = 0;

@@ -389,8 +389,8 @@ float ms_between(cudaEvent_t a, cudaEvent_t b) {
 
 }  // namespace
 
-// What the caller's stream (the legacy default stream where the batch was given none) still has to do with a buffer or
-// a network it hands over comes before the work on the batch's own stream, which waits for no other by itself.
+// What the caller's stream (the legacy default stream where the batch was given none) still has to do with a network it
+// attached comes before the work on the batch's own stream, which waits for no other by itself.
 static pe_status after_caller(pe_batch* b) {
   PE_CUDA_TRY(cudaEventRecord(b->ev_order, b->user_stream));
   PE_CUDA_TRY(cudaStreamWaitEvent(b->stream, b->ev_order, 0));
@@ -557,11 +557,12 @@ extern "C" pe_status pe_batch_get_modal(pe_batch* b, int32_t problem, int32_t sl
   if (slice < 0 || slice > B.N) return pe_fail(PE_EINVAL, "pe_batch_get_modal: slice out of range");
   if (!b->have_problem) return pe_fail(PE_ESTATE, "pe_batch_get_modal: no solve has completed");
   const bool dev = pe_is_device_ptr(out);
-  std::lock_guard<std::mutex> lock(b->fetch);
-  PE_TRY(after_caller(b));
+  // fetches run on the caller's stream (the batch's own has nothing left to do after a solve): after whatever that
+  // still does with the buffer, without an event in between (1 us a fetch)
+  const cudaStream_t st = b->user_stream;
   PE_CUDA_TRY(cudaMemcpyAsync(out, b->U + B.oU + (int64_t)slice * B.g.ndof, sizeof(double) * B.g.ndof,
-                              dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, b->stream));
-  PE_CUDA_TRY(cudaStreamSynchronize(b->stream));
+                              dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
+  PE_CUDA_TRY(cudaStreamSynchronize(st));
   return PE_OK;
 }
 
@@ -576,14 +577,14 @@ extern "C" pe_status pe_batch_get_solution(pe_batch* b, int32_t problem, double*
   for (int a = 0; a < B.g.d; ++a) rows[a] = b->rows + B.oMu + B.g.off[a];
   const bool dev = pe_is_device_ptr(nodal_out);
   double* out = dev ? nodal_out : b->scratch + b->ndof_max;
+  const cudaStream_t stream = b->user_stream;  // (as in pe_batch_get_modal)
   std::lock_guard<std::mutex> lock(b->fetch);
-  PE_TRY(after_caller(b));
-  pe_status st = dst_rows_f64(B.g.d, n, rows, last, out, b->scratch, b->stream);
+  pe_status st = dst_rows_f64(B.g.d, n, rows, last, out, b->scratch, stream);
   if (st == PE_OK && !dev) {
-    cudaError_t e = cudaMemcpyAsync(nodal_out, out, sizeof(double) * B.g.ndof, cudaMemcpyDeviceToHost, b->stream);
+    cudaError_t e = cudaMemcpyAsync(nodal_out, out, sizeof(double) * B.g.ndof, cudaMemcpyDeviceToHost, stream);
     if (e != cudaSuccess) st = pe_cuda_fail(e, "pe_batch_get_solution");
   }
-  cudaError_t e = cudaStreamSynchronize(b->stream);
+  cudaError_t e = cudaStreamSynchronize(stream);
   if (st == PE_OK && e != cudaSuccess) st = pe_cuda_fail(e, "pe_batch_get_solution");
   return st;
 }

@@ -9,11 +9,9 @@
 
 #include <algorithm>
 #include <climits>
-#include <map>
 #include <mutex>
 #include <new>
 #include <string>
-#include <utility>
 
 #include "pe_contract.cuh"
 #include "pe_internal.h"
@@ -107,15 +105,23 @@ void pe_lagrange_coeffs(int s, const double* c, double a[PE_MAX_S][PE_MAX_S]) {
 
 pe_status allow_smem(const void* kern, size_t bytes) {
   if (bytes <= 40 * 1024) return PE_OK;  // (48 KB without asking, a kernel's static shared memory included)
-  static std::map<std::pair<const void*, int>, size_t> allowed;
+  struct Limit {
+    const void* kern;
+    int dev;
+    size_t bytes;
+  };
+  static Limit limits[512];  // (about thirty kernels a device)
+  static int used = 0;
   static std::mutex mu;
   int dev = 0;
   PE_CUDA_TRY(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lock(mu);
-  size_t& have = allowed[{kern, dev}];
-  if (bytes <= have) return PE_OK;
+  int i = 0;
+  while (i < used && !(limits[i].kern == kern && limits[i].dev == dev)) ++i;
+  if (i < used && bytes <= limits[i].bytes) return PE_OK;
   PE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-  have = bytes;
+  if (i < 512) limits[i] = Limit{kern, dev, bytes};
+  if (i == used && used < 512) ++used;
   return PE_OK;
 }
 

@@ -83,7 +83,8 @@ enum { PE_DST_AUTO = 0, PE_DST_MATRIX = 1, PE_DST_TC = 2 };
 enum { PE_S_ONE = 0, PE_S_SIN = 1, PE_S_GAUSS = 2, PE_S_POLY = 3, PE_S_MOVING_HAT = 4 };
 
 /* how P_h f(t) is formed (pe_options.forcing_path) */
-enum { PE_FORCING_SEPARABLE = 0, /* modal factors of every term once, products per mode and stage */
+enum { PE_FORCING_SEPARABLE = 0, /* modal factors of every term once; per mode a weight of every time column, and
+                                    per mode and slice the sum over the columns */
        PE_FORCING_GENERAL = 1    /* also terms with moving factors: at every stage time the consistent
                                     1D loads of their moving axes (element Gauss quadrature), the DST-I along
                                     those axes, division by Lambda_M; terms that do not move as above */ };
@@ -150,20 +151,21 @@ typedef struct {
   void (*residual_reduce)(double* sums, void* user);
   void* residual_reduce_user;
   /* 1: pe_solve runs Algorithm 1's loop on the device -- one CUDA graph whose conditional
-   * (while) node repeats {fine sweep, correction + residual} and whose correction kernel
-   * decides, from the float64 residual, whether to go on (r > tol and k < max_iter) -- so the
+   * (while) node repeats the iteration; its last kernel (fine step, correction and residual in
+   * one) decides, from the float64 residual, whether to go on (r > tol and k < max_iter), so the
    * host waits once per solve instead of once per iteration.  Same kernels and results as the
    * host-driven loop; per-kernel times (pe_result.ms_fine_kernel, ms_correction_kernel) are not
    * measured in this mode (0).  The graph is built at the first such solve of a column count K
-   * and reused.  Falls back to the host loop for cache_forced, the general forcing path and
-   * contexts with residual_reduce.  0 (default): the host-driven loop of the paper's Algorithm 1.
+   * and reused until K changes or more columns need larger weight tables.  Falls back to the
+   * host loop for cache_forced, the general forcing path and contexts with residual_reduce.
+   * 0 (default): the host-driven loop of the paper's Algorithm 1.
    * 2: as 1, and a problem solved again -- the same u0 description (or the same device pointer
    * of nodal u0: its values are read anew each solve), forcing terms, Dirichlet data and network
-   * pointer -- replays the set-up (transform of u0, forcing factors, stage weights, coarse
-   * sweep) and output (inverse transform, lifting) phases as CUDA graphs captured at its second
-   * solve, so that a solve costs a few graph launches.  Same kernels, same results.  Nodal u0 in
-   * host memory, or any pe_set_problem / pe_set_dirichlet / pe_set_learned call in between, runs
-   * the phases directly (and drops the graphs).  Other values: PE_EINVAL. */
+   * pointer -- replays the set-up (transform of u0, forcing factors, column weights) and output
+   * (inverse transform, lifting) phases as CUDA graphs captured at its second solve, so that a
+   * solve costs a few graph launches.  Same kernels, same results.  A solve of nodal u0 in host
+   * memory, or any pe_set_problem / pe_set_dirichlet / pe_set_learned call in between, runs the
+   * phases directly (and drops the graphs).  Other values: PE_EINVAL. */
   int32_t device_loop;
 } pe_options;
 
@@ -496,7 +498,7 @@ pe_status pe_dst_tc(int32_t d, const int32_t* n, const float* in, float* out, in
  * pe_measure_fma_peak -- FMA throughput of the CUDA cores in TFLOP/s (2 FLOP per FMA),
  * measured by a kernel of independent FMA chains (8 per thread, 2048 threads per SM), the
  * best of five timed launches after one warm-up: precision PE_FP64 for float64 FMAs,
- * PE_MIXED for float32 FMAs.  The ALU-bound fine kernels are quoted against it beside
+ * PE_MIXED for float32 FMAs.  The ALU-bound kernels are quoted against it beside
  * the peak derived from unit counts and the clock.  tflops_out: host.  Allocates 40 KB
  * with cudaMallocAsync on the stream for the duration of the call.
  */

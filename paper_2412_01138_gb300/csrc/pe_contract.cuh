@@ -33,13 +33,12 @@ __host__ __device__ inline int chain_steps(int M) {
   return s;
 }
 
-// Chain tables of one term: entry (s, e), e = 0..3: Re D, Im D, Re A, Im A of step s at
-// [(s * R + r) * 4 + e]; the float form holds (hi, lo) pairs of the same.
 // Step s of M (0 = the first doubling): the length before it, and whether one more is added.
 __host__ __device__ inline int chain_length(int M, int steps, int s) { return M >> (steps - s); }
 __host__ __device__ inline bool chain_adds(int M, int steps, int s) { return (M >> (steps - s - 1)) & 1; }
 
-// S_M for x (= E, or E e^{-a dt}), float64.  tab: the term's entries, `stride` doubles per step.
+// S_M for x (= E, or E e^{-a dt}), float64.  tab: the term's entries, `stride` doubles per step.  The tables hold Re D, Im D,
+// Re A, Im A of step s and term r at [(s * R + r) * 4 ..]; the float form (hi, lo) pairs of the same.
 __device__ __forceinline__ void chain_sum(double x, int M, int steps, const double* __restrict__ tab, int stride,
                                           double& Sr, double& Si) {
   double xL = x;

@@ -281,7 +281,8 @@ template <typename T, int RW, int CW>
 pe_status folded_launch(const T* row, const T* in, T* out, int n, int64_t inner, int64_t np, cudaStream_t st) {
   const dim3 grid((unsigned)((np + 32 * CW - 1) / (32 * CW)), (unsigned)((n + 8 * RW - 1) / (8 * RW)));
   // a plain launch: CTAs let in while the kernel before still runs pile up on the SMs that have room, and
-  // the busiest SM is the run time (two transforms of 405 x 279 in a solve: 706 us with an early launch, 538 without)
+  // the busiest SM is the run time (two transforms of 405 x 279 in a solve, more than a wave of CTAs each: 706 us with
+  // an early launch, 538 without; grids of less than a wave follow the same rule, unmeasured)
   folded_dst_kernel<T, RW, CW><<<grid, 128, 0, st>>>(row, in, out, n, inner, np);
   PE_CUDA_TRY(cudaGetLastError());
   return PE_OK;

@@ -88,7 +88,7 @@ struct ColumnTables {
   float *Y32, *ZF32, *ZG32, *chain32, *xs32;
 };
 // Device-resident state of a solve whose Parareal loop runs as a CUDA graph (device_loop):
-// the correction kernel's last CTA appends r_k, advances k and sets the graph's loop condition.
+// the walk's last CTA appends r_k, advances k and sets the graph's loop condition.
 struct LoopCtl {
   int k, max_iter, nonfinite, hist_cap;
   double tol, r;
@@ -199,7 +199,7 @@ struct pe_ctx {
   // accounting
   int64_t launches = 0;     // kernels launched since the last reset
   double ms_fine = 0.0;     // device time of fine-propagator kernels since the last reset
-  double ms_corr = 0.0;     // device time of correction kernels since the last reset
+  double ms_corr = 0.0;     // device time between the forced parts and the end of an iteration since the last reset
   // state
   int k = 0;
   bool have_problem = false;
@@ -312,11 +312,6 @@ inline int per_mode_block(int64_t units, int sms, int cap = 512) {
   return (int)(t < 64 ? 64 : t);
 }
 
-// Programmatic dependent launch: a kernel launched by launch_pdl may be scheduled while its
-// predecessor on the stream is still running.  Each such kernel calls pdl_wait() first, before
-// it touches global memory: it waits there until the predecessor has completed and its writes
-// are visible, then lets its own successor be scheduled early in turn.  Without the launch
-// attribute (a plain launch) both instructions do nothing.
 // Exact float32 -> float64 widening.  GB300 runs the F2F conversion on its float64 pipe (two
 // lanes per SM), where the recurrences that add a float32 sum into a float64 state already
 // spend their float64 budget; a normal float32 is widened here with integer operations instead
@@ -332,6 +327,12 @@ __device__ __forceinline__ double widen_f32(float x) {
   return widen_f32_rare(x);
 }
 
+// Programmatic dependent launch: a kernel launched by launch_pdl may be scheduled while its
+// predecessor on the stream is still running.  Each such kernel calls pdl_wait() before it touches
+// global memory that a kernel of the stream may have written (tables of the process, which were
+// waited for when they were made, may be read earlier): it waits there until the predecessor has completed
+// and its writes are visible, then lets its own successor be scheduled early in turn.  Without
+// the launch attribute (a plain launch) both instructions do nothing.
 __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

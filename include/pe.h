@@ -425,7 +425,10 @@ pe_status pe_batch_autotune(pe_batch* b, const char* cache_path);
  * until every problem has r <= tol or k = N.  res may be NULL. */
 pe_status pe_batch_solve(pe_batch* b, double tol, pe_batch_result* res);
 
-/* Per-problem modal U^{slice} / nodal u_h(T) (host or device out, Ndof of that problem). */
+/* Per-problem modal U^{slice} / nodal u_h(T) (host or device out, Ndof of that problem).  They run
+ * on the stream of pe_options.cuda_stream (NULL: the legacy default stream), after what was
+ * enqueued there before, and return when the values are in `out`.  Several threads may fetch
+ * from one batch. */
 pe_status pe_batch_get_modal(pe_batch* b, int32_t problem, int32_t slice, double* out);
 pe_status pe_batch_get_solution(pe_batch* b, int32_t problem, double* nodal_out);
 

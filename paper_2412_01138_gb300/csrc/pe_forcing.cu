@@ -619,8 +619,10 @@ static pe_status grow_weights(pe_ctx* c, T** W, int* cap) {
   const int K = c->K;
   if (K <= *cap) return PE_OK;
   PE_CUDA_TRY(cudaStreamSynchronize(c->stream));
-  drop_loop_graph(c);  // it was captured with the address given back here
-  if (*W) cudaFree(*W);
+  if (*W) {
+    drop_loop_graph(c);  // it was captured with the address given back here
+    cudaFree(*W);
+  }
   *W = nullptr;
   *cap = 0;
   if (cudaMalloc((void**)W, (size_t)K * (size_t)c->g.ndof * sizeof(T)) != cudaSuccess) {

@@ -387,3 +387,17 @@ def test_forced_parts_are_allocated_where_something_fills_them(rt, form, at_setu
         s.refine()
         s.refine()
         assert count() == at_setup + by_refine
+
+
+def test_loop_graph_is_kept_where_no_weights_were_given_back(rt):
+    """The float64 weights of a mixed context's first refinement are one more table: the loop graph stays."""
+    from paper_2412_01138_gb300 import pe
+
+    with pe.Solver(_prob(5), precision=1, device_loop=1) as s:
+        _solve(s)
+        s.set_problem()
+        s.refine()
+        rt.clear()
+        _solve(s)
+        log = rt.log()
+    assert any(l[0] == "exec_launch" for l in log) and not any(l[0] == "exec_new" for l in log)

@@ -548,8 +548,10 @@ pe_status setup_response_nodes(pe_ctx* c) {
 // its n-th derivative in lam is the weight times a mean of s^n, at most dT^n and, where lam > alpha, n! / (lam - alpha)^n.  With
 // n! >= (n/e)^n the interpolation error on an interval of width w lam, 2 (w lam / 4)^n max |H^(n)| / n!, is at most
 //   2 ((w lam / 4) min(e dT / n, 1 / (lam - alpha)))^n H,
-// largest where the two meet, lam = alpha + n / (e dT), or at the end of the spectrum next to it.  (160^2 modes, one
-// source, mixed: dT = 3, alpha = 30, lam_min = 20 gave 7e-5 in the solution by the table; float64 5e-11 on 208^2.)
+// largest where the two meet, lam = alpha + n / (e dT), or at the end of the spectrum next to it.  One source, lam_min about 20,
+// relative L2 by the table and directly: dT = 1.5, alpha = 30, 7.2e-5 and 9.1e-9 (mixed, 160^2 modes), 4.4e-11 and 4.3e-16
+// (float64, 208^2); dT = 3, alpha = 40, 3.4e-3 and 3.0e-8, 1.2e-8 and 2.2e-15; just inside the rule by the table: 1.0e-7 and
+// 4.0e-16.
 static bool response_exact(const pe_ctx* c, const pe_term& t) {
   if (t.tkind == PE_T_SIN || !(t.tp[0] < 0.0)) return true;
   const bool f32 = c->precision == PE_MIXED;
